@@ -29,6 +29,10 @@ def nvcc_path():
     raise RuntimeError("nvcc not found: the planner's CUDA library cannot be built")
 
 
+# -fmad=false: fused multiply-adds are written out (csrc/twa_math.cuh), so that
+# a factor rounds alike in every kernel that computes it
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     """Compile libplan.so unless it is newer than every source.  Returns its path."""
     os.makedirs(BUILD, exist_ok=True)
@@ -37,7 +41,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         if all(os.path.getmtime(d) <= t for d in DEPS):
             return LIB
     tmp = LIB + ".tmp"
-    cmd = [nvcc_path(), ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
+    cmd = [nvcc_path(), ARCH, "-O3", "-fmad=false", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
            "-shared", "-I", INCLUDE, "-I", CSRC, "-o", tmp, *SOURCES, *extra_flags]
     if verbose:
         print(" ".join(cmd), flush=True)

@@ -2,15 +2,17 @@
 // planner (Bento, Derbinsky, Alonso-Mora, Yedidia, NIPS 2013): workspace
 // layout, input checks, state reset / import / export, the residual, and the
 // per-iteration launch sequence.  The iteration's per-block work lives in
-// twa_iter.cuh; one iteration is three kernels on one stream:
+// twa_iter.cuh.  Gated state (default), two kernels per iteration on one
+// stream:
 //
-//   test_kernel      every collision factor: deferred u step, n = z - u,
-//                    collision test, activity bits, worklist of active pairs;
-//                    in the same launch, the kinetic factors and the wall
-//                    tests (worklist of active walls)
-//   prox_kernel      the minimizer of every active wall and pair, adding
-//                    m = x + u into exact fixed-point consensus sums
-//   consensus_kernel z = sum m / count per free break-point
+//   factor_kernel    every factor: deferred u step, n = z - u, test, and the
+//                    minimizer of the active ones, adding m = x + u into exact
+//                    fixed-point consensus sums
+//   node_kernel      z = sum m / count per free break-point
+//
+// Dense state, three: test_kernel (tests, with the kinetic, wall and velocity
+// factors whole), prox_kernel (the minimizer of every active pair) and
+// node_kernel.
 //
 // Iterations after the first are replayed from captured CUDA graphs.
 #include <cuda_runtime.h>
@@ -30,7 +32,7 @@
 
 namespace {
 
-// Programmatic dependent launch: the three kernels of an iteration are
+// Programmatic dependent launch: the kernels of an iteration are
 // launched with programmatic stream serialization, so each one's CTAs can be
 // scheduled while the previous kernel drains (every CTA lets its dependents
 // launch as soon as it starts); griddepcontrol.wait then holds them until the
@@ -41,63 +43,48 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// The single-planner kernels: thin wrappers over the per-block work.
+// The single-planner kernels: thin wrappers over the per-warp work.
 constexpr int TEST_WARPS = 4;
 constexpr int TEST_ROWS = TILE / TEST_WARPS;
 
-// Pass 1 is one launch: its first nseg = eta x (agent tiles) blocks take the
-// kinetic and wall factors of one (segment, agent tile) each (segment_block,
-// dispatched first), the rest the collision blocks.  Both kinds of work
-// depend only on z^k, so one launch replaces two streams and their join.
-template <bool DENSE>
-__global__ void __launch_bounds__(32 * TEST_WARPS, 8) test_kernel(Dev P, int nseg) {
-  pdl_begin();
-  if ((int)blockIdx.x < nseg) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) *P.res_cur = 0u;
-    segment_block<true>(P, blockIdx.x);
-    return;
-  }
-  test_block<DENSE, TEST_ROWS>(P, blockIdx.x - nseg);
-}
-
-// Gated state: one warp per tile, lane = row agent (test_tile_rows).  The
-// register cap keeps the collision blocks at their own count (48), which
-// sets the occupancy; the kinetic and wall blocks spill a little under it.
-constexpr int TILES_PER_CTA = 4;  // the batched test pass
-constexpr int ROWS_WARPS = 4;     // tiles (warps) per CTA of test_rows_kernel (2 and 8 measured slower)
-__global__ void __launch_bounds__(32 * ROWS_WARPS, 40 / ROWS_WARPS) test_rows_kernel(Dev P, int nseg) {
-  __shared__ float4 col[ROWS_WARPS][72];
-  __shared__ uint32_t nws[ROWS_WARPS][32];
+// Gated state, every factor in one launch.  The first CTAs take the worklist
+// (the longest chains: a minimizer each), then the kinetic, wall and velocity
+// warps, then the tiles.  A chunk of 32 list entries goes to the warp of the
+// same number, and consecutive warps sit on different CTAs, so a short list
+// spreads over the SMs.
+constexpr int FACTOR_WARPS = 4;
+template <bool CLASSES>
+__global__ void __launch_bounds__(32 * FACTOR_WARPS, 6) factor_kernel(Dev P, int list_ctas, int seg_ctas,
+                                                                     int seg_warps, int tile_warps) {
+  __shared__ TileMem mem[FACTOR_WARPS];
   pdl_begin();
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.res_cur = 0u;
-  if ((int)blockIdx.x < nseg) {
-    segment_block<true>(P, blockIdx.x);
+  const int warp = threadIdx.x >> 5, nlist = list_ctas * FACTOR_WARPS;
+  int b = (int)blockIdx.x, item = warp * list_ctas + b;
+  if (b >= list_ctas) {
+    b -= list_ctas;
+    if (b < seg_ctas) {
+      if (b * FACTOR_WARPS + warp < seg_warps) segment_warp(P, b * FACTOR_WARPS + warp);
+      return;
+    }
+    item = (b - seg_ctas) * FACTOR_WARPS + warp;
+    if (item >= tile_warps) return;  // warp-uniform
+    item += nlist;
+  }
+  collision_warp<CLASSES>(P, item, nlist, mem + warp);
+}
+
+// Dense state, pass 1: the first CTAs take the kinetic, wall and velocity
+// warps, the rest a collision tile each.
+__global__ void __launch_bounds__(32 * TEST_WARPS, 8) test_kernel(Dev P, int seg_ctas, int seg_warps) {
+  pdl_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *P.res_cur = 0u;
+  if ((int)blockIdx.x < seg_ctas) {
+    const int w = (int)blockIdx.x * TEST_WARPS + (threadIdx.x >> 5);
+    if (w < seg_warps) segment_warp(P, w);
     return;
   }
-  const int warp = threadIdx.x >> 5;
-  // the first hcap warps take the tiles listed heavy by the previous
-  // iteration; the others go through every tile segment-minor (t -> segment
-  // t mod eta, so that a crowded segment spreads over the launch), skipping
-  // the listed ones
-  const int t = ((int)blockIdx.x - nseg) * ROWS_WARPS + warp;
-  int blk;
-  bool check_stamp = false;
-  if (t < P.hcap) {
-    // the list's length and this warp's entry are loaded together (t < hcap
-    // keeps the entry in bounds; it is used only below the length)
-    const unsigned hc = ld_now(P.hcount_cur);
-    const unsigned hb = ld_now(P.heavy_cur + t);
-    if (t >= (int)hc) return;  // warp-uniform
-    blk = (int)hb;
-  } else {
-    const int tr = t - P.hcap;
-    if (tr >= P.eta * P.ntp) return;  // warp-uniform
-    const int s = tr % P.eta;
-    if (P.vo && s != 0) return;  // no collision factors on the second segment
-    blk = s * P.ntp + tr / P.eta;
-    check_stamp = P.hcap != 0;  // skipped there if a heavy warp takes it
-  }
-  test_tile_rows(P, blk, col[warp], nws[warp], check_stamp);
+  test_block<TEST_ROWS>(P, blockIdx.x - seg_ctas);
 }
 
 // Worklist items are dealt to warps round-robin (item t to warp t mod W,
@@ -110,61 +97,32 @@ __device__ __forceinline__ unsigned long long dealt_first(unsigned long long& st
   return (unsigned long long)(threadIdx.x & 31) * W + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
 }
 
-// Pass 2: every active wall's minimizer on a warp of its own (all lanes
-// cooperating), the first warp of each of the first n_wall CTAs, so that
-// these long chains sit on different SMs.  The collision minimizers go in
-// groups of 32 consecutive worklist entries (pairs of one tile, so of one
-// segment: the lanes take the same branches) to the other warps, ordered so
-// that consecutive groups land on different CTAs and so spread over the SMs.
-// (More active walls than CTAs: walls over all warps, then pairs.)
+// Dense state, pass 2: groups of 32 consecutive worklist entries (pairs of
+// one tile, so of one segment: the lanes take the same branches), consecutive
+// groups on different CTAs, so that they spread over the SMs.
 __global__ void __launch_bounds__(256) prox_kernel(Dev P) {
   pdl_begin();
-  const unsigned long long nc = *P.work_count, nwl = *P.wwork_count;
-  const unsigned long long wpb = blockDim.x >> 5, G = gridDim.x, b = blockIdx.x;
-  const unsigned long long wib = threadIdx.x >> 5;
-  const unsigned lane = threadIdx.x & 31;
-  unsigned long long v, Wc;  // this warp's place among the collision warps, their number
-  // The wall items of this warp: first, first + stride, ... below nwl.  Both
-  // dealings go through this one call of the wall minimizer: with two call
-  // sites the compiler inlined two copies whose floating-point contractions
-  // differed, so the result of a wall factor depended on whether the active
-  // walls outnumbered the CTAs (that is, on the GPU's SM count).
-  unsigned long long first, stride;
-  bool wall_only;
-  if (nwl <= G) {
-    wall_only = b < nwl && wib == 0;
-    first = wall_only ? b : nwl;
-    stride = G;
-    Wc = G * wpb - nwl;
-    v = wib == 0 ? b - nwl : (G - nwl) + (wib - 1) * G + b;
-  } else {
-    wall_only = false;
-    first = b * wpb + wib;
-    stride = G * wpb;
-    Wc = G * wpb;
-    v = wib * G + b;
-  }
-  for (unsigned long long t = first; t < nwl; t += stride) wall_prox_item_warp(P, P.wwork[t]);
-  if (wall_only) return;
-  for (unsigned long long t = 32ull * v + lane; t < nc; t += 32ull * Wc) prox_item(P, P.work[t]);
+  const unsigned long long nc = *P.work_count, G = gridDim.x, wpb = blockDim.x >> 5;
+  const unsigned long long v = (threadIdx.x >> 5) * G + blockIdx.x;
+  for (unsigned long long t = 32ull * v + (threadIdx.x & 31); t < nc; t += 32ull * G * wpb) prox_item(P, P.work[t]);
 }
 
-__global__ void consensus_kernel(Dev P) {
+constexpr int NODE_WARPS = 2;
+__global__ void __launch_bounds__(32 * NODE_WARPS) node_kernel(Dev P) {
   pdl_begin();
-  const int nfree = (P.eta - 1) * P.p;
+  const int warp = (int)blockIdx.x * NODE_WARPS + (threadIdx.x >> 5);
+  if (blockIdx.x == 0 && threadIdx.x == 0) advance_worklist(P, false);
+  consensus_warp(P, warp);
+}
+
+// The segment records of the factor pass after z, a fixed end or a radius was
+// changed by something else than an iteration.
+__global__ void segments_kernel(Dev P) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *P.work_count_next = 0u;
-    *P.wwork_count_next = 0u;
-    if (P.hcap) {
-      *P.hcount_cur = 0u;  // read by this iteration's pass 1; the next-but-one builds into it
-      *P.iter += 1u;
-    }
-  }
-  float dz = 0.f;
-  bool bad = false;
-  if (t < nfree) consensus_node(P, t, dz, bad);
-  consensus_reduce(P, dz, bad);
+  if (t >= P.p * P.eta) return;
+  const int s = t / P.p, i = t - s * P.p;
+  const size_t node = (size_t)i * (P.eta + 1) + s;
+  store_segment(P, i, s, P.z[node], P.z[node + 1]);
 }
 
 // Fixed-point scale of the consensus sums: the largest power of two with
@@ -217,11 +175,11 @@ __global__ void fix_kernel(Dev P, const float2* start, const float2* goal) {
 
 // Squared distance from the origin to the segment a -> b.
 __device__ __forceinline__ double origin_seg_dist2(double ax, double ay, double bx, double by) {
-  const double dx = bx - ax, dy = by - ay, dd = dx * dx + dy * dy;
-  double t = dd > 0.0 ? -(ax * dx + ay * dy) / dd : 0.0;
+  const double dx = bx - ax, dy = by - ay, dd = fma(dx, dx, dy * dy);
+  double t = dd > 0.0 ? -fma(ax, dx, ay * dy) / dd : 0.0;
   t = fmin(1.0, fmax(0.0, t));
-  const double cx = ax + t * dx, cy = ay + t * dy;
-  return cx * cx + cy * cy;
+  const double cx = fma(t, dx, ax), cy = fma(t, dy, ay);
+  return fma(cx, cx, cy * cy);
 }
 
 __device__ __forceinline__ void block_min_u64(unsigned long long v, unsigned long long* out) {
@@ -285,10 +243,10 @@ __global__ void check_walls_kernel(Dev P, int nseg, unsigned long long* out) {
     const float2 a = P.z[(size_t)i * E1 + s], b = P.z[(size_t)i * E1 + s + 1];
     const double ax = a.x, ay = a.y, bx = b.x, by = b.y;
     const double cx = W.x, cy = W.y, dx = W.z, dy = W.w;
-    const double o1 = (dx - cx) * (ay - cy) - (dy - cy) * (ax - cx);
-    const double o2 = (dx - cx) * (by - cy) - (dy - cy) * (bx - cx);
-    const double o3 = (bx - ax) * (cy - ay) - (by - ay) * (cx - ax);
-    const double o4 = (bx - ax) * (dy - ay) - (by - ay) * (dx - ax);
+    const double o1 = fma(dx - cx, ay - cy, -((dy - cy) * (ax - cx)));
+    const double o2 = fma(dx - cx, by - cy, -((dy - cy) * (bx - cx)));
+    const double o3 = fma(bx - ax, cy - ay, -((by - ay) * (cx - ax)));
+    const double o4 = fma(bx - ax, dy - ay, -((by - ay) * (dx - ax)));
     double d2;
     if (((o1 > 0.0 && o2 < 0.0) || (o1 < 0.0 && o2 > 0.0)) &&
         ((o3 > 0.0 && o4 < 0.0) || (o3 < 0.0 && o4 > 0.0))) {
@@ -317,7 +275,7 @@ __global__ void check_cost_kernel(Dev P, const double* ccost, const float2* star
     if (s >= s_lo && s < s_hi) {
       const float2 a = P.z[(size_t)i * E1 + s], b = P.z[(size_t)i * E1 + s + 1];
       const double dx = (double)b.x - (double)a.x, dy = (double)b.y - (double)a.y;
-      c += ccost[t] * (dx * dx + dy * dy);
+      c = fma(ccost[t], fma(dx, dx, dy * dy), c);
     }
   }
   for (int i = threadIdx.x; i < P.p; i += blockDim.x) {
@@ -352,44 +310,31 @@ __global__ void residual_kernel(Dev P) {
   const int nwarps = (gridDim.x * blockDim.x) >> 5;
   const int E1 = P.eta + 1;
   const size_t nrows = (size_t)P.eta * P.ntp * TILE;
-  for (size_t row = gw; row < nrows; row += nwarps) {
-    uint32_t word = P.bits[row];
-    if (P.admm && !((word >> lane) & 1u)) {
-      // standard ADMM: a feasible pair's x is z^{k-1} - u^{k-1}
-      const size_t blk = row / TILE;
-      const int r = (int)(row - blk * TILE);
-      const int s = (int)(blk / P.ntp);
-      const int2 IJ = P.tiles[blk - (size_t)s * P.ntp];
-      const int i = IJ.x * TILE + r, j = IJ.y * TILE + lane;
-      if (i >= P.p || j >= P.p || (IJ.x == IJ.y && r >= lane)) continue;
-      const size_t fid = row * TILE + lane;
-      const float4 a = P.ulo[fid], b = P.uhi[fid];
-      if (s != 0) {
-        finish_u_feasible(false, lo2(a), P.z_next[(size_t)i * E1 + s], P.z[(size_t)i * E1 + s], P.alpha, res);
-        finish_u_feasible(false, hi2(a), P.z_next[(size_t)j * E1 + s], P.z[(size_t)j * E1 + s], P.alpha, res);
-      }
-      if (s != P.eta - 1) {
-        finish_u_feasible(false, lo2(b), P.z_next[(size_t)i * E1 + s + 1], P.z[(size_t)i * E1 + s + 1], P.alpha, res);
-        finish_u_feasible(false, hi2(b), P.z_next[(size_t)j * E1 + s + 1], P.z[(size_t)j * E1 + s + 1], P.alpha, res);
-      }
-      continue;
-    }
-    if (!((word >> lane) & 1u)) continue;
+  // the pair in column c of a row: active (x pending) or, in standard ADMM,
+  // feasible (x is z^{k-1} - u^{k-1})
+  auto pair = [&](size_t row, int c, bool active) {
     const size_t blk = row / TILE;
     const int r = (int)(row - blk * TILE);
     const int s = (int)(blk / P.ntp);
     const int2 IJ = P.tiles[blk - (size_t)s * P.ntp];
-    const int i = IJ.x * TILE + r, j = IJ.y * TILE + lane;
-    const size_t fid = row * TILE + lane;
-    float4 xl = P.xlo[fid], xh = P.xhi[fid];
+    const int i = IJ.x * TILE + r, j = IJ.y * TILE + c;
+    if (i >= P.p || j >= P.p || (IJ.x == IJ.y && r >= c)) return;
+    const size_t fid = row * TILE + c, ni = (size_t)i * E1 + s, nj = (size_t)j * E1 + s;
+    const float4 a = active ? P.xlo[fid] : P.ulo[fid], b = active ? P.xhi[fid] : P.uhi[fid];
     if (s != 0) {
-      res = fmaxf(res, maxabs2(lo2(xl) - P.z[(size_t)i * E1 + s]));
-      res = fmaxf(res, maxabs2(hi2(xl) - P.z[(size_t)j * E1 + s]));
+      const float2 xi = active ? lo2(a) : P.z_next[ni] - lo2(a), xj = active ? hi2(a) : P.z_next[nj] - hi2(a);
+      res = fmaxf(res, fmaxf(maxabs2(xi - P.z[ni]), maxabs2(xj - P.z[nj])));
     }
     if (s != P.eta - 1) {
-      res = fmaxf(res, maxabs2(lo2(xh) - P.z[(size_t)i * E1 + s + 1]));
-      res = fmaxf(res, maxabs2(hi2(xh) - P.z[(size_t)j * E1 + s + 1]));
+      const float2 xi = active ? lo2(b) : P.z_next[ni + 1] - lo2(b), xj = active ? hi2(b) : P.z_next[nj + 1] - hi2(b);
+      res = fmaxf(res, fmaxf(maxabs2(xi - P.z[ni + 1]), maxabs2(xj - P.z[nj + 1])));
     }
+  };
+  if (P.admm) {  // every pair: a warp per row
+    for (size_t row = gw; row < nrows; row += nwarps) pair(row, lane, (P.bits[row] >> lane) & 1u);
+  } else {  // the few active ones: a lane per row
+    for (size_t row = (size_t)gw * 32 + lane; row < nrows; row += (size_t)nwarps * 32)
+      for (uint32_t w = P.bits[row]; w; w &= w - 1u) pair(row, __ffs(w) - 1, true);
   }
   const int gt = blockIdx.x * blockDim.x + threadIdx.x;
   const int nth = gridDim.x * blockDim.x;
@@ -421,24 +366,50 @@ __global__ void residual_kernel(Dev P) {
   if (lane == 0 && res > 0.f) atomic_max_nonneg(P.res_prev, res);
 }
 
-// Initial state (Section 4): z = start except the goal node; u = 0; the
-// kinetic pending x equals z so that the first finishing step gives u = 0.
-__global__ void reset_kernel(Dev P, float2* z0, float2* z1, const float2* start,
-                             const float2* goal) {
+// Initial state (Section 4): z = start except the goal node; u = 0 (the gated
+// state's records are read only where a bit is set); the kinetic pending x
+// equals z so that the first finishing step gives u = 0.  One launch for all
+// of it (fourteen memsets and two kernels cost 30 us of launches): block 0
+// derives the fixed-point scale, the others clear and fill.
+__global__ void __launch_bounds__(256) reset_kernel(Dev P, float2* z0, float2* z1, const float2* start,
+                                                    const float2* goal, unsigned* res, unsigned* wcount,
+                                                    unsigned long long* ekey) {
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < 4) { res[threadIdx.x] = 0u; wcount[threadIdx.x] = 0u; P.ctl[threadIdx.x] = 0u; }
+    if (threadIdx.x == 4) *P.status = 0u;
+    // plan_set_endpoints' words: no violation, extent 0, no fix-up block done
+    if (threadIdx.x == 5) { ekey[0] = ~0ull; ekey[1] = 0ull; ekey[2] = 0ull; }
+    fix_block(P, start, goal);
+    return;
+  }
+  const size_t t0 = (size_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x, nt = (size_t)(gridDim.x - 1) * blockDim.x;
   const int E1 = P.eta + 1;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < P.p * E1) {
-    const int i = t / E1, s = t - i * E1;
-    float2 v = (s == P.eta) ? goal[i] : start[i];
+  const size_t nodes = (size_t)P.p * E1, nkin = (size_t)P.eta * P.p;
+  const size_t nwords = (size_t)P.eta * P.ntp * TILE, nwb = (size_t)(P.nw + P.nv) * P.eta * P.nt;
+  uint4* b4 = reinterpret_cast<uint4*>(P.bits);
+  uint4* l4 = reinterpret_cast<uint4*>(P.listed);
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t t = t0; t < nwords / 4; t += nt) {
+    b4[t] = zero;
+    if (!P.dense) l4[t] = zero;
+  }
+  for (size_t t = t0; t < nwb; t += nt) P.wbits[t] = 0u;
+  for (size_t t = t0; t < nodes; t += nt) {
+    const int i = (int)(t / E1), s = (int)(t - (size_t)i * E1);
+    const float2 v = (s == P.eta) ? goal[i] : start[i];
     z0[t] = v;
     z1[t] = v;
+    P.wnode[t] = 1;
+    P.accx[t] = 0ull;
+    P.accy[t] = 0ull;
+    P.accc[t] = 0u;
   }
-  if (t < P.eta * P.p) {
-    const int s = t / P.p, i = t - s * P.p;
-    float2 zl = start[i];
-    float2 zh = (s + 1 == P.eta) ? goal[i] : start[i];
+  for (size_t t = t0; t < nkin; t += nt) {
+    const int s = (int)(t / P.p), i = (int)(t - (size_t)s * P.p);
+    const float2 zl = start[i], zh = (s + 1 == P.eta) ? goal[i] : start[i];
     P.xkin[t] = pack(zl, zh);
     P.ukin[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!P.dense) store_segment(P, i, s, zl, zh);
   }
 }
 
@@ -626,6 +597,13 @@ __global__ void __launch_bounds__(256) endpoint_update_kernel(Dev P, const float
       start[i] = a; goal[i] = b;
       z0[i * E1] = a; P.z_next[i * E1] = a;
       z0[i * E1 + P.eta] = b; P.z_next[i * E1 + P.eta] = b;
+      if (!P.dense) {  // the segment records at the fixed ends
+        const int last = P.eta - 1;
+        const float2 zh = last ? hi2(P.zseg[i]) : b;
+        const float2 zl = last ? lo2(P.zseg[(size_t)last * p + i]) : a;
+        store_segment(P, i, 0, a, zh);
+        if (last) store_segment(P, i, last, zl, b);
+      }
     }
   }
 }
@@ -951,9 +929,12 @@ constexpr size_t kDeviceEndpointCheck = 8192;
 
 struct Layout {
   size_t z0, z1, start, goal, radius, cost, walls, vlim, wnode, tiles;
-  size_t ulo, uhi, xlo, xhi, bits, ukin, xkin, uwall, xwall, wbits, work, wwork, wcount, sched,
-      stamps, heavy, accx, accy, accc, fix,
+  size_t ulo, uhi, xlo, xhi, bits, ukin, xkin, uwall, xwall, wbits, work, wcount, ctl,
+      accx, accy, accc, fix,
       res, status, count, ccost, chk, ekey, eshadow;
+  // inside the worklist's space (gated state): its capacity, and what takes
+  // the space behind it
+  size_t cap, listed, zseg, circ;
   size_t total;
 };
 
@@ -965,9 +946,6 @@ bool sizes_ok(const plan_config* c) {
   if ((unsigned long long)c->eta * ntp * TILE * TILE > 0xffffffffull) return false;
   return true;
 }
-
-// Heavy-tile slots at the front of pass 1: an eighth of the tiles.
-size_t heavy_cap(size_t ntiles) { return std::max<size_t>(32, ntiles / 8); }
 
 Layout layout_for(const plan_config* c) {
   const size_t p = c->p, eta = c->eta, nw = c->n_walls;
@@ -998,12 +976,17 @@ Layout layout_for(const plan_config* c) {
   L.uwall = take(ng * eta * p * 16);
   L.xwall = take(ng * eta * p * 16);
   L.wbits = take(ng * eta * nt * 4);
+  // the dense state's worklist may need every slot; the gated state's is only
+  // an order of work (it is rebuilt when it runs out), so the pairs-on-it
+  // words and the segment records share its space
   L.work = take(slots * 4);
-  L.wwork = take(nw * eta * p * 4);
-  L.wcount = take(4 * 4);  // collision and wall worklist counters, by iteration parity
-  L.sched = take(4 * 4);   // iteration number, heavy-tile counts by parity
-  L.stamps = take(2 * eta * ntp * 4);
-  L.heavy = take(2 * heavy_cap(eta * ntp) * 4);
+  L.circ = L.work + slots * 4 - p * eta * 16;
+  L.zseg = L.circ - p * eta * 16;
+  L.listed = L.zseg - slots / 8;
+  // a list entry holds a 31-bit slot
+  L.cap = slots <= 0x80000000ull ? (L.listed - L.work) / 4 : 0;
+  L.wcount = take(4 * 4);  // worklist length by iteration parity
+  L.ctl = take(4 * 4);     // worklist mode (Dev::ctl)
   L.accx = take(p * (eta + 1) * 8);
   L.accy = take(p * (eta + 1) * 8);
   L.accc = take(p * (eta + 1) * 4);
@@ -1161,7 +1144,8 @@ struct plan_s {
   bool own_ws;
   int k;
   int cur;  // which z buffer holds z^k
-  int prox_grid = 0;  // CTAs of the minimizer pass (resident CTAs per SM x SMs)
+  int sms = 0;        // SMs of the device
+  int prox_grid = 0;  // CTAs of the dense state's minimizer pass (resident CTAs per SM x SMs)
   cudaStream_t cap = nullptr;    // private stream for capturing the iteration graphs
   bool profiling = false;        // plan_profile: per-kernel event timing
   cudaEvent_t pev[6] = {};
@@ -1231,23 +1215,13 @@ struct plan_s {
     P.uwall = at<float4>(L.uwall); P.xwall = at<float4>(L.xwall);
     P.wbits = at<uint32_t>(L.wbits);
     P.work = at<uint32_t>(L.work);
+    P.cap = (unsigned)L.cap;
+    P.listed = at<uint32_t>(L.listed);
+    P.zseg = at<float4>(L.zseg);
+    P.circ = at<float4>(L.circ);
     P.work_count = at<unsigned>(L.wcount) + (kk & 1);
-    P.work_count_next = at<unsigned>(L.wcount) + ((kk + 1) & 1);
-    P.wwork = at<uint32_t>(L.wwork);
-    P.wwork_count = at<unsigned>(L.wcount) + 2 + (kk & 1);
-    P.wwork_count_next = at<unsigned>(L.wcount) + 2 + ((kk + 1) & 1);
-    {
-      const size_t cap = heavy_cap((size_t)eta * ntp);
-      P.hcap = (int)cap;
-      P.iter = at<unsigned>(L.sched);
-      P.hcount_cur = at<unsigned>(L.sched) + 1 + (kk & 1);
-      P.hcount_next = at<unsigned>(L.sched) + 1 + ((kk + 1) & 1);
-      P.heavy_cur = at<uint32_t>(L.heavy) + (kk & 1) * cap;
-      P.heavy_next = at<uint32_t>(L.heavy) + ((kk + 1) & 1) * cap;
-      const size_t ntiles = (size_t)eta * ntp;
-      P.stamp_cur = at<unsigned>(L.stamps) + (kk & 1) * ntiles;
-      P.stamp_next = at<unsigned>(L.stamps) + ((kk + 1) & 1) * ntiles;
-    }
+    P.work_count_prev = at<unsigned>(L.wcount) + ((kk + 1) & 1);
+    P.ctl = at<unsigned>(L.ctl);
     P.accx = at<unsigned long long>(L.accx);
     P.accy = at<unsigned long long>(L.accy);
     P.accc = at<unsigned>(L.accc);
@@ -1275,6 +1249,25 @@ cudaError_t clear_sums(plan_t h) {
   return e;
 }
 
+// The gated state's records after a change of z, the fixed ends or the radii
+// from outside an iteration.
+plan_status refresh_segments(plan_t h) {
+  Dev P = h->dev(h->k);
+  if (P.dense) return PLAN_OK;
+  const int n = h->p * h->eta;
+  segments_kernel<<<(n + 255) / 256, 256, 0, h->stream>>>(P);
+  CK(cudaGetLastError());
+  return PLAN_OK;
+}
+
+// No worklist: the next iteration builds it from the activity bits.
+plan_status drop_worklist(plan_t h) {
+  CK(cudaMemsetAsync(h->at<void>(h->L.wcount), 0, 16, h->stream));
+  CK(cudaMemsetAsync(h->at<void>(h->L.ctl), 0, 16, h->stream));
+  CK(cudaMemsetAsync(h->at<void>(h->L.ctl), 1, 1, h->stream));  // ctl[0] = 1 (rebuild)
+  return PLAN_OK;
+}
+
 plan_status ensure_prox_grid(plan_t h) {
   if (h->prox_grid == 0) {
     int dev = 0, sms = 0, nb = 0;
@@ -1282,6 +1275,7 @@ plan_status ensure_prox_grid(plan_t h) {
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, prox_kernel, 256, 0));
     h->prox_grid = std::max(1, sms * std::max(nb, 1));
+    h->sms = sms;
   }
   return PLAN_OK;
 }
@@ -1303,32 +1297,45 @@ cudaError_t launch_pdl(void (*kern)(Args...), unsigned grid, unsigned block, cud
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// Segment warps and list warps of a problem's factor pass.  List warps: one
+// per 32 pairs up to two CTAs' worth per SM; longer lists go round.
+int segment_warps(const plan_s* h) { return (1 + h->nw + h->nv) * h->eta * h->nt; }
+int list_ctas(const plan_s* h) {
+  const long long pairs = (long long)(h->vo ? 1 : h->eta) * h->p * (h->p - 1) / 2;
+  return (int)std::max<long long>(1, std::min<long long>((pairs + 32 * FACTOR_WARPS - 1) / (32 * FACTOR_WARPS), 2ll * h->sms));
+}
+
 // Enqueue the kernels of iteration h->k (no state change on the host).
 plan_status enqueue_iteration(plan_t h, cudaStream_t ms) {
   Dev P = h->dev(h->k);
-  const unsigned grid = (unsigned)((size_t)h->eta * h->ntp);
-  const int nseg = h->eta * h->nt;  // kinetic and wall blocks, ahead of the collision blocks
+  const int segw = segment_warps(h);
   const bool prof = h->profiling;
   if (prof) CK(cudaEventRecord(h->pev[0], ms));
-  if (P.dense)
-    CK(launch_pdl(test_kernel<true>, nseg + grid, 32 * TEST_WARPS, ms, P, nseg));
-  else
-    CK(launch_pdl(test_rows_kernel, nseg + (P.hcap + grid + ROWS_WARPS - 1) / ROWS_WARPS,
-                  32 * ROWS_WARPS, ms, P, nseg));
-  if (prof) CK(cudaEventRecord(h->pev[1], ms));
-  CK(launch_pdl(prox_kernel, h->prox_grid, 256, ms, P));
+  if (P.dense) {
+    const int segc = (segw + TEST_WARPS - 1) / TEST_WARPS;
+    CK(launch_pdl(test_kernel, (unsigned)(segc + (size_t)h->eta * h->ntp), 32u * TEST_WARPS, ms, P, segc, segw));
+    if (prof) CK(cudaEventRecord(h->pev[1], ms));
+    CK(launch_pdl(prox_kernel, (unsigned)h->prox_grid, 256u, ms, P));
+  } else {
+    const int lc = list_ctas(h), segc = (segw + FACTOR_WARPS - 1) / FACTOR_WARPS;
+    const int tiles = (h->vo ? 1 : h->eta) * h->ntp;
+    const unsigned grid = (unsigned)(lc + segc + (tiles + FACTOR_WARPS - 1) / FACTOR_WARPS);
+    CK(launch_pdl(h->noenergy ? factor_kernel<true> : factor_kernel<false>, grid, 32u * FACTOR_WARPS, ms, P, lc,
+                  segc, segw, tiles));
+    if (prof) CK(cudaEventRecord(h->pev[1], ms));
+  }
   if (prof) CK(cudaEventRecord(h->pev[2], ms));
-  // the consensus kernel also clears the next iteration's worklist counter, so
-  // it runs even when there is no free break-point (eta = 1)
-  const int nfree = (h->eta - 1) * h->p;
-  CK(launch_pdl(consensus_kernel, std::max(1, (nfree + 63) / 64), 64, ms, P));
+  // the node pass also sets up the next iteration's worklist, so it runs even
+  // when there is no free break-point (eta = 1)
+  const int nodew = node_warps(h->p, h->eta);
+  CK(launch_pdl(node_kernel, (unsigned)((nodew + NODE_WARPS - 1) / NODE_WARPS), 32u * NODE_WARPS, ms, P));
   if (prof) {
     CK(cudaEventRecord(h->pend, ms));
     CK(cudaEventSynchronize(h->pend));
     float t[4];
     CK(cudaEventElapsedTime(&t[0], h->pev[0], h->pev[1]));
     CK(cudaEventElapsedTime(&t[1], h->pev[1], h->pev[2]));
-    t[2] = 0.f;  // the kinetic and wall blocks run inside the pass-1 launch
+    t[2] = 0.f;  // the kinetic, wall and velocity factors run inside the first launch
     CK(cudaEventElapsedTime(&t[3], h->pev[2], h->pend));
     for (int q = 0; q < 4; ++q) h->ptime[q] += t[q];
     h->pcount += 1;
@@ -1490,31 +1497,16 @@ plan_status plan_reset(plan_t h) {
   h->k = 0;
   h->cur = 0;
   Dev P = h->dev(0);
-  const size_t zbytes = (size_t)h->p * (h->eta + 1) * 8;
-  (void)zbytes;
-  CK(cudaMemsetAsync(h->at<void>(h->L.bits), 0, (size_t)h->eta * h->ntp * TILE * 4, h->stream));
-  const size_t ng = (size_t)h->nw + h->nv;
-  if (ng) CK(cudaMemsetAsync(h->at<void>(h->L.wbits), 0, ng * h->eta * h->nt * 4, h->stream));
-  CK(cudaMemsetAsync(h->at<void>(h->L.wnode), 1, (size_t)h->p * (h->eta + 1), h->stream));
-  if (h->cfg.flags & (PLAN_DENSE_STATE | PLAN_U_KEEP | PLAN_ADMM)) {
+  if (P.dense) {
+    const size_t ng = (size_t)h->nw + h->nv;
     CK(cudaMemsetAsync(h->at<void>(h->L.ulo), 0, h->slots * 16, h->stream));
     CK(cudaMemsetAsync(h->at<void>(h->L.uhi), 0, h->slots * 16, h->stream));
     if (ng) CK(cudaMemsetAsync(h->at<void>(h->L.uwall), 0, ng * h->eta * h->p * 16, h->stream));
   }
-  CK(cudaMemsetAsync(h->at<void>(h->L.res), 0, 16, h->stream));
-  CK(cudaMemsetAsync(h->at<void>(h->L.wcount), 0, 16, h->stream));
-  CK(cudaMemsetAsync(h->at<void>(h->L.sched), 0, 16, h->stream));
-
-  CK(cudaMemsetAsync(h->at<void>(h->L.stamps), 0xff, 2 * (size_t)h->eta * h->ntp * 4, h->stream));
-  CK(clear_sums(h));
-  CK(cudaMemsetAsync(h->at<void>(h->L.status), 0, 4, h->stream));
-  // plan_set_endpoints' words: no violation, extent 0, no fix-up block done
-  CK(cudaMemsetAsync(h->at<void>(h->L.ekey), 0xff, 8, h->stream));
-  CK(cudaMemsetAsync(h->at<char>(h->L.ekey) + 8, 0, 16, h->stream));
-  fix_kernel<<<1, 256, 0, h->stream>>>(P, h->at<float2>(h->L.start), h->at<float2>(h->L.goal));
-  const int n = std::max(h->p * (h->eta + 1), h->eta * h->p);
-  reset_kernel<<<(n + 255) / 256, 256, 0, h->stream>>>(P, h->at<float2>(h->L.z0), h->at<float2>(h->L.z1),
-                                                      h->at<float2>(h->L.start), h->at<float2>(h->L.goal));
+  const size_t words = std::max((size_t)h->eta * h->ntp * TILE / 4, (size_t)h->p * (h->eta + 1));
+  reset_kernel<<<1 + (unsigned)std::min<size_t>((words + 255) / 256, 1216), 256, 0, h->stream>>>(
+      P, h->at<float2>(h->L.z0), h->at<float2>(h->L.z1), h->at<float2>(h->L.start), h->at<float2>(h->L.goal),
+      h->at<unsigned>(h->L.res), h->at<unsigned>(h->L.wcount), h->at<unsigned long long>(h->L.ekey));
   CK(cudaGetLastError());
   return PLAN_OK;
 }
@@ -1776,6 +1768,7 @@ plan_status plan_set_endpoints(plan_t h, const float* start, const float* goal) 
     CK(cudaMemcpyAsync(d_goal, goal, p * 8, cudaMemcpyHostToDevice, h->stream));
     endpoints_fix_kernel<<<1, 256, 0, h->stream>>>(h->dev(h->k), d_start, d_goal);
     CK(cudaGetLastError());
+    if ((st = refresh_segments(h)) != PLAN_OK) return st;
     // the caller's host buffers may be reused once this returns
     CK(cudaStreamSynchronize(h->stream));
     h->adj_valid = false;
@@ -1890,14 +1883,12 @@ plan_status plan_import_state(plan_t h, const float* z, const float* u_coll, con
   plan_status wst = derive_wnode(h);
   if (wst != PLAN_OK) return wst;
   CK(cudaMemsetAsync(h->at<void>(h->L.res), 0, 16, h->stream));
-  CK(cudaMemsetAsync(h->at<void>(h->L.wcount), 0, 16, h->stream));
-  CK(cudaMemsetAsync(h->at<void>(h->L.sched), 0, 16, h->stream));
-  CK(cudaMemsetAsync(h->at<void>(h->L.stamps), 0xff, 2 * (size_t)h->eta * h->ntp * 4, h->stream));
+  if ((wst = drop_worklist(h)) != PLAN_OK) return wst;
   CK(clear_sums(h));
   CK(cudaMemsetAsync(h->at<void>(h->L.status), 0, 4, h->stream));
   fix_kernel<<<1, 256, 0, h->stream>>>(P, h->at<float2>(h->L.start), h->at<float2>(h->L.goal));
   CK(cudaGetLastError());
-  return PLAN_OK;
+  return refresh_segments(h);
 }
 
 plan_status plan_check(plan_t h, double* total_cost, double* min_pair_clearance,
@@ -1978,25 +1969,38 @@ plan_status plan_profile(plan_t h, int enable, float* ms, int* iterations) {
 // ---------------------------------------------------------------------------
 namespace {
 
+// The tape of one iteration: z^k, the kinetic u^k, and the active pairs and
+// gated segment factors with their u^k, compacted (both counts zeroed before).
 __global__ void record_kernel(Dev P, const float2* zk, float2* tz, float4* tukin, uint32_t* tfid,
                               float4* tucl, float4* tuch, unsigned* tcount, uint32_t* tsidx,
                               float4* tsu, unsigned* tscount) {
   pdl_begin();
-  const unsigned cnt = *P.work_count;
   const unsigned nz = (unsigned)P.p * (P.eta + 1), nk = (unsigned)P.eta * P.p;
-  const unsigned nseg = (unsigned)(P.nw + P.nv) * nk;
-  const unsigned n = max(max(max(nz, nk), cnt), nseg);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *tcount = cnt;
+  const unsigned nseg = (unsigned)(P.nw + P.nv) * nk, nrows = (unsigned)P.eta * P.ntp * TILE;
+  const unsigned n = (max(max(nz, nrows), nseg) + 31u) & ~31u;  // whole warps
+  const int lane = threadIdx.x & 31;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     if (t < nz) tz[t] = zk[t];
     if (t < nk) tukin[t] = P.ukin[t];
-    if (t < cnt) {
-      const uint32_t f = P.work[t];
-      tfid[t] = f;
-      tucl[t] = P.ulo[f];
-      tuch[t] = P.uhi[f];
+    const uint32_t word = t < nrows ? P.bits[t] : 0u;
+    if (__any_sync(FULL, word != 0u)) {
+      const unsigned cnt = __popc(word);
+      unsigned incl = cnt;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += v;
+      }
+      unsigned at = 0;
+      if (lane == 31) at = atomicAdd(tcount, incl);
+      at = __shfl_sync(FULL, at, 31) + (incl - cnt);
+      for (uint32_t w = word; w; w &= w - 1u, ++at) {
+        const uint32_t f = t * TILE + (uint32_t)(__ffs(w) - 1);
+        tfid[at] = f;
+        tucl[at] = P.ulo[f];
+        tuch[at] = P.uhi[f];
+      }
     }
-    if (t < nseg) {  // active walls and velocity limits, compacted (tscount zeroed before)
+    if (t < nseg) {
       const unsigned i = t % P.p, ws = t / P.p;
       if ((P.wbits[(size_t)ws * P.nt + i / TILE] >> (i % TILE)) & 1u) {
         const unsigned at = atomicAdd(tscount, 1u);
@@ -2007,10 +2011,13 @@ __global__ void record_kernel(Dev P, const float2* zk, float2* tz, float4* tukin
   }
 }
 
-// Zeroes n 32-bit counters spaced stride bytes apart (the compaction counter
-// of every tape slot of a segment, before its replay).
-__global__ void zero_strided_kernel(char* base, size_t stride, int n) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) *reinterpret_cast<unsigned*>(base + i * stride) = 0u;
+// Zeroes two 32-bit counters in each of n slots stride bytes apart (the
+// compaction counters of every tape slot of a segment, before its replay).
+__global__ void zero_strided_kernel(char* a, char* b, size_t stride, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    *reinterpret_cast<unsigned*>(a + i * stride) = 0u;
+    *reinterpret_cast<unsigned*>(b + i * stride) = 0u;
+  }
 }
 
 // The adjoint passes run with programmatic dependent launch, like the
@@ -2074,7 +2081,7 @@ std::vector<Region> ck_regions(plan_t h) {
   std::vector<Region> r = {
       {h->L.z0, zb}, {h->L.z1, zb}, {h->L.bits, (size_t)h->eta * h->ntp * TILE * 4},
       {h->L.ulo, h->slots * 16}, {h->L.uhi, h->slots * 16}, {h->L.xlo, h->slots * 16},
-      {h->L.xhi, h->slots * 16}, {h->L.ukin, kin}, {h->L.xkin, kin}, {h->L.wcount, 16},
+      {h->L.xhi, h->slots * 16}, {h->L.ukin, kin}, {h->L.xkin, kin},
       {h->L.res, 16}, {h->L.status, 4}};
   if (ng) {
     r.push_back({h->L.uwall, ng * kin});
@@ -2145,10 +2152,9 @@ plan_status snapshot(plan_t h, const AdjLayout& A, int idx, bool save) {
     ck += a256(r.bytes);
   }
   if (!save) {
-    // the pass-1 heavy-tile lists belong to the iteration order that ran, not
-    // to the restored state: start over with none (results do not depend on it)
-    CK(cudaMemsetAsync(h->at<void>(h->L.sched), 0, 16, h->stream));
-    CK(cudaMemsetAsync(h->at<void>(h->L.stamps), 0xff, 2 * (size_t)h->eta * h->ntp * 4, h->stream));
+    // the worklist is not part of the state
+    plan_status st = drop_worklist(h);
+    if (st != PLAN_OK) return st;
   }
   return PLAN_OK;
 }
@@ -2389,6 +2395,10 @@ plan_status plan_set_params(plan_t h, const float* radius, const float* cost_w) 
     CK(cudaMemcpyAsync(h->at<void>(h->L.cost), cost.data(), p * eta * 4, cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(h->at<void>(h->L.ccost), ccost.data(), p * eta * 8, cudaMemcpyHostToDevice, h->stream));
   }
+  if (radius) {
+    plan_status st = refresh_segments(h);
+    if (st != PLAN_OK) return st;
+  }
   CK(cudaStreamSynchronize(h->stream));
   return PLAN_OK;
 }
@@ -2463,7 +2473,9 @@ plan_status plan_backward(plan_t h, int K, const float* dL_dz, float* d_start, f
     if ((st = snapshot(h, A, seg, false)) != PLAN_OK) return st;
     h->k = c0;
     h->cur = h->ck_cur[seg];
-    zero_strided_kernel<<<1, 64, 0, h->stream>>>(h->adj + A.tape0 + A.t_scount, A.slot_bytes, c1 - c0);
+    if ((st = refresh_segments(h)) != PLAN_OK) return st;
+    zero_strided_kernel<<<1, 64, 0, h->stream>>>(h->adj + A.tape0 + A.t_count, h->adj + A.tape0 + A.t_scount,
+                                                 A.slot_bytes, c1 - c0);
     CK(cudaGetLastError());
     for (int k = c0; k < c1; ++k) {
       const float2* zk = h->cur ? h->at<float2>(h->L.z1) : h->at<float2>(h->L.z0);
@@ -2496,7 +2508,7 @@ plan_status plan_backward(plan_t h, int K, const float* dL_dz, float* d_start, f
   if ((st = snapshot(h, A, nseg, false)) != PLAN_OK) return st;
   h->k = K;
   h->cur = h->ck_cur[nseg];
-  return PLAN_OK;
+  return refresh_segments(h);
 }
 
 
@@ -2644,10 +2656,11 @@ plan_status plan_iterate_static(const plan_config* cfg, const float* start, cons
 // ---------------------------------------------------------------------------
 // Each member is an ordinary plan (its own workspace slice, no streams of its
 // own).  Every pass of an iteration is a single launch over the union of all
-// members' blocks: a block finds its member by binary search over a prefix
-// table of block counts and runs the same per-block code as a single plan,
-// on the member's descriptor copied into shared memory.  All members advance
-// in lockstep, so the descriptors only depend on the iteration's parity; a
+// members' warps: a warp finds its member and its work in a table built at
+// creation (one 8-byte load; a binary search over prefix sums took six to
+// nine dependent ones) and runs the same per-warp code as a single plan, on
+// the member's descriptor copied into shared memory.  All members advance in
+// lockstep, so the descriptors only depend on the iteration's parity; a
 // member that has converged is frozen (its passes do nothing and its z is
 // carried over unchanged).  Iterations are replayed from CUDA graphs, and
 // three launch-shape knobs are chosen by timing (plan_batch_autotune).
@@ -2663,7 +2676,16 @@ __device__ __forceinline__ int find_member(const int* pre, int n, int x) {
   return lo;
 }
 
-template <bool DENSE, int TROWS>
+// The member's descriptor into a warp's shared slot.
+__device__ __forceinline__ const Dev& load_member(const Dev* tab, int b, Dev* slot) {
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(tab + b);
+  uint32_t* dst = reinterpret_cast<uint32_t*>(slot);
+  for (int w = threadIdx.x & 31; w < (int)(sizeof(Dev) / 4); w += 32) dst[w] = src[w];
+  __syncwarp();
+  return *slot;
+}
+
+template <int TROWS>
 __global__ void __launch_bounds__(32 * (TILE / TROWS)) batch_test_kernel(const Dev* tab, const int* pre,
                                                                           int n, const uint8_t* frozen) {
   __shared__ Dev sP;
@@ -2676,44 +2698,42 @@ __global__ void __launch_bounds__(32 * (TILE / TROWS)) batch_test_kernel(const D
   }
   __syncthreads();
   if (frozen[sb]) return;
-  test_block<DENSE, TROWS>(sP, sblk);
+  if (sblk == 0 && threadIdx.x == 0) *sP.res_cur = 0u;
+  test_block<TROWS>(sP, sblk);
 }
 
-// Gated state, one warp per tile (lane = row agent): each warp finds its own
-// member, since the 4 tiles of a CTA may belong to different members.
-__global__ void __launch_bounds__(32 * TILES_PER_CTA) batch_test_rows_kernel(const Dev* tab, const int* pre,
-                                                                         int n, int ntiles,
-                                                                         const uint8_t* frozen) {
-  __shared__ Dev sP[TILES_PER_CTA];
-  __shared__ float4 col[TILES_PER_CTA][72];
-  __shared__ uint32_t nws[TILES_PER_CTA][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * TILES_PER_CTA + warp;
-  if (t >= ntiles) return;  // warp-uniform
-  const int b = find_member(pre, n, t);
-  if (frozen[b]) return;
-  // the member's descriptor into this warp's shared slot
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(tab + b);
-  uint32_t* dst = reinterpret_cast<uint32_t*>(&sP[warp]);
-  for (int w = lane; w < (int)(sizeof(Dev) / 4); w += 32) dst[w] = src[w];
-  __syncwarp();
-  const int blk = t - pre[b];
-  if (blk == 0 && lane == 0) *sP[warp].res_cur = 0u;
-  test_tile_rows(sP[warp], blk, col[warp], nws[warp]);
-}
+// Table entry of a factor-pass warp: the member, and an item of its own
+// numbering: list warps, then segment warps, then tiles (dense state: segment
+// warps only).
+struct BatchItem { int member, item; };
 
-__global__ void batch_segment_kernel(const Dev* tab, const int* pre, int n, const uint8_t* frozen) {
-  __shared__ Dev sP;
-  __shared__ int sb, sblk;
-  if (threadIdx.x == 0) {
-    const int b = find_member(pre, n, blockIdx.x);
-    sb = b;
-    sblk = blockIdx.x - pre[b];
-    sP = tab[b];
+// What the numbering is made of, per member.
+struct BatchShape { int nlist, nseg; };
+
+// Every factor of every member (gated state), or the kinetic, wall and
+// velocity factors (dense state, after batch_test_kernel).
+template <bool DENSE>
+__global__ void __launch_bounds__(32 * FACTOR_WARPS, 6) batch_factor_kernel(const Dev* tab, const BatchItem* items,
+                                                                           int nitems, const BatchShape* shapes,
+                                                                           const uint8_t* frozen) {
+  __shared__ Dev sP[FACTOR_WARPS];
+  __shared__ TileMem mem[DENSE ? 1 : FACTOR_WARPS];
+  pdl_begin();
+  const int warp = threadIdx.x >> 5;
+  const int t = (int)blockIdx.x * FACTOR_WARPS + warp;
+  if (t >= nitems) return;  // warp-uniform
+  const BatchItem it = items[t];
+  if (frozen[it.member]) return;
+  const BatchShape sh = shapes[it.member];
+  const Dev& P = load_member(tab, it.member, sP + warp);
+  if (DENSE) {
+    segment_warp(P, it.item);
+  } else {
+    if (it.item == 0 && (threadIdx.x & 31) == 0) *P.res_cur = 0u;
+    const int g = it.item - sh.nlist;
+    if (g >= 0 && g < sh.nseg) segment_warp(P, g);
+    else collision_warp<false>(P, g < 0 ? it.item : it.item - sh.nseg, sh.nlist, mem + warp);
   }
-  __syncthreads();
-  if (frozen[sb]) return;
-  segment_block<false>(sP, sblk);
 }
 
 // Exclusive prefix of the members' worklist lengths (frozen members: 0).
@@ -2748,20 +2768,18 @@ __global__ void __launch_bounds__(256) batch_prox_kernel(const Dev* tab, const i
   }
 }
 
-// One thread per free break-point; each member's range is padded to whole
-// warps (and at least one warp, which also clears the member's next worklist
-// counter), so a warp never spans two members.
-__global__ void batch_consensus_kernel(const Dev* tab, const int* pre, int n) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= pre[n]) return;  // whole warps past the end
-  const int b = find_member(pre, n, t);
-  const Dev& P = tab[b];
-  const int tl = t - pre[b];
-  if (tl == 0) *P.work_count_next = 0u;
-  float dz = 0.f;
-  bool bad = false;
-  if (tl < (P.eta - 1) * P.p) consensus_node(P, tl, dz, bad);
-  consensus_reduce(P, dz, bad);
+// Node pass: a warp per table entry (member, node warp).
+__global__ void __launch_bounds__(32 * NODE_WARPS) batch_node_kernel(const Dev* tab, const BatchItem* nodes, int nnodes,
+                                                                    const uint8_t* frozen) {
+  __shared__ Dev sP[NODE_WARPS];
+  pdl_begin();
+  const int warp = threadIdx.x >> 5;
+  const int t = (int)blockIdx.x * NODE_WARPS + warp;
+  if (t >= nnodes) return;  // warp-uniform
+  const BatchItem it = nodes[t];
+  const Dev& P = load_member(tab, it.member, sP + warp);
+  if (it.item == 0 && (threadIdx.x & 31) == 0) advance_worklist(P, frozen[it.member] != 0);
+  consensus_warp(P, it.item);
 }
 
 // The residual slot of each member's last iteration, gathered contiguously.
@@ -2783,10 +2801,12 @@ struct plan_batch_s {
   bool dense = false;
   // device tables (in the workspace tail)
   Dev* tab[2] = {nullptr, nullptr};
-  int *pre_test = nullptr, *pre_seg = nullptr, *pre_node = nullptr, *pre_work = nullptr;
+  int *pre_test = nullptr, *pre_work = nullptr;  // dense state
+  BatchItem *items = nullptr, *nodes = nullptr;
+  BatchShape* shapes = nullptr;
   uint8_t* frozen = nullptr;
   float* res = nullptr;
-  int ntest = 0, nseg = 0, nnode = 0;
+  int ntest = 0, nitems = 0, nnodes = 0;
   std::vector<uint8_t> h_frozen;
   std::vector<int> conv_iter;
   int warm = 0;  // largest warm-up length among members
@@ -2799,8 +2819,32 @@ struct plan_batch_s {
 
 namespace {
 
-size_t batch_tables_bytes(int n) {
-  return a256(2 * (size_t)n * sizeof(Dev)) + 4 * a256(((size_t)n + 1) * 4) + a256(n) + a256((size_t)n * 4);
+// The warps of one member's passes: list warps enough for a chunk of 32 pairs
+// each in a small member, shared out over the GPU (32 warps an SM) in a large
+// batch; one warp per tile, per segment kind and per node group.
+struct MemberWarps { int list, seg, tiles, nodes; };
+MemberWarps member_warps(const plan_config& c, int n) {
+  const int nt = (c.p + TILE - 1) / TILE, ntp = nt * (nt + 1) / 2;
+  const long long pairs = (long long)c.eta * c.p * (c.p - 1) / 2;
+  const bool dense = (c.flags & (PLAN_DENSE_STATE | PLAN_U_KEEP | PLAN_ADMM)) != 0;
+  MemberWarps w;
+  w.list = (int)std::max<long long>(1, std::min<long long>((pairs + 127) / 128, std::max(8, 4864 / n)));
+  w.seg = (1 + c.n_walls) * c.eta * nt;
+  w.tiles = c.eta * ntp;
+  w.nodes = node_warps(c.p, c.eta);
+  if (dense) w.list = w.tiles = 0;  // collisions: batch_test_kernel
+  return w;
+}
+
+size_t batch_tables_bytes(int n, const plan_config* cfgs) {
+  size_t items = 0, nodes = 0;
+  for (int b = 0; b < n; ++b) {
+    const MemberWarps w = member_warps(cfgs[b], n);
+    items += (size_t)w.list + w.seg + w.tiles;
+    nodes += w.nodes;
+  }
+  return a256(2 * (size_t)n * sizeof(Dev)) + 2 * a256(((size_t)n + 1) * 4) + a256(n) + a256((size_t)n * 4) +
+         a256(items * sizeof(BatchItem)) + a256(nodes * sizeof(BatchItem)) + a256(n * sizeof(BatchShape));
 }
 
 plan_status batch_tables(plan_batch_s* B) {
@@ -2814,7 +2858,6 @@ plan_status batch_tables(plan_batch_s* B) {
       h->k = kk;
       h->cur = (h->eta > 1) ? (kk & 1) : 0;
       d[b] = h->dev(kk);
-      d[b].hcap = 0;  // the batched test pass keeps its own order
       // the table serves every later iteration of this parity, so the
       // previous iteration's residual slot is always the other one
       d[b].res_prev = h->at<unsigned>(h->L.res) + ((kk + 1) & 1);
@@ -2832,23 +2875,30 @@ plan_status batch_tables(plan_batch_s* B) {
 
 template <int TROWS>
 void launch_batch_test(plan_batch_s* B, const Dev* tab, cudaStream_t s) {
-  constexpr int threads = 32 * (TILE / TROWS);
-  if (B->dense) batch_test_kernel<true, TROWS><<<B->ntest, threads, 0, s>>>(tab, B->pre_test, B->n, B->frozen);
-  else batch_test_kernel<false, TROWS><<<B->ntest, threads, 0, s>>>(tab, B->pre_test, B->n, B->frozen);
+  batch_test_kernel<TROWS><<<B->ntest, 32 * (TILE / TROWS), 0, s>>>(tab, B->pre_test, B->n, B->frozen);
 }
 
+// Gated state: two launches with programmatic serialization, as a single
+// plan.  Dense state: the collision tests in the chosen shape, the other
+// factors, the minimizers over the members' concatenated worklists, the nodes.
 plan_status enqueue_batch_iteration(plan_batch_s* B, int parity, cudaStream_t s) {
   const Dev* tab = B->tab[parity];
-  if (B->trows == 32 && !B->dense)
-    batch_test_rows_kernel<<<(B->ntest + TILES_PER_CTA - 1) / TILES_PER_CTA, 32 * TILES_PER_CTA, 0, s>>>(
-        tab, B->pre_test, B->n, B->ntest, B->frozen);
-  else if (B->trows == 4) launch_batch_test<4>(B, tab, s);
+  const unsigned fgrid = (unsigned)((B->nitems + FACTOR_WARPS - 1) / FACTOR_WARPS);
+  const unsigned ngrid = (unsigned)((B->nnodes + NODE_WARPS - 1) / NODE_WARPS);
+  if (!B->dense) {
+    CK(launch_pdl(batch_factor_kernel<false>, fgrid, 32u * FACTOR_WARPS, s, tab, (const BatchItem*)B->items,
+                  B->nitems, (const BatchShape*)B->shapes, (const uint8_t*)B->frozen));
+    CK(launch_pdl(batch_node_kernel, ngrid, 32u * NODE_WARPS, s, tab, (const BatchItem*)B->nodes, B->nnodes,
+                  (const uint8_t*)B->frozen));
+    return PLAN_OK;
+  }
+  if (B->trows == 4) launch_batch_test<4>(B, tab, s);
   else if (B->trows == 16) launch_batch_test<16>(B, tab, s);
   else launch_batch_test<8>(B, tab, s);
-  batch_segment_kernel<<<B->nseg, THREADS, 0, s>>>(tab, B->pre_seg, B->n, B->frozen);
+  batch_factor_kernel<true><<<fgrid, 32 * FACTOR_WARPS, 0, s>>>(tab, B->items, B->nitems, B->shapes, B->frozen);
   batch_scan_kernel<<<1, 1024, 0, s>>>(tab, B->n, B->frozen, B->pre_work);
   batch_prox_kernel<<<B->prox_grid * B->prox_mult, 256, 0, s>>>(tab, B->pre_work, B->n);
-  batch_consensus_kernel<<<(B->nnode + 255) / 256, 256, 0, s>>>(tab, B->pre_node, B->n);
+  batch_node_kernel<<<ngrid, 32 * NODE_WARPS, 0, s>>>(tab, B->nodes, B->nnodes, B->frozen);
   CK(cudaGetLastError());
   return PLAN_OK;
 }
@@ -2910,7 +2960,7 @@ plan_status plan_batch_workspace_size(int n, const plan_config* cfgs, size_t* by
     if (!sizes_ok(&cfgs[b])) return fail(PLAN_EINVAL, "member %d: p, eta or n_walls out of range", b);
     tot += a256(layout_for(&cfgs[b]).total);
   }
-  *bytes = tot + batch_tables_bytes(n);
+  *bytes = tot + batch_tables_bytes(n, cfgs);
   return PLAN_OK;
 }
 
@@ -2968,26 +3018,37 @@ plan_status plan_batch_create(int n, const plan_config* cfgs, const float* const
   B->tab[1] = B->tab[0] + n;
   t += a256(2 * (size_t)n * sizeof(Dev));
   B->pre_test = reinterpret_cast<int*>(t); t += a256(((size_t)n + 1) * 4);
-  B->pre_seg = reinterpret_cast<int*>(t); t += a256(((size_t)n + 1) * 4);
-  B->pre_node = reinterpret_cast<int*>(t); t += a256(((size_t)n + 1) * 4);
   B->pre_work = reinterpret_cast<int*>(t); t += a256(((size_t)n + 1) * 4);
   B->frozen = reinterpret_cast<uint8_t*>(t); t += a256(n);
-  B->res = reinterpret_cast<float*>(t);
-  std::vector<int> pt(n + 1, 0), ps(n + 1, 0), pn(n + 1, 0);
+  B->res = reinterpret_cast<float*>(t); t += a256((size_t)n * 4);
+  std::vector<int> pt(n + 1, 0);
+  std::vector<BatchItem> items, nodes;
+  std::vector<BatchShape> shapes(n);
+  // the longest chains first: list warps, then segment warps, then tiles
+  for (int part = 0; part < 3; ++part)
+    for (int b = 0; b < n; ++b) {
+      const MemberWarps w = member_warps(cfgs[b], n);
+      const int lo = part == 0 ? 0 : part == 1 ? w.list : w.list + w.seg;
+      const int hi = part == 0 ? w.list : part == 1 ? w.list + w.seg : w.list + w.seg + w.tiles;
+      for (int q = lo; q < hi; ++q) items.push_back({b, q});
+    }
   for (int b = 0; b < n; ++b) {
-    plan_t h = B->m[b];
-    pt[b + 1] = pt[b] + h->eta * h->ntp;
-    ps[b + 1] = ps[b] + h->eta * h->nt;
-    const int nfree = (h->eta - 1) * h->p;
-    pn[b + 1] = pn[b] + std::max(32, (nfree + 31) / 32 * 32);
+    const MemberWarps w = member_warps(cfgs[b], n);
+    shapes[b] = {w.list, w.seg};
+    for (int q = 0; q < w.nodes; ++q) nodes.push_back({b, q});
+    pt[b + 1] = pt[b] + B->m[b]->eta * B->m[b]->ntp;
   }
-  B->ntest = pt[n]; B->nseg = ps[n]; B->nnode = pn[n];
+  B->ntest = pt[n]; B->nitems = (int)items.size(); B->nnodes = (int)nodes.size();
+  B->items = reinterpret_cast<BatchItem*>(t); t += a256(items.size() * sizeof(BatchItem));
+  B->nodes = reinterpret_cast<BatchItem*>(t); t += a256(nodes.size() * sizeof(BatchItem));
+  B->shapes = reinterpret_cast<BatchShape*>(t);
   B->h_frozen.assign(n, 0);
   B->conv_iter.assign(n, -1);
   cudaError_t e = cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMemcpyAsync(B->pre_test, pt.data(), (n + 1) * 4, cudaMemcpyHostToDevice, B->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(B->pre_seg, ps.data(), (n + 1) * 4, cudaMemcpyHostToDevice, B->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(B->pre_node, pn.data(), (n + 1) * 4, cudaMemcpyHostToDevice, B->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(B->items, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, B->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(B->nodes, nodes.data(), nodes.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, B->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(B->shapes, shapes.data(), n * sizeof(BatchShape), cudaMemcpyHostToDevice, B->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(B->frozen, B->h_frozen.data(), n, cudaMemcpyHostToDevice, B->stream);
   if (e != cudaSuccess) { plan_batch_destroy(B); return fail(PLAN_ECUDA, "batch setup failed: %s", cudaGetErrorString(e)); }
   st = ensure_prox_grid(B->m[0]);

@@ -1,18 +1,20 @@
-// twa_iter.cuh -- the per-block work of one TWA iteration (Appendix B steps
+// twa_iter.cuh -- the per-warp work of one TWA iteration (Appendix B steps
 // 1-7 over the factor graph of Section 3.3 of Bento et al., NIPS 2013), shared
 // by the single-planner kernels and the batched ones (both in plan.cu).
 //
-// Pass 1, test_block: one block per (segment s, agent tiles I <= J) of 32 x 32
-//   collision factors: finish the deferred dual update of the pairs that were
-//   active (step 7 of the previous iteration), n = z - u (step 1), collision
-//   test and weight (steps 2-3), activity bits, worklist of active pairs.
-// segment_block: the kinetic and wall factors of one (segment, agent tile);
-//   the single-planner kernels run these blocks in the same launch as pass 1
-//   and leave the active walls' capsule minimizers to pass 2
-//   (wall_prox_item_warp, one warp per wall), which spreads them over the GPU.
-// Pass 2, prox_item: the collision minimizer of one active pair; adds its
-//   m = x + u to the consensus sums (wall_prox_item_warp: the same for a wall).
-// Pass 3, consensus_node: z = sum m / count per free break-point (step 5).
+// Gated state (default): two launches.
+//   Factor pass, collision_warp and segment_warp: every factor.  The pairs
+//     that were active lately are on a worklist, 32 to a warp; a tile warp
+//     looks through one (segment, agent tiles I <= J) block of 32 x 32 pairs
+//     for others that collide; a segment warp takes one kinetic, wall or
+//     velocity kind of one (segment, agent tile).  Whoever finds a factor
+//     active runs its minimizer at once and adds m = x + u to the consensus
+//     sums.
+//   Node pass, consensus_warp: z = sum m / count per free break-point (step
+//     5), and the per-segment records the next factor pass starts from.
+// Dense state: test_block (every pair's u record streamed, lane = column
+//   agent) and segment_warp in one launch, then prox_item over the worklist of
+//   active pairs, then the node pass.
 //
 // Step 7 needs z^{k+1}, which exists only after every factor ran, so x^{k+1}
 // of the active factors is stored and u^{k+1} = u^k + alpha (x^{k+1} -
@@ -30,6 +32,18 @@
 // With the dense state the u record of every slot is read and written each
 // iteration; otherwise only those of factors whose bit is set (every other u
 // is 0 by the reset rule), which leaves 1 bit per factor of state traffic.
+//
+// Worklist of the gated state.  work[0 .. n) holds slots, bit 31 set where
+// the pair was active in the last iteration; listed[row] bit c says that the
+// pair is on it.  A pair joins when a tile warp finds it active, and stays on
+// it after it turns inactive (a pair that left often comes back; its u is 0
+// then), so the tile warps of an iteration can read `listed` while the list
+// warps work: nothing in it changes but the words of a tile's own warp.  When
+// more than half of the list is inactive, or an append did not fit, the next
+// iteration builds it anew from `bits` (the tile warps then take the pairs
+// active before, the list warps nothing): `bits` and the slot records are
+// the state, the list only an order of work, and any list gives the same
+// iterates.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -41,9 +55,6 @@ namespace {
 using namespace twa;
 
 constexpr int TILE = 32;
-constexpr int WARPS = 8;
-constexpr int THREADS = TILE * WARPS;
-constexpr int ROWS = TILE / WARPS;  // rows of a tile per warp
 constexpr unsigned FULL = 0xffffffffu;
 
 struct Dev {
@@ -69,28 +80,15 @@ struct Dev {
   float4 *ukin, *xkin;   // [eta][p]
   float4 *uwall, *xwall; // [nw][eta][p]
   uint32_t* wbits;       // [nw][eta][nt]
-  uint32_t* work;        // active collision slots of this iteration
-  unsigned* work_count;  // their number
-  unsigned* work_count_next;  // the counter the next iteration appends to
-  // pass-1 scheduling (single plans; hcap = 0 turns it off): tiles whose
-  // exact-test work was large in the previous iteration are listed and
-  // dispatched first, on the first hcap warps of the launch, and stamped so
-  // that their place in the ordinary order is skipped
-  int hcap;                    // heavy-tile slots at the front of the launch
-  const uint32_t* heavy_cur;   // this iteration's heavy tiles (built by the previous one)
-  unsigned* hcount_cur;        // their number (cleared by the consensus pass for reuse)
-  uint32_t* heavy_next;        // the next iteration's heavy tiles (built by this pass 1)
-  unsigned* hcount_next;
-  // [eta ntp] iteration number for which the tile is listed heavy, one array
-  // per iteration parity: this iteration's list is only read (ordinary warps
-  // skip the tiles listed in it) while the next one's is written
-  const unsigned* stamp_cur;
-  unsigned* stamp_next;
-  unsigned* iter;              // iteration number (advanced by the consensus pass)
-  uint32_t* wwork;       // active wall factors ((w eta + s) p + i) of this iteration whose
-                         // minimizer runs in pass 2 (wall_prox_item_warp)
-  unsigned* wwork_count;       // their number
-  unsigned* wwork_count_next;  // the counter the next iteration appends to
+  float4* zseg;          // [eta][p] (z(s), z(s+1)) of z^k (gated state)
+  float4* circ;          // [eta][p] bounding circle (m.x, m.y, b, bounding_offset) of z^k
+  uint32_t* work;        // collision worklist (dense state: the active slots of this iteration)
+  unsigned cap;          // its capacity
+  uint32_t* listed;      // [eta * ntp * 32] pairs on the worklist (gated state)
+  unsigned* work_count;  // its length, by iteration parity: entries are appended here
+  unsigned* work_count_prev;  // ... its length at the start of this iteration
+  unsigned* ctl;         // gated state: [0] rebuild the worklist in this iteration, [1] entries
+                         // of inactive pairs on it, [2] an append did not fit
   unsigned long long* accx;  // [p][eta+1] fixed-point sums of rho0-weighted m.x
   unsigned long long* accy;  //                                 ... of m.y
   unsigned* accc;        // [p][eta+1] number of rho0-weighted incoming edges
@@ -111,7 +109,7 @@ __device__ __forceinline__ float2 finish_u(bool bprev, bool pinned, bool keep, f
   if (bprev) {
     float2 d = x_pend - zk;
     res = fmaxf(res, maxabs2(d));
-    return mk(u_prev.x + alpha * d.x, u_prev.y + alpha * d.y);
+    return axpy(alpha, d, u_prev);
   }
   return keep ? u_prev : mk(0.f, 0.f);
 }
@@ -147,7 +145,7 @@ __device__ __forceinline__ float2 finish_u_feasible(bool pinned, float2 u_prev, 
   if (pinned) return mk(0.f, 0.f);
   const float2 d = (z_prev - u_prev) - zk;
   res = fmaxf(res, maxabs2(d));
-  return mk(u_prev.x + alpha * d.x, u_prev.y + alpha * d.y);
+  return axpy(alpha, d, u_prev);
 }
 
 __device__ __forceinline__ float2 lo2(float4 v) { return mk(v.x, v.y); }
@@ -158,24 +156,22 @@ __device__ __forceinline__ void atomic_max_nonneg(unsigned* slot, float v) {
   atomicMax(slot, __float_as_uint(v));
 }
 
-// Global loads issued where they stand.  A volatile asm is never moved into
-// a later branch, so loads placed ahead of an early exit are in flight
-// together with the loads after it: one memory round trip instead of two on
-// a warp's dependent chain.  For data that no other thread of the launch
-// writes (and that the loading thread writes, if at all, only afterwards).
-__device__ __forceinline__ float2 ld_now(const float2* p) {
-  float2 v;
-  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+// Four single-precision lanes as two pairs, and paired operations on them
+// (one instruction for two multiply-adds).
+__device__ __forceinline__ unsigned long long pair_of(float lo, float hi) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
   return v;
 }
-__device__ __forceinline__ float ld_now(const float* p) {
-  float v;
-  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
+                                                   unsigned long long c) {
+  unsigned long long v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
   return v;
 }
-__device__ __forceinline__ unsigned ld_now(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long v;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
   return v;
 }
 
@@ -267,9 +263,7 @@ __device__ __forceinline__ void end_classes(const Dev& P, int i, int s, bool pin
 // Gated segment factor w of (i, s): a wall (w < nw, Eq. wall_minimizer) or a
 // maximum / minimum velocity factor (w >= nw, Eq. max_vel_min).  Forward
 // weight rho0 when the n's violate it, else 0.  Called by a full warp (lane =
-// agent of tile I).  DEFER: the capsule minimizers of active walls go to the
-// wall worklist (P.wwork) instead of running here.
-template <bool DEFER>
+// agent of tile I).
 __device__ __forceinline__ void wall_factor(const Dev& P, int w, int i, bool vi, int s, int I,
                                             float2 zl, float2 zh, float r, bool pin_lo,
                                             bool pin_hi, float& res) {
@@ -277,6 +271,25 @@ __device__ __forceinline__ void wall_factor(const Dev& P, int w, int i, bool vi,
   const size_t widx = ((size_t)w * P.eta + s) * P.nt + I;
   const uint32_t word = P.wbits[widx];
   const bool bprev = vi && ((word >> lane) & 1u);
+  const bool vel = w >= P.nw;
+  float2 c0 = mk(0.f, 0.f), c1 = c0;
+  if (!vel) {
+    const float4 W = P.walls[w];
+    c0 = mk(W.x, W.y); c1 = mk(W.z, W.w);
+    // A wall none of the warp's agents was pushing against, and none can
+    // reach: the segment lies in the disk of half its length about its
+    // midpoint, so it is out of reach when the midpoint is farther than that
+    // plus r from the wall (with a margin of 1e-4 of the radii and 1e-5 of
+    // the coordinates, a hundred times the rounding).  Most walls of a warp
+    // end here: the exact test costs about ten times as much.
+    if (word == 0u && !P.dense) {
+      const float2 m = 0.5f * (zl + zh), d = zh - zl;
+      const float b = fmaf(0.5f, sqrtf(dot(d, d)), r);
+      const float L = fmaxf(fmaxf(maxabs2(c0), maxabs2(c1)), maxabs2(m));
+      const float reach = fmaf(1e-5f, L, 1.0001f * b);
+      if (!__any_sync(FULL, vi && !(dist2_point_segment(m, c0, c1) > reach * reach))) return;
+    }
+  }
   const size_t idx = ((size_t)w * P.eta + s) * P.p + i;
   float4 u4 = make_float4(0.f, 0.f, 0.f, 0.f), x4 = u4;
   if (vi && (P.dense || bprev)) u4 = P.uwall[idx];
@@ -291,47 +304,28 @@ __device__ __forceinline__ void wall_factor(const Dev& P, int w, int i, bool vi,
     uh = finish_u(bprev, pin_hi, P.keep, hi2(u4), hi2(x4), zh, P.alpha, res);
   }
   const float2 nl = zl - ul, nh = zh - uh;
-  const bool vel = w >= P.nw;
   bool act;
-  float2 c0 = mk(0.f, 0.f), c1 = c0;
   float C = 0.f;
-  bool vmin = false;
   if (vel) {
     const int v = w - P.nw;
-    vmin = (P.vmin_mask >> v) & 1u;
+    const bool vmin = (P.vmin_mask >> v) & 1u;
     if (vi) C = P.vlim[((size_t)v * P.p + i) * P.eta + s];
     const float2 d = nl - nh;
     const float d2 = dot(d, d);
     act = vi && (vmin ? d2 < C * C : d2 > C * C);
   } else {
-    const float4 W = P.walls[w];
-    c0 = mk(W.x, W.y); c1 = mk(W.z, W.w);
     act = vi && dist2_segment_segment(nl, nh, c0, c1) < r * r;
   }
   const uint32_t nw = __ballot_sync(FULL, act);
   if (lane == 0 && nw != word) P.wbits[widx] = nw;
-  if (DEFER && !vel) {
-    // the capsule minimizers go to the minimizer pass, spread over the GPU
-    // (one warp with several active walls would run them one after another)
-    if (act) P.uwall[idx] = pack(ul, uh);
-    else if (vi && P.dense) P.uwall[idx] = pack(ul, uh);
-    if (nw) {
-      unsigned base = 0;
-      if (lane == 0) base = atomicAdd(P.wwork_count, (unsigned)__popc(nw));
-      base = __shfl_sync(FULL, base, 0);
-      if (act) P.wwork[base + __popc(nw & ((1u << lane) - 1u))] = (uint32_t)idx;
-    }
-    return;
-  }
   if (act) {
     float2 xl = nl, xh = nh;
     int cl, ch;
     end_classes(P, i, s, pin_lo, pin_hi, cl, ch);
     if (vel) {
       velocity_prox(nl, nh, cl, ch, C, xl, xh);
-    } else if (!DEFER) {
-      if (!capsule_prox_classes(nl, nh, cl, ch, c0, c1, r, 0.5f * P.rho, xl, xh))
-        atomicOr(P.status, 1u);
+    } else if (!capsule_prox_classes(nl, nh, cl, ch, c0, c1, r, 0.5f * P.rho, xl, xh)) {
+      atomicOr(P.status, 1u);
     }
     P.xwall[idx] = pack(xl, xh);
     P.uwall[idx] = pack(ul, uh);
@@ -339,6 +333,41 @@ __device__ __forceinline__ void wall_factor(const Dev& P, int w, int i, bool vi,
     if (!pin_hi) contribute(P, i, s + 1, xh + uh);
   } else if (vi && P.dense) {
     P.uwall[idx] = pack(ul, uh);
+  }
+}
+
+// Kinetic, wall and velocity factors (steps 1-3 and the pending step 7): one
+// warp per (kind f, segment s, agent tile I), lane = agent; item = (s nt + I)
+// kinds + f, kind 0 the kinetic factor.
+__device__ __forceinline__ void segment_warp(const Dev& P, int item) {
+  const int kinds = 1 + P.nw + P.nv;
+  const int sI = item / kinds, f = item - sI * kinds;
+  const int s = sI / P.nt, I = sI - s * P.nt;
+  if (P.vo && (f == 0) == (s == 0)) return;  // kinetic on segment 1 only, the rest on segment 0
+  const int lane = threadIdx.x & 31, i = I * TILE + lane;
+  const bool vi = i < P.p;
+  const int E1 = P.eta + 1;
+  const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
+  float2 zl = mk(0.f, 0.f), zh = zl;
+  float r = 0.f;
+  if (vi) {
+    if (P.dense) {
+      zl = P.z[(size_t)i * E1 + s]; zh = P.z[(size_t)i * E1 + s + 1];
+    } else {
+      const float4 z4 = P.zseg[(size_t)s * P.p + i];
+      zl = lo2(z4); zh = hi2(z4);
+    }
+    r = P.radius[i];
+  }
+  float res = 0.f;
+  if (f == 0) {
+    if (vi && !P.noenergy) kinetic_factor(P, i, s, zl, zh, pin_lo, pin_hi, res);
+  } else {
+    wall_factor(P, f - 1, i, vi, s, I, zl, zh, r, pin_lo, pin_hi, res);
+  }
+  if (__any_sync(FULL, res > 0.f)) {
+    res = warp_max(res);
+    if (lane == 0 && P.res_prev) atomic_max_nonneg(P.res_prev, res);
   }
 }
 
@@ -372,38 +401,28 @@ __device__ __forceinline__ void tile_of(int nt, int t, int& I, int& J) {
   J = i + (t - tile_pair(nt, i, i));
 }
 
-// Pass 1 of an iteration.  One CTA of 4 warps per (segment s, agent tiles
-// I <= J) block of 32 x 32 collision factors; each warp takes 8 rows, lane =
-// column agent j, and the row agents' data is held one per lane and broadcast
-// by shuffles.  Per row, the warp finishes the pending dual update of the
-// pairs that were active (step 7 of the previous iteration), forms n = z - u
+// Dense state, pass 1: one CTA of TILE / TROWS warps per (segment s, agent
+// tiles I <= J) block of 32 x 32 collision factors; each warp takes TROWS
+// rows (the launch shape the batched autotuner varies), lane = column agent j,
+// and the row agents' data is held one per lane and broadcast by shuffles.
+// Per row, the warp streams the u records of its 32 pairs, finishes the
+// pending dual update (step 7 of the previous iteration), forms n = z - u
 // (step 1), runs the collision test (steps 2-3: weight rho0 or 0), stores the
-// row's activity bits, and appends its active pairs to the global worklist.
-// DENSE streams the u record of every pair (PLAN_DENSE_STATE).
-//
-// Early out (gated state): agent i's segment lies in the disk of centre m_i
-// (its midpoint) and radius h_i (half its length), so the relative segment of
-// a pair stays at distance >= |m_j - m_i| - h_i - h_j from the origin.  Rows
-// where every pair has |m_j - m_i| > (h_i + h_j + r_i + r_j)(1 + 1e-5) cannot
-// collide and skip the exact test; the margin keeps the outcome identical to
-// running the exact test everywhere.
-// TROWS rows per warp, TILE / TROWS warps per block (the launch shape the
-// batched autotuner varies).
-template <bool DENSE, int TROWS>
+// records and the row's activity bits, and appends its active pairs to the
+// global worklist.
+template <int TROWS>
 __device__ __forceinline__ void test_block(const Dev& P, int blk) {
-  constexpr int TEST_ROWS = TROWS;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int E1 = P.eta + 1;
   float res = 0.f;
-  if (blk == 0 && threadIdx.x == 0) *P.res_cur = 0u;
   const int s = blk / P.ntp;
   if (P.vo && s != 0) return;  // no collision factors between x and x_ref
   const int2 IJ = P.tiles[blk - s * P.ntp];
   const int I = IJ.x, J = IJ.y;
   const bool diag = (I == J);
   const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
-  const int r0 = warp * TEST_ROWS;
-  const int nrows = min(TEST_ROWS, P.p - I * TILE - r0);
+  const int r0 = warp * TROWS;
+  const int nrows = min(TROWS, P.p - I * TILE - r0);
   if (nrows > 0) {  // warp-uniform
     // column agent of this lane
     const int j = J * TILE + lane;
@@ -411,7 +430,7 @@ __device__ __forceinline__ void test_block(const Dev& P, int blk) {
     float2 zjl = mk(0.f, 0.f), zjh = zjl;
     float rj = 0.f;
     if (vj) { zjl = P.z[(size_t)j * E1 + s]; zjh = P.z[(size_t)j * E1 + s + 1]; rj = P.radius[j]; }
-    // row agents r0 .. r0 + 7, held by lanes 0 .. 7
+    // row agents, held by the first nrows lanes
     float2 ill = mk(0.f, 0.f), ilh = ill;
     float rl = 0.f;
     uint32_t wordl = 0u;
@@ -420,80 +439,51 @@ __device__ __forceinline__ void test_block(const Dev& P, int blk) {
       ill = P.z[(size_t)il * E1 + s]; ilh = P.z[(size_t)il * E1 + s + 1]; rl = P.radius[il];
       wordl = P.bits[(size_t)blk * TILE + r0 + lane];
     }
-    float2 mj = mk(0.f, 0.f), ml = mj;
-    float bj = 0.f, bl = 0.f;
-    if (!DENSE) {
-      mj = 0.5f * (zjl + zjh);
-      bj = 0.5f * sqrtf(dot(zjh - zjl, zjh - zjl)) + rj;
-      ml = 0.5f * (ill + ilh);
-      bl = 0.5f * sqrtf(dot(ilh - ill, ilh - ill)) + rl;
-    }
 #pragma unroll 2
     for (int q = 0; q < nrows; ++q) {
       const int r = r0 + q;
       const uint32_t word = __shfl_sync(FULL, wordl, q);
       const bool valid = vj && (!diag || r < lane);
       const float ri = __shfl_sync(FULL, rl, q);
-      bool act = false;
       float2 uil = mk(0.f, 0.f), ujl = uil, uih = uil, ujh = uil;
       const size_t row = (size_t)blk * TILE + r;
       const size_t fid = row * TILE + lane;
-      if (!DENSE && word == 0u) {
-        // no pair of this row was active: every u is 0 by the reset rule, n = z
-        const float2 mi = mk(__shfl_sync(FULL, ml.x, q), __shfl_sync(FULL, ml.y, q));
-        const float br = __shfl_sync(FULL, bl, q) + bj;
-        const float2 dm = mj - mi;
-        const bool near = valid && dot(dm, dm) <= br * br * 1.00002f;
-        if (__any_sync(FULL, near)) {
-          const float2 zil = mk(__shfl_sync(FULL, ill.x, q), __shfl_sync(FULL, ill.y, q));
-          const float2 zih = mk(__shfl_sync(FULL, ilh.x, q), __shfl_sync(FULL, ilh.y, q));
-          act = near && collides(zjl - zil, zjh - zih, ri + rj);
-        }
-      } else {
-        const float2 zil = mk(__shfl_sync(FULL, ill.x, q), __shfl_sync(FULL, ill.y, q));
-        const float2 zih = mk(__shfl_sync(FULL, ilh.x, q), __shfl_sync(FULL, ilh.y, q));
-        const bool bprev = (word >> lane) & 1u;  // set only for valid pairs
-        if (DENSE && valid) {
-          const float4 a = P.ulo[fid], b = P.uhi[fid];
-          uil = lo2(a); ujl = hi2(a); uih = lo2(b); ujh = hi2(b);
-        }
-        if (bprev) {
-          // finish step 7 of the previous iteration for this pair
-          const float4 xa = P.xlo[fid], xb = P.xhi[fid];
-          float4 a, b;
-          if (DENSE) { a = pack(uil, ujl); b = pack(uih, ujh); }
-          else { a = P.ulo[fid]; b = P.uhi[fid]; }
-          uil = finish_u(true, pin_lo, false, lo2(a), lo2(xa), zil, P.alpha, res);
-          ujl = finish_u(true, pin_lo, false, hi2(a), hi2(xa), zjl, P.alpha, res);
-          uih = finish_u(true, pin_hi, false, lo2(b), lo2(xb), zih, P.alpha, res);
-          ujh = finish_u(true, pin_hi, false, hi2(b), hi2(xb), zjh, P.alpha, res);
-        } else if (DENSE && P.admm && valid) {
-          // standard ADMM: the pair was feasible, so x^k = z^{k-1} - u^{k-1}
-          const float2 pil = P.z_next[(size_t)(I * TILE + r) * E1 + s];
-          const float2 pih = P.z_next[(size_t)(I * TILE + r) * E1 + s + 1];
-          const float2 pjl = P.z_next[(size_t)j * E1 + s], pjh = P.z_next[(size_t)j * E1 + s + 1];
-          uil = finish_u_feasible(pin_lo, uil, pil, zil, P.alpha, res);
-          ujl = finish_u_feasible(pin_lo, ujl, pjl, zjl, P.alpha, res);
-          uih = finish_u_feasible(pin_hi, uih, pih, zih, P.alpha, res);
-          ujh = finish_u_feasible(pin_hi, ujh, pjh, zjh, P.alpha, res);
-        } else if (DENSE && !P.keep) {
-          uil = ujl = uih = ujh = mk(0.f, 0.f);  // reset rule: inactive edges carry u = 0
-        }
-        if (pin_lo) { uil = mk(0.f, 0.f); ujl = uil; }
-        if (pin_hi) { uih = mk(0.f, 0.f); ujh = uih; }
-        act = valid && collides((zjl - ujl) - (zil - uil), (zjh - ujh) - (zih - uih), ri + rj);
-        if (DENSE && valid) {
-          P.ulo[fid] = pack(uil, ujl);
-          P.uhi[fid] = pack(uih, ujh);
-        }
+      const float2 zil = mk(__shfl_sync(FULL, ill.x, q), __shfl_sync(FULL, ill.y, q));
+      const float2 zih = mk(__shfl_sync(FULL, ilh.x, q), __shfl_sync(FULL, ilh.y, q));
+      const bool bprev = (word >> lane) & 1u;  // set only for valid pairs
+      if (valid) {
+        const float4 a = P.ulo[fid], b = P.uhi[fid];
+        uil = lo2(a); ujl = hi2(a); uih = lo2(b); ujh = hi2(b);
+      }
+      if (bprev) {
+        // finish step 7 of the previous iteration for this pair
+        const float4 xa = P.xlo[fid], xb = P.xhi[fid];
+        uil = finish_u(true, pin_lo, false, uil, lo2(xa), zil, P.alpha, res);
+        ujl = finish_u(true, pin_lo, false, ujl, hi2(xa), zjl, P.alpha, res);
+        uih = finish_u(true, pin_hi, false, uih, lo2(xb), zih, P.alpha, res);
+        ujh = finish_u(true, pin_hi, false, ujh, hi2(xb), zjh, P.alpha, res);
+      } else if (P.admm && valid) {
+        // standard ADMM: the pair was feasible, so x^k = z^{k-1} - u^{k-1}
+        const float2 pil = P.z_next[(size_t)(I * TILE + r) * E1 + s];
+        const float2 pih = P.z_next[(size_t)(I * TILE + r) * E1 + s + 1];
+        const float2 pjl = P.z_next[(size_t)j * E1 + s], pjh = P.z_next[(size_t)j * E1 + s + 1];
+        uil = finish_u_feasible(pin_lo, uil, pil, zil, P.alpha, res);
+        ujl = finish_u_feasible(pin_lo, ujl, pjl, zjl, P.alpha, res);
+        uih = finish_u_feasible(pin_hi, uih, pih, zih, P.alpha, res);
+        ujh = finish_u_feasible(pin_hi, ujh, pjh, zjh, P.alpha, res);
+      } else if (!P.keep) {
+        uil = ujl = uih = ujh = mk(0.f, 0.f);  // reset rule: inactive edges carry u = 0
+      }
+      if (pin_lo) { uil = mk(0.f, 0.f); ujl = uil; }
+      if (pin_hi) { uih = mk(0.f, 0.f); ujh = uih; }
+      const bool act = valid && collides((zjl - ujl) - (zil - uil), (zjh - ujh) - (zih - uih), ri + rj);
+      if (valid) {
+        P.ulo[fid] = pack(uil, ujl);
+        P.uhi[fid] = pack(uih, ujh);
       }
       const uint32_t nword = __ballot_sync(FULL, act);
       if (nword != word && lane == 0) P.bits[row] = nword;
       if (nword) {
-        if (!DENSE && act) {
-          P.ulo[fid] = pack(uil, ujl);
-          P.uhi[fid] = pack(uih, ujh);
-        }
         unsigned base = 0;
         if (lane == 0) base = atomicAdd(P.work_count, (unsigned)__popc(nword));
         base = __shfl_sync(FULL, base, 0);
@@ -505,252 +495,297 @@ __device__ __forceinline__ void test_block(const Dev& P, int blk) {
   if (lane == 0 && res > 0.f && P.res_prev) atomic_max_nonneg(P.res_prev, res);
 }
 
-// Pass 1 of an iteration, gated state, one warp per (segment s, agent tiles
-// I <= J) block with lane = ROW agent i: each lane keeps its row agent in
-// registers and walks the 32 column agents, whose data the warp stages in
-// shared memory (one broadcast 16-byte load per column).  A lane accumulates
-// its row's activity word itself, so a row costs no shuffles, ballots or
-// per-row bookkeeping; the pairs of the row that were active in the last
-// iteration (set bits) are finished first (deferred step 7, exact test on
-// n = z - u), every other valid pair has u = 0 by the reset rule and takes the
-// bounding-circle early out before the exact test.  Same decisions and
-// stores as test_block<false>; only the worklist order differs.
-// col: 64 float4 of shared memory per warp.
-// Bounding-circle filter of pass 1.  Agent i's segment lies in the disk of
-// centre m_i (its midpoint) and radius b_i (half its length plus r_i), so a
-// pair can only collide when |m_i - m_j| <= b_i + b_j, i.e. when
+// Bounding-circle filter of the gated state.  Agent i's segment lies in the
+// disk of centre m_i (its midpoint) and radius b_i (half its length plus
+// r_i), so a pair can only collide when |m_i - m_j| <= b_i + b_j, i.e. when
 //     m_i . m_j + b_i b_j >= Q_i / 2 + Q_j / 2,   Q = |m|^2 - b^2.
 // With a_i = Q_i / 2 - 2e-6 (|m_i|^2 + b_i^2) the test is
-// m_i . m_j + b_i b_j - a_i >= a_j.  The margin, 4e-6 of the magnitudes
+// m_i . m_j + b_i b_j - a_i - a_j >= 0.  The margin, 4e-6 of the magnitudes
 // involved, is about ten times the rounding of the expression and of the
 // bounding radii, so the filter never drops a pair that the exact test would
 // find colliding: the outcome is that of testing every pair exactly.
 __device__ __forceinline__ float bounding_offset(float2 m, float b) {
   const float mm = dot(m, m), bb = b * b;
-  return 0.5f * (mm - bb) - 2e-6f * (mm + bb);
+  return fmaf(-2e-6f, mm + bb, 0.5f * (mm - bb));
 }
 
-// A tile with at least this many exact tests (pairs past the bounding-circle
-// filter plus pairs active before) is listed heavy for the next iteration.
-constexpr unsigned HEAVY_TESTS = 160;
+// The records the factor pass starts from (gated state), of agent i on
+// segment s: both break-points together, and the bounding circle with the
+// offset negated.  Written by the node pass (and after z changed by other
+// means), so that a tile warp loads 16 bytes per agent, coalesced, and
+// derives nothing.
+__device__ __forceinline__ void store_segment(const Dev& P, int i, int s, float2 zl, float2 zh) {
+  const float2 m = 0.5f * (zl + zh), d = zh - zl;
+  const float b = fmaf(0.5f, sqrtf(dot(d, d)), P.radius[i]);
+  const size_t q = (size_t)s * P.p + i;
+  P.zseg[q] = pack(zl, zh);
+  P.circ[q] = make_float4(m.x, m.y, b, -bounding_offset(m, b));
+}
 
-// check_stamp: the tile is skipped when the heavy-tile stamps show that a
-// heavy warp takes it in this iteration.
-__device__ __forceinline__ void test_tile_rows(const Dev& P, int blk, float4* col, uint32_t* nws,
-                                               bool check_stamp = false) {
-  const int lane = threadIdx.x & 31;
-  const int E1 = P.eta + 1;
-  float res = 0.f;
-  const int s = blk / P.ntp;
-  int I, J;
-  tile_of(P.nt, blk - s * P.ntp, I, J);
+// Position of the n-th set bit of w (n counted from 0, less than popc(w)).
+__device__ __forceinline__ int nth_bit(uint32_t w, unsigned n) {
+  int at = 0;
+#pragma unroll
+  for (int k = 16; k > 0; k >>= 1) {
+    const unsigned low = __popc(w & ((1u << k) - 1u));
+    if (n >= low) { n -= low; w >>= k; at += k; }
+  }
+  return at;
+}
+
+// Shared memory of one tile warp: its 32 column agents' circles by
+// component, their segments and radii, and the rows' new activity words.
+struct TileMem {
+  float mx[32], my[32], b[32], na[32], r[32];
+  uint32_t act[32];
+  float4 z[32];
+};
+
+// A pair of one warp item: (i, j) on segment s with slot fid; prev: active in
+// the last iteration.  Finishes its dual update, tests it and, when it is
+// active, runs the minimizer, stores its record and adds its messages to the
+// sums (steps 7, 1-4).  CLASSES: per-node back weights (the feasibility
+// problem).
+template <bool CLASSES>
+__device__ __forceinline__ bool pair_factor(const Dev& P, int s, int i, int j, uint32_t fid,
+                                            bool prev, float& res) {
   const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
-  // Every load the tile starts from is issued here, before any is used: the
-  // column agent and the row agent of this lane, the row's activity word,
-  // the iteration number and the tile's stamp.
-  const int j = J * TILE + lane;
-  const bool vj = j < P.p;
-  float2 zjl = mk(0.f, 0.f), zjh = zjl;
-  float rj = 0.f;
-  if (vj) { zjl = ld_now(P.z + (size_t)j * E1 + s); zjh = ld_now(P.z + (size_t)j * E1 + s + 1); rj = ld_now(P.radius + j); }
-  const int i = I * TILE + lane;
-  const bool vi = i < P.p;
-  const size_t row = (size_t)blk * TILE + lane;
-  float2 zil = mk(0.f, 0.f), zih = zil;
-  float ri = 0.f;
-  uint32_t word = 0u;
-  if (vi) {
-    zil = ld_now(P.z + (size_t)i * E1 + s); zih = ld_now(P.z + (size_t)i * E1 + s + 1); ri = ld_now(P.radius + i);
-    word = ld_now(P.bits + row);
+  const float4 zi = P.zseg[(size_t)s * P.p + i], zj = P.zseg[(size_t)s * P.p + j];
+  const float R = P.radius[i] + P.radius[j];
+  const float scale = P.fix[0], bound = P.fix[1];
+  float2 uil = mk(0.f, 0.f), ujl = uil, uih = uil, ujh = uil;
+  if (prev) {
+    const float4 a = P.ulo[fid], b = P.uhi[fid], xa = P.xlo[fid], xb = P.xhi[fid];
+    uil = finish_u(true, pin_lo, false, lo2(a), lo2(xa), lo2(zi), P.alpha, res);
+    ujl = finish_u(true, pin_lo, false, hi2(a), hi2(xa), lo2(zj), P.alpha, res);
+    uih = finish_u(true, pin_hi, false, lo2(b), lo2(xb), hi2(zi), P.alpha, res);
+    ujh = finish_u(true, pin_hi, false, hi2(b), hi2(xb), hi2(zj), P.alpha, res);
   }
-  const unsigned it = P.hcap ? ld_now(P.iter) : 0u;
-  if (check_stamp && ld_now(P.stamp_cur + blk) == it) return;  // warp-uniform: taken by a heavy warp
-  // column agents: (midpoint, bounding radius, bounding_offset), (z lo, z hi)
-  // and r_j (col holds 72 float4: the last 8 are the 32 radii)
-  float* rcol = reinterpret_cast<float*>(col + 64);
-  {
-    const float2 m = 0.5f * (zjl + zjh);
-    const float b = 0.5f * sqrtf(dot(zjh - zjl, zjh - zjl)) + rj;
-    col[lane] = make_float4(m.x, m.y, b, bounding_offset(m, b));
-    col[32 + lane] = pack(zjl, zjh);
-    rcol[lane] = rj;
+  const float2 nil = lo2(zi) - uil, nih = hi2(zi) - uih, njl = lo2(zj) - ujl, njh = hi2(zj) - ujh;
+  if (!collides(njl - nil, njh - nih, R)) return false;
+  float2 xil, xih, xjl, xjh;
+  if (CLASSES) {
+    int cil, cih, cjl, cjh;
+    end_classes(P, i, s, pin_lo, pin_hi, cil, cih);
+    end_classes(P, j, s, pin_lo, pin_hi, cjl, cjh);
+    coll_minimizer_classes(nil, nih, njl, njh, cil, cih, cjl, cjh, R, P.rho, xil, xih, xjl, xjh);
+  } else {
+    coll_minimizer(nil, nih, njl, njh, pin_lo, pin_hi, R, P.rho, xil, xih, xjl, xjh);
   }
-  const uint32_t vmask = __ballot_sync(FULL, vj);
-  __syncwarp();
-  uint32_t valid = vi ? vmask : 0u;
-  if (I == J) valid &= (lane == 31) ? 0u : (~0u << (lane + 1));  // pairs i < j
-  uint32_t nword = 0u;
-  // pairs active in the last iteration: finish step 7, test n = z - u
-  // exactly.  They are dealt over the whole warp, one pair per lane per
-  // round, so that their u / x loads overlap (a row's own pairs would be
-  // fetched one after another); the activity bits come back through nws.
-  if (__any_sync(FULL, word != 0u)) {
-    unsigned pincl = __popc(word);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v = __shfl_up_sync(FULL, pincl, o);
-      if (lane >= o) pincl += v;
-    }
-    const unsigned ptot = __shfl_sync(FULL, pincl, 31);
-    nws[lane] = 0u;
+  P.ulo[fid] = pack(uil, ujl);
+  P.uhi[fid] = pack(uih, ujh);
+  P.xlo[fid] = pack(xil, xjl);
+  P.xhi[fid] = pack(xih, xjh);
+  if (!pin_lo) {
+    contribute(P, scale, bound, i, s, xil + uil);
+    contribute(P, scale, bound, j, s, xjl + ujl);
+  }
+  if (!pin_hi) {
+    contribute(P, scale, bound, i, s + 1, xih + uih);
+    contribute(P, scale, bound, j, s + 1, xjh + ujh);
+  }
+  return true;
+}
+
+// Activity flag of a worklist entry.  Problems of more than 2^31 slots keep no
+// list (capacity 0: every iteration takes the rebuilding form).
+constexpr uint32_t ACTIVE = 0x80000000u;
+
+// Collision factors of the gated state, one warp.  item < nlist: list warp
+// `item` of nlist takes the chunks of 32 worklist entries item, item + nlist,
+// ...; else tile warp item - nlist takes one 32 x 32 block of pairs.
+//
+// Tile warp: lane = row agent.  The bounding circles of the 32 columns come
+// from shared memory four columns at a time and are tested two columns per
+// instruction; the sign of the result is shifted into the row's word, so a
+// pair costs about four instructions (the scalar form with a compare and a
+// select took seven).  Near pairs that are not on the worklist take the exact
+// test, and those that collide are dealt over the whole warp, one pair per
+// lane per round (row found by a shuffle binary search over the rows' prefix
+// counts), to run the minimizer.  Both kinds of warp share one copy of that
+// code (one loop, one call site): it is most of the kernel's instructions.
+template <bool CLASSES>
+__device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist, TileMem* M) {
+  const int lane = threadIdx.x & 31;
+  const bool rebuild = P.ctl[0] != 0u;
+  const bool lister = item < nlist;
+  float res = 0.f;
+  // list warp
+  unsigned n = 0, chunk = (unsigned)item;
+  int gone = 0;  // entries turned inactive less entries turned active
+  // tile warp
+  int s = 0, I = 0, J = 0, blk = 0, phase = 0;
+  size_t row = 0;
+  uint32_t listed = 0u, todo = 0u, near = 0u;
+  unsigned tincl = 0, total = 0, base = 0;
+  if (lister) {
+    if (rebuild) return;
+    n = *P.work_count_prev;
+  } else {
+    const int nseg = P.vo ? 1 : P.eta;
+    const int t = item - nlist;
+    s = nseg - 1 - t / P.ntp;  // the last segment spans the longest way early in a solve: first
+    const int tp = t - (nseg - 1 - s) * P.ntp;
+    tile_of(P.nt, tp, I, J);
+    blk = s * P.ntp + tp;
+    const int i = I * TILE + lane, j = J * TILE + lane;
+    const bool vi = i < P.p, vj = j < P.p;
+    const size_t so = (size_t)s * P.p;
+    const float4 none = make_float4(0.f, 0.f, 0.f, -INFINITY);
+    const float4 ci = vi ? P.circ[so + i] : none, cj = vj ? P.circ[so + j] : none;
+    row = (size_t)blk * TILE + lane;
+    listed = (rebuild ? P.bits : P.listed)[row];
+    M->mx[lane] = cj.x; M->my[lane] = cj.y; M->b[lane] = cj.z; M->na[lane] = cj.w;
+    uint32_t valid = __ballot_sync(FULL, vj);  // (also orders the stores before the loads below)
     __syncwarp();
-    for (unsigned base = 0; base < ptot; base += 32) {  // warp-uniform
-      const unsigned g = base + lane;
-      int r = 0;  // the row of pair g: the first lane whose inclusive count exceeds g
+    if (!vi) valid = 0u;
+    if (I == J) valid &= (lane == 31) ? 0u : (~0u << (lane + 1));  // pairs i < j
+    const unsigned long long mx = pair_of(ci.x, ci.x), my = pair_of(ci.y, ci.y), b = pair_of(ci.z, ci.z),
+                             na = pair_of(ci.w, ci.w);
+    uint32_t far = 0u;
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1)
-        if (__shfl_sync(FULL, pincl, r + step - 1) <= g) r += step;
-      const uint32_t wr = __shfl_sync(FULL, word, r);
-      const unsigned first = __shfl_sync(FULL, pincl, r) - __popc(wr);
-      const float2 zrl = mk(__shfl_sync(FULL, zil.x, r), __shfl_sync(FULL, zil.y, r));
-      const float2 zrh = mk(__shfl_sync(FULL, zih.x, r), __shfl_sync(FULL, zih.y, r));
-      const float rr = __shfl_sync(FULL, ri, r);
-      if (g < ptot) {
-        uint32_t w = wr;
-        for (unsigned q = first; q < g; ++q) w &= w - 1u;
+    for (int c = TILE - 4; c >= 0; c -= 4) {
+      const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(M->mx + c);
+      const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(M->my + c);
+      const ulonglong2 B = *reinterpret_cast<const ulonglong2*>(M->b + c);
+      const ulonglong2 A = *reinterpret_cast<const ulonglong2*>(M->na + c);
+      const unsigned long long t1 = fma2(mx, X.y, fma2(my, Y.y, fma2(b, B.y, add2(na, A.y))));
+      const unsigned long long t0 = fma2(mx, X.x, fma2(my, Y.x, fma2(b, B.x, add2(na, A.x))));
+      // sign bits, highest column first
+      far = __funnelshift_l((uint32_t)(t1 >> 32), far, 1);
+      far = __funnelshift_l((uint32_t)t1, far, 1);
+      far = __funnelshift_l((uint32_t)(t0 >> 32), far, 1);
+      far = __funnelshift_l((uint32_t)t0, far, 1);
+    }
+    near = ~far & valid & ~listed;
+    M->act[lane] = 0u;
+    todo = rebuild ? listed : 0u;
+    phase = rebuild ? 0 : 1;
+    if (__any_sync(FULL, near != 0u)) {
+      float4 zi = make_float4(0.f, 0.f, 0.f, 0.f), zj = zi;
+      float ri = 0.f, rj = 0.f;
+      if (vi) { zi = P.zseg[so + i]; ri = P.radius[i]; }
+      if (vj) { zj = P.zseg[so + j]; rj = P.radius[j]; }
+      M->z[lane] = zj;
+      M->r[lane] = rj;
+      __syncwarp();
+      uint32_t hit = 0u;
+      for (uint32_t w = near; w; w &= w - 1u) {
         const int c = __ffs(w) - 1;
-        const size_t fid = ((size_t)blk * TILE + r) * TILE + c;
-        const float4 cb = col[32 + c];
-        const float rjc = rcol[c];
-        const float4 a = P.ulo[fid], b = P.uhi[fid], xa = P.xlo[fid], xb = P.xhi[fid];
-        const float2 uil = finish_u(true, pin_lo, false, lo2(a), lo2(xa), zrl, P.alpha, res);
-        const float2 ujl = finish_u(true, pin_lo, false, hi2(a), hi2(xa), lo2(cb), P.alpha, res);
-        const float2 uih = finish_u(true, pin_hi, false, lo2(b), lo2(xb), zrh, P.alpha, res);
-        const float2 ujh = finish_u(true, pin_hi, false, hi2(b), hi2(xb), hi2(cb), P.alpha, res);
-        if (collides((lo2(cb) - ujl) - (zrl - uil), (hi2(cb) - ujh) - (zrh - uih), rr + rjc)) {
-          P.ulo[fid] = pack(uil, ujl);
-          P.uhi[fid] = pack(uih, ujh);
-          atomicOr(&nws[r], 1u << c);
-        }
+        const float4 B = M->z[c];
+        if (collides(lo2(B) - lo2(zi), hi2(B) - hi2(zi), ri + M->r[c])) hit |= 1u << c;
       }
+      near = hit;
     }
     __syncwarp();
-    nword = nws[lane];
   }
-  // every other valid pair: u = 0, n = z.  The bounding circles of all 32
-  // columns first (branch-free), then the exact test on the near ones.
-  const uint32_t rest = valid & ~word;
-  unsigned work = __popc(word);  // exact tests of this row (scheduling of the next iteration)
-  if (__any_sync(FULL, rest != 0u)) {
-    const float2 mi = 0.5f * (zil + zih);
-    const float bi = 0.5f * sqrtf(dot(zih - zil, zih - zil)) + ri;
-    const float ai = bounding_offset(mi, bi);
-    uint32_t near = 0u;
-#pragma unroll
-    for (int c = 0; c < TILE; ++c) {
-      const float4 A = col[c];
-      // m_i . m_j + b_i b_j - a_i >= a_j: three FMAs and a compare per pair
-      const float t = fmaf(mi.x, A.x, fmaf(mi.y, A.y, fmaf(bi, A.z, -ai)));
-      near |= (t >= A.w) ? (1u << c) : 0u;
-    }
-    work += __popc(near & rest);
-    for (near &= rest; near; near &= near - 1u) {
-      const int c = __ffs(near) - 1;
-      const float4 B = col[32 + c];
-      if (collides(lo2(B) - zil, hi2(B) - zih, ri + rcol[c])) {
-        // a newly active pair starts from u = 0 (the slot may hold an old u)
-        const size_t fid = row * TILE + c;
-        P.ulo[fid] = make_float4(0.f, 0.f, 0.f, 0.f);
-        P.uhi[fid] = make_float4(0.f, 0.f, 0.f, 0.f);
-        nword |= 1u << c;
+  for (;;) {
+    // the next 32 pairs
+    int pi = 0, pj = 0, ps = 0, r = 0, c = 0;
+    uint32_t fid = 0u, entry = 0u;
+    bool on = false, prev = false;
+    if (lister) {
+      const unsigned long long t = 32ull * chunk + lane;
+      if (32ull * chunk >= n) break;  // warp-uniform
+      on = t < n;
+      if (on) {
+        entry = P.work[t];
+        fid = entry & ~ACTIVE;
+        prev = (entry & ACTIVE) != 0u;
+        const uint32_t prow = fid >> 5, pblk = prow >> 5;
+        ps = (int)(pblk / (uint32_t)P.ntp);
+        int pI, pJ;
+        tile_of(P.nt, (int)(pblk - (uint32_t)ps * P.ntp), pI, pJ);
+        pi = pI * TILE + (int)(prow & 31);
+        pj = pJ * TILE + (int)(fid & 31);
       }
-    }
-  }
-  if (vi && nword != word) P.bits[row] = nword;
-  // a heavy tile goes first in the next iteration: its slot is claimed here,
-  // so that this atomic and the worklist's below are in flight together
-  unsigned hk = ~0u;
-  if (P.hcap) {
-    const unsigned total = __reduce_add_sync(FULL, work);
-    if (lane == 0 && total >= HEAVY_TESTS) hk = atomicAdd(P.hcount_next, 1u);
-  }
-  // worklist: warp prefix sum of the rows' active counts, one atomic per warp
-  if (__any_sync(FULL, nword != 0u)) {
-    const unsigned cnt = __popc(nword);
-    unsigned incl = cnt;
+    } else {
+      if (base >= total) {  // start a phase: 0 the pairs active before (rebuild), 1 the new ones
+        if (phase > 1) break;
+        if (phase == 1) todo = near;
+        ++phase;
+        tincl = __popc(todo);
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v = __shfl_up_sync(FULL, incl, o);
-      if (lane >= o) incl += v;
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned v = __shfl_up_sync(FULL, tincl, o);
+          if (lane >= o) tincl += v;
+        }
+        total = __shfl_sync(FULL, tincl, 31);
+        base = 0;
+        if (total == 0) continue;
+      }
+      prev = phase == 1;  // (the phase was advanced as it started)
+      const unsigned g = base + lane;
+      base += 32;
+      on = g < total;
+#pragma unroll
+      for (int step = 16; step > 0; step >>= 1)  // the row of pair g: the first whose inclusive count exceeds g
+        if (__shfl_sync(FULL, tincl, r + step - 1) <= g) r += step;
+      const uint32_t wr = __shfl_sync(FULL, todo, r);
+      const unsigned first = __shfl_sync(FULL, tincl, r) - __popc(wr);
+      c = on ? nth_bit(wr, g - first) : 0;
+      ps = s;
+      pi = I * TILE + r;
+      pj = J * TILE + c;
+      fid = (uint32_t)(((size_t)blk * TILE + r) * TILE + c);
     }
-    const unsigned total = __shfl_sync(FULL, incl, 31);
-    unsigned base = 0;
-    if (lane == 31) base = atomicAdd(P.work_count, total);
-    base = __shfl_sync(FULL, base, 31) + (incl - cnt);
-    for (uint32_t w = nword; w; w &= w - 1u) P.work[base++] = (uint32_t)(row * TILE + (__ffs(w) - 1));
+    bool act = false;
+    if (on) act = pair_factor<CLASSES>(P, ps, pi, pj, fid, prev, res);
+    if (lister) {
+      if (on && act != prev) {
+        P.work[32ull * chunk + lane] = fid | (act ? ACTIVE : 0u);
+        const uint32_t bit = 1u << (fid & 31);
+        if (act) atomicOr(P.bits + (fid >> 5), bit); else atomicAnd(P.bits + (fid >> 5), ~bit);
+        gone += act ? -1 : 1;
+      }
+      chunk += (unsigned)nlist;
+    } else if (act) {
+      atomicOr(&M->act[r], 1u << c);
+    }
+  }
+  if (lister) {
+    if (__any_sync(FULL, gone != 0)) {
+      gone = __reduce_add_sync(FULL, gone);
+      if (lane == 0 && gone != 0) atomicAdd(P.ctl + 1, (unsigned)gone);
+    }
+  } else {
+    __syncwarp();
+    const uint32_t nword = M->act[lane];
+    if (rebuild) {
+      if (nword != listed) P.bits[row] = nword;
+      P.listed[row] = nword;
+    } else if (nword) {
+      atomicOr(P.bits + row, nword);
+      P.listed[row] = listed | nword;
+    }
+    if (__any_sync(FULL, nword != 0u)) {  // append: one atomic per warp
+      const unsigned cnt = __popc(nword);
+      unsigned incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const unsigned all = __shfl_sync(FULL, incl, 31);
+      unsigned at = 0;
+      if (lane == 31) {
+        at = atomicAdd(P.work_count, all);
+        if ((unsigned long long)at + all > P.cap) atomicOr(P.ctl + 2, 1u);
+      }
+      at = __shfl_sync(FULL, at, 31) + (incl - cnt);
+      for (uint32_t w = nword; w; w &= w - 1u, ++at)
+        if (at < P.cap) P.work[at] = (uint32_t)(row * TILE + (__ffs(w) - 1)) | ACTIVE;
+    }
   }
   if (__any_sync(FULL, res > 0.f)) {  // only pairs active before have a residual
     res = warp_max(res);
     if (lane == 0 && P.res_prev) atomic_max_nonneg(P.res_prev, res);
   }
-  if (hk < (unsigned)P.hcap) {  // lane 0 of a heavy tile with a free slot
-    P.heavy_next[hk] = (uint32_t)blk;
-    P.stamp_next[blk] = it + 1u;
-  }
 }
 
-// Kinetic and wall factors (steps 1-3 and the pending step 7) of one segment
-// s and one agent tile: warp f < 1 + n_walls takes factor kind f (0 =
-// kinetic, else wall f - 1), lane = agent.  DEFER: see wall_factor.
-template <bool DEFER>
-__device__ __forceinline__ void segment_block(const Dev& P, int blk) {
-  const int s = blk / P.nt;
-  const int I = blk - s * P.nt;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = I * TILE + lane;
-  const bool vi = i < P.p;
-  const int E1 = P.eta + 1;
-  const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
-  float2 zl = mk(0.f, 0.f), zh = zl;
-  float r = 0.f;
-  if (vi) { zl = P.z[(size_t)i * E1 + s]; zh = P.z[(size_t)i * E1 + s + 1]; r = P.radius[i]; }
-  float res = 0.f;
-  for (int f = warp; f < 1 + P.nw + P.nv; f += blockDim.x >> 5) {
-    if (f == 0) {
-      if (vi && !P.noenergy && !(P.vo && s == 0)) kinetic_factor(P, i, s, zl, zh, pin_lo, pin_hi, res);
-    } else if (!(P.vo && s != 0)) {
-      wall_factor<DEFER>(P, f - 1, i, vi, s, I, zl, zh, r, pin_lo, pin_hi, res);
-    }
-  }
-  res = warp_max(res);
-  if (lane == 0 && res > 0.f && P.res_prev) atomic_max_nonneg(P.res_prev, res);
-}
-
-// The capsule minimizer (Eq. wall_minimizer) of one active wall factor from
-// the wall worklist, with the u that its segment block finished (so n = z - u
-// is the value it tested).  Called by all 32 lanes of a warp with the same
-// item: both ends free (the common case) shares the candidate solves out
-// over the lanes; lane 0 stores the result.
-__device__ __forceinline__ void wall_prox_item_warp(const Dev& P, uint32_t idx) {
-  const uint32_t i = idx % (uint32_t)P.p, ws = idx / (uint32_t)P.p;
-  const int s = (int)(ws % (uint32_t)P.eta), w = (int)(ws / (uint32_t)P.eta);
-  const int E1 = P.eta + 1;
-  const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
-  const float4 u4 = P.uwall[idx];
-  const float2 ul = lo2(u4), uh = hi2(u4);
-  const float2 nl = P.z[(size_t)i * E1 + s] - ul, nh = P.z[(size_t)i * E1 + s + 1] - uh;
-  const float4 W = P.walls[w];
-  const float2 c0 = mk(W.x, W.y), c1 = mk(W.z, W.w);
-  const float r = P.radius[i];
-  int cl, ch;
-  end_classes(P, (int)i, s, pin_lo, pin_hi, cl, ch);
-  float2 xl = nl, xh = nh;
-  bool ok = true;
-  if (cl == 1 && ch == 1) {
-    const float wgt = 0.5f * P.rho;
-    capsule_prox_free_warp(nl, nh, wgt, wgt, c0, c1, r, xl, xh);
-  } else {
-    ok = capsule_prox_classes(nl, nh, cl, ch, c0, c1, r, 0.5f * P.rho, xl, xh);
-  }
-  if ((threadIdx.x & 31) != 0) return;
-  if (!ok) atomicOr(P.status, 1u);
-  P.xwall[idx] = pack(xl, xh);
-  if (!pin_lo) contribute(P, (int)i, s, xl + ul);
-  if (!pin_hi) contribute(P, (int)i, s + 1, xh + uh);
-}
-
-// Pass 2: the collision minimizer (Eq. coll_minimizer_problem through
-// App. C/D/I) of every active pair in the worklist, one thread per pair.
+// Dense state, pass 2: the collision minimizer (Eq. coll_minimizer_problem
+// through App. C/D/I) of every active pair in the worklist, one thread per
+// pair.
 __device__ __forceinline__ void prox_item(const Dev& P, uint32_t fid) {
   const int E1 = P.eta + 1;
   const uint32_t row = fid >> 5, c = fid & 31;
@@ -787,20 +822,14 @@ __device__ __forceinline__ void prox_item(const Dev& P, uint32_t fid) {
   }
 }
 
-// Pass 3 (steps 5-6): z = sum(rho m) / sum(rho) per free break-point from the
+// Steps 5-6 for one free break-point: z = sum(rho m) / sum(rho) from the
 // fixed-point sums (every weight is rho0, so z is the mean of the incoming m;
 // no incoming weight means z is unchanged).  Clears the sums for the next
 // iteration.
-__device__ __forceinline__ void consensus_node(const Dev& P, int t, float& dz, bool& bad) {
-  // consecutive threads take consecutive break-points of one agent, which
-  // are adjacent in the [p][eta+1] arrays (coalesced)
-  const int i = t / (P.eta - 1);
-  const int sp = 1 + (t - i * (P.eta - 1));
-  const size_t node = (size_t)i * (P.eta + 1) + sp;
-  const unsigned status = *P.status;  // issued with the sums, not after them
+__device__ __forceinline__ float2 consensus_node(const Dev& P, size_t node, float2 zo, unsigned status,
+                                                 float& dz, bool& bad) {
   const long long sx = (long long)P.accx[node], sy = (long long)P.accy[node];
   const unsigned cnt = P.accc[node];
-  const float2 zo = P.z[node];  // every load before the stores, so that they overlap
   P.accx[node] = 0ull;
   P.accy[node] = 0ull;
   P.accc[node] = 0u;
@@ -821,8 +850,11 @@ __device__ __forceinline__ void consensus_node(const Dev& P, int t, float& dz, b
   // step 6: the back weight is rho0 where some factor sent rho0, else 0
   if (P.noenergy) P.wnode[node] = cnt > 0u ? 1 : 0;
   P.z_next[node] = zn;
-  bad = (status & 2u) != 0u || !(fabsf(zn.x - zo.x) + fabsf(zn.y - zo.y) >= 0.f);
-  dz = bad ? 0.f : maxabs2(zn - zo);
+  const float2 d = zn - zo;
+  const bool odd = (status & 2u) != 0u || !(fabsf(d.x) + fabsf(d.y) >= 0.f);
+  bad |= odd;
+  if (!odd) dz = fmaxf(dz, maxabs2(d));
+  return zn;
 }
 
 // Warp-level end of the consensus pass: a NaN or overflow anywhere makes the
@@ -834,6 +866,69 @@ __device__ __forceinline__ void consensus_reduce(const Dev& P, float dz, bool ba
     if (anybad) atomicMax(P.res_cur, 0x7fc00000u);
     else if (dz > 0.f) atomic_max_nonneg(P.res_cur, dz);
   }
+}
+
+// Agents a node warp takes: as many whole agents as fit its 32 lanes.
+__host__ __device__ __forceinline__ int agents_per_warp(int eta) { return eta + 1 <= 32 ? 32 / (eta + 1) : 1; }
+
+// Node pass of one warp: every break-point of its agents, lane = break-point
+// (consecutive in the [p][eta+1] arrays, so coalesced), longer agents in
+// rounds of 32 from the far end.  A lane gets the next break-point's z from
+// its neighbour and writes the segment records of the next factor pass.
+__device__ __forceinline__ void consensus_warp(const Dev& P, int warp) {
+  const int lane = threadIdx.x & 31, E1 = P.eta + 1, apw = agents_per_warp(P.eta);
+  const unsigned status = *P.status;
+  float dz = 0.f;
+  bool bad = false;
+  if (E1 <= 32) {
+    const int a = lane / E1, s = lane - a * E1, i = warp * apw + a;
+    const bool on = a < apw && i < P.p;
+    float2 z = mk(0.f, 0.f);
+    if (on) {
+      const size_t node = (size_t)i * E1 + s;
+      z = P.z[node];
+      if (s > 0 && s < P.eta) z = consensus_node(P, node, z, status, dz, bad);
+    }
+    const float2 zh = mk(__shfl_down_sync(FULL, z.x, 1), __shfl_down_sync(FULL, z.y, 1));
+    if (on && s < P.eta && !P.dense) store_segment(P, i, s, z, zh);
+  } else if (warp < P.p) {
+    float2 next = mk(0.f, 0.f);  // z of the round's far neighbour
+    for (int s0 = (P.eta / 32) * 32; s0 >= 0; s0 -= 32) {
+      const int s = s0 + lane;
+      const size_t node = (size_t)warp * E1 + s;
+      float2 z = mk(0.f, 0.f);
+      if (s <= P.eta) {
+        z = P.z[node];
+        if (s > 0 && s < P.eta) z = consensus_node(P, node, z, status, dz, bad);
+      }
+      float2 zh = mk(__shfl_down_sync(FULL, z.x, 1), __shfl_down_sync(FULL, z.y, 1));
+      if (lane == 31) zh = next;
+      if (s < P.eta && !P.dense) store_segment(P, warp, s, z, zh);
+      next = mk(__shfl_sync(FULL, z.x, 0), __shfl_sync(FULL, z.y, 0));
+    }
+  }
+  consensus_reduce(P, dz, bad);
+}
+
+// Node warps of a problem.
+__host__ __device__ __forceinline__ int node_warps(int p, int eta) {
+  const int apw = agents_per_warp(eta);
+  return (p + apw - 1) / apw;
+}
+
+// The worklist's length and mode for the next iteration, by one thread of
+// the node pass.  frozen: the problem took no factor pass.
+__device__ __forceinline__ void advance_worklist(const Dev& P, bool frozen) {
+  unsigned n = *P.work_count;
+  if (P.dense) n = 0u;  // the dense state's list is that of one iteration
+  else if (!frozen) {
+    // half of the list inactive (and more than a few warps' worth), or longer
+    // than it fits, or slots that a list entry cannot hold
+    const bool again = P.ctl[2] != 0u || 2u * P.ctl[1] > n + 1024u || P.cap == 0u;
+    P.ctl[0] = again ? 1u : 0u;
+    if (again) { n = 0u; P.ctl[1] = 0u; P.ctl[2] = 0u; }
+  }
+  *P.work_count_prev = n;  // the next iteration appends to the other parity's counter
 }
 
 }  // namespace

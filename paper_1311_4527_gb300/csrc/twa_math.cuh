@@ -60,14 +60,19 @@ TWA_DEV float2 operator+(float2 a, float2 b) { return mk(a.x + b.x, a.y + b.y); 
 TWA_DEV float2 operator-(float2 a, float2 b) { return mk(a.x - b.x, a.y - b.y); }
 TWA_DEV float2 operator-(float2 a) { return mk(-a.x, -a.y); }
 TWA_DEV float2 operator*(float s, float2 a) { return mk(s * a.x, s * a.y); }
-TWA_DEV float dot(float2 a, float2 b) { return a.x * b.x + a.y * b.y; }
-TWA_DEV float cross(float2 a, float2 b) { return a.x * b.y - a.y * b.x; }
+// The library is compiled without implicit multiply-add fusion: which pairs
+// the compiler fuses depends on the code around an inlined function, and the
+// same factor has to round alike in every kernel that computes it.  The fused
+// operations are written out instead.
+TWA_DEV float dot(float2 a, float2 b) { return fmaf(a.x, b.x, a.y * b.y); }
+TWA_DEV float cross(float2 a, float2 b) { return fmaf(a.x, b.y, -(a.y * b.x)); }
+TWA_DEV float2 axpy(float s, float2 a, float2 b) { return mk(fmaf(s, a.x, b.x), fmaf(s, a.y, b.y)); }  // s a + b
 TWA_DEV float2 perp(float2 a) { return mk(-a.y, a.x); }
 TWA_DEV float2 normalized(float2 a) {
 #ifdef __CUDA_ARCH__
   // one reciprocal square root (2 ulp) where |a|^2 is a normal float; the
   // directions are unit to a few ulp either way
-  const float dd = a.x * a.x + a.y * a.y;
+  const float dd = dot(a, a);
   if (dd > 1e-30f && dd < 1e30f) {
     const float s = rsqrtf(dd);
     return mk(a.x * s, a.y * s);
@@ -165,23 +170,24 @@ struct Best {
 TWA_DEV void energy_prox(float2 n_lo, float2 n_hi, float rho, bool pin_lo, bool pin_hi, float c,
                          float2& x_lo, float2& x_hi) {
   if (pin_lo && pin_hi) { x_lo = n_lo; x_hi = n_hi; return; }
+  const float c2 = 2.f * c;
   if (pin_lo) {
     x_lo = n_lo;
-    float inv = 1.f / (2.f * c + rho);
-    x_hi = mk((rho * n_hi.x + 2.f * c * n_lo.x) * inv, (rho * n_hi.y + 2.f * c * n_lo.y) * inv);
+    const float inv = 1.f / (c2 + rho);
+    x_hi = inv * axpy(rho, n_hi, c2 * n_lo);
     return;
   }
   if (pin_hi) {
     x_hi = n_hi;
-    float inv = 1.f / (2.f * c + rho);
-    x_lo = mk((rho * n_lo.x + 2.f * c * n_hi.x) * inv, (rho * n_lo.y + 2.f * c * n_hi.y) * inv);
+    const float inv = 1.f / (c2 + rho);
+    x_lo = inv * axpy(rho, n_lo, c2 * n_hi);
     return;
   }
   // equal weights rho on both ends
-  float inv = 1.f / (4.f * c + rho);
-  float2 s = n_lo + n_hi;
-  x_lo = mk((rho * n_lo.x + 2.f * c * s.x) * inv, (rho * n_lo.y + 2.f * c * s.y) * inv);
-  x_hi = mk((rho * n_hi.x + 2.f * c * s.x) * inv, (rho * n_hi.y + 2.f * c * s.y) * inv);
+  const float inv = 1.f / fmaf(4.f, c, rho);
+  const float2 s = c2 * (n_lo + n_hi);
+  x_lo = inv * axpy(rho, n_lo, s);
+  x_hi = inv * axpy(rho, n_hi, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -189,17 +195,18 @@ TWA_DEV void energy_prox(float2 n_lo, float2 n_hi, float rho, bool pin_lo, bool 
 // ---------------------------------------------------------------------------
 TWA_DEV float hinge_E(float2 a, float2 b, float wl, float wh, float R, float2 n) {
   float ga = fmaxf(R - dot(a, n), 0.f), gb = fmaxf(R - dot(b, n), 0.f);
-  return 0.5f * wl * ga * ga + 0.5f * wh * gb * gb;
+  return fmaf(0.5f * wl * ga, ga, 0.5f * wh * gb * gb);
 }
 
 // Global minimiser(s) of f(n) = wl (R - <a,n>)^2 + wh (R - <b,n>)^2 on the
 // unit circle.  Writes 1 or 2 directions (2 only for exact ties).
 TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
                                        float2* out) {
-  float m11 = wl * a.x * a.x + wh * b.x * b.x;
-  float m22 = wl * a.y * a.y + wh * b.y * b.y;
-  float m12 = wl * a.x * a.y + wh * b.x * b.y;
-  float2 S = mk(wl * a.x + wh * b.x, wl * a.y + wh * b.y);
+  const float2 wa = wl * a, wb = wh * b;
+  float m11 = fmaf(wa.x, a.x, wb.x * b.x);
+  float m22 = fmaf(wa.y, a.y, wb.y * b.y);
+  float m12 = fmaf(wa.x, a.y, wb.x * b.y);
+  float2 S = wa + wb;
   float hd = 0.5f * (m11 - m22);
   float disc = hypotf(hd, m12);
   float d = 2.f * disc;  // lambda2 - lambda1 >= 0
@@ -214,9 +221,9 @@ TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
   float A1 = R * fabsf(s1), A2 = R * fabsf(s2);
   if (A1 <= 1e-7f * R * Sn && A2 < d) {  // hard case: t = 0
     float n2 = R * s2 / d;
-    float n1 = sqrtf(fmaxf(0.f, 1.f - n2 * n2));
-    out[0] = n1 * e1 + n2 * e2;
-    out[1] = (-n1) * e1 + n2 * e2;
+    float n1 = sqrtf(fmaxf(0.f, fmaf(-n2, n2, 1.f)));
+    out[0] = axpy(n1, e1, n2 * e2);
+    out[1] = axpy(-n1, e1, n2 * e2);
     return 2;
   }
   // Root of h(t) = phi(t)^{-1/2} - 1 with phi = (A1/t)^2 + (A2/(d+t))^2.
@@ -229,12 +236,12 @@ TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
     TWA_ITER_HOOK(0);
     float it_ = fdiv(1.f, t), id = fdiv(1.f, d + t);
     float q1 = A1 * it_, q2 = A2 * id;
-    float phi = q1 * q1 + q2 * q2;
+    float phi = fmaf(q1, q1, q2 * q2);
     float ip = frsqrt(phi);
     float h = ip - 1.f;
     if (h > 0.f) hi = t; else lo = t;
     if (h == 0.f) break;
-    float dh = ip * ip * ip * (q1 * q1 * it_ + q2 * q2 * id);
+    float dh = ip * ip * ip * fmaf(q1 * q1, it_, q2 * q2 * id);
     float tn = t - fdiv(h, dh);
     if (!(tn > lo && tn < hi)) tn = 0.5f * (lo + hi);
     // FP32 noise in h limits t to ~1e-7 relative; stop at 1e-6
@@ -246,12 +253,12 @@ TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
   float n1, n2;
   if (fabsf(p1) <= fabsf(p2)) {
     n1 = p1;
-    n2 = copysignf(sqrtf(fmaxf(0.f, 1.f - p1 * p1)), s2);
+    n2 = copysignf(sqrtf(fmaxf(0.f, fmaf(-p1, p1, 1.f))), s2);
   } else {
     n2 = p2;
-    n1 = copysignf(sqrtf(fmaxf(0.f, 1.f - p2 * p2)), s1);
+    n1 = copysignf(sqrtf(fmaxf(0.f, fmaf(-p2, p2, 1.f))), s1);
   }
-  out[0] = normalized(n1 * e1 + n2 * e2);
+  out[0] = normalized(axpy(n1, e1, n2 * e2));
   return 1;
 }
 
@@ -267,10 +274,11 @@ TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
 // split the work over threads; -1 writes all.
 TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, float2* out,
                            int part = -1) {
-  float m11 = wl * a.x * a.x + wh * b.x * b.x;
-  float m22 = wl * a.y * a.y + wh * b.y * b.y;
-  float m12 = wl * a.x * a.y + wh * b.x * b.y;
-  float2 S = mk(wl * a.x + wh * b.x, wl * a.y + wh * b.y);
+  const float2 wa = wl * a, wb = wh * b;
+  float m11 = fmaf(wa.x, a.x, wb.x * b.x);
+  float m22 = fmaf(wa.y, a.y, wb.y * b.y);
+  float m12 = fmaf(wa.x, a.y, wb.x * b.y);
+  float2 S = wa + wb;
   float hd = 0.5f * (m11 - m22);
   float disc = hypotf(hd, m12);
   float d = 2.f * disc;
@@ -285,9 +293,9 @@ TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, floa
   if (A2 == 0.f) {  // hard case at mu = lambda2, and the root t = A1
     if (A1 < d) {
       float n1 = -R * s1 / d;
-      float n2 = sqrtf(fmaxf(0.f, 1.f - n1 * n1));
-      out[0] = n1 * e1 + n2 * e2;
-      out[1] = n1 * e1 + (-n2) * e2;
+      float n2 = sqrtf(fmaxf(0.f, fmaf(-n1, n1, 1.f)));
+      out[0] = axpy(n1, e1, n2 * e2);
+      out[1] = axpy(n1, e1, (-n2) * e2);
       out[2] = (s1 > 0.f ? -1.f : 1.f) * e1;
       n = 3;
     }
@@ -299,7 +307,8 @@ TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, floa
   }
   float c1 = cbrtf(A1 * A1), c2 = cbrtf(A2 * A2);
   float tm = d * c1 / (c1 + c2);
-  float phim = (A1 / tm) * (A1 / tm) + (A2 / (d - tm)) * (A2 / (d - tm));
+  const float r1 = A1 / tm, r2 = A2 / (d - tm);
+  float phim = fmaf(r1, r1, r2 * r2);
   if (!(phim <= 1.f)) return 0;
   for (int side = (part == 1) ? 1 : 0; side < ((part == 0) ? 1 : 2); ++side) {
     // h(t) = phi(t)^(-1/2) - 1 is increasing on (0, tm] and decreasing on
@@ -312,13 +321,13 @@ TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, floa
       TWA_ITER_HOOK(1);
       float it_ = fdiv(1.f, t), id = fdiv(1.f, d - t);
       float q1 = A1 * it_, q2 = A2 * id;
-      float phi = q1 * q1 + q2 * q2;
+      float phi = fmaf(q1, q1, q2 * q2);
       float ip = frsqrt(phi);
       float h = ip - 1.f;
       bool right = side ? (h < 0.f) : (h > 0.f);  // root lies left of t
       if (right) hi = t; else lo = t;
       if (h == 0.f || hi - lo <= 1e-6f * hi) break;
-      float dphi = -2.f * (q1 * q1 * it_) + 2.f * (q2 * q2 * id);
+      float dphi = 2.f * fmaf(q2 * q2, id, -(q1 * q1 * it_));
       float dh = -0.5f * ip * ip * ip * dphi;
       float tn = (dh != 0.f) ? t - fdiv(h, dh) : 0.5f * (lo + hi);
       if (!(tn > lo && tn < hi)) tn = 0.5f * (lo + hi);
@@ -328,9 +337,9 @@ TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, floa
     }
     float p1 = fdiv(-R * s1, t), p2 = fdiv(R * s2, d - t);
     float n1, n2;
-    if (fabsf(p1) <= fabsf(p2)) { n1 = p1; n2 = copysignf(sqrtf(fmaxf(0.f, 1.f - p1 * p1)), p2); }
-    else { n2 = p2; n1 = copysignf(sqrtf(fmaxf(0.f, 1.f - p2 * p2)), p1); }
-    put_dir(out, n, normalized(n1 * e1 + n2 * e2));
+    if (fabsf(p1) <= fabsf(p2)) { n1 = p1; n2 = copysignf(sqrtf(fmaxf(0.f, fmaf(-p1, p1, 1.f))), p2); }
+    else { n2 = p2; n1 = copysignf(sqrtf(fmaxf(0.f, fmaf(-p2, p2, 1.f))), p1); }
+    put_dir(out, n, normalized(axpy(n1, e1, n2 * e2)));
   }
   return n;
 }
@@ -338,11 +347,11 @@ TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, floa
 // Tangent normals n with <q, n> = R from a point q (|q| >= R).
 TWA_DEV void tangent_normals(float2 q, float R, float2& t0, float2& t1) {
   float L2 = dot(q, q);
-  float s = sqrtf(fmaxf(L2 - R * R, 0.f));
+  float s = sqrtf(fmaxf(fmaf(-R, R, L2), 0.f));
   float inv = fdiv(1.f, L2);
-  float2 pq = perp(q);
-  t0 = mk((R * q.x + s * pq.x) * inv, (R * q.y + s * pq.y) * inv);
-  t1 = mk((R * q.x - s * pq.x) * inv, (R * q.y - s * pq.y) * inv);
+  float2 pq = perp(q), Rq = R * q;
+  t0 = inv * axpy(s, pq, Rq);
+  t1 = inv * axpy(-s, pq, Rq);
 }
 
 // Direction in the arc {n : <q,n> >= R} (|q| >= R) maximising <w, n>.
@@ -409,15 +418,15 @@ TWA_NOINLINE void disk_prox_free(float2 a, float2 b, float wl, float wh, float R
                                             float2& vl, float2& vh) {
   int tag;
   float2 n = disk_dir_free(a, b, wl, wh, R, tag);
-  vl = a + fmaxf(R - dot(a, n), 0.f) * n;
-  vh = b + fmaxf(R - dot(b, n), 0.f) * n;
+  vl = axpy(fmaxf(R - dot(a, n), 0.f), n, a);
+  vh = axpy(fmaxf(R - dot(b, n), 0.f), n, b);
 }
 
 // One end pinned at q (weight infinite): the free end's target is w.  The
 // separating direction ranges over the arc {<q,n> >= R}.
 TWA_NOINLINE float2 disk_prox_pinned(float2 q, float2 w, float R) {
   float2 n = arc_argmax(q, R, w);
-  return w + fmaxf(R - dot(w, n), 0.f) * n;
+  return axpy(fmaxf(R - dot(w, n), 0.f), n, w);
 }
 
 // ---------------------------------------------------------------------------
@@ -431,7 +440,7 @@ TWA_DEV float capsule_E(float2 a, float2 b, float wl, float wh, float2 c0, float
                         float2 n) {
   float h = capsule_h(c0, c1, r, n);
   float ga = fmaxf(h - dot(a, n), 0.f), gb = fmaxf(h - dot(b, n), 0.f);
-  return 0.5f * wl * ga * ga + 0.5f * wh * gb * gb;
+  return fmaf(0.5f * wl * ga, ga, 0.5f * wh * gb * gb);
 }
 
 // On the half-plane of directions where end circle ci gives the capsule's
@@ -512,8 +521,8 @@ TWA_NOINLINE void capsule_prox_free(float2 a, float2 b, float wl, float wh, floa
   int tag;
   float2 n = capsule_dir_free(a, b, wl, wh, c0, c1, r, tag);
   float h = capsule_h(c0, c1, r, n);
-  vl = a + fmaxf(h - dot(a, n), 0.f) * n;
-  vh = b + fmaxf(h - dot(b, n), 0.f) * n;
+  vl = axpy(fmaxf(h - dot(a, n), 0.f), n, a);
+  vh = axpy(fmaxf(h - dot(b, n), 0.f), n, b);
 }
 
 #ifdef __CUDACC__
@@ -585,8 +594,8 @@ __device__ __forceinline__ void capsule_prox_free_warp(float2 a, float2 b, float
     if (take) { E = E2; n = mk(nx, ny); src = src2; }
   }
   const float h = capsule_h(c0, c1, r, n);
-  vl = a + fmaxf(h - dot(a, n), 0.f) * n;
-  vh = b + fmaxf(h - dot(b, n), 0.f) * n;
+  vl = axpy(fmaxf(h - dot(a, n), 0.f), n, a);
+  vh = axpy(fmaxf(h - dot(b, n), 0.f), n, b);
 }
 #endif
 
@@ -641,7 +650,7 @@ TWA_NOINLINE bool capsule_prox_pinned(float2 q, float2 w, float2 c0, float2 c1, 
   int tag;
   if (!capsule_dir_pinned(q, w, c0, c1, r, n, tag)) { vw = w; return false; }
   float h = capsule_h(c0, c1, r, n);
-  vw = w + fmaxf(h - dot(w, n), 0.f) * n;
+  vw = axpy(fmaxf(h - dot(w, n), 0.f), n, w);
   return true;
 }
 
@@ -669,14 +678,14 @@ TWA_DEV float2 capsule_project_out(float2 q, float2 c0, float2 c1, float r) {
   const float ee = dot(e, e);
   float t = ee > 0.f ? dot(q - c0, e) / ee : 0.f;
   t = fminf(1.f, fmaxf(0.f, t));
-  const float2 c = c0 + t * e;
+  const float2 c = axpy(t, e, c0);
   const float2 d = q - c;
   const float L = hypotf(d.x, d.y);
   if (L >= r) return q;
-  if (L > 0.f) return c + (r / L) * d;
+  if (L > 0.f) return axpy(r / L, d, c);
   if (!(ee > 0.f)) return c + mk(r, 0.f);
   const float2 n1 = normalized(perp(e));
-  return c + r * ((angle_of(n1) < angle_of(-n1)) ? n1 : -n1);
+  return axpy(r, (angle_of(n1) < angle_of(-n1)) ? n1 : -n1, c);
 }
 
 // Disk minimizer for weight classes (cl, ch) of the two ends of the relative
@@ -725,11 +734,11 @@ TWA_DEV void velocity_prox(float2 n_lo, float2 n_hi, int cl, int ch, float C, fl
   const float2 d = n_lo - n_hi;
   const float L = hypotf(d.x, d.y);
   const float2 u = L > 0.f ? (1.f / L) * d : mk(-1.f, 0.f);
-  if (cl == 2 || (ch == 0 && cl != 0)) { x_hi = n_lo - C * u; return; }
-  if (ch == 2 || (cl == 0 && ch != 0)) { x_lo = n_hi + C * u; return; }
+  if (cl == 2 || (ch == 0 && cl != 0)) { x_hi = axpy(-C, u, n_lo); return; }
+  if (ch == 2 || (cl == 0 && ch != 0)) { x_lo = axpy(C, u, n_hi); return; }
   const float2 m = 0.5f * (n_lo + n_hi);
-  x_lo = m + (0.5f * C) * u;
-  x_hi = m - (0.5f * C) * u;
+  x_lo = axpy(0.5f * C, u, m);
+  x_hi = axpy(-0.5f * C, u, m);
 }
 
 }  // namespace twa
