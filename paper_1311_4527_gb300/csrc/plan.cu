@@ -172,6 +172,11 @@ __global__ void fix_kernel(Dev P, const float2* start, const float2* goal) {
 // velo_cost_pair_wise, Eq. basic_opt_prob) on the FP32 break-points z^k.
 // Smallest clearances are kept as squared ratios; a non-negative double's bit
 // pattern orders like the double, so 64-bit atomicMin takes their minimum.
+// FP64 runs at a sixty-fourth of the FP32 rate here, and one FP64 test of
+// every pair and segment (8.4 M at p = 1024, eta = 16) took 720 of the
+// check's 845 us.  Only a pair that can be its block's closest needs it: FP32
+// gives every distance with a bound on its error, and the pairs whose lower
+// bound is above the block's least upper bound are left at that.
 
 // Squared distance from the origin to the segment a -> b.
 __device__ __forceinline__ double origin_seg_dist2(double ax, double ay, double bx, double by) {
@@ -182,44 +187,83 @@ __device__ __forceinline__ double origin_seg_dist2(double ax, double ay, double 
   return fma(cx, cx, cy * cy);
 }
 
-__device__ __forceinline__ void block_min_u64(unsigned long long v, unsigned long long* out) {
-  __shared__ unsigned long long red[32];
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-    v = w < v ? w : v;
+// Distance bounds of one ratio in FP32: the distance of the origin from the
+// segment cl -> ch (or any other distance d found from coordinates of size
+// mag), with an error of at most 4e-6 mag (sixty times the rounding of one
+// operation on such coordinates, of which the distance takes about ten), over
+// the radius sum R.  Beyond the range where FP32 squares are safe the bounds
+// are those that always ask for FP64.
+struct Bounds { float lo, hi; };
+__device__ __forceinline__ Bounds ratio_bounds(float d, float mag, float R) {
+  Bounds b = {-1.f, INFINITY};
+  if (mag < 1e15f && d < INFINITY) {
+    const float err = fmaf(4e-6f, mag, 1e-18f);
+    b.lo = (d - err) / R * 0.999999f;
+    b.hi = (d + err) / R * 1.000001f;
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    v = lane < (int)(blockDim.x >> 5) ? red[lane] : ~0ull;
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-      v = w < v ? w : v;
-    }
-    if (lane == 0 && v != ~0ull) atomicMin(out, v);  // nothing to report: no atomic
-  }
+  return b;
 }
 
-// One block per (segment s, agent tile pair): min over its pairs i < j of
-// dist^2 / (r_i + r_j)^2, dist the smallest distance between the agents
-// over the segment (the origin against their relative motion).
-__global__ void check_pairs_kernel(Dev P, unsigned long long* out) {
-  const int s = blockIdx.x / P.ntp, tp = blockIdx.x - s * P.ntp;
+// The least of a value over the block's threads, to all of them.
+__device__ __forceinline__ float block_min(float v) {
+  __shared__ float red[32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(FULL, v, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = red[0];
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = fminf(v, red[w]);
+  return v;
+}
+
+// An upper bound of the smallest ratio found so far by any block.
+__device__ __forceinline__ float least_so_far(const unsigned long long* out) {
+  return sqrtf((float)__longlong_as_double((long long)__ldcg(out))) * 1.000001f;
+}
+
+// A candidate's squared ratio into the global minimum.
+__device__ __forceinline__ void offer_ratio(double q, unsigned long long* out) {
+  const unsigned long long v = (unsigned long long)__double_as_longlong(q);
+  if (q >= 0.0 && v < __ldcg(out)) atomicMin(out, v);
+}
+
+// Pairs of one (segment s, agent tile pair): min over i < j of
+// dist^2 / (r_i + r_j)^2, dist the smallest distance between the agents over
+// the segment (the origin against their relative motion).  256 threads, four
+// rows each, lane = column.
+__device__ __forceinline__ void check_pairs(const Dev& P, int block, unsigned long long* out) {
+  constexpr int PER = TILE * TILE / 256;
+  const int s = block / P.ntp, tp = block - s * P.ntp;
   const int2 IJ = P.tiles[tp];
   const int E1 = P.eta + 1;
-  double best = __longlong_as_double(0x7ff0000000000000ll);
-  for (int q = threadIdx.x; q < TILE * TILE; q += blockDim.x) {
-    const int i = IJ.x * TILE + (q >> 5), j = IJ.y * TILE + (q & 31);
-    if (i >= j || j >= P.p) continue;
-    const float2 zil = P.z[(size_t)i * E1 + s], zih = P.z[(size_t)i * E1 + s + 1];
-    const float2 zjl = P.z[(size_t)j * E1 + s], zjh = P.z[(size_t)j * E1 + s + 1];
-    const double ax = (double)zjl.x - (double)zil.x, ay = (double)zjl.y - (double)zil.y;
-    const double bx = (double)zjh.x - (double)zih.x, by = (double)zjh.y - (double)zih.y;
-    const double R = (double)P.radius[i] + (double)P.radius[j];
-    best = fmin(best, origin_seg_dist2(ax, ay, bx, by) / (R * R));
+  const int j = IJ.y * TILE + (threadIdx.x & 31);
+  float2 zjl = mk(0.f, 0.f), zjh = zjl;
+  float rj = 1.f;
+  if (j < P.p) { zjl = P.z[(size_t)j * E1 + s]; zjh = P.z[(size_t)j * E1 + s + 1]; rj = P.radius[j]; }
+  float lo[PER], least = INFINITY;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int i = IJ.x * TILE + (threadIdx.x >> 5) + q * (256 / TILE);
+    lo[q] = INFINITY;
+    if (i < j && j < P.p) {
+      const float2 cl = zjl - P.z[(size_t)i * E1 + s], ch = zjh - P.z[(size_t)i * E1 + s + 1];
+      const float mag = fmaxf(maxabs2(cl), maxabs2(ch));
+      const Bounds b = ratio_bounds(sqrtf(dist2_origin_segment(cl, ch)), mag, P.radius[i] + rj);
+      lo[q] = b.lo;
+      least = fminf(least, b.hi);
+    }
   }
-  block_min_u64((unsigned long long)__double_as_longlong(best), out);
+  least = fminf(block_min(least), least_so_far(out));
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int i = IJ.x * TILE + (threadIdx.x >> 5) + q * (256 / TILE);
+    if (!(i < j && j < P.p) || lo[q] > least) continue;
+    const float2 zil = P.z[(size_t)i * E1 + s], zih = P.z[(size_t)i * E1 + s + 1];
+    const double R = (double)P.radius[i] + (double)rj;
+    offer_ratio(origin_seg_dist2((double)zjl.x - (double)zil.x, (double)zjl.y - (double)zil.y,
+                                 (double)zjh.x - (double)zih.x, (double)zjh.y - (double)zih.y) / (R * R), out);
+  }
 }
 
 // Squared distance from point (px, py) to the segment a -> b.
@@ -228,77 +272,122 @@ __device__ __forceinline__ double point_seg_dist2(double px, double py, double a
   return origin_seg_dist2(ax - px, ay - py, bx - px, by - py);
 }
 
-// One thread per (wall, segment, agent): dist^2 / r_i^2, dist the distance
-// between the agent's segment and the wall segment (0 if they cross).
-__global__ void check_walls_kernel(Dev P, int nseg, unsigned long long* out) {
-  const int E1 = P.eta + 1;
-  double best = __longlong_as_double(0x7ff0000000000000ll);
-  const long long n = (long long)P.nw * nseg * P.p;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(t % P.p);
-    const int s = (int)((t / P.p) % nseg);
-    const int w = (int)(t / ((long long)P.p * nseg));
-    const float4 W = P.walls[w];
-    const float2 a = P.z[(size_t)i * E1 + s], b = P.z[(size_t)i * E1 + s + 1];
-    const double ax = a.x, ay = a.y, bx = b.x, by = b.y;
-    const double cx = W.x, cy = W.y, dx = W.z, dy = W.w;
-    const double o1 = fma(dx - cx, ay - cy, -((dy - cy) * (ax - cx)));
-    const double o2 = fma(dx - cx, by - cy, -((dy - cy) * (bx - cx)));
-    const double o3 = fma(bx - ax, cy - ay, -((by - ay) * (cx - ax)));
-    const double o4 = fma(bx - ax, dy - ay, -((by - ay) * (dx - ax)));
-    double d2;
-    if (((o1 > 0.0 && o2 < 0.0) || (o1 < 0.0 && o2 > 0.0)) &&
-        ((o3 > 0.0 && o4 < 0.0) || (o3 < 0.0 && o4 > 0.0))) {
-      d2 = 0.0;  // the segments cross
-    } else {
-      d2 = fmin(fmin(point_seg_dist2(ax, ay, cx, cy, dx, dy), point_seg_dist2(bx, by, cx, cy, dx, dy)),
-                fmin(point_seg_dist2(cx, cy, ax, ay, bx, by), point_seg_dist2(dx, dy, ax, ay, bx, by)));
-    }
-    const double r = P.radius[i];
-    best = fmin(best, d2 / (r * r));
+// dist^2 / r_i^2 of one (wall, segment, agent), dist the distance between the
+// agent's segment and the wall segment (0 if they cross).
+__device__ double wall_ratio2(const Dev& P, float4 W, float2 a, float2 b, float ri) {
+  const double ax = a.x, ay = a.y, bx = b.x, by = b.y;
+  const double cx = W.x, cy = W.y, dx = W.z, dy = W.w;
+  const double o1 = fma(dx - cx, ay - cy, -((dy - cy) * (ax - cx)));
+  const double o2 = fma(dx - cx, by - cy, -((dy - cy) * (bx - cx)));
+  const double o3 = fma(bx - ax, cy - ay, -((by - ay) * (cx - ax)));
+  const double o4 = fma(bx - ax, dy - ay, -((by - ay) * (dx - ax)));
+  double d2;
+  if (((o1 > 0.0 && o2 < 0.0) || (o1 < 0.0 && o2 > 0.0)) &&
+      ((o3 > 0.0 && o4 < 0.0) || (o3 < 0.0 && o4 > 0.0))) {
+    d2 = 0.0;  // the segments cross
+  } else {
+    d2 = fmin(fmin(point_seg_dist2(ax, ay, cx, cy, dx, dy), point_seg_dist2(bx, by, cx, cy, dx, dy)),
+              fmin(point_seg_dist2(cx, cy, ax, ay, bx, by), point_seg_dist2(dx, dy, ax, ay, bx, by)));
   }
-  block_min_u64((unsigned long long)__double_as_longlong(best), out);
+  return d2 / ((double)ri * (double)ri);
 }
 
-// One block: the total kinetic cost sum c_{i,s} |z_i(s+1) - z_i(s)|^2 over
-// the kinetic segments (fixed summation order, so the result is
-// deterministic), the largest endpoint error |z - start|, |z - goal|, and
-// the two clearance minima set to +inf for the kernels that follow.
-__global__ void check_cost_kernel(Dev P, const double* ccost, const float2* start, const float2* goal,
-                                  int s_lo, int s_hi, double* out) {
-  __shared__ double sc[256], se[256];
+// One thread per (wall, segment, agent), grid-stride over whole blocks.  A
+// wall that the FP32 test finds crossed is 0 within its bound only if the
+// crossing is not one of rounding, so it asks for FP64 like a distance of 0.
+__device__ __forceinline__ void check_walls(const Dev& P, int nseg, int block, int blocks, unsigned long long* out) {
   const int E1 = P.eta + 1;
-  double c = 0.0, e = 0.0;
-  for (int t = threadIdx.x; t < P.p * P.eta; t += blockDim.x) {
-    const int i = t / P.eta, s = t - i * P.eta;
-    if (s >= s_lo && s < s_hi) {
-      const float2 a = P.z[(size_t)i * E1 + s], b = P.z[(size_t)i * E1 + s + 1];
-      const double dx = (double)b.x - (double)a.x, dy = (double)b.y - (double)a.y;
-      c = fma(ccost[t], fma(dx, dx, dy * dy), c);
+  const long long n = (long long)P.nw * nseg * P.p;
+  for (long long t0 = (long long)block * blockDim.x; t0 < n; t0 += (long long)blocks * blockDim.x) {
+    const long long t = t0 + threadIdx.x;
+    float lo = INFINITY, hi = INFINITY, ri = 1.f;
+    float4 W = make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 a = mk(0.f, 0.f), b = a;
+    if (t < n) {
+      const int i = (int)(t % P.p), s = (int)((t / P.p) % nseg);
+      W = P.walls[(int)(t / ((long long)P.p * nseg))];
+      a = P.z[(size_t)i * E1 + s];
+      b = P.z[(size_t)i * E1 + s + 1];
+      ri = P.radius[i];
+      const float2 c0 = mk(W.x, W.y), c1 = mk(W.z, W.w);
+      // the differences the distances are made of
+      const float mag = fmaxf(fmaxf(maxabs2(a - c0), maxabs2(a - c1)), fmaxf(maxabs2(b - c0), maxabs2(b - c1)));
+      const Bounds q = ratio_bounds(sqrtf(dist2_segment_segment(a, b, c0, c1)), mag, ri);
+      lo = q.lo;
+      hi = q.hi;
     }
+    const float least = fminf(block_min(hi), least_so_far(out));
+    if (t < n && !(lo > least)) offer_ratio(wall_ratio2(P, W, a, b, ri), out);
   }
-  for (int i = threadIdx.x; i < P.p; i += blockDim.x) {
-    const float2 a = P.z[(size_t)i * E1], b = P.z[(size_t)i * E1 + P.eta];
-    e = fmax(e, fmax(fabs((double)a.x - (double)start[i].x), fabs((double)a.y - (double)start[i].y)));
-    e = fmax(e, fmax(fabs((double)b.x - (double)goal[i].x), fabs((double)b.y - (double)goal[i].y)));
-  }
-  sc[threadIdx.x] = c;
-  se[threadIdx.x] = e;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) {
-      sc[threadIdx.x] += sc[threadIdx.x + o];
-      se[threadIdx.x] = fmax(se[threadIdx.x], se[threadIdx.x + o]);
+}
+
+// The whole check in one launch.  Blocks: `costs` for the total kinetic cost
+// sum c_{i,s} |z_i(s+1) - z_i(s)|^2 over the kinetic segments (each block's
+// share by a fixed tree, the blocks' shares in order, so the sum is
+// deterministic) and the largest endpoint error |z - start|, |z - goal|; one
+// per tile of pairs; the rest walls.  The last block to finish hands the four
+// numbers over and leaves the words as it found them.
+// words: pair and wall minima (bits), endpoint error (bits), finished blocks.
+constexpr int CHECK_COST_BLOCKS = 64;
+__device__ __forceinline__ void init_check_words(unsigned long long* words) {
+  words[0] = words[1] = 0x7ff0000000000000ull;  // +inf
+  words[2] = words[3] = 0ull;
+}
+__global__ void __launch_bounds__(256) check_kernel(Dev P, const double* ccost, const float2* start,
+                                                    const float2* goal, int s_lo, int nseg, int costs, int pairs,
+                                                    double* part, unsigned long long* words, double* out) {
+  __shared__ double sc[256], se[256];
+  __shared__ bool last;
+  const int block = (int)blockIdx.x, tid = threadIdx.x;
+  if (block < costs) {
+    const int E1 = P.eta + 1, stride = costs * 256;
+    double c = 0.0, e = 0.0;
+#pragma unroll 4
+    for (int t = block * 256 + tid; t < P.p * P.eta; t += stride) {
+      const int i = t / P.eta, s = t - i * P.eta;
+      if (s >= s_lo) {
+        const float2 a = P.z[(size_t)i * E1 + s], b = P.z[(size_t)i * E1 + s + 1];
+        const double dx = (double)b.x - (double)a.x, dy = (double)b.y - (double)a.y;
+        c = fma(ccost[t], fma(dx, dx, dy * dy), c);
+      }
     }
+    for (int i = block * 256 + tid; i < P.p; i += stride) {
+      const float2 a = P.z[(size_t)i * E1], b = P.z[(size_t)i * E1 + P.eta];
+      e = fmax(e, fmax(fabs((double)a.x - (double)start[i].x), fabs((double)a.y - (double)start[i].y)));
+      e = fmax(e, fmax(fabs((double)b.x - (double)goal[i].x), fabs((double)b.y - (double)goal[i].y)));
+    }
+    sc[tid] = c;
+    se[tid] = e;
     __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+      if (tid < o) {
+        sc[tid] += sc[tid + o];
+        se[tid] = fmax(se[tid], se[tid + o]);
+      }
+      __syncthreads();
+    }
+    if (tid == 0) {
+      part[block] = sc[0];
+      if (se[0] > 0.0) atomicMax(words + 2, (unsigned long long)__double_as_longlong(se[0]));
+    }
+  } else if (block < costs + pairs) {
+    check_pairs(P, block - costs, words);
+  } else {
+    check_walls(P, nseg, block - costs - pairs, (int)gridDim.x - costs - pairs, words + 1);
   }
-  if (threadIdx.x == 0) {
-    out[0] = sc[0];
-    out[1] = __longlong_as_double(0x7ff0000000000000ll);
-    out[2] = __longlong_as_double(0x7ff0000000000000ll);
-    out[3] = se[0];
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();
+    last = atomicAdd(words + 3, 1ull) == (unsigned long long)gridDim.x - 1;
   }
+  __syncthreads();
+  if (!last || tid != 0) return;
+  __threadfence();
+  double c = 0.0;
+  for (int q = 0; q < costs; ++q) c += __ldcg(part + q);
+  out[0] = c;
+  for (int q = 0; q < 3; ++q) out[1 + q] = __longlong_as_double((long long)__ldcg(words + q));
+  init_check_words(words);
 }
 
 // Primal residual max |x^k - z^k| over weighted edges, without changing state
@@ -373,12 +462,13 @@ __global__ void residual_kernel(Dev P) {
 // derives the fixed-point scale, the others clear and fill.
 __global__ void __launch_bounds__(256) reset_kernel(Dev P, float2* z0, float2* z1, const float2* start,
                                                     const float2* goal, unsigned* res, unsigned* wcount,
-                                                    unsigned long long* ekey) {
+                                                    unsigned long long* ekey, unsigned long long* check) {
   if (blockIdx.x == 0) {
     if (threadIdx.x < 4) { res[threadIdx.x] = 0u; wcount[threadIdx.x] = 0u; P.ctl[threadIdx.x] = 0u; }
     if (threadIdx.x == 4) *P.status = 0u;
     // plan_set_endpoints' words: no violation, extent 0, no fix-up block done
     if (threadIdx.x == 5) { ekey[0] = ~0ull; ekey[1] = 0ull; ekey[2] = 0ull; }
+    if (threadIdx.x == 6) init_check_words(check);
     fix_block(P, start, goal);
     return;
   }
@@ -995,7 +1085,7 @@ Layout layout_for(const plan_config* c) {
   L.status = take(4);
   L.count = take(16);
   L.ccost = take(p * eta * 8);  // FP64 kinetic coefficients for plan_check
-  L.chk = take(4 * 8);          // plan_check results
+  L.chk = take((4 + CHECK_COST_BLOCKS) * 8);  // plan_check: its words and the cost blocks' shares
   L.ekey = take(24);            // plan_set_endpoints: first violation, extent, finished blocks
   // a device copy of the endpoints of a device-checked update, made while
   // they are checked
@@ -1155,7 +1245,7 @@ struct plan_s {
   cudaGraphExec_t gexec64[4] = {}; // ... and of ITERS_PER_LONG_GRAPH iterations
   double ptime[4] = {0, 0, 0, 0};
   int pcount = 0;
-  unsigned* h_res;  // pinned host words: residual readback (0), endpoint check key (2..3)
+  unsigned* h_res;  // pinned host words: residual readback (0), endpoint check key (2..3), plan_check (4..11)
   float* h_stage = nullptr;  // pinned staging of new endpoints (plan_set_endpoints)
   cudaGraphExec_t gset = nullptr;  // plan_set_endpoints' device work (fixed pointers)
   cudaEvent_t ep_event = nullptr;  // after the last endpoint update's graph
@@ -1506,7 +1596,8 @@ plan_status plan_reset(plan_t h) {
   const size_t words = std::max((size_t)h->eta * h->ntp * TILE / 4, (size_t)h->p * (h->eta + 1));
   reset_kernel<<<1 + (unsigned)std::min<size_t>((words + 255) / 256, 1216), 256, 0, h->stream>>>(
       P, h->at<float2>(h->L.z0), h->at<float2>(h->L.z1), h->at<float2>(h->L.start), h->at<float2>(h->L.goal),
-      h->at<unsigned>(h->L.res), h->at<unsigned>(h->L.wcount), h->at<unsigned long long>(h->L.ekey));
+      h->at<unsigned>(h->L.res), h->at<unsigned>(h->L.wcount), h->at<unsigned long long>(h->L.ekey),
+      h->at<unsigned long long>(h->L.chk));
   CK(cudaGetLastError());
   return PLAN_OK;
 }
@@ -1591,7 +1682,7 @@ plan_status create_plan(const plan_config* cfg, const float* start, const float*
     h->own_ws = true;
   }
   if (!member) {
-    cudaError_t e = cudaMallocHost(&h->h_res, 16);
+    cudaError_t e = cudaMallocHost(&h->h_res, 48);
     if (e == cudaSuccess && (size_t)cfg->p <= kDeviceEndpointCheck)
       e = cudaMallocHost(&h->h_stage, (size_t)cfg->p * 16);
     if (e != cudaSuccess) {
@@ -1895,23 +1986,23 @@ plan_status plan_check(plan_t h, double* total_cost, double* min_pair_clearance,
                        double* min_wall_clearance, double* max_endpoint_error) {
   if (!h) return fail(PLAN_EINVAL, "null plan");
   Dev P = h->dev(h->k);
-  double* out = h->at<double>(h->L.chk);
   // the local planner's graph: kinetic factor on segment 1, the rest on segment 0
   const int s_lo = h->vo ? 1 : 0;
   const int nseg = h->vo ? 1 : h->eta;
-  check_cost_kernel<<<1, 256, 0, h->stream>>>(P, h->at<double>(h->L.ccost), h->at<float2>(h->L.start),
-                                              h->at<float2>(h->L.goal), s_lo, h->eta, out);
-  if (h->p > 1)
-    check_pairs_kernel<<<(unsigned)(nseg * h->ntp), 256, 0, h->stream>>>(
-        P, reinterpret_cast<unsigned long long*>(out + 1));
-  if (h->nw) {
-    const long long n = (long long)h->nw * nseg * h->p;
-    check_walls_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 4096), 256, 0, h->stream>>>(
-        P, nseg, reinterpret_cast<unsigned long long*>(out + 2));
-  }
+  const int costs = (int)std::min<long long>(((long long)h->p * h->eta + 255) / 256, CHECK_COST_BLOCKS);
+  const int pairs = h->p > 1 ? nseg * h->ntp : 0;
+  const long long nwall = (long long)h->nw * nseg * h->p;
+  const int walls = (int)std::min<long long>((nwall + 255) / 256, 4096);
+  // the last block writes the results into pinned host memory: a copy behind
+  // the kernel would cost more than it
+  unsigned long long* words = h->at<unsigned long long>(h->L.chk);
+  double* v = reinterpret_cast<double*>(h->h_res + 4);
+  double* dv = nullptr;
+  CK(cudaHostGetDevicePointer(reinterpret_cast<void**>(&dv), v, 0));
+  check_kernel<<<(unsigned)(costs + pairs + walls), 256, 0, h->stream>>>(
+      P, h->at<double>(h->L.ccost), h->at<float2>(h->L.start), h->at<float2>(h->L.goal), s_lo, nseg, costs, pairs,
+      reinterpret_cast<double*>(words + 4), words, dv);
   CK(cudaGetLastError());
-  double v[4];
-  CK(cudaMemcpyAsync(v, out, sizeof v, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   if (total_cost) *total_cost = v[0];
   if (min_pair_clearance) *min_pair_clearance = std::sqrt(v[1]);
