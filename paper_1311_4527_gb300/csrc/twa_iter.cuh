@@ -234,6 +234,31 @@ __device__ __forceinline__ void coll_minimizer_classes(float2 nil, float2 nih, f
   pair_end(nih, njh, cih, cjh, vh, xih, xjh);
 }
 
+// Collision test of the n-trajectories (Eq. f_coll_def): does the relative
+// segment [cl, ch] pass closer than R to the origin?  Strict, so touching is
+// inactive.  Division-free: for an interior closest point, dist^2 =
+// cross(cl, d)^2 / |d|^2 is compared as cross^2 < R^2 |d|^2.
+__device__ __forceinline__ bool collides(float2 cl, float2 ch, float R) {
+  const float2 d = ch - cl;
+  const float dd = dot(d, d);
+  const float t = -dot(cl, d);
+  const float R2 = R * R;
+  const float c = cross(cl, d);
+  // endpoints, or an interior closest point (0 < t < |d|^2)
+  return (dot(cl, cl) < R2) | (dot(ch, ch) < R2) | ((t > 0.f) & (t < dd) & (c * c < R2 * dd));
+}
+
+// Do the segments [a0, a1] and [b0, b1] come closer than r (strict)?  They do
+// if they cross, or if an end of one is that close to the other.
+__device__ __forceinline__ bool within(float2 a0, float2 a1, float2 b0, float2 b1, float r) {
+  const float2 da = a1 - a0, db = b1 - b0;
+  const float2 p00 = b0 - a0, p01 = b1 - a0, p10 = b0 - a1, p11 = b1 - a1;
+  const float d1 = cross(da, p00), d2 = cross(da, p01), d3 = -cross(db, p00), d4 = -cross(db, p10);
+  const bool crossing = ((d1 < 0.f && d2 > 0.f) || (d1 > 0.f && d2 < 0.f)) &&
+                        ((d3 < 0.f && d4 > 0.f) || (d3 > 0.f && d4 < 0.f));
+  return crossing || collides(p00, p01, r) || collides(p10, p11, r) || collides(p00, p10, r) || collides(p01, p11, r);
+}
+
 // Kinetic factor (i, s): always active (it always sends rho0).  Finishes its
 // pending dual update, runs the closed-form minimizer and stores x and u.
 __device__ __forceinline__ void kinetic_factor(const Dev& P, int i, int s, float2 zl, float2 zh,
@@ -314,7 +339,7 @@ __device__ __forceinline__ void wall_factor(const Dev& P, int w, int i, bool vi,
     const float d2 = dot(d, d);
     act = vi && (vmin ? d2 < C * C : d2 > C * C);
   } else {
-    act = vi && dist2_segment_segment(nl, nh, c0, c1) < r * r;
+    act = vi && within(nl, nh, c0, c1, r);
   }
   const uint32_t nw = __ballot_sync(FULL, act);
   if (lane == 0 && nw != word) P.wbits[widx] = nw;
@@ -369,20 +394,6 @@ __device__ __forceinline__ void segment_warp(const Dev& P, int item) {
     res = warp_max(res);
     if (lane == 0 && P.res_prev) atomic_max_nonneg(P.res_prev, res);
   }
-}
-
-// Collision test of the n-trajectories (Eq. f_coll_def): does the relative
-// segment [cl, ch] pass closer than R to the origin?  Strict, so touching is
-// inactive.  Division-free: for an interior closest point, dist^2 =
-// cross(cl, d)^2 / |d|^2 is compared as cross^2 < R^2 |d|^2.
-__device__ __forceinline__ bool collides(float2 cl, float2 ch, float R) {
-  const float2 d = ch - cl;
-  const float dd = dot(d, d);
-  const float t = -dot(cl, d);
-  const float R2 = R * R;
-  const float c = cross(cl, d);
-  // endpoints, or an interior closest point (0 < t < |d|^2)
-  return (dot(cl, cl) < R2) | (dot(ch, ch) < R2) | ((t > 0.f) & (t < dd) & (c * c < R2 * dd));
 }
 
 __device__ __forceinline__ int tile_pair(int nt, int I, int J) {  // I <= J

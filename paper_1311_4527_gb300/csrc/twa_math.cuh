@@ -37,7 +37,8 @@
 // on each half-plane of directions.  The global minimum is at one of the two
 // kink directions or at a local minimum of one end circle's energy: a local
 // minimum of its both-stretched piece (global or local-nonglobal, both from
-// the secular equation) or a single-hinge direction.  All are candidates.
+// the secular equation) or a single-hinge direction.  A circle whose
+// half-plane cannot beat the kinks is skipped (capsule_end_dominated).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
@@ -49,7 +50,7 @@ namespace twa {
 // Host and device: the same FP32 code is also compiled into a host-side test
 // harness (tests/minimizer_harness.cu) that compares it with the FP64 oracle.
 // Everything is inlined, and candidate directions are written to fixed
-// array slots only (put_dir, unrolled loops), so that the minimizers keep
+// array slots only (unrolled loops), so that the minimizers keep
 // their candidates in registers: a call or a dynamically indexed array puts
 // them in local memory, whose latency sits on the minimizer's long dependent
 // chain.
@@ -117,15 +118,6 @@ TWA_DEV float pow2_inverse(float x) {
   memcpy(&x, &u, 4);
   return x;
 #endif
-}
-
-// out[n++] = v with constant indices (up to 4 slots).
-TWA_DEV void put_dir(float2* out, int& n, float2 v) {
-  if (n == 0) out[0] = v;
-  else if (n == 1) out[1] = v;
-  else if (n == 2) out[2] = v;
-  else out[3] = v;
-  ++n;
 }
 
 // Angle of a unit vector in [0, 2 pi): the tie-break order of directions.
@@ -271,86 +263,53 @@ TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
   return 1;
 }
 
-// The other stationary points of f: mu in (lambda1, lambda2), where
-// t = mu - lambda1 solves (A1/t)^2 + (A2/(d - t))^2 = 1.  The left side is
-// convex on (0, d) with its minimum at t_m = d A1^(2/3) / (A1^(2/3) + A2^(2/3)),
-// so there are 0 or 2 roots (one is the local-but-not-global minimum); with
-// s1 = 0 or s2 = 0 the stationary points at mu = lambda1 or lambda2 are added.
-// Writes up to 4 directions; used by the wall minimizer, whose capsule
-// restricts each end circle to a half-plane of directions.  part = 0 or 1
-// writes only the directions of that part of the sequence (0: the special
-// cases or the root left of t_m, 1: the root right of it), for callers that
-// split the work over threads; -1 writes all.
-TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, float2* out,
-                           int part = -1) {
+// The other local minimum of f, where there is one: mu in (lambda1, lambda2),
+// where t = mu - lambda1 solves phi = (A1/t)^2 + (A2/(d - t))^2 = 1.  phi is
+// convex on (0, d), so there are 0 or 2 roots; the curvature of f along the
+// circle is (d - t) n1^2 - t n2^2, which has the sign of -dphi/dt, so the root
+// left of phi's minimum is the local minimum (the other one a local maximum).
+// Newton on 1/|n(t)| from the pole side, t = A1, where phi >= 1, climbs to it;
+// when the climb passes phi's minimum (dphi/dt >= 0) there is no root.  With
+// s2 = 0 the root is t = A1 < d; with s1 = 0 there is none left of the
+// minimum.  Writes 0 or 1 direction; used by the wall minimizer, whose capsule
+// restricts each end circle to a half-plane of directions.
+TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, float2* out) {
+  const float sc = pow2_inverse(R);
+  a = sc * a; b = sc * b; R *= sc;
   const float2 wa = wl * a, wb = wh * b;
-  float m11 = fmaf(wa.x, a.x, wb.x * b.x);
-  float m22 = fmaf(wa.y, a.y, wb.y * b.y);
-  float m12 = fmaf(wa.x, a.y, wb.x * b.y);
-  float2 S = wa + wb;
-  float hd = 0.5f * (m11 - m22);
-  float disc = hypotf(hd, m12);
-  float d = 2.f * disc;
+  const float m11 = fmaf(wa.x, a.x, wb.x * b.x);
+  const float m22 = fmaf(wa.y, a.y, wb.y * b.y);
+  const float m12 = fmaf(wa.x, a.y, wb.x * b.y);
+  const float2 S = wa + wb;
+  const float hd = 0.5f * (m11 - m22);
+  const float disc = sqrtf(fmaf(hd, hd, m12 * m12));
+  const float d = 2.f * disc;
   if (!(d > 0.f)) return 0;
-  float2 e2 = (hd >= 0.f) ? normalized(mk(hd + disc, m12)) : normalized(mk(m12, disc - hd));
-  float2 e1 = perp(e2);
-  float s1 = dot(S, e1), s2 = dot(S, e2);
-  float A1 = R * fabsf(s1), A2 = R * fabsf(s2);
-  int n = 0;
-  if (A1 == 0.f && A2 == 0.f) return 0;
-  if ((A2 == 0.f || A1 == 0.f) && part == 1) return 0;
-  if (A2 == 0.f) {  // hard case at mu = lambda2, and the root t = A1
-    if (A1 < d) {
-      float n1 = -R * s1 / d;
-      float n2 = sqrtf(fmaxf(0.f, fmaf(-n1, n1, 1.f)));
-      out[0] = axpy(n1, e1, n2 * e2);
-      out[1] = axpy(n1, e1, (-n2) * e2);
-      out[2] = (s1 > 0.f ? -1.f : 1.f) * e1;
-      n = 3;
-    }
-    return n;
+  const float q = fabsf(hd) + disc;
+  const float2 e2 = normalized((hd >= 0.f) ? mk(q, m12) : mk(m12, q));
+  const float2 e1 = perp(e2);
+  const float s1 = dot(S, e1), s2 = dot(S, e2);
+  const float A1 = R * fabsf(s1), A2 = R * fabsf(s2);
+  if (!(A1 > 0.f && A1 < d)) return 0;
+  float t = A1;
+  bool found = A2 == 0.f;
+#pragma unroll 1
+  for (int it = 0; it < 40 && !found; ++it) {
+    TWA_ITER_HOOK(1);
+    const float it_ = fdiv(1.f, t), id = fdiv(1.f, d - t);
+    const float q1 = A1 * it_, q2 = A2 * id;
+    const float w1 = q1 * q1, w2 = q2 * q2;
+    const float phi = w1 + w2, slope = fmaf(w1, it_, -(w2 * id));
+    if (!(slope > 0.f)) break;  // past the minimum of phi
+    const float step = (phi * frsqrt(phi) - 1.f) * fdiv(phi, slope);
+    t += step;
+    if (!(t > 0.f && t < d)) break;
+    found = fabsf(step) <= 1e-6f * t;
   }
-  if (A1 == 0.f) {  // the root t = d - A2
-    if (A2 < d) { out[0] = (s2 > 0.f ? 1.f : -1.f) * e2; n = 1; }
-    return n;
-  }
-  float c1 = cbrtf(A1 * A1), c2 = cbrtf(A2 * A2);
-  float tm = d * c1 / (c1 + c2);
-  const float r1 = A1 / tm, r2 = A2 / (d - tm);
-  float phim = fmaf(r1, r1, r2 * r2);
-  if (!(phim <= 1.f)) return 0;
-  for (int side = (part == 1) ? 1 : 0; side < ((part == 0) ? 1 : 2); ++side) {
-    // h(t) = phi(t)^(-1/2) - 1 is increasing on (0, tm] and decreasing on
-    // [tm, d); each root is approached from its pole side, where h <= 0 (at
-    // t = A1, resp. t = d - A2), so that the Newton steps move monotonically.
-    float lo = side ? tm : 0.f, hi = side ? d : tm;
-    float t = side ? fminf(fmaxf(d - A2, tm), d) : fmaxf(fminf(A1, tm), 0.f);
-    if (!(t > lo && t < hi)) t = 0.5f * (lo + hi);
-    for (int it = 0; it < 40; ++it) {
-      TWA_ITER_HOOK(1);
-      float it_ = fdiv(1.f, t), id = fdiv(1.f, d - t);
-      float q1 = A1 * it_, q2 = A2 * id;
-      float phi = fmaf(q1, q1, q2 * q2);
-      float ip = frsqrt(phi);
-      float h = ip - 1.f;
-      bool right = side ? (h < 0.f) : (h > 0.f);  // root lies left of t
-      if (right) hi = t; else lo = t;
-      if (h == 0.f || hi - lo <= 1e-6f * hi) break;
-      float dphi = 2.f * fmaf(q2 * q2, id, -(q1 * q1 * it_));
-      float dh = -0.5f * ip * ip * ip * dphi;
-      float tn = (dh != 0.f) ? t - fdiv(h, dh) : 0.5f * (lo + hi);
-      if (!(tn > lo && tn < hi)) tn = 0.5f * (lo + hi);
-      const bool done = fabsf(tn - t) <= 1e-6f * fmaxf(t, tn);
-      t = tn;
-      if (done) break;
-    }
-    float p1 = fdiv(-R * s1, t), p2 = fdiv(R * s2, d - t);
-    float n1, n2;
-    if (fabsf(p1) <= fabsf(p2)) { n1 = p1; n2 = copysignf(sqrtf(fmaxf(0.f, fmaf(-p1, p1, 1.f))), p2); }
-    else { n2 = p2; n1 = copysignf(sqrtf(fmaxf(0.f, fmaf(-p2, p2, 1.f))), p1); }
-    put_dir(out, n, normalized(axpy(n1, e1, n2 * e2)));
-  }
-  return n;
+  if (!found) return 0;
+  // (n1, n2) = (-R s1 / t, R s2 / (d - t)) up to its length
+  out[0] = normalized(axpy(-s1 * (d - t), e1, (s2 * t) * e2));
+  return 1;
 }
 
 // Tangent normals n with <q, n> = R from a point q (|q| >= R).
@@ -457,16 +416,21 @@ TWA_DEV float capsule_E(float2 a, float2 b, float wl, float wh, float2 c0, float
 // support (<c_ci - c_other, n> >= 0), the energy is that circle's disk
 // energy.  Write n = c nu + s e (e the outward wall direction at that end, nu
 // its normal, s >= 0) and beta_x, gamma_x for the coordinates of x - c_ci
-// along nu and e.  When neither target lies beyond the end (gamma <= 0),
-// <x - c_ci, n> <= c beta_x, so the energy is at least
-// G(c) = wl/2 [r - c beta_a]_+^2 + wh/2 [r - c beta_b]_+^2, which equals the
-// kink energies at c = +-1; with both targets on one side of the wall's line
-// (beta_a, beta_b of one sign) G is monotone in c, so nothing in that
-// half-plane is below the better kink and the circle's candidates can be
-// skipped.  False for a zero-length wall.  The signs are decided in FP32, so
-// each coordinate must clear a margin of 1e-6 |e| |x - c_ci| (a few units in
-// the last place of the products): a target on the wall's line, on the
-// perpendicular through the end or at the end centre keeps the circle's
+// along nu and e.  With no target beyond the end (gamma <= 0) the hinge of
+// target x is [r - c beta_x + s |gamma_x|]_+.
+// (1) Both targets on one side of the wall's line (beta_a, beta_b of one
+// sign): dropping s |gamma| gives a lower bound monotone in c.
+// (2) Both in the quarter-turn cone behind the end (|beta_x| <= |gamma_x|):
+// s >= 1 - |c| bounds the hinge from below by [r + |gamma_x| -
+// |c| (|gamma_x| +- beta_x)]_+, which does not increase with |c|.
+// Either way nothing in that half-plane is below the better kink (c = +-1,
+// where the bounds are met), and the circle's candidates can be skipped; with
+// one end pinned at a the constraint <a, n> >= h(n) asks for a's hinge to be
+// zero, which holds at the kink if it holds anywhere on that side, so the rule
+// is the same.  False for a zero-length wall.  The signs are decided in
+// FP32, so each coordinate must clear a margin of 1e-6 |e| |x - c_ci| (a few
+// units in the last place of the products): a target on the wall's line, on
+// the perpendicular through the end or at the end centre keeps the circle's
 // candidates (which are then computed exactly) instead of trusting a sign
 // that rounding may have flipped.
 TWA_DEV bool capsule_end_dominated(float2 a, float2 b, float2 c0, float2 c1, int ci) {
@@ -480,7 +444,8 @@ TWA_DEV bool capsule_end_dominated(float2 a, float2 b, float2 c0, float2 c1, int
   const float ta = 1e-6f * sqrtf(ee * dot(da, da)), tb = 1e-6f * sqrtf(ee * dot(db, db));
   const float ga = dot(da, out), gb = dot(db, out);
   const float ba = dot(da, nu), bb = dot(db, nu);
-  return ga < -ta && gb < -tb && ((ba > ta && bb > tb) || (ba < -ta && bb < -tb));
+  return ga < -ta && gb < -tb &&
+         ((ba > ta && bb > tb) || (ba < -ta && bb < -tb) || (fabsf(ba) < -ga - ta && fabsf(bb) < -gb - tb));
 }
 
 // Kinds of winning capsule direction (Best::tag): 0 the (1, 0) fallback,
@@ -504,15 +469,18 @@ TWA_DEV float2 capsule_dir_free(float2 a, float2 b, float wl, float wh, float2 c
     if (capsule_end_dominated(a, b, c0, c1, ci)) continue;
     float2 cc = ci ? c1 : c0;
     float2 ac = a - cc, bc = b - cc;
-    float2 t[4];
-    int nt = trs_global(ac, bc, wl, wh, r, t);
+    float2 t[2];
+    const int nt = trs_global(ac, bc, wl, wh, r, t);
+    bool mine = false;  // a global minimiser in this circle's half-plane
 #pragma unroll
     for (int k = 0; k < 2; ++k)
-      if (k < nt) best.offer(t[k], capsule_E(a, b, wl, wh, c0, c1, r, t[k]), 2 + 4 * ci);
-    nt = trs_local(ac, bc, wl, wh, r, t);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      if (k < nt) best.offer(t[k], capsule_E(a, b, wl, wh, c0, c1, r, t[k]), 2 + 4 * ci);
+      if (k < nt) {
+        best.offer(t[k], capsule_E(a, b, wl, wh, c0, c1, r, t[k]), 2 + 4 * ci);
+        mine |= (ci ? dot(e, t[k]) : -dot(e, t[k])) >= 0.f;
+      }
+    // (then nothing stretched in the half-plane is lower)
+    if (!mine && trs_local(ac, bc, wl, wh, r, t))
+      best.offer(t[0], capsule_E(a, b, wl, wh, c0, c1, r, t[0]), 2 + 4 * ci);
     if (dot(ac, ac) > 0.f) {
       float2 n = normalized(ac);
       best.offer(n, capsule_E(a, b, wl, wh, c0, c1, r, n), 3 + 4 * ci);
@@ -538,9 +506,9 @@ TWA_NOINLINE void capsule_prox_free(float2 a, float2 b, float wl, float wh, floa
 #ifdef __CUDACC__
 // capsule_prox_free by a whole warp (every lane calls it with the same
 // arguments and gets the same result): the candidate directions of
-// capsule_dir_free are shared out over 9 lanes (the fallback and kinks; per
-// end circle the global stationary point, the two halves of trs_local and the
-// single-hinge directions), each lane keeps its best in the same order, and a
+// capsule_dir_free are shared out over 7 lanes (the fallback and kinks; per
+// end circle the global and the local stationary point and the single-hinge
+// directions), each lane keeps its best in the same order, and a
 // warp reduction on (E, angle, position in the sequence) picks the candidate
 // that the sequential scan keeps.  The secular solves then run side by side
 // instead of one after another.
@@ -563,18 +531,18 @@ __device__ __forceinline__ void capsule_prox_free_warp(float2 a, float2 b, float
       offer(k0);
       offer(-k0);
     }
-  } else if (lane < 9 && !capsule_end_dominated(a, b, c0, c1, (lane - 1) >> 2)) {
-    const int ci = (lane - 1) >> 2, task = (lane - 1) & 3;
+  } else if (lane < 7 && !capsule_end_dominated(a, b, c0, c1, (lane - 1) / 3)) {
+    const int ci = (lane - 1) / 3, task = (lane - 1) % 3;
     const float2 cc = ci ? c1 : c0;
     const float2 ac = a - cc, bc = b - cc;
-    float2 t[4];
+    float2 t[2];
     int nt = 0;
     if (task == 0) nt = trs_global(ac, bc, wl, wh, r, t);
-    else if (task < 3) nt = trs_local(ac, bc, wl, wh, r, t, task - 1);
+    else if (task == 1) nt = trs_local(ac, bc, wl, wh, r, t);
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 2; ++k)
       if (k < nt) offer(t[k]);
-    if (task == 3) {
+    if (task == 2) {
       if (dot(ac, ac) > 0.f) offer(normalized(ac));
       if (dot(bc, bc) > 0.f) offer(normalized(bc));
     }
@@ -630,8 +598,15 @@ TWA_DEV bool capsule_dir_pinned(float2 q, float2 w, float2 c0, float2 c1, float 
       any = true;
     }
   };
-#pragma unroll
+  float2 e = c1 - c0;
+  if (e.x != 0.f || e.y != 0.f) {
+    float2 k0 = normalized(perp(e));
+    offer(k0, 1);
+    offer(-k0, 1);
+  }
+#pragma unroll 1
   for (int ci = 0; ci < 2; ++ci) {
+    if (any && capsule_end_dominated(q, w, c0, c1, ci)) continue;
     float2 cc = ci ? c1 : c0;
     float2 qc = q - cc;
     if (dot(qc, qc) >= r * r) {
@@ -642,12 +617,6 @@ TWA_DEV bool capsule_dir_pinned(float2 q, float2 w, float2 c0, float2 c1, float 
     }
     float2 wc = w - cc;
     if (dot(wc, wc) > 0.f) offer(normalized(wc), 3 + 4 * ci);
-  }
-  float2 e = c1 - c0;
-  if (e.x != 0.f || e.y != 0.f) {
-    float2 k0 = normalized(perp(e));
-    offer(k0, 1);
-    offer(-k0, 1);
   }
   dir = best.n;
   tag = best.tag;
