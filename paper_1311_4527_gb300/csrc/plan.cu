@@ -48,30 +48,40 @@ constexpr int TEST_WARPS = 4;
 constexpr int TEST_ROWS = TILE / TEST_WARPS;
 
 // Gated state, every factor in one launch.  The first CTAs take the worklist
-// (the longest chains: a minimizer each), then the kinetic, wall and velocity
-// warps, then the tiles.  A chunk of 32 list entries goes to the warp of the
+// (long chains: a minimizer each), then the tiles of the last segment (early
+// in a solve it spans each agent's whole way, and nearly all its pairs take
+// the exact test), then the kinetic, wall and velocity warps, then the other
+// tiles.  A chunk of 32 list entries goes to the warp of the
 // same number, and consecutive warps sit on different CTAs, so a short list
 // spreads over the SMs.
 constexpr int FACTOR_WARPS = 4;
+struct FactorGrid {
+  int list_ctas, lead_ctas;  // CTAs of the worklist, and of tiles ahead of the segment warps
+  int seg_ctas, seg_warps, tile_warps;
+  int mode;                  // FactorMode
+};
 template <bool CLASSES>
-__global__ void __launch_bounds__(32 * FACTOR_WARPS, 6) factor_kernel(Dev P, int list_ctas, int seg_ctas,
-                                                                     int seg_warps, int tile_warps) {
+__global__ void __launch_bounds__(32 * FACTOR_WARPS, 6) factor_kernel(Dev P, FactorGrid G) {
   __shared__ TileMem mem[FACTOR_WARPS];
   pdl_begin();
-  if (blockIdx.x == 0 && threadIdx.x == 0) *P.res_cur = 0u;
-  const int warp = threadIdx.x >> 5, nlist = list_ctas * FACTOR_WARPS;
-  int b = (int)blockIdx.x, item = warp * list_ctas + b;
-  if (b >= list_ctas) {
-    b -= list_ctas;
-    if (b < seg_ctas) {
-      if (b * FACTOR_WARPS + warp < seg_warps) segment_warp(P, b * FACTOR_WARPS + warp);
-      return;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && G.mode != LISTED) *P.res_cur = 0u;
+  const int warp = threadIdx.x >> 5, nlist = G.list_ctas * FACTOR_WARPS;
+  int b = (int)blockIdx.x, item = warp * G.list_ctas + b;
+  if (b >= G.list_ctas) {
+    b -= G.list_ctas;  // tile CTA, once the segment CTAs are taken out
+    if (b >= G.lead_ctas) {
+      b -= G.seg_ctas;
+      if (b < G.lead_ctas) {
+        const int w = (b + G.seg_ctas - G.lead_ctas) * FACTOR_WARPS + warp;
+        if (w < G.seg_warps) segment_warp(P, w);
+        return;
+      }
     }
-    item = (b - seg_ctas) * FACTOR_WARPS + warp;
-    if (item >= tile_warps) return;  // warp-uniform
+    item = b * FACTOR_WARPS + warp;
+    if (item >= G.tile_warps) return;  // warp-uniform
     item += nlist;
   }
-  collision_warp<CLASSES>(P, item, nlist, mem + warp);
+  collision_warp<CLASSES>(P, item, nlist, mem + warp, G.mode);
 }
 
 // Dense state, pass 1: the first CTAs take the kinetic, wall and velocity
@@ -421,7 +431,13 @@ __global__ void residual_kernel(Dev P) {
   };
   if (P.admm) {  // every pair: a warp per row
     for (size_t row = gw; row < nrows; row += nwarps) pair(row, lane, (P.bits[row] >> lane) & 1u);
-  } else {  // the few active ones: a lane per row
+  } else if (!P.dense && P.ctl[0] == 0u) {  // the active ones from the worklist, a lane each
+    const unsigned n = *P.work_count;
+    for (unsigned t = (unsigned)gw * 32 + lane; t < n; t += (unsigned)nwarps * 32) {
+      const uint32_t e = P.work[t];
+      if (e & ACTIVE) pair((e & ~ACTIVE) >> 5, (int)(e & 31), true);
+    }
+  } else {  // or from the bits, a lane per row
     for (size_t row = (size_t)gw * 32 + lane; row < nrows; row += (size_t)nwarps * 32)
       for (uint32_t w = P.bits[row]; w; w &= w - 1u) pair(row, __ffs(w) - 1, true);
   }
@@ -1234,6 +1250,7 @@ struct plan_s {
   bool own_ws;
   int k;
   int cur;  // which z buffer holds z^k
+  bool fresh = true;  // no worklist yet: the next iteration runs in two launches (FactorMode)
   int sms = 0;        // SMs of the device
   int prox_grid = 0;  // CTAs of the dense state's minimizer pass (resident CTAs per SM x SMs)
   cudaStream_t cap = nullptr;    // private stream for capturing the iteration graphs
@@ -1355,6 +1372,7 @@ plan_status drop_worklist(plan_t h) {
   CK(cudaMemsetAsync(h->at<void>(h->L.wcount), 0, 16, h->stream));
   CK(cudaMemsetAsync(h->at<void>(h->L.ctl), 0, 16, h->stream));
   CK(cudaMemsetAsync(h->at<void>(h->L.ctl), 1, 1, h->stream));  // ctl[0] = 1 (rebuild)
+  h->fresh = true;
   return PLAN_OK;
 }
 
@@ -1395,6 +1413,12 @@ int list_ctas(const plan_s* h) {
   return (int)std::max<long long>(1, std::min<long long>((pairs + 32 * FACTOR_WARPS - 1) / (32 * FACTOR_WARPS), 2ll * h->sms));
 }
 
+// Every pair fits the worklist, so that an iteration may be split in listing
+// and processing the list.
+bool lists_every_pair(const plan_s* h) {
+  return (unsigned long long)(h->vo ? 1 : h->eta) * h->p * (h->p - 1) / 2 <= h->L.cap;
+}
+
 // Enqueue the kernels of iteration h->k (no state change on the host).
 plan_status enqueue_iteration(plan_t h, cudaStream_t ms) {
   Dev P = h->dev(h->k);
@@ -1407,11 +1431,21 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms) {
     if (prof) CK(cudaEventRecord(h->pev[1], ms));
     CK(launch_pdl(prox_kernel, (unsigned)h->prox_grid, 256u, ms, P));
   } else {
-    const int lc = list_ctas(h), segc = (segw + FACTOR_WARPS - 1) / FACTOR_WARPS;
-    const int tiles = (h->vo ? 1 : h->eta) * h->ntp;
-    const unsigned grid = (unsigned)(lc + segc + (tiles + FACTOR_WARPS - 1) / FACTOR_WARPS);
-    CK(launch_pdl(h->noenergy ? factor_kernel<true> : factor_kernel<false>, grid, 32u * FACTOR_WARPS, ms, P, lc,
-                  segc, segw, tiles));
+    FactorGrid G;
+    const int tiles = (h->vo ? 1 : h->eta) * h->ntp, tile_ctas = (tiles + FACTOR_WARPS - 1) / FACTOR_WARPS;
+    G.list_ctas = list_ctas(h);
+    G.lead_ctas = std::min(tile_ctas, (h->ntp + FACTOR_WARPS - 1) / FACTOR_WARPS);
+    G.seg_ctas = (segw + FACTOR_WARPS - 1) / FACTOR_WARPS;
+    G.seg_warps = segw;
+    G.tile_warps = tiles;
+    const bool listing = h->fresh && lists_every_pair(h);
+    G.mode = listing ? LISTING : FUSED;
+    auto kern = h->noenergy ? factor_kernel<true> : factor_kernel<false>;
+    CK(launch_pdl(kern, (unsigned)(G.list_ctas + G.seg_ctas + tile_ctas), 32u * FACTOR_WARPS, ms, P, G));
+    if (listing) {
+      G.mode = LISTED;
+      CK(launch_pdl(kern, (unsigned)G.list_ctas, 32u * FACTOR_WARPS, ms, P, G));
+    }
     if (prof) CK(cudaEventRecord(h->pev[1], ms));
   }
   if (prof) CK(cudaEventRecord(h->pev[2], ms));
@@ -1439,7 +1473,7 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms) {
 plan_status run_iteration(plan_t h) {
   plan_status st = ensure_prox_grid(h);
   if (st != PLAN_OK) return st;
-  const bool graphable = h->cap && !h->profiling && h->k >= h->graph_from();
+  const bool graphable = h->cap && !h->profiling && h->k >= h->graph_from() && !h->fresh;
   if (graphable) {
     const int key = ((h->k & 1) << 1) | h->cur;
     if (!h->gexec[key]) {
@@ -1459,6 +1493,7 @@ plan_status run_iteration(plan_t h) {
   } else {
     st = enqueue_iteration(h, h->stream);
     if (st != PLAN_OK) return st;
+    h->fresh = false;
   }
   if (h->eta > 1) h->cur ^= 1;
   h->k += 1;
@@ -1505,6 +1540,10 @@ plan_status run_graph_runs(plan_t h, int& n, int len, cudaGraphExec_t* execs) {
 plan_status run_iterations(plan_t h, int n) {
   plan_status st = ensure_prox_grid(h);
   if (st != PLAN_OK) return st;
+  if (n > 0 && h->fresh) {
+    if ((st = run_iteration(h)) != PLAN_OK) return st;
+    --n;
+  }
   if ((st = run_graph_runs(h, n, ITERS_PER_LONG_GRAPH, h->gexec64)) != PLAN_OK) return st;
   if ((st = run_graph_runs(h, n, ITERS_PER_GRAPH, h->gexec8)) != PLAN_OK) return st;
   for (; n > 0; --n)
@@ -1586,6 +1625,7 @@ plan_status plan_reset(plan_t h) {
   h->adj_valid = false;
   h->k = 0;
   h->cur = 0;
+  h->fresh = true;
   Dev P = h->dev(0);
   if (P.dense) {
     const size_t ng = (size_t)h->nw + h->nv;
@@ -2823,7 +2863,7 @@ __global__ void __launch_bounds__(32 * FACTOR_WARPS, 6) batch_factor_kernel(cons
     if (it.item == 0 && (threadIdx.x & 31) == 0) *P.res_cur = 0u;
     const int g = it.item - sh.nlist;
     if (g >= 0 && g < sh.nseg) segment_warp(P, g);
-    else collision_warp<false>(P, g < 0 ? it.item : it.item - sh.nseg, sh.nlist, mem + warp);
+    else collision_warp<false>(P, g < 0 ? it.item : it.item - sh.nseg, sh.nlist, mem + warp, FUSED);
   }
 }
 

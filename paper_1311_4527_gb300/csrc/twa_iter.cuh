@@ -615,10 +615,17 @@ constexpr uint32_t ACTIVE = 0x80000000u;
 // lane per round (row found by a shuffle binary search over the rows' prefix
 // counts), to run the minimizer.  Both kinds of warp share one copy of that
 // code (one loop, one call site): it is most of the kernel's instructions.
+//
+// mode FUSED is the above.  After a reset or an import nearly every active
+// pair is new to the tile warps, which then run many rounds one after another
+// where a layout is crowded (41 us for the p = 100 circle), so that iteration
+// is two launches: LISTING (tile warps put every pair that was active or
+// collides on the worklist) and LISTED (list warps only).
+enum FactorMode { FUSED = 0, LISTING = 1, LISTED = 2 };
 template <bool CLASSES>
-__device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist, TileMem* M) {
+__device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist, TileMem* M, int mode) {
   const int lane = threadIdx.x & 31;
-  const bool rebuild = P.ctl[0] != 0u;
+  const bool rebuild = mode == LISTED ? false : P.ctl[0] != 0u;
   const bool lister = item < nlist;
   float res = 0.f;
   // list warp
@@ -630,8 +637,8 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
   uint32_t listed = 0u, todo = 0u, near = 0u;
   unsigned tincl = 0, total = 0, base = 0;
   if (lister) {
-    if (rebuild) return;
-    n = *P.work_count_prev;
+    if (rebuild || mode == LISTING) return;
+    n = mode == LISTED ? *P.work_count : *P.work_count_prev;
   } else {
     const int nseg = P.vo ? 1 : P.eta;
     const int t = item - nlist;
@@ -671,7 +678,7 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
     near = ~far & valid & ~listed;
     M->act[lane] = 0u;
     todo = rebuild ? listed : 0u;
-    phase = rebuild ? 0 : 1;
+    phase = mode == LISTING ? 2 : rebuild ? 0 : 1;
     if (__any_sync(FULL, near != 0u)) {
       float4 zi = make_float4(0.f, 0.f, 0.f, 0.f), zj = zi;
       float ri = 0.f, rj = 0.f;
@@ -680,11 +687,18 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
       M->z[lane] = zj;
       M->r[lane] = rj;
       __syncwarp();
+      // two columns a round: their chains overlap (on the segment that spans
+      // the whole way nearly every pair is near)
       uint32_t hit = 0u;
-      for (uint32_t w = near; w; w &= w - 1u) {
+      for (uint32_t w = near; w; ) {
         const int c = __ffs(w) - 1;
-        const float4 B = M->z[c];
-        if (collides(lo2(B) - lo2(zi), hi2(B) - hi2(zi), ri + M->r[c])) hit |= 1u << c;
+        w &= w - 1u;
+        const int k = w ? __ffs(w) - 1 : c;
+        w &= w - 1u;
+        const float4 B = M->z[c], D = M->z[k];
+        const bool h0 = collides(lo2(B) - lo2(zi), hi2(B) - hi2(zi), ri + M->r[c]);
+        const bool h1 = collides(lo2(D) - lo2(zi), hi2(D) - hi2(zi), ri + M->r[k]);
+        hit |= (h0 ? 1u << c : 0u) | (h1 ? 1u << k : 0u);
       }
       near = hit;
     }
@@ -761,8 +775,15 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
     }
   } else {
     __syncwarp();
-    const uint32_t nword = M->act[lane];
-    if (rebuild) {
+    uint32_t nword = M->act[lane];
+    const uint32_t flagged = mode == LISTING ? (rebuild ? listed : 0u) : ~0u;  // entries active so far
+    if (mode == LISTING) {
+      // (a reset leaves nothing active and `listed` clear; an import, rebuild)
+      nword = near | flagged;
+      P.listed[row] = nword;
+      const int fresh = __reduce_add_sync(FULL, __popc(near));
+      if (lane == 0 && fresh) atomicAdd(P.ctl + 1, (unsigned)fresh);
+    } else if (rebuild) {
       if (nword != listed) P.bits[row] = nword;
       P.listed[row] = nword;
     } else if (nword) {
@@ -785,7 +806,10 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
       }
       at = __shfl_sync(FULL, at, 31) + (incl - cnt);
       for (uint32_t w = nword; w; w &= w - 1u, ++at)
-        if (at < P.cap) P.work[at] = (uint32_t)(row * TILE + (__ffs(w) - 1)) | ACTIVE;
+        if (at < P.cap) {
+          const int bit = __ffs(w) - 1;
+          P.work[at] = (uint32_t)(row * TILE + bit) | ((flagged >> bit) & 1u ? ACTIVE : 0u);
+        }
     }
   }
   if (__any_sync(FULL, res > 0.f)) {  // only pairs active before have a residual
