@@ -24,6 +24,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "plan.h"
@@ -133,6 +134,54 @@ __global__ void segments_kernel(Dev P) {
   const int s = t / P.p, i = t - s * P.p;
   const size_t node = (size_t)i * (P.eta + 1) + s;
   store_segment(P, i, s, P.z[node], P.z[node + 1]);
+}
+
+// Small problems, gated state: whole runs of iterations in one launch of one
+// CTA.  The two kernels of an iteration are bound by their launches and by
+// dependent loads through L2 there, not by work (a p = 4 iteration's factor
+// pass takes 3 us, its launches and node pass another 3.4).  The CTA's 16
+// warps take the factor pass's warps' work in turn, meet at a barrier, take
+// the node pass's, and meet again; the state stays in the SM's L1.  Every
+// warp-level routine is the one the per-pass kernels run, so the iterates are
+// the same.  A cluster of two to eight CTAs was no faster than two launches
+// (5.5 to 8 us at p = 8 to 48): its barrier makes every load go to L2 again.
+// tape (differentiation): each iteration's record is written beside its node
+// pass.
+constexpr int SOLO_WARPS = 16;
+struct Tape {
+  char* at;  // the first iteration's slot (null: nothing is recorded)
+  size_t stride, z, ukin, count, fid, ucl, uch, scount, sidx, su;
+};
+__device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, char* slot, unsigned t0, unsigned nt);
+
+template <bool CLASSES>
+__global__ void __launch_bounds__(32 * SOLO_WARPS, 1) run_kernel(Dev P0, Dev P1, int iters, int nlist, int seg_warps,
+                                                                 int tile_warps, int nodes, Tape T) {
+  __shared__ TileMem mem[SOLO_WARPS];
+  __shared__ Dev sP[2];
+  for (int w = threadIdx.x; w < (int)(sizeof(Dev) / 4); w += blockDim.x) {
+    reinterpret_cast<uint32_t*>(&sP[0])[w] = reinterpret_cast<const uint32_t*>(&P0)[w];
+    reinterpret_cast<uint32_t*>(&sP[1])[w] = reinterpret_cast<const uint32_t*>(&P1)[w];
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, coll = nlist + tile_warps;
+#pragma unroll 1
+  for (int it = 0; it < iters; ++it) {
+    const Dev& P = sP[it & 1];
+    if (threadIdx.x == 0) *P.res_cur = 0u;
+#pragma unroll 1
+    for (int item = warp; item < coll + seg_warps; item += SOLO_WARPS) {
+      if (item < coll) collision_warp<CLASSES>(P, item, nlist, mem + warp, FUSED);
+      else segment_warp(P, item - coll);
+      __syncwarp();
+    }
+    __syncthreads();
+    if (threadIdx.x == 32 * (SOLO_WARPS - 1)) advance_worklist(P, false);
+#pragma unroll 1
+    for (int w = warp; w < nodes; w += SOLO_WARPS) consensus_warp(P, w);
+    if (T.at) record_iteration(P, T, T.at + (size_t)it * T.stride, threadIdx.x, blockDim.x);
+    __syncthreads();
+  }
 }
 
 // Fixed-point scale of the consensus sums: the largest power of two with
@@ -1236,6 +1285,13 @@ plan_status check_endpoints(int p, const float* start, const float* goal, const 
 
 }  // namespace
 
+// A captured segment of the backward pass and what it was captured for.
+struct SegmentGraph {
+  int n, parity, cur;
+  bool first, zb;
+  cudaGraphExec_t exec;
+};
+
 struct plan_s {
   plan_config cfg;
   int p, eta, nw, nt, ntp;
@@ -1278,6 +1334,7 @@ struct plan_s {
   int adj_K = -1, adj_C = 0;     // the last unroll
   bool adj_valid = false;        // state unchanged since that unroll
   std::vector<int> ck_cur;       // z buffer holding z at each checkpoint
+  std::vector<SegmentGraph> adj_graphs;  // plan_backward's captured segments (segment_steps)
 
   template <class T> T* at(size_t off) const { return reinterpret_cast<T*>(ws + off); }
 
@@ -1288,6 +1345,7 @@ struct plan_s {
   // are captured from there): past the warm-up, and past the deferred dual
   // step of its last iteration
   int graph_from() const { return cfg.warm_iters > 0 ? cfg.warm_iters + 1 : 1; }
+  bool dense() const { return (cfg.flags & (PLAN_DENSE_STATE | PLAN_U_KEEP | PLAN_ADMM)) != 0; }
 
   Dev dev(int kk) const {
     Dev P{};
@@ -1304,7 +1362,7 @@ struct plan_s {
     P.alpha = (cfg.flags & PLAN_U_LITERAL) ? cfg.alpha / rho_at(kk > 0 ? kk - 1 : 0) : cfg.alpha;
     // keeping u on inactive edges (or standard ADMM, which updates every u)
     // needs every u record, so both imply the dense state
-    P.dense = (cfg.flags & (PLAN_DENSE_STATE | PLAN_U_KEEP | PLAN_ADMM)) ? 1 : 0;
+    P.dense = dense() ? 1 : 0;
     P.admm = (cfg.flags & PLAN_ADMM) ? 1 : 0;
     P.keep = (cfg.flags & PLAN_U_KEEP) ? 1 : 0;
     float2* z0 = at<float2>(L.z0);
@@ -1347,6 +1405,11 @@ plan_status settle_endpoints(plan_t h);
 }  // namespace
 
 namespace {
+
+void drop_segment_graphs(plan_t h) {
+  for (SegmentGraph& g : h->adj_graphs) cudaGraphExecDestroy(g.exec);
+  h->adj_graphs.clear();
+}
 
 cudaError_t clear_sums(plan_t h) {
   const size_t nodes = (size_t)h->p * (h->eta + 1);
@@ -1411,6 +1474,45 @@ int segment_warps(const plan_s* h) { return (1 + h->nw + h->nv) * h->eta * h->nt
 int list_ctas(const plan_s* h) {
   const long long pairs = (long long)(h->vo ? 1 : h->eta) * h->p * (h->p - 1) / 2;
   return (int)std::max<long long>(1, std::min<long long>((pairs + 32 * FACTOR_WARPS - 1) / (32 * FACTOR_WARPS), 2ll * h->sms));
+}
+
+// Problems that one CTA serves better than two launches per iteration over the
+// whole GPU.  Measured (circle swaps, us per iteration, one CTA / two
+// launches): eta = 4: 3.9 / 6.5 at p = 4, 4.3 / 6.3 at 16, 5.0 / 6.6 at 20,
+// 6.1 / 6.8 at 28, 6.9 / 7.3 at 32, 8.6 / 7.1 at 33; eta = 8: 5.6 / 6.3 at
+// p = 4, 6.5 / 6.8 at 20, 7.4 / 6.8 at 24; eta = 16: 6.9 / 6.4 at p = 4.  So:
+// tiles and segment warps within the CTA's warps, and pairs that make, with a
+// third of them active, about one list chunk per warp.
+bool solo(const plan_s* h) {
+  const long long eta = h->vo ? 1 : h->eta;
+  return h->cap && !h->profiling && !h->dense() && eta * h->ntp + segment_warps(h) <= SOLO_WARPS &&
+         eta * h->p * (h->p - 1) / 2 <= 1536;
+}
+
+// n iterations of a small problem from h->k on, past the warm-up, in launches
+// of at most SOLO_ITERS (a few milliseconds, so that a long solve leaves the
+// GPU to others now and then).  tape: where to record them, or null.
+constexpr int SOLO_ITERS = 512;
+plan_status run_solo(plan_t h, int n, const Tape* tape) {
+  while (n > 0) {
+    const int m = std::min(n, SOLO_ITERS), c0 = h->cur;
+    const Dev P0 = h->dev(h->k);
+    if (h->eta > 1) h->cur ^= 1;
+    const Dev P1 = h->dev(h->k + 1);
+    h->cur = c0;
+    Tape T{};
+    if (tape) T = *tape;
+    const int segw = segment_warps(h), tiles = (h->vo ? 1 : h->eta) * h->ntp;
+    // list warps: those the tiles and segments leave, at least half of the CTA's
+    const int nlist = std::min(list_ctas(h) * FACTOR_WARPS, std::max(SOLO_WARPS - tiles - segw, SOLO_WARPS / 2));
+    auto kern = h->noenergy ? run_kernel<true> : run_kernel<false>;
+    kern<<<1, 32 * SOLO_WARPS, 0, h->stream>>>(P0, P1, m, nlist, segw, tiles, node_warps(h->p, h->eta), T);
+    CK(cudaGetLastError());
+    if (h->eta > 1 && (m & 1)) h->cur ^= 1;
+    h->k += m;
+    n -= m;
+  }
+  return PLAN_OK;
 }
 
 // Every pair fits the worklist, so that an iteration may be split in listing
@@ -1543,6 +1645,11 @@ plan_status run_iterations(plan_t h, int n) {
   if (n > 0 && h->fresh) {
     if ((st = run_iteration(h)) != PLAN_OK) return st;
     --n;
+  }
+  if (solo(h)) {
+    for (; n > 0 && h->k < h->graph_from(); --n)
+      if ((st = run_iteration(h)) != PLAN_OK) return st;
+    return run_solo(h, n, nullptr);
   }
   if ((st = run_graph_runs(h, n, ITERS_PER_LONG_GRAPH, h->gexec64)) != PLAN_OK) return st;
   if ((st = run_graph_runs(h, n, ITERS_PER_GRAPH, h->gexec8)) != PLAN_OK) return st;
@@ -1782,6 +1889,7 @@ void plan_destroy(plan_t h) {
   if (h->gset) cudaGraphExecDestroy(h->gset);
   if (h->ep_event) cudaEventDestroy(h->ep_event);
   if (h->cap) cudaStreamDestroy(h->cap);
+  drop_segment_graphs(h);
   if (h->adj) cudaFree(h->adj);
   delete h;
 }
@@ -2102,16 +2210,21 @@ namespace {
 
 // The tape of one iteration: z^k, the kinetic u^k, and the active pairs and
 // gated segment factors with their u^k, compacted (both counts zeroed before).
-__global__ void record_kernel(Dev P, const float2* zk, float2* tz, float4* tukin, uint32_t* tfid,
-                              float4* tucl, float4* tuch, unsigned* tcount, uint32_t* tsidx,
-                              float4* tsu, unsigned* tscount) {
-  pdl_begin();
+// P is the iteration's own descriptor; threads t0, t0 + nt, ... (whole warps).
+__device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, char* slot, unsigned t0, unsigned nt) {
+  float2* tz = reinterpret_cast<float2*>(slot + T.z);
+  float4* tukin = reinterpret_cast<float4*>(slot + T.ukin);
+  uint32_t* tfid = reinterpret_cast<uint32_t*>(slot + T.fid);
+  float4 *tucl = reinterpret_cast<float4*>(slot + T.ucl), *tuch = reinterpret_cast<float4*>(slot + T.uch);
+  unsigned *tcount = reinterpret_cast<unsigned*>(slot + T.count), *tscount = reinterpret_cast<unsigned*>(slot + T.scount);
+  uint32_t* tsidx = reinterpret_cast<uint32_t*>(slot + T.sidx);
+  float4* tsu = reinterpret_cast<float4*>(slot + T.su);
   const unsigned nz = (unsigned)P.p * (P.eta + 1), nk = (unsigned)P.eta * P.p;
   const unsigned nseg = (unsigned)(P.nw + P.nv) * nk, nrows = (unsigned)P.eta * P.ntp * TILE;
   const unsigned n = (max(max(nz, nrows), nseg) + 31u) & ~31u;  // whole warps
   const int lane = threadIdx.x & 31;
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    if (t < nz) tz[t] = zk[t];
+  for (unsigned t = t0; t < n; t += nt) {
+    if (t < nz) tz[t] = P.z[t];
     if (t < nk) tukin[t] = P.ukin[t];
     const uint32_t word = t < nrows ? P.bits[t] : 0u;
     if (__any_sync(FULL, word != 0u)) {
@@ -2141,14 +2254,20 @@ __global__ void record_kernel(Dev P, const float2* zk, float2* tz, float4* tukin
     }
   }
 }
+__global__ void record_kernel(Dev P, Tape T) {
+  pdl_begin();
+  record_iteration(P, T, T.at, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
 
-// Zeroes two 32-bit counters in each of n slots stride bytes apart (the
-// compaction counters of every tape slot of a segment, before its replay).
-__global__ void zero_strided_kernel(char* a, char* b, size_t stride, int n) {
+// Before a segment's replay: zeroes the two compaction counters in each of its
+// n tape slots, stride bytes apart, and notes its first iteration, which the
+// adjoint kernels add to their own (so that one graph serves every segment).
+__global__ void begin_segment_kernel(char* a, char* b, size_t stride, int n, int* k0, int first) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     *reinterpret_cast<unsigned*>(a + i * stride) = 0u;
     *reinterpret_cast<unsigned*>(b + i * stride) = 0u;
   }
+  if (threadIdx.x == 0) *k0 = first;
 }
 
 // The adjoint passes run with programmatic dependent launch, like the
@@ -2156,6 +2275,7 @@ __global__ void zero_strided_kernel(char* a, char* b, size_t stride, int n) {
 // writes, but its CTAs are scheduled while the predecessor drains.
 __global__ void __launch_bounds__(256) bw_scatter_kernel(AdjDev A) {
   pdl_begin();
+  A.k += *A.k0;
   const unsigned n = (unsigned)(A.eta * A.p) + *A.count + *A.scount;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
     bw_scatter_item(A, t);
@@ -2169,9 +2289,38 @@ __global__ void bw_node_kernel(AdjDev A) {
 
 __global__ void __launch_bounds__(256) bw_factor_kernel(AdjDev A) {
   pdl_begin();
+  A.k += *A.k0;
   const unsigned n = (unsigned)(A.eta * A.p) + *A.count + *A.scount;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
     bw_factor_item(A, t);
+}
+
+// A small problem's adjoint steps of a whole segment, last iteration first, by
+// one CTA (run_kernel): A is the last iteration's descriptor, the tape slots
+// before it stride bytes apart.
+__global__ void __launch_bounds__(32 * SOLO_WARPS, 1) bw_run_kernel(AdjDev A, int iters, size_t stride) {
+  A.k += *A.k0;
+  auto back = [&](auto*& p) {
+    p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(reinterpret_cast<const char*>(p) - stride);
+  };
+#pragma unroll 1
+  for (int it = 0; it < iters; ++it) {
+    const unsigned n = (unsigned)(A.eta * A.p) + *A.count + *A.scount, nodes = (unsigned)(A.p * (A.eta + 1));
+    for (unsigned t = threadIdx.x; t < n; t += blockDim.x) bw_scatter_item(A, t);
+    __syncthreads();
+    for (unsigned t = threadIdx.x; t < nodes; t += blockDim.x) bw_node(A, (int)t);
+    __syncthreads();
+    for (unsigned t = threadIdx.x; t < n; t += blockDim.x) bw_factor_item(A, t);
+    __syncthreads();
+    A.k -= 1;
+    double2* in = const_cast<double2*>(A.zb_in);
+    A.zb_in = A.zb_out;
+    A.zb_out = in;
+    if (it + 1 < iters) {  // the tape slot of the iteration before
+      back(A.z); back(A.ukin); back(A.fid); back(A.ucl); back(A.uch); back(A.count); back(A.sidx); back(A.su);
+      back(A.scount);
+    }
+  }
 }
 
 __global__ void bw_init_kernel(int n, const float2* dz, double2* zb) {
@@ -2229,7 +2378,7 @@ struct AdjLayout {
   size_t cap, slot_bytes, tape0;
   size_t t_z, t_ukin, t_count, t_fid, t_ucl, t_uch;  // within one tape slot
   size_t t_scount, t_sidx, t_su, scap;
-  size_t ubk, ubl, ubh, stamp, ubs, sstamp, zbA, zbB, S, cnt, mbar, gs, gg, gr, gc;
+  size_t ubk, ubl, ubh, stamp, ubs, sstamp, zbA, zbB, S, cnt, mbar, gs, gg, gr, gc, k0;
   size_t total;
 };
 
@@ -2271,17 +2420,43 @@ AdjLayout adj_layout(plan_t h, int K, int C) {
   A.gg = take(p * 16);
   A.gr = take(p * 8);
   A.gc = take(p * eta * 8);
+  A.k0 = take(4);
   A.total = o;
   return A;
 }
 
+// The checkpoint's regions, copied by one launch (a dozen copies before): 16
+// bytes a thread, one grid row per region.  Every region starts and ends on a
+// 256-byte boundary, so whole float4 are copied.
+constexpr int CK_MAX = 16;
+struct CkCopy {
+  const float4* from[CK_MAX];
+  float4* to[CK_MAX];
+  size_t n[CK_MAX];  // float4 of each region
+};
+__global__ void __launch_bounds__(256) checkpoint_kernel(CkCopy C) {
+  const float4* from = C.from[blockIdx.y];
+  float4* to = C.to[blockIdx.y];
+  const size_t n = C.n[blockIdx.y];
+  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
+    to[t] = from[t];
+}
+
 plan_status snapshot(plan_t h, const AdjLayout& A, int idx, bool save) {
   char* ck = h->adj + A.ck0 + (size_t)idx * A.ck_bytes;
+  CkCopy C{};
+  int n = 0;
+  size_t largest = 0;
   for (const Region& r : ck_regions(h)) {
     char* ws = h->ws + r.off;
-    CK(cudaMemcpyAsync(save ? ck : ws, save ? ws : ck, r.bytes, cudaMemcpyDeviceToDevice, h->stream));
+    C.from[n] = reinterpret_cast<const float4*>(save ? ws : ck);
+    C.to[n] = reinterpret_cast<float4*>(save ? ck : ws);
+    C.n[n] = (r.bytes + 15) / 16;
+    largest = std::max(largest, C.n[n++]);
     ck += a256(r.bytes);
   }
+  checkpoint_kernel<<<dim3((unsigned)std::min<size_t>((largest + 255) / 256, 608), (unsigned)n), 256, 0, h->stream>>>(C);
+  CK(cudaGetLastError());
   if (!save) {
     // the worklist is not part of the state
     plan_status st = drop_worklist(h);
@@ -2290,9 +2465,16 @@ plan_status snapshot(plan_t h, const AdjLayout& A, int idx, bool save) {
   return PLAN_OK;
 }
 
-AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, int k, char* zb_in, char* zb_out) {
+Tape adj_tape(plan_t h, const AdjLayout& A) {
+  return {h->adj + A.tape0, A.slot_bytes, A.t_z, A.t_ukin, A.t_count, A.t_fid, A.t_ucl, A.t_uch, A.t_scount, A.t_sidx,
+          A.t_su};
+}
+
+// Adjoint of the iteration `slot` of a segment (iterations count from the
+// segment's first, AdjDev::k0).
+AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, char* zb_in, char* zb_out) {
   AdjDev D{};
-  D.p = h->p; D.eta = h->eta; D.ntp = h->ntp; D.k = k;
+  D.p = h->p; D.eta = h->eta; D.ntp = h->ntp; D.k = slot;
   D.rho = h->cfg.rho0;
   D.alpha = (h->cfg.flags & PLAN_U_LITERAL) ? h->cfg.alpha / h->cfg.rho0 : h->cfg.alpha;
   D.tiles = h->at<int2>(h->L.tiles);
@@ -2318,6 +2500,7 @@ AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, int k, char* zb_in, char*
   D.ubl = reinterpret_cast<float4*>(h->adj + A.ubl);
   D.ubh = reinterpret_cast<float4*>(h->adj + A.ubh);
   D.stamp = reinterpret_cast<int*>(h->adj + A.stamp);
+  D.k0 = reinterpret_cast<const int*>(h->adj + A.k0);
   D.zb_in = reinterpret_cast<const double2*>(zb_in);
   D.zb_out = reinterpret_cast<double2*>(zb_out);
   D.S = reinterpret_cast<double2*>(h->adj + A.S);
@@ -2328,6 +2511,92 @@ AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, int k, char* zb_in, char*
   D.g_r = reinterpret_cast<double*>(h->adj + A.gr);
   D.g_c = reinterpret_cast<double*>(h->adj + A.gc);
   return D;
+}
+
+// One segment of the backward pass on the given stream: n iterations from h->k
+// recorded, then their adjoint steps, last iteration first (no state change
+// on the host).
+plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, char* zb_in, char* zb_out, cudaStream_t ms) {
+  const int k0 = h->k, c0 = h->cur;
+  const bool fresh = h->fresh;
+  Tape T = adj_tape(h, A);
+  plan_status st = PLAN_OK;
+  cudaError_t e = cudaSuccess;
+  for (int q = 0; q < n && st == PLAN_OK && e == cudaSuccess; ++q) {
+    st = enqueue_iteration(h, ms);
+    if (st != PLAN_OK) break;
+    e = launch_pdl(record_kernel, (unsigned)h->prox_grid, 256u, ms, h->dev(h->k), T);
+    T.at += T.stride;
+    h->fresh = false;
+    if (h->eta > 1) h->cur ^= 1;
+    h->k += 1;
+  }
+  h->k = k0;
+  h->cur = c0;
+  h->fresh = fresh;
+  const unsigned node_grid = (unsigned)((h->p * (h->eta + 1) + 255) / 256);
+  for (int q = n - 1; q >= 0 && st == PLAN_OK && e == cudaSuccess; --q) {
+    const AdjDev D = adj_dev(h, A, q, zb_in, zb_out);
+    e = launch_pdl(bw_scatter_kernel, (unsigned)h->prox_grid, 256u, ms, D);
+    if (e == cudaSuccess) e = launch_pdl(bw_node_kernel, node_grid, 256u, ms, D);
+    if (e == cudaSuccess) e = launch_pdl(bw_factor_kernel, (unsigned)h->prox_grid, 256u, ms, D);
+    std::swap(zb_in, zb_out);
+  }
+  if (st == PLAN_OK && e != cudaSuccess) st = fail(PLAN_ECUDA, "adjoint launch failed: %s", cudaGetErrorString(e));
+  return st;
+}
+
+// The same, run: by one CTA for a small problem; else replayed from a graph,
+// kept with the plan (six launches an iteration, each about 6 us of host time
+// when made one by one, bound the backward pass at any size: 34 us an
+// iteration at p = 64).  Segments differ in their length, in the parity and z
+// buffer of their first iteration, in where the adjoint of z stands, and
+// iteration 0 has no residual slot before it; the rest is the same for all of
+// them, the iteration number coming from AdjDev::k0.
+plan_status segment_steps(plan_t h, const AdjLayout& A, int n, char* zb_in, char* zb_out) {
+  plan_status st = ensure_prox_grid(h);
+  if (st != PLAN_OK) return st;
+  if (solo(h)) {
+    Tape T = adj_tape(h, A);
+    const int end = h->k + n;
+    while (h->k < end && (h->fresh || h->k < h->graph_from())) {  // the first one has no worklist yet
+      const Dev P = h->dev(h->k);
+      if ((st = run_iteration(h)) != PLAN_OK) return st;
+      CK(launch_pdl(record_kernel, (unsigned)h->prox_grid, 256u, h->stream, P, T));
+      T.at += T.stride;
+    }
+    if (h->k < end && (st = run_solo(h, end - h->k, &T)) != PLAN_OK) return st;
+    bw_run_kernel<<<1, 32 * SOLO_WARPS, 0, h->stream>>>(adj_dev(h, A, n - 1, zb_in, zb_out), n, A.slot_bytes);
+    CK(cudaGetLastError());
+    return PLAN_OK;
+  }
+  if (h->profiling) {  // each kernel is timed on its own: launched one by one
+    if ((st = enqueue_segment(h, A, n, zb_in, zb_out, h->stream)) != PLAN_OK) return st;
+  } else {
+    const SegmentGraph key = {n, h->k & 1, h->cur, h->k == 0, zb_in == h->adj + A.zbA, nullptr};
+    const SegmentGraph* found = nullptr;
+    for (const SegmentGraph& g : h->adj_graphs)
+      if (g.n == key.n && g.parity == key.parity && g.cur == key.cur && g.first == key.first && g.zb == key.zb) found = &g;
+    if (!found) {
+      if (h->adj_graphs.size() >= 8) drop_segment_graphs(h);
+      cudaGraph_t g = nullptr;
+      CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
+      st = enqueue_segment(h, A, n, zb_in, zb_out, h->cap);
+      cudaError_t e = cudaStreamEndCapture(h->cap, &g);
+      SegmentGraph made = key;
+      if (st == PLAN_OK && e == cudaSuccess) e = cudaGraphInstantiate(&made.exec, g, 0);
+      if (g) cudaGraphDestroy(g);
+      if (st != PLAN_OK) return st;
+      if (e != cudaSuccess) return fail(PLAN_ECUDA, "backward graph: %s", cudaGetErrorString(e));
+      h->adj_graphs.push_back(made);
+      found = &h->adj_graphs.back();
+    }
+    CK(cudaGraphLaunch(found->exec, h->stream));
+  }
+  h->fresh = false;
+  if (h->eta > 1 && (n & 1)) h->cur ^= 1;
+  h->k += n;
+  return PLAN_OK;
 }
 
 plan_status adj_supported(plan_t h) {
@@ -2542,9 +2811,14 @@ plan_status plan_unroll(plan_t h, int K, int checkpoint_every) {
   int C = checkpoint_every ? checkpoint_every : (int)std::ceil(std::sqrt((double)std::max(K, 1)));
   C = std::max(1, std::min(C, std::max(K, 1)));
   const AdjLayout A = adj_layout(h, K, C);
+  if ((K != h->adj_K || C != h->adj_C) && !h->adj_graphs.empty()) {  // captured for other offsets
+    CK(cudaStreamSynchronize(h->stream));
+    drop_segment_graphs(h);
+  }
   if (h->adj_bytes < A.total) {
     if (h->adj) {
       CK(cudaStreamSynchronize(h->stream));
+      drop_segment_graphs(h);
       cudaFree(h->adj);
       h->adj = nullptr;
       h->adj_bytes = 0;
@@ -2583,7 +2857,7 @@ plan_status plan_backward(plan_t h, int K, const float* dL_dz, float* d_start, f
   if ((st = ensure_prox_grid(h)) != PLAN_OK) return st;
   const int C = h->adj_C;
   const AdjLayout A = adj_layout(h, K, C);
-  const size_t p = h->p, E1 = h->eta + 1, nodes = p * E1;
+  const size_t p = h->p, nodes = p * (h->eta + 1);
   // adjoint state: u adjoints 0, no stamps, gradients 0, zbar = dL/dz^K
   CK(cudaMemsetAsync(h->adj + A.ubk, 0, (size_t)h->eta * p * 16, h->stream));
   CK(cudaMemsetAsync(h->adj + A.stamp, 0xff, h->slots * 4, h->stream));
@@ -2597,39 +2871,20 @@ plan_status plan_backward(plan_t h, int K, const float* dL_dz, float* d_start, f
   char* zb_in = h->adj + A.zbA;
   char* zb_out = h->adj + A.zbB;
   const int nseg = A.nck - 1;
-  const unsigned node_grid = (unsigned)((nodes + 255) / 256);
   for (int seg = nseg - 1; seg >= 0; --seg) {
-    const int c0 = seg * C, c1 = std::min(K, c0 + C);
+    const int c0 = seg * C, n = std::min(K, c0 + C) - c0;
     // recompute the segment from its checkpoint, recording each iteration
     if ((st = snapshot(h, A, seg, false)) != PLAN_OK) return st;
     h->k = c0;
     h->cur = h->ck_cur[seg];
     if ((st = refresh_segments(h)) != PLAN_OK) return st;
-    zero_strided_kernel<<<1, 64, 0, h->stream>>>(h->adj + A.tape0 + A.t_count, h->adj + A.tape0 + A.t_scount,
-                                                 A.slot_bytes, c1 - c0);
+    begin_segment_kernel<<<1, 64, 0, h->stream>>>(h->adj + A.tape0 + A.t_count, h->adj + A.tape0 + A.t_scount,
+                                                  A.slot_bytes, n, reinterpret_cast<int*>(h->adj + A.k0), c0);
     CK(cudaGetLastError());
-    for (int k = c0; k < c1; ++k) {
-      const float2* zk = h->cur ? h->at<float2>(h->L.z1) : h->at<float2>(h->L.z0);
-      if ((st = run_iteration(h)) != PLAN_OK) return st;
-      char* t = h->adj + A.tape0 + (size_t)(k - c0) * A.slot_bytes;
-      CK(launch_pdl(record_kernel, (unsigned)h->prox_grid, 256u, h->stream, h->dev(k), zk,
-                    reinterpret_cast<float2*>(t + A.t_z), reinterpret_cast<float4*>(t + A.t_ukin),
-                    reinterpret_cast<uint32_t*>(t + A.t_fid), reinterpret_cast<float4*>(t + A.t_ucl),
-                    reinterpret_cast<float4*>(t + A.t_uch), reinterpret_cast<unsigned*>(t + A.t_count),
-                    reinterpret_cast<uint32_t*>(t + A.t_sidx), reinterpret_cast<float4*>(t + A.t_su),
-                    reinterpret_cast<unsigned*>(t + A.t_scount)));
-    }
-    // the adjoint steps of the segment, last iteration first
-    for (int k = c1 - 1; k >= c0; --k) {
-      const AdjDev D = adj_dev(h, A, k - c0, k, zb_in, zb_out);
-      CK(launch_pdl(bw_scatter_kernel, (unsigned)h->prox_grid, 256u, h->stream, D));
-      CK(launch_pdl(bw_node_kernel, node_grid, 256u, h->stream, D));
-      CK(launch_pdl(bw_factor_kernel, (unsigned)h->prox_grid, 256u, h->stream, D));
-      CK(cudaGetLastError());
-      std::swap(zb_in, zb_out);
-    }
+    if ((st = segment_steps(h, A, n, zb_in, zb_out)) != PLAN_OK) return st;
+    if (n & 1) std::swap(zb_in, zb_out);
   }
-  const AdjDev D = adj_dev(h, A, 0, 0, zb_in, zb_out);
+  const AdjDev D = adj_dev(h, A, 0, zb_in, zb_out);
   const double norm = (h->cfg.flags & (PLAN_COST_UNNORM | PLAN_VO)) ? 1.0 : 1.0 / ((double)p * h->eta);
   bw_final_kernel<<<(unsigned)((p + 127) / 128), 128, 0, h->stream>>>(
       D, reinterpret_cast<const double2*>(zb_in), norm, (h->cfg.flags & PLAN_COST_PER_SEGMENT) ? 1 : 0,

@@ -25,7 +25,7 @@
 namespace {
 
 struct AdjDev {
-  int p, eta, ntp, k;
+  int p, eta, ntp, k;       // k: iteration (kernels add *k0, the first one of their segment)
   float rho, alpha;
   const int2* tiles;
   const float* radius;
@@ -49,6 +49,7 @@ struct AdjDev {
   float4* ubk;              // kinetic u adjoints, [eta][p]: of u^{k+1} in, u^k out
   float4* ubl;              // collision u adjoints by slot (lower, upper)
   float4* ubh;
+  const int* k0;
   int* stamp;               // the iteration whose u adjoint a slot holds
   float4* ubs;              // gated segment factor u adjoints, [(nw + nv) eta p]
   int* sstamp;              // ... and the iteration that wrote them
@@ -75,6 +76,14 @@ __device__ __forceinline__ void decode_slot(const AdjDev& A, uint32_t f, int& s,
   const int2 IJ = A.tiles[blk - (uint32_t)s * A.ntp];
   i = IJ.x * TILE + (int)r;
   j = IJ.y * TILE + (int)c;
+}
+
+// The u adjoint of pair slot f, 0 unless the iteration after this one wrote
+// it.  Loaded beside the stamp, not after it (a slot never written holds
+// anything, and is not used).
+__device__ __forceinline__ float4 live_ub(const AdjDev& A, const float4* ub, uint32_t f) {
+  const float4 v = ub[f];
+  return A.stamp[f] == A.k + 1 ? v : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 __device__ __forceinline__ void scatter_edge(const AdjDev& A, int i, int s, float2 ub) {
@@ -106,9 +115,7 @@ __device__ __forceinline__ void bw_scatter_item(const AdjDev& A, unsigned t) {
   const uint32_t f = A.fid[t - nkin];
   int s, i, j;
   decode_slot(A, f, s, i, j);
-  const bool live = A.stamp[f] == A.k + 1;
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4 bl = live ? A.ubl[f] : zero, bh = live ? A.ubh[f] : zero;
+  const float4 bl = live_ub(A, A.ubl, f), bh = live_ub(A, A.ubh, f);
   if (s > 0) { scatter_edge(A, i, s, lo2(bl)); scatter_edge(A, j, s, hi2(bl)); }
   if (s + 1 < A.eta) { scatter_edge(A, i, s + 1, lo2(bh)); scatter_edge(A, j, s + 1, hi2(bh)); }
 }
@@ -208,9 +215,7 @@ __device__ __forceinline__ void bw_factor_item(const AdjDev& A, unsigned t) {
   // n exactly as the forward minimizer pass formed it
   const float2 nil = A.z[(size_t)i * E1 + s] - lo2(a), nih = A.z[(size_t)i * E1 + s + 1] - lo2(b);
   const float2 njl = A.z[(size_t)j * E1 + s] - hi2(a), njh = A.z[(size_t)j * E1 + s + 1] - hi2(b);
-  const bool live = A.stamp[f] == A.k + 1;
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4 bl = live ? A.ubl[f] : zero, bh = live ? A.ubh[f] : zero;
+  const float4 bl = live_ub(A, A.ubl, f), bh = live_ub(A, A.ubh, f);
   float2 mil, mjl, mih, mjh;
   const float2 xil = edge_xbar(A, pin_lo, i, s, lo2(bl), mil);
   const float2 xjl = edge_xbar(A, pin_lo, j, s, hi2(bl), mjl);

@@ -55,3 +55,48 @@ def test_break_point_counts_around_a_node_warp(eta):
     st = par.oracle_state(prob, 4)
     new, info = twa.iterate(prob, st, record_branches=True)
     par.compare(prob, new, info, par.gpu_step(prob, st))
+
+
+@pytest.mark.parametrize("p,eta", [(2, 1), (5, 3), (20, 8), (28, 4), (29, 4), (16, 8)])
+def test_single_cta_runs_equal_iterations_one_kernel_at_a_time(p, eta):
+    """Problems on both sides of the single-CTA rule: runs of iterations
+    against the same iterations launched kernel by kernel (profiling), with
+    odd run lengths, the feasibility mode and walls."""
+    import paper_1311_4527_gb300 as pk
+    for inst, kw in ((workloads.circle_swap(p, eta, 0.04, 0.005, 3), {}),
+                     (workloads.circle_swap(p, eta, 0.04, 0.005, 3), {"energy": False}),
+                     (workloads.small_square(p, eta, seed=p), {"vmax": 0.4})):
+        out = []
+        for single in (True, False):
+            with pk.Planner.from_instance(inst, **kw) as pl:
+                if not single:
+                    pl.profile_start()
+                zs = []
+                for n in (1, 1, 6, 33):
+                    pl.iterate(n)
+                    zs.append(pl.trajectory().cpu().numpy())
+                out.append(zs + [pl.iterate(2, residual=True)])
+        for a, b in zip(*out):
+            assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("p,eta,K,C", [(4, 4, 23, 5), (40, 4, 23, 5), (40, 4, 24, 6), (33, 2, 7, 7)])
+def test_backward_by_graph_and_by_one_cta_match_single_launches(p, eta, K, C):
+    """The captured segments (odd and even lengths, the first one and the
+    rest, called again with another loss) and the single-CTA form against the
+    same steps launched one by one: equal up to the order of FP64 atomics."""
+    import torch
+    import paper_1311_4527_gb300 as pk
+    inst = workloads.circle_swap(p, eta, 0.03, 0.005, 7)
+    gen = torch.Generator().manual_seed(3)
+    losses = [torch.randn(p, eta + 1, 2, generator=gen) for _ in range(2)]
+    with pk.Planner.from_instance(inst) as pl, pk.Planner.from_instance(inst) as ref:
+        pl.unroll(3, 2)  # another layout first
+        pl.backward(losses[0])
+        ref.profile_start()
+        for g in losses:
+            pl.unroll(K, C)
+            ref.unroll(K, C)
+            assert torch.equal(pl.trajectory(), ref.trajectory())
+            for a, b in zip(pl.backward(g), ref.backward(g)):
+                assert torch.allclose(a, b, rtol=1e-5, atol=1e-6 * float(b.abs().max()))
