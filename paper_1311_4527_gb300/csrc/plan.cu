@@ -118,12 +118,90 @@ __global__ void __launch_bounds__(256) prox_kernel(Dev P) {
   for (unsigned long long t = 32ull * v + (threadIdx.x & 31); t < nc; t += 32ull * G * wpb) prox_item(P, P.work[t]);
 }
 
+// Where an iteration is recorded for the backward pass: z^k, the kinetic u^k,
+// and the active pairs and gated segment factors with their u^k, compacted
+// (both counts zeroed before).
+struct Tape {
+  char* at;  // the iteration's slot (null: nothing is recorded)
+  size_t stride, z, ukin, count, fid, ucl, uch, scount, sidx, su;
+  int from_list;  // the worklist holds every active pair (it cannot run out): else from the bits
+};
+
+// Records the iteration of descriptor P after its factor pass; threads t0, t0
+// + nt, ... (whole warps).
+__device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, char* slot, unsigned t0, unsigned nt) {
+  float2* tz = reinterpret_cast<float2*>(slot + T.z);
+  float4* tukin = reinterpret_cast<float4*>(slot + T.ukin);
+  uint32_t* tfid = reinterpret_cast<uint32_t*>(slot + T.fid);
+  float4 *tucl = reinterpret_cast<float4*>(slot + T.ucl), *tuch = reinterpret_cast<float4*>(slot + T.uch);
+  unsigned *tcount = reinterpret_cast<unsigned*>(slot + T.count), *tscount = reinterpret_cast<unsigned*>(slot + T.scount);
+  uint32_t* tsidx = reinterpret_cast<uint32_t*>(slot + T.sidx);
+  float4* tsu = reinterpret_cast<float4*>(slot + T.su);
+  const unsigned nz = (unsigned)P.p * (P.eta + 1), nk = (unsigned)P.eta * P.p;
+  const unsigned nseg = (unsigned)(P.nw + P.nv) * nk;
+  const unsigned npairs = T.from_list ? *P.work_count : (unsigned)P.eta * P.ntp * TILE;
+  const unsigned n = (max(max(nz, npairs), nseg) + 31u) & ~31u;  // whole warps
+  const int lane = threadIdx.x & 31;
+  for (unsigned t = t0; t < n; t += nt) {
+    if (t < nz) tz[t] = P.z[t];
+    if (t < nk) tukin[t] = P.ukin[t];
+    // this lane's active pairs: one list entry's, or a row's bits
+    uint32_t word = 0u, first = t * TILE;
+    if (t < npairs) {
+      if (T.from_list) {
+        const uint32_t e = P.work[t];
+        word = e >> 31;
+        first = e & ~ACTIVE;
+      } else {
+        word = P.bits[t];
+      }
+    }
+    if (__any_sync(FULL, word != 0u)) {
+      const unsigned cnt = __popc(word);
+      unsigned incl = cnt;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += v;
+      }
+      unsigned at = 0;
+      if (lane == 31) at = atomicAdd(tcount, incl);
+      at = __shfl_sync(FULL, at, 31) + (incl - cnt);
+      for (uint32_t w = word; w; w &= w - 1u, ++at) {
+        const uint32_t f = first + (uint32_t)(__ffs(w) - 1);
+        tfid[at] = f;
+        tucl[at] = P.ulo[f];
+        tuch[at] = P.uhi[f];
+      }
+    }
+    if (t < nseg) {
+      const unsigned i = t % P.p, ws = t / P.p;
+      if ((P.wbits[(size_t)ws * P.nt + i / TILE] >> (i % TILE)) & 1u) {
+        const unsigned at = atomicAdd(tscount, 1u);
+        tsidx[at] = t;
+        tsu[at] = P.uwall[t];
+      }
+    }
+  }
+}
+
+// Node pass.
 constexpr int NODE_WARPS = 2;
-__global__ void __launch_bounds__(32 * NODE_WARPS) node_kernel(Dev P) {
-  pdl_begin();
+__device__ __forceinline__ void node_pass(const Dev& P) {
   const int warp = (int)blockIdx.x * NODE_WARPS + (threadIdx.x >> 5);
   if (blockIdx.x == 0 && threadIdx.x == 0) advance_worklist(P, false);
   consensus_warp(P, warp);
+}
+__global__ void __launch_bounds__(32 * NODE_WARPS) node_kernel(Dev P) {
+  pdl_begin();
+  node_pass(P);
+}
+// The node pass beside the record of the iteration (the CTAs past node_ctas),
+// which like it needs the factor pass only.  A kernel of its own: the tape's
+// parameters cost the plain pass 0.1 us of each iteration.
+__global__ void __launch_bounds__(32 * NODE_WARPS) node_record_kernel(Dev P, Tape T, int node_ctas) {
+  pdl_begin();
+  if ((int)blockIdx.x < node_ctas) node_pass(P);
+  else record_iteration(P, T, T.at, (blockIdx.x - node_ctas) * blockDim.x + threadIdx.x, (gridDim.x - node_ctas) * blockDim.x);
 }
 
 // The segment records of the factor pass after z, a fixed end or a radius was
@@ -148,12 +226,6 @@ __global__ void segments_kernel(Dev P) {
 // tape (differentiation): each iteration's record is written beside its node
 // pass.
 constexpr int SOLO_WARPS = 16;
-struct Tape {
-  char* at;  // the first iteration's slot (null: nothing is recorded)
-  size_t stride, z, ukin, count, fid, ucl, uch, scount, sidx, su;
-};
-__device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, char* slot, unsigned t0, unsigned nt);
-
 template <bool CLASSES>
 __global__ void __launch_bounds__(32 * SOLO_WARPS, 1) run_kernel(Dev P0, Dev P1, int iters, int nlist, int seg_warps,
                                                                  int tile_warps, int nodes, Tape T) {
@@ -1521,8 +1593,17 @@ bool lists_every_pair(const plan_s* h) {
   return (unsigned long long)(h->vo ? 1 : h->eta) * h->p * (h->p - 1) / 2 <= h->L.cap;
 }
 
+// CTAs that record an iteration: a thread per break-point, list entry (or
+// activity word) and segment factor, up to four CTAs an SM.
+int record_ctas(const plan_s* h) {
+  const long long pairs = (long long)h->eta * h->p * (h->p - 1) / 2;
+  const long long n = std::max({(long long)h->p * (h->eta + 1), std::min<long long>(pairs, (long long)h->eta * h->ntp * TILE * 4),
+                                (long long)(h->nw + h->nv) * h->eta * h->p});
+  return (int)std::min<long long>((n + 32 * NODE_WARPS - 1) / (32 * NODE_WARPS), 4ll * h->sms);
+}
+
 // Enqueue the kernels of iteration h->k (no state change on the host).
-plan_status enqueue_iteration(plan_t h, cudaStream_t ms) {
+plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = nullptr) {
   Dev P = h->dev(h->k);
   const int segw = segment_warps(h);
   const bool prof = h->profiling;
@@ -1553,8 +1634,11 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms) {
   if (prof) CK(cudaEventRecord(h->pev[2], ms));
   // the node pass also sets up the next iteration's worklist, so it runs even
   // when there is no free break-point (eta = 1)
-  const int nodew = node_warps(h->p, h->eta);
-  CK(launch_pdl(node_kernel, (unsigned)((nodew + NODE_WARPS - 1) / NODE_WARPS), 32u * NODE_WARPS, ms, P));
+  const int node_ctas = (node_warps(h->p, h->eta) + NODE_WARPS - 1) / NODE_WARPS;
+  if (tape)
+    CK(launch_pdl(node_record_kernel, (unsigned)(node_ctas + record_ctas(h)), 32u * NODE_WARPS, ms, P, *tape, node_ctas));
+  else
+    CK(launch_pdl(node_kernel, (unsigned)node_ctas, 32u * NODE_WARPS, ms, P));
   if (prof) {
     CK(cudaEventRecord(h->pend, ms));
     CK(cudaEventSynchronize(h->pend));
@@ -2208,57 +2292,6 @@ plan_status plan_profile(plan_t h, int enable, float* ms, int* iterations) {
 // ---------------------------------------------------------------------------
 namespace {
 
-// The tape of one iteration: z^k, the kinetic u^k, and the active pairs and
-// gated segment factors with their u^k, compacted (both counts zeroed before).
-// P is the iteration's own descriptor; threads t0, t0 + nt, ... (whole warps).
-__device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, char* slot, unsigned t0, unsigned nt) {
-  float2* tz = reinterpret_cast<float2*>(slot + T.z);
-  float4* tukin = reinterpret_cast<float4*>(slot + T.ukin);
-  uint32_t* tfid = reinterpret_cast<uint32_t*>(slot + T.fid);
-  float4 *tucl = reinterpret_cast<float4*>(slot + T.ucl), *tuch = reinterpret_cast<float4*>(slot + T.uch);
-  unsigned *tcount = reinterpret_cast<unsigned*>(slot + T.count), *tscount = reinterpret_cast<unsigned*>(slot + T.scount);
-  uint32_t* tsidx = reinterpret_cast<uint32_t*>(slot + T.sidx);
-  float4* tsu = reinterpret_cast<float4*>(slot + T.su);
-  const unsigned nz = (unsigned)P.p * (P.eta + 1), nk = (unsigned)P.eta * P.p;
-  const unsigned nseg = (unsigned)(P.nw + P.nv) * nk, nrows = (unsigned)P.eta * P.ntp * TILE;
-  const unsigned n = (max(max(nz, nrows), nseg) + 31u) & ~31u;  // whole warps
-  const int lane = threadIdx.x & 31;
-  for (unsigned t = t0; t < n; t += nt) {
-    if (t < nz) tz[t] = P.z[t];
-    if (t < nk) tukin[t] = P.ukin[t];
-    const uint32_t word = t < nrows ? P.bits[t] : 0u;
-    if (__any_sync(FULL, word != 0u)) {
-      const unsigned cnt = __popc(word);
-      unsigned incl = cnt;
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned v = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += v;
-      }
-      unsigned at = 0;
-      if (lane == 31) at = atomicAdd(tcount, incl);
-      at = __shfl_sync(FULL, at, 31) + (incl - cnt);
-      for (uint32_t w = word; w; w &= w - 1u, ++at) {
-        const uint32_t f = t * TILE + (uint32_t)(__ffs(w) - 1);
-        tfid[at] = f;
-        tucl[at] = P.ulo[f];
-        tuch[at] = P.uhi[f];
-      }
-    }
-    if (t < nseg) {
-      const unsigned i = t % P.p, ws = t / P.p;
-      if ((P.wbits[(size_t)ws * P.nt + i / TILE] >> (i % TILE)) & 1u) {
-        const unsigned at = atomicAdd(tscount, 1u);
-        tsidx[at] = t;
-        tsu[at] = P.uwall[t];
-      }
-    }
-  }
-}
-__global__ void record_kernel(Dev P, Tape T) {
-  pdl_begin();
-  record_iteration(P, T, T.at, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-}
-
 // Before a segment's replay: zeroes the two compaction counters in each of its
 // n tape slots, stride bytes apart, and notes its first iteration, which the
 // adjoint kernels add to their own (so that one graph serves every segment).
@@ -2273,7 +2306,7 @@ __global__ void begin_segment_kernel(char* a, char* b, size_t stride, int n, int
 // The adjoint passes run with programmatic dependent launch, like the
 // forward ones: each waits (griddepcontrol.wait) for its predecessor's
 // writes, but its CTAs are scheduled while the predecessor drains.
-__global__ void __launch_bounds__(256) bw_scatter_kernel(AdjDev A) {
+__global__ void __launch_bounds__(128) bw_scatter_kernel(AdjDev A) {
   pdl_begin();
   A.k += *A.k0;
   const unsigned n = (unsigned)(A.eta * A.p) + *A.count + *A.scount;
@@ -2287,7 +2320,7 @@ __global__ void bw_node_kernel(AdjDev A) {
   if (t < A.p * (A.eta + 1)) bw_node(A, t);
 }
 
-__global__ void __launch_bounds__(256) bw_factor_kernel(AdjDev A) {
+__global__ void __launch_bounds__(128) bw_factor_kernel(AdjDev A) {
   pdl_begin();
   A.k += *A.k0;
   const unsigned n = (unsigned)(A.eta * A.p) + *A.count + *A.scount;
@@ -2467,7 +2500,7 @@ plan_status snapshot(plan_t h, const AdjLayout& A, int idx, bool save) {
 
 Tape adj_tape(plan_t h, const AdjLayout& A) {
   return {h->adj + A.tape0, A.slot_bytes, A.t_z, A.t_ukin, A.t_count, A.t_fid, A.t_ucl, A.t_uch, A.t_scount, A.t_sidx,
-          A.t_su};
+          A.t_su, !h->dense() && lists_every_pair(h) ? 1 : 0};
 }
 
 // Adjoint of the iteration `slot` of a segment (iterations count from the
@@ -2523,9 +2556,7 @@ plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, char* zb_in, ch
   plan_status st = PLAN_OK;
   cudaError_t e = cudaSuccess;
   for (int q = 0; q < n && st == PLAN_OK && e == cudaSuccess; ++q) {
-    st = enqueue_iteration(h, ms);
-    if (st != PLAN_OK) break;
-    e = launch_pdl(record_kernel, (unsigned)h->prox_grid, 256u, ms, h->dev(h->k), T);
+    st = enqueue_iteration(h, ms, &T);
     T.at += T.stride;
     h->fresh = false;
     if (h->eta > 1) h->cur ^= 1;
@@ -2535,11 +2566,14 @@ plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, char* zb_in, ch
   h->cur = c0;
   h->fresh = fresh;
   const unsigned node_grid = (unsigned)((h->p * (h->eta + 1) + 255) / 256);
+  // a thread per edge group that may be active (more CTAs than that only cost their launch)
+  const long long items = (long long)(1 + h->nw + h->nv) * h->eta * h->p + (long long)h->eta * h->p * (h->p - 1) / 2;
+  const unsigned grid = (unsigned)std::min<long long>((items + 127) / 128, 2ll * h->prox_grid);
   for (int q = n - 1; q >= 0 && st == PLAN_OK && e == cudaSuccess; --q) {
     const AdjDev D = adj_dev(h, A, q, zb_in, zb_out);
-    e = launch_pdl(bw_scatter_kernel, (unsigned)h->prox_grid, 256u, ms, D);
+    e = launch_pdl(bw_scatter_kernel, grid, 128u, ms, D);
     if (e == cudaSuccess) e = launch_pdl(bw_node_kernel, node_grid, 256u, ms, D);
-    if (e == cudaSuccess) e = launch_pdl(bw_factor_kernel, (unsigned)h->prox_grid, 256u, ms, D);
+    if (e == cudaSuccess) e = launch_pdl(bw_factor_kernel, grid, 128u, ms, D);
     std::swap(zb_in, zb_out);
   }
   if (st == PLAN_OK && e != cudaSuccess) st = fail(PLAN_ECUDA, "adjoint launch failed: %s", cudaGetErrorString(e));
@@ -2560,10 +2594,11 @@ plan_status segment_steps(plan_t h, const AdjLayout& A, int n, char* zb_in, char
     Tape T = adj_tape(h, A);
     const int end = h->k + n;
     while (h->k < end && (h->fresh || h->k < h->graph_from())) {  // the first one has no worklist yet
-      const Dev P = h->dev(h->k);
-      if ((st = run_iteration(h)) != PLAN_OK) return st;
-      CK(launch_pdl(record_kernel, (unsigned)h->prox_grid, 256u, h->stream, P, T));
+      if ((st = enqueue_iteration(h, h->stream, &T)) != PLAN_OK) return st;
       T.at += T.stride;
+      h->fresh = false;
+      if (h->eta > 1) h->cur ^= 1;
+      h->k += 1;
     }
     if (h->k < end && (st = run_solo(h, end - h->k, &T)) != PLAN_OK) return st;
     bw_run_kernel<<<1, 32 * SOLO_WARPS, 0, h->stream>>>(adj_dev(h, A, n - 1, zb_in, zb_out), n, A.slot_bytes);
