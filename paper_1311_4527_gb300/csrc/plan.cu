@@ -58,10 +58,10 @@ constexpr int TEST_ROWS = TILE / TEST_WARPS;
 constexpr int FACTOR_WARPS = 4;
 struct FactorGrid {
   int list_ctas, lead_ctas;  // CTAs of the worklist, and of tiles ahead of the segment warps
-  int seg_ctas, seg_warps, tile_warps;
+  int seg_ctas, seg_warps, tile_warps, strip;
   int mode;                  // FactorMode
 };
-template <bool CLASSES>
+template <bool CLASSES, bool SORTED>
 __global__ void __launch_bounds__(32 * FACTOR_WARPS, 6) factor_kernel(Dev P, FactorGrid G) {
   __shared__ TileMem mem[FACTOR_WARPS];
   pdl_begin();
@@ -82,7 +82,8 @@ __global__ void __launch_bounds__(32 * FACTOR_WARPS, 6) factor_kernel(Dev P, Fac
     if (item >= G.tile_warps) return;  // warp-uniform
     item += nlist;
   }
-  collision_warp<CLASSES>(P, item, nlist, mem + warp, G.mode);
+  if (SORTED) sorted_collision_warp<CLASSES>(P, item, nlist, G.strip, mem + warp, G.mode);
+  else collision_warp<CLASSES>(P, item, nlist, mem + warp, G.mode);
 }
 
 // Dense state, pass 1: the first CTAs take the kinetic, wall and velocity
@@ -205,13 +206,86 @@ __global__ void __launch_bounds__(32 * NODE_WARPS) node_record_kernel(Dev P, Tap
 }
 
 // The segment records of the factor pass after z, a fixed end or a radius was
-// changed by something else than an iteration.
+// changed by something else than an iteration (sorted plans: sort_kernel
+// follows and writes the circles).
 __global__ void segments_kernel(Dev P) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= P.p * P.eta) return;
   const int s = t / P.p, i = t - s * P.p;
   const size_t node = (size_t)i * (P.eta + 1) + s;
-  store_segment(P, i, s, P.z[node], P.z[node + 1]);
+  const float2 zl = P.z[node], zh = P.z[node + 1];
+  if (P.sorted) P.zseg[t] = pack(zl, zh);
+  else store_segment(P, i, s, zl, zh);
+}
+
+// Search order of sorted plans: one CTA per segment deals the agents into the
+// cells of a 64 x 64 grid by their segments' midpoints, the cells in the order
+// of a Morton curve (a counting sort: a bitonic sort took 45 us at p = 4,095),
+// and writes the order, its inverse, the circles in that order and the boxes
+// of its groups of 32.  Any order gives the same iterates, so the agents of a
+// cell come as they come, and it is done at a reset and every SORT_EVERY
+// iterations.
+__device__ __forceinline__ unsigned spread6(unsigned v) {  // the bits of v at even places
+  v = (v | (v << 4)) & 0x0f0fu;
+  v = (v | (v << 2)) & 0x3333u;
+  return (v | (v << 1)) & 0x5555u;
+}
+constexpr int SORT_CELLS = 4096;
+__global__ void __launch_bounds__(1024) sort_kernel(Dev P) {
+  __shared__ int first[SORT_CELLS];
+  __shared__ int sums[32];
+  const int s = blockIdx.x, p = P.p, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const size_t so = (size_t)s * p;
+  const float reach = P.fix[1] * 0.125f, scale = 63.99f / (2.f * reach);  // fix[1] = 8 (largest coordinate + 1)
+  for (int c = threadIdx.x; c < SORT_CELLS; c += 1024) first[c] = 0;
+  __syncthreads();
+  auto cell = [&](int i) {
+    const float4 z = P.zseg[so + i];
+    const float x = fminf(fmaxf((0.5f * (z.x + z.z) + reach) * scale, 0.f), 63.f);
+    const float y = fminf(fmaxf((0.5f * (z.y + z.w) + reach) * scale, 0.f), 63.f);
+    return (int)(spread6((unsigned)x) | (spread6((unsigned)y) << 1));
+  };
+  for (int i = threadIdx.x; i < p; i += 1024) P.inv[so + i] = atomicAdd(&first[cell(i)], 1);
+  __syncthreads();
+  // exclusive prefix over the cells, four a thread
+  int c[4], sum = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) { c[q] = first[4 * threadIdx.x + q]; sum += c[q]; }
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(FULL, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) sums[warp] = incl;
+  __syncthreads();
+  int before = incl - sum;
+  for (int w = 0; w < warp; ++w) before += sums[w];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) { first[4 * threadIdx.x + q] = before; before += c[q]; }
+  __syncthreads();
+  for (int i = threadIdx.x; i < p; i += 1024) {
+    const int at = first[cell(i)] + P.inv[so + i];
+    P.inv[so + i] = at;
+    P.perm[so + at] = i;
+  }
+  __syncthreads();
+  const int none = 0x7fffffff;
+  for (int t = threadIdx.x; t < P.nt * TILE; t += 1024) {  // whole warps
+    int4 box = make_int4(none, none, -none, -none);
+    if (t < p) {
+      const int i = P.perm[so + t];
+      const float4 z = P.zseg[so + i];
+      const float4 circle = segment_circle(lo2(z), hi2(z), P.radius[i]);
+      P.circ[so + t] = circle;
+      box = circle_box(circle);
+    }
+    box.x = __reduce_min_sync(FULL, box.x);
+    box.y = __reduce_min_sync(FULL, box.y);
+    box.z = __reduce_max_sync(FULL, box.z);
+    box.w = __reduce_max_sync(FULL, box.w);
+    if (lane == 0) P.box[(size_t)s * P.nt + (t >> 5)] = box;
+  }
 }
 
 // Small problems, gated state: whole runs of iterations in one launch of one
@@ -636,7 +710,8 @@ __global__ void __launch_bounds__(256) reset_kernel(Dev P, float2* z0, float2* z
     const float2 zl = start[i], zh = (s + 1 == P.eta) ? goal[i] : start[i];
     P.xkin[t] = pack(zl, zh);
     P.ukin[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!P.dense) store_segment(P, i, s, zl, zh);
+    if (P.sorted) P.zseg[t] = pack(zl, zh);  // (sort_kernel follows)
+    else if (!P.dense) store_segment(P, i, s, zl, zh);
   }
 }
 
@@ -1149,6 +1224,19 @@ plan_status fail(plan_status s, const char* fmt, ...) {
   } while (0)
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
+size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
+
+// Sorted tiles pay where the segments before the last have at least this many
+// blocks of pairs.  Measured (us per iteration, squares, first 4 / after 200
+// iterations, agents' order against sorted): p = 1,536, eta = 16 (18,000
+// blocks) 26.5 / 25.2 against 27.5 / 29.2; 2,048, 16 (31,000) 39.2 / 37.8
+// against 34.2 / 39.8; 4,095, 4 (25,000) 49.2 / 54.8 against 47.5 / 57.5;
+// 6,000, 4 (53,000) 98 / 112 against 81 / 107; 4,095, 16 (124,000) 119 / 124
+// against 66 / 94.
+#ifndef SORT_MIN
+#define SORT_MIN 40000
+#endif
+constexpr int SORT_EVERY = 16;
 
 // plan_set_endpoints checks new endpoints on the device up to this many
 // agents (an all-pairs test), and with the host grid above it.
@@ -1161,7 +1249,8 @@ struct Layout {
       res, status, count, ccost, chk, ekey, eshadow;
   // inside the worklist's space (gated state): its capacity, and what takes
   // the space behind it
-  size_t cap, listed, zseg, circ;
+  size_t cap, listed, zseg, circ, perm, inv, box;
+  bool sorted;
   size_t total;
 };
 
@@ -1207,9 +1296,13 @@ Layout layout_for(const plan_config* c) {
   // an order of work (it is rebuilt when it runs out), so the pairs-on-it
   // words and the segment records share its space
   L.work = take(slots * 4);
+  L.sorted = !(c->flags & (PLAN_DENSE_STATE | PLAN_U_KEEP | PLAN_ADMM | PLAN_VO)) && (eta - 1) * ntp >= SORT_MIN;
   L.circ = L.work + slots * 4 - p * eta * 16;
   L.zseg = L.circ - p * eta * 16;
-  L.listed = L.zseg - slots / 8;
+  L.box = L.zseg - (L.sorted ? eta * nt * 16 : 0);
+  L.perm = L.box - (L.sorted ? a16(p * eta * 4) : 0);
+  L.inv = L.perm - (L.sorted ? a16(p * eta * 4) : 0);
+  L.listed = L.inv - slots / 8;
   // a list entry holds a 31-bit slot
   L.cap = slots <= 0x80000000ull ? (L.listed - L.work) / 4 : 0;
   L.wcount = take(4 * 4);  // worklist length by iteration parity
@@ -1378,6 +1471,8 @@ struct plan_s {
   bool own_ws;
   int k;
   int cur;  // which z buffer holds z^k
+  bool sorted = false;  // sorted tiles (single plans, Layout::sorted)
+  int sorted_at = 0;    // iteration of the last sort
   bool fresh = true;  // no worklist yet: the next iteration runs in two launches (FactorMode)
   int sms = 0;        // SMs of the device
   int prox_grid = 0;  // CTAs of the dense state's minimizer pass (resident CTAs per SM x SMs)
@@ -1456,6 +1551,10 @@ struct plan_s {
     P.listed = at<uint32_t>(L.listed);
     P.zseg = at<float4>(L.zseg);
     P.circ = at<float4>(L.circ);
+    P.sorted = sorted ? 1 : 0;
+    P.perm = at<int>(L.perm);
+    P.inv = at<int>(L.inv);
+    P.box = at<int4>(L.box);
     P.work_count = at<unsigned>(L.wcount) + (kk & 1);
     P.work_count_prev = at<unsigned>(L.wcount) + ((kk + 1) & 1);
     P.ctl = at<unsigned>(L.ctl);
@@ -1493,17 +1592,28 @@ cudaError_t clear_sums(plan_t h) {
 
 // The gated state's records after a change of z, the fixed ends or the radii
 // from outside an iteration.
+plan_status sort_agents(plan_t h) {
+  if (!h->sorted) return PLAN_OK;
+  sort_kernel<<<h->eta, 1024, 0, h->stream>>>(h->dev(h->k));
+  CK(cudaGetLastError());
+  h->sorted_at = h->k;
+  return PLAN_OK;
+}
+
 plan_status refresh_segments(plan_t h) {
   Dev P = h->dev(h->k);
   if (P.dense) return PLAN_OK;
   const int n = h->p * h->eta;
   segments_kernel<<<(n + 255) / 256, 256, 0, h->stream>>>(P);
   CK(cudaGetLastError());
-  return PLAN_OK;
+  return sort_agents(h);
 }
 
 // No worklist: the next iteration builds it from the activity bits.
 plan_status drop_worklist(plan_t h) {
+  if (h->dense()) return PLAN_OK;
+  CK(cudaMemcpyAsync(h->at<void>(h->L.listed), h->at<void>(h->L.bits), (size_t)h->eta * h->ntp * TILE * 4,
+                     cudaMemcpyDeviceToDevice, h->stream));
   CK(cudaMemsetAsync(h->at<void>(h->L.wcount), 0, 16, h->stream));
   CK(cudaMemsetAsync(h->at<void>(h->L.ctl), 0, 16, h->stream));
   CK(cudaMemsetAsync(h->at<void>(h->L.ctl), 1, 1, h->stream));  // ctl[0] = 1 (rebuild)
@@ -1557,7 +1667,7 @@ int list_ctas(const plan_s* h) {
 // third of them active, about one list chunk per warp.
 bool solo(const plan_s* h) {
   const long long eta = h->vo ? 1 : h->eta;
-  return h->cap && !h->profiling && !h->dense() && eta * h->ntp + segment_warps(h) <= SOLO_WARPS &&
+  return h->cap && !h->profiling && !h->dense() && !h->sorted && eta * h->ntp + segment_warps(h) <= SOLO_WARPS &&
          eta * h->p * (h->p - 1) / 2 <= 1536;
 }
 
@@ -1585,6 +1695,15 @@ plan_status run_solo(plan_t h, int n, const Tape* tape) {
     n -= m;
   }
   return PLAN_OK;
+}
+
+// Blocks per tile warp on the segments before the last: enough for two rounds
+// of the warps that the GPU holds (24 an SM), at most 32 (a lane tests each
+// block's boxes), one where the tiles are not sorted (every block is work).
+int tile_strip(const plan_s* h) {
+  if (!h->sorted) return 1;
+  const long long tiles = (long long)(h->eta - 1) * h->ntp;
+  return (int)std::max<long long>(1, std::min<long long>(32, tiles / (48ll * h->sms)));
 }
 
 // Every pair fits the worklist, so that an iteration may be split in listing
@@ -1615,7 +1734,9 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = null
     CK(launch_pdl(prox_kernel, (unsigned)h->prox_grid, 256u, ms, P));
   } else {
     FactorGrid G;
-    const int tiles = (h->vo ? 1 : h->eta) * h->ntp, tile_ctas = (tiles + FACTOR_WARPS - 1) / FACTOR_WARPS;
+    const int nseg = h->vo ? 1 : h->eta;
+    G.strip = tile_strip(h);
+    const int tiles = tile_warps(nseg, h->ntp, G.strip), tile_ctas = (tiles + FACTOR_WARPS - 1) / FACTOR_WARPS;
     G.list_ctas = list_ctas(h);
     G.lead_ctas = std::min(tile_ctas, (h->ntp + FACTOR_WARPS - 1) / FACTOR_WARPS);
     G.seg_ctas = (segw + FACTOR_WARPS - 1) / FACTOR_WARPS;
@@ -1623,7 +1744,8 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = null
     G.tile_warps = tiles;
     const bool listing = h->fresh && lists_every_pair(h);
     G.mode = listing ? LISTING : FUSED;
-    auto kern = h->noenergy ? factor_kernel<true> : factor_kernel<false>;
+    auto kern = h->noenergy ? (h->sorted ? factor_kernel<true, true> : factor_kernel<true, false>)
+                            : (h->sorted ? factor_kernel<false, true> : factor_kernel<false, false>);
     CK(launch_pdl(kern, (unsigned)(G.list_ctas + G.seg_ctas + tile_ctas), 32u * FACTOR_WARPS, ms, P, G));
     if (listing) {
       G.mode = LISTED;
@@ -1658,6 +1780,7 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = null
 // fits (past the rho warm-up, not profiling), else launch them directly.
 plan_status run_iteration(plan_t h) {
   plan_status st = ensure_prox_grid(h);
+  if (st == PLAN_OK && h->sorted && h->k - h->sorted_at >= SORT_EVERY) st = sort_agents(h);
   if (st != PLAN_OK) return st;
   const bool graphable = h->cap && !h->profiling && h->k >= h->graph_from() && !h->fresh;
   if (graphable) {
@@ -1703,6 +1826,7 @@ plan_status run_graph_runs(plan_t h, int& n, int len, cudaGraphExec_t* execs) {
       CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
       plan_status cst = PLAN_OK;
       for (int q = 0; q < len && cst == PLAN_OK; ++q) {
+        if (q > 0 && q % SORT_EVERY == 0 && h->sorted) sort_kernel<<<h->eta, 1024, 0, h->cap>>>(h->dev(h->k));
         cst = enqueue_iteration(h, h->cap);
         if (h->eta > 1) h->cur ^= 1;
         h->k += 1;
@@ -1716,7 +1840,12 @@ plan_status run_graph_runs(plan_t h, int& n, int len, cudaGraphExec_t* execs) {
       cudaGraphDestroy(g);
       if (e != cudaSuccess) return fail(PLAN_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e));
     }
+    if (h->sorted && h->k - h->sorted_at >= SORT_EVERY) {
+      plan_status sst = sort_agents(h);
+      if (sst != PLAN_OK) return sst;
+    }
     CK(cudaGraphLaunch(execs[key], h->stream));
+    if (len > SORT_EVERY) h->sorted_at = h->k + len - SORT_EVERY;
     h->k += len;
     n -= len;
   }
@@ -1830,7 +1959,7 @@ plan_status plan_reset(plan_t h) {
       h->at<unsigned>(h->L.res), h->at<unsigned>(h->L.wcount), h->at<unsigned long long>(h->L.ekey),
       h->at<unsigned long long>(h->L.chk));
   CK(cudaGetLastError());
-  return PLAN_OK;
+  return sort_agents(h);
 }
 
 }  // extern "C"
@@ -1913,6 +2042,7 @@ plan_status create_plan(const plan_config* cfg, const float* start, const float*
     h->own_ws = true;
   }
   if (!member) {
+    h->sorted = L.sorted;
     cudaError_t e = cudaMallocHost(&h->h_res, 48);
     if (e == cudaSuccess && (size_t)cfg->p <= kDeviceEndpointCheck)
       e = cudaMallocHost(&h->h_stage, (size_t)cfg->p * 16);

@@ -38,12 +38,22 @@
 // pair is on it.  A pair joins when a tile warp finds it active, and stays on
 // it after it turns inactive (a pair that left often comes back; its u is 0
 // then), so the tile warps of an iteration can read `listed` while the list
-// warps work: nothing in it changes but the words of a tile's own warp.  When
-// more than half of the list is inactive, or an append did not fit, the next
-// iteration builds it anew from `bits` (the tile warps then take the pairs
-// active before, the list warps nothing): `bits` and the slot records are
-// the state, the list only an order of work, and any list gives the same
-// iterates.
+// warps work: no pair leaves it meanwhile.  When more than half of the list is
+// inactive, or an append did not fit, the next iteration builds it anew: the
+// tile warps then take the pairs of `listed` too and the list warps nothing;
+// a pair drops out if it was inactive and still is, which the test on z that a
+// tile warp makes would also find.  `bits` and the slot records are the
+// state, the list only an order of work, and any list gives the same
+// iterates.  (An iteration that rebuilds goes through the tiles in the agents'
+// own order, also where they are sorted, so that a block's listed pairs and
+// its new ones are one warp's.)
+//
+// Sorted tiles (large single plans).  The tiles of the search are made of
+// agents in the order of a Morton curve through their segments' midpoints,
+// sorted anew now and then (perm / inv), with a box around each group of 32:
+// two groups whose boxes do not meet hold no near pair.  The slots stay in
+// agent order.  Boxes only grow between sorts (the node pass widens the box
+// of an agent that left it), so they hold whatever the order's age.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -81,7 +91,13 @@ struct Dev {
   float4 *uwall, *xwall; // [nw][eta][p]
   uint32_t* wbits;       // [nw][eta][nt]
   float4* zseg;          // [eta][p] (z(s), z(s+1)) of z^k (gated state)
-  float4* circ;          // [eta][p] bounding circle (m.x, m.y, b, bounding_offset) of z^k
+  float4* circ;          // [eta][p] bounding circle (m.x, m.y, b, -bounding_offset) of z^k, by
+                         // place in the search order
+  int sorted;            // sorted tiles (else the search order is the agents' own)
+  int* perm;             // [eta][p] agent at a place of the search order
+  int* inv;              // [eta][p] place of an agent
+  int4* box;             // [eta][nt] box of the circles at 32 places (x, y least, x, y largest;
+                         // floats as ordered integers)
   uint32_t* work;        // collision worklist (dense state: the active slots of this iteration)
   unsigned cap;          // its capacity
   uint32_t* listed;      // [eta * ntp * 32] pairs on the worklist (gated state)
@@ -169,6 +185,13 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
   return v;
 }
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long v;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ float lo_of(unsigned long long v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi_of(unsigned long long v) { return __uint_as_float((uint32_t)(v >> 32)); }
 __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
   unsigned long long v;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
@@ -400,6 +423,13 @@ __device__ __forceinline__ int tile_pair(int nt, int I, int J) {  // I <= J
   return I * nt - I * (I - 1) / 2 + (J - I);
 }
 
+// Slot of the pair (a, b), either order, on segment s.
+__device__ __forceinline__ uint32_t pair_slot(const Dev& P, int s, int a, int b) {
+  const int i = min(a, b), j = max(a, b);
+  const uint32_t blk = (uint32_t)s * P.ntp + tile_pair(P.nt, i >> 5, j >> 5);
+  return (blk * TILE + (i & 31)) * TILE + (j & 31);
+}
+
 // Inverse of tile_pair: the tiles (I, J), I <= J, of pair index t, without
 // the table lookup (a square root, then an exact integer correction).
 __device__ __forceinline__ void tile_of(int nt, int t, int& I, int& J) {
@@ -520,17 +550,43 @@ __device__ __forceinline__ float bounding_offset(float2 m, float b) {
   return fmaf(-2e-6f, mm + bb, 0.5f * (mm - bb));
 }
 
+// Floats as integers of the same order, for integer atomics.
+__device__ __forceinline__ int ordered(float f) {
+  const int i = __float_as_int(f);
+  return i ^ ((i >> 31) & 0x7fffffff);
+}
+// The box of a bounding circle, a little wide (1e-5 of its size and place, a
+// hundred times the rounding here and in the exact test): two agents that the
+// exact test finds colliding have boxes that meet.  (One with an infinity or a
+// NaN never passes that test, whatever its box.)
+__device__ __forceinline__ int4 circle_box(float4 c) {
+  const float ex = fmaf(1e-5f, fabsf(c.x) + c.z, c.z), ey = fmaf(1e-5f, fabsf(c.y) + c.z, c.z);
+  return make_int4(ordered(c.x - ex), ordered(c.y - ey), ordered(c.x + ex), ordered(c.y + ey));
+}
+__device__ __forceinline__ float4 segment_circle(float2 zl, float2 zh, float r) {
+  const float2 m = 0.5f * (zl + zh), d = zh - zl;
+  const float b = fmaf(0.5f, sqrtf(dot(d, d)), r);
+  return make_float4(m.x, m.y, b, -bounding_offset(m, b));
+}
+
 // The records the factor pass starts from (gated state), of agent i on
 // segment s: both break-points together, and the bounding circle with the
-// offset negated.  Written by the node pass (and after z changed by other
-// means), so that a tile warp loads 16 bytes per agent, coalesced, and
-// derives nothing.
+// offset negated, at the agent's place in the search order.  Written by the
+// node pass (and after z changed by other means), so that a tile warp loads
+// 16 bytes per agent, coalesced, and derives nothing.
 __device__ __forceinline__ void store_segment(const Dev& P, int i, int s, float2 zl, float2 zh) {
-  const float2 m = 0.5f * (zl + zh), d = zh - zl;
-  const float b = fmaf(0.5f, sqrtf(dot(d, d)), P.radius[i]);
-  const size_t q = (size_t)s * P.p + i;
-  P.zseg[q] = pack(zl, zh);
-  P.circ[q] = make_float4(m.x, m.y, b, -bounding_offset(m, b));
+  const size_t so = (size_t)s * P.p;
+  const float4 c = segment_circle(zl, zh, P.radius[i]);
+  P.zseg[so + i] = pack(zl, zh);
+  if (!P.sorted) { P.circ[so + i] = c; return; }
+  const int at = P.inv[so + i];
+  P.circ[so + at] = c;
+  int4* box = P.box + (size_t)s * P.nt + (at >> 5);
+  const int4 have = *box, need = circle_box(c);
+  if (need.x < have.x) atomicMin(&box->x, need.x);
+  if (need.y < have.y) atomicMin(&box->y, need.y);
+  if (need.z > have.z) atomicMax(&box->z, need.z);
+  if (need.w > have.w) atomicMax(&box->w, need.w);
 }
 
 // Position of the n-th set bit of w (n counted from 0, less than popc(w)).
@@ -544,13 +600,43 @@ __device__ __forceinline__ int nth_bit(uint32_t w, unsigned n) {
   return at;
 }
 
-// Shared memory of one tile warp: its 32 column agents' circles by
-// component, their segments and radii, and the rows' new activity words.
-struct TileMem {
-  float mx[32], my[32], b[32], na[32], r[32];
+// Shared memory of one tile warp: its 32 column agents' circles by component,
+// their segments (by component with sorted tiles, where a pair of columns is
+// one 8-byte load, else whole) and radii, their numbers, and the activity of
+// the pairs of the current phase by row.
+struct __align__(16) TileMem {
+  float mx[32], my[32], b[32], na[32];
+  union {
+    float4 z[32];
+    struct { float zlx[32], zly[32], zhx[32], zhy[32]; };
+  };
+  float r[32];
+  int id[32];
   uint32_t act[32];
-  float4 z[32];
 };
+
+// collides() of a row agent (segment z, negated, and radius in both halves)
+// with columns 2 k and 2 k + 1: the same operations, two at a time; bits 0 and
+// 1 of the result.
+struct RowPair { unsigned long long nlx, nly, nhx, nhy, r; };
+__device__ __forceinline__ uint32_t collides2(const RowPair& A, const TileMem* M, int k) {
+  auto at = [&](const float* v) { return reinterpret_cast<const unsigned long long*>(v)[k]; };
+  const unsigned long long minus = pair_of(-1.f, -1.f);
+  const unsigned long long lx = add2(at(M->zlx), A.nlx), ly = add2(at(M->zly), A.nly);
+  const unsigned long long hx = add2(at(M->zhx), A.nhx), hy = add2(at(M->zhy), A.nhy);
+  const unsigned long long R = add2(A.r, at(M->r)), R2 = mul2(R, R);
+  const unsigned long long dx = fma2(lx, minus, hx), dy = fma2(ly, minus, hy);  // hx - lx, one rounding
+  const unsigned long long dd = fma2(dx, dx, mul2(dy, dy)), ld = fma2(lx, dx, mul2(ly, dy));
+  const unsigned long long c = fma2(lx, dy, mul2(mul2(ly, dx), minus));
+  const unsigned long long ll = fma2(lx, lx, mul2(ly, ly)), hh = fma2(hx, hx, mul2(hy, hy));
+  const unsigned long long cc = mul2(c, c), Rd = mul2(R2, dd);
+  auto one = [](float ll, float hh, float ld, float dd, float cc, float R2, float Rd) {
+    const float t = -ld;
+    return (ll < R2) | (hh < R2) | ((t > 0.f) & (t < dd) & (cc < Rd));
+  };
+  return (one(lo_of(ll), lo_of(hh), lo_of(ld), lo_of(dd), lo_of(cc), lo_of(R2), lo_of(Rd)) ? 1u : 0u) |
+         (one(hi_of(ll), hi_of(hh), hi_of(ld), hi_of(dd), hi_of(cc), hi_of(R2), hi_of(Rd)) ? 2u : 0u);
+}
 
 // A pair of one warp item: (i, j) on segment s with slot fid; prev: active in
 // the last iteration.  Finishes its dual update, tests it and, when it is
@@ -602,17 +688,28 @@ __device__ __forceinline__ bool pair_factor(const Dev& P, int s, int i, int j, u
 // list (capacity 0: every iteration takes the rebuilding form).
 constexpr uint32_t ACTIVE = 0x80000000u;
 
+// Tile warps of a problem: one per 32 x 32 block on the last segment (early in
+// a solve it spans each agent's whole way, nearly all its pairs take the exact
+// test, and it goes first), `strip` blocks elsewhere (most of which the boxes
+// rule out when the tiles are sorted), taken at equal distances so that the
+// neighbouring groups, whose boxes meet, go to different warps (strips of 16
+// consecutive blocks left one warp with all of them: 81 us at p = 4,095).
+__host__ __device__ __forceinline__ int tile_warps(int nseg, int ntp, int strip) {
+  return ntp + (nseg - 1) * ((ntp + strip - 1) / strip);
+}
+
 // Collision factors of the gated state, one warp.  item < nlist: list warp
 // `item` of nlist takes the chunks of 32 worklist entries item, item + nlist,
-// ...; else tile warp item - nlist takes one 32 x 32 block of pairs.
+// ...; else tile warp item - nlist takes one 32 x 32 block of pairs or a strip
+// of them.
 //
 // Tile warp: lane = row agent.  The bounding circles of the 32 columns come
 // from shared memory four columns at a time and are tested two columns per
 // instruction; the sign of the result is shifted into the row's word, so a
 // pair costs about four instructions (the scalar form with a compare and a
-// select took seven).  Near pairs that are not on the worklist take the exact
-// test, and those that collide are dealt over the whole warp, one pair per
-// lane per round (row found by a shuffle binary search over the rows' prefix
+// select took seven).  Near pairs take the exact test, and those that collide
+// and are not on the worklist are dealt over the whole warp, one pair per lane
+// per round (row found by a shuffle binary search over the rows' prefix
 // counts), to run the minimizer.  Both kinds of warp share one copy of that
 // code (one loop, one call site): it is most of the kernel's instructions.
 //
@@ -622,6 +719,86 @@ constexpr uint32_t ACTIVE = 0x80000000u;
 // is two launches: LISTING (tile warps put every pair that was active or
 // collides on the worklist) and LISTED (list warps only).
 enum FactorMode { FUSED = 0, LISTING = 1, LISTED = 2 };
+
+// Columns of a 32 x 32 block whose bounding circles (in M) come near the
+// lane's row circle ci, as a word.
+__device__ __forceinline__ uint32_t near_columns(const float4 ci, const TileMem* M) {
+  const unsigned long long mx = pair_of(ci.x, ci.x), my = pair_of(ci.y, ci.y), b = pair_of(ci.z, ci.z),
+                           na = pair_of(ci.w, ci.w);
+  uint32_t far = 0u;
+#pragma unroll
+  for (int c = TILE - 4; c >= 0; c -= 4) {
+    const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(M->mx + c);
+    const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(M->my + c);
+    const ulonglong2 B = *reinterpret_cast<const ulonglong2*>(M->b + c);
+    const ulonglong2 A = *reinterpret_cast<const ulonglong2*>(M->na + c);
+    const unsigned long long t1 = fma2(mx, X.y, fma2(my, Y.y, fma2(b, B.y, add2(na, A.y))));
+    const unsigned long long t0 = fma2(mx, X.x, fma2(my, Y.x, fma2(b, B.x, add2(na, A.x))));
+    // sign bits, highest column first
+    far = __funnelshift_l((uint32_t)(t1 >> 32), far, 1);
+    far = __funnelshift_l((uint32_t)t1, far, 1);
+    far = __funnelshift_l((uint32_t)(t0 >> 32), far, 1);
+    far = __funnelshift_l((uint32_t)t0, far, 1);
+  }
+  return ~far;
+}
+
+// Inclusive prefix sums over the warp.
+__device__ __forceinline__ unsigned warp_inclusive(unsigned v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned w = __shfl_up_sync(FULL, v, o);
+    if (lane >= o) v += w;
+  }
+  return v;
+}
+
+// Room for every lane's n worklist entries (one atomic): the lane's first.
+__device__ __forceinline__ unsigned claim_entries(const Dev& P, unsigned n) {
+  const unsigned incl = warp_inclusive(n);
+  unsigned at = 0;
+  if ((threadIdx.x & 31) == 31) {
+    at = atomicAdd(P.work_count, incl);
+    if ((unsigned long long)at + incl > P.cap) atomicOr(P.ctl + 2, 1u);
+  }
+  return __shfl_sync(FULL, at, 31) + (incl - n);
+}
+
+// A lane's worklist entry `entry` (position t): slot, segment, agents i < j.
+__device__ __forceinline__ void entry_pair(const Dev& P, uint32_t entry, uint32_t& fid, int& s, int& i, int& j) {
+  fid = entry & ~ACTIVE;
+  const uint32_t row = fid >> 5, blk = row >> 5;
+  s = (int)(blk / (uint32_t)P.ntp);
+  int I, J;
+  tile_of(P.nt, (int)(blk - (uint32_t)s * P.ntp), I, J);
+  i = I * TILE + (int)(row & 31);
+  j = J * TILE + (int)(fid & 31);
+}
+
+// A list warp's lane after its pair: the entry and the activity bit, where
+// that changed.  Returns by how much the list's inactive entries grew.
+__device__ __forceinline__ int entry_done(const Dev& P, unsigned long long t, uint32_t fid, bool prev, bool act) {
+  if (act == prev) return 0;
+  P.work[t] = fid | (act ? ACTIVE : 0u);
+  const uint32_t bit = 1u << (fid & 31);
+  if (act) atomicOr(P.bits + (fid >> 5), bit); else atomicAnd(P.bits + (fid >> 5), ~bit);
+  return act ? -1 : 1;
+}
+
+// Pair g of a warp's pairs, dealt from the rows' words todo with inclusive
+// prefix counts tincl and `total` in all: its row (the first whose count
+// exceeds g) and column (0 past the end).
+__device__ __forceinline__ void nth_pair(uint32_t todo, unsigned tincl, unsigned total, unsigned g, int& r, int& c) {
+  r = 0;
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1)
+    if (__shfl_sync(FULL, tincl, r + step - 1) <= g) r += step;
+  const uint32_t w = __shfl_sync(FULL, todo, r);
+  const unsigned first = __shfl_sync(FULL, tincl, r) - __popc(w);
+  c = g < total ? nth_bit(w, g - first) : 0;
+}
+
 template <bool CLASSES>
 __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist, TileMem* M, int mode) {
   const int lane = threadIdx.x & 31;
@@ -658,24 +835,7 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
     __syncwarp();
     if (!vi) valid = 0u;
     if (I == J) valid &= (lane == 31) ? 0u : (~0u << (lane + 1));  // pairs i < j
-    const unsigned long long mx = pair_of(ci.x, ci.x), my = pair_of(ci.y, ci.y), b = pair_of(ci.z, ci.z),
-                             na = pair_of(ci.w, ci.w);
-    uint32_t far = 0u;
-#pragma unroll
-    for (int c = TILE - 4; c >= 0; c -= 4) {
-      const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(M->mx + c);
-      const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(M->my + c);
-      const ulonglong2 B = *reinterpret_cast<const ulonglong2*>(M->b + c);
-      const ulonglong2 A = *reinterpret_cast<const ulonglong2*>(M->na + c);
-      const unsigned long long t1 = fma2(mx, X.y, fma2(my, Y.y, fma2(b, B.y, add2(na, A.y))));
-      const unsigned long long t0 = fma2(mx, X.x, fma2(my, Y.x, fma2(b, B.x, add2(na, A.x))));
-      // sign bits, highest column first
-      far = __funnelshift_l((uint32_t)(t1 >> 32), far, 1);
-      far = __funnelshift_l((uint32_t)t1, far, 1);
-      far = __funnelshift_l((uint32_t)(t0 >> 32), far, 1);
-      far = __funnelshift_l((uint32_t)t0, far, 1);
-    }
-    near = ~far & valid & ~listed;
+    near = near_columns(ci, M) & valid & ~listed;
     M->act[lane] = 0u;
     todo = rebuild ? listed : 0u;
     phase = mode == LISTING ? 2 : rebuild ? 0 : 1;
@@ -702,39 +862,29 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
       }
       near = hit;
     }
+    if (!rebuild && !__any_sync(FULL, near != 0u)) return;  // most tiles: nothing to run, nothing to note
     __syncwarp();
   }
   for (;;) {
     // the next 32 pairs
     int pi = 0, pj = 0, ps = 0, r = 0, c = 0;
-    uint32_t fid = 0u, entry = 0u;
+    uint32_t fid = 0u;
     bool on = false, prev = false;
+    const unsigned long long t = 32ull * chunk + lane;
     if (lister) {
-      const unsigned long long t = 32ull * chunk + lane;
       if (32ull * chunk >= n) break;  // warp-uniform
       on = t < n;
       if (on) {
-        entry = P.work[t];
-        fid = entry & ~ACTIVE;
+        const uint32_t entry = P.work[t];
         prev = (entry & ACTIVE) != 0u;
-        const uint32_t prow = fid >> 5, pblk = prow >> 5;
-        ps = (int)(pblk / (uint32_t)P.ntp);
-        int pI, pJ;
-        tile_of(P.nt, (int)(pblk - (uint32_t)ps * P.ntp), pI, pJ);
-        pi = pI * TILE + (int)(prow & 31);
-        pj = pJ * TILE + (int)(fid & 31);
+        entry_pair(P, entry, fid, ps, pi, pj);
       }
     } else {
       if (base >= total) {  // start a phase: 0 the pairs active before (rebuild), 1 the new ones
         if (phase > 1) break;
         if (phase == 1) todo = near;
         ++phase;
-        tincl = __popc(todo);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned v = __shfl_up_sync(FULL, tincl, o);
-          if (lane >= o) tincl += v;
-        }
+        tincl = warp_inclusive(__popc(todo));
         total = __shfl_sync(FULL, tincl, 31);
         base = 0;
         if (total == 0) continue;
@@ -743,12 +893,7 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
       const unsigned g = base + lane;
       base += 32;
       on = g < total;
-#pragma unroll
-      for (int step = 16; step > 0; step >>= 1)  // the row of pair g: the first whose inclusive count exceeds g
-        if (__shfl_sync(FULL, tincl, r + step - 1) <= g) r += step;
-      const uint32_t wr = __shfl_sync(FULL, todo, r);
-      const unsigned first = __shfl_sync(FULL, tincl, r) - __popc(wr);
-      c = on ? nth_bit(wr, g - first) : 0;
+      nth_pair(todo, tincl, total, g, r, c);
       ps = s;
       pi = I * TILE + r;
       pj = J * TILE + c;
@@ -757,12 +902,7 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
     bool act = false;
     if (on) act = pair_factor<CLASSES>(P, ps, pi, pj, fid, prev, res);
     if (lister) {
-      if (on && act != prev) {
-        P.work[32ull * chunk + lane] = fid | (act ? ACTIVE : 0u);
-        const uint32_t bit = 1u << (fid & 31);
-        if (act) atomicOr(P.bits + (fid >> 5), bit); else atomicAnd(P.bits + (fid >> 5), ~bit);
-        gone += act ? -1 : 1;
-      }
+      if (on) gone += entry_done(P, t, fid, prev, act);
       chunk += (unsigned)nlist;
     } else if (act) {
       atomicOr(&M->act[r], 1u << c);
@@ -790,27 +930,233 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
       atomicOr(P.bits + row, nword);
       P.listed[row] = listed | nword;
     }
-    if (__any_sync(FULL, nword != 0u)) {  // append: one atomic per warp
-      const unsigned cnt = __popc(nword);
-      unsigned incl = cnt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned v = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const unsigned all = __shfl_sync(FULL, incl, 31);
-      unsigned at = 0;
-      if (lane == 31) {
-        at = atomicAdd(P.work_count, all);
-        if ((unsigned long long)at + all > P.cap) atomicOr(P.ctl + 2, 1u);
-      }
-      at = __shfl_sync(FULL, at, 31) + (incl - cnt);
+    if (__any_sync(FULL, nword != 0u)) {
+      unsigned at = claim_entries(P, __popc(nword));
       for (uint32_t w = nword; w; w &= w - 1u, ++at)
         if (at < P.cap) {
           const int bit = __ffs(w) - 1;
           P.work[at] = (uint32_t)(row * TILE + bit) | ((flagged >> bit) & 1u ? ACTIVE : 0u);
         }
     }
+  }
+  if (__any_sync(FULL, res > 0.f)) {  // only pairs active before have a residual
+    res = warp_max(res);
+    if (lane == 0 && P.res_prev) atomic_max_nonneg(P.res_prev, res);
+  }
+}
+
+// Sorted tiles: pairs of tile t of segment s that collide with u = 0 and are
+// not on the worklist, by row (lane) a word of columns.  sorted: the tile's
+// agents come in the search order, else in their own (a rebuild).  rid: the
+// lane's row agent.
+__device__ __forceinline__ uint32_t tile_candidates(const Dev& P, int s, int t, int I, int J, bool sorted, TileMem* M,
+                                                    int& rid) {
+  const int lane = threadIdx.x & 31;
+  const int ri = I * TILE + lane, cj = J * TILE + lane;
+  const bool vi = ri < P.p, vj = cj < P.p;
+  const size_t so = (size_t)s * P.p;
+  const float4 none = make_float4(0.f, 0.f, 0.f, -INFINITY);
+  rid = ri;
+  int cid = cj, rat = ri, cat = cj;  // row and column agent, and the places of their circles
+  if (sorted) {
+    if (vi) rid = P.perm[so + ri];
+    if (vj) cid = P.perm[so + cj];
+  } else {
+    if (vi) rat = P.inv[so + ri];
+    if (vj) cat = P.inv[so + cj];
+  }
+  const float4 ci = vi ? P.circ[so + rat] : none, cc = vj ? P.circ[so + cat] : none;
+  // with the agents' own order the block's listed pairs are known
+  const uint32_t known = sorted ? 0u : P.listed[((size_t)s * P.ntp + t) * TILE + lane];
+  __syncwarp();
+  M->mx[lane] = cc.x; M->my[lane] = cc.y; M->b[lane] = cc.z; M->na[lane] = cc.w;
+  M->id[lane] = cid;
+  uint32_t valid = __ballot_sync(FULL, vj);
+  __syncwarp();
+  if (!vi) valid = 0u;
+  if (I == J) valid &= (lane == 31) ? 0u : (~0u << (lane + 1));  // each pair once
+  const uint32_t near = near_columns(ci, M) & valid & ~known;
+  if (!__any_sync(FULL, near != 0u)) return 0u;
+  float4 zi = make_float4(0.f, 0.f, 0.f, 0.f), zj = zi;
+  float r = 0.f, rj = 0.f;
+  if (vi) { zi = P.zseg[so + rid]; r = P.radius[rid]; }
+  if (vj) { zj = P.zseg[so + cid]; rj = P.radius[cid]; }
+  M->r[lane] = rj;
+  M->zlx[lane] = zj.x; M->zly[lane] = zj.y; M->zhx[lane] = zj.z; M->zhy[lane] = zj.w;
+  __syncwarp();
+  uint32_t hit = 0u;
+  if (__reduce_max_sync(FULL, __popc(near)) >= 12) {
+    // near a third of the columns or more (the segment that spans the whole
+    // way): every column, two an instruction (8.5 to 7.5 us a tile there)
+    const RowPair A = {pair_of(-zi.x, -zi.x), pair_of(-zi.y, -zi.y), pair_of(-zi.z, -zi.z), pair_of(-zi.w, -zi.w),
+                       pair_of(r, r)};
+#pragma unroll 2
+    for (int k = 0; k < TILE / 2; ++k) hit |= collides2(A, M, k) << (2 * k);
+    hit &= near;
+  } else {
+    for (uint32_t w = near; w; w &= w - 1u) {
+      const int c = __ffs(w) - 1;
+      if (collides(mk(M->zlx[c], M->zly[c]) - lo2(zi), mk(M->zhx[c], M->zhy[c]) - hi2(zi), r + M->r[c]))
+        hit |= 1u << c;
+    }
+  }
+  if (sorted) {  // (those on the worklist are the list warps')
+#pragma unroll 4
+    for (uint32_t w = hit; w; w &= w - 1u) {
+      const int c = __ffs(w) - 1;
+      const uint32_t f = pair_slot(P, s, rid, M->id[c]);
+      if ((P.listed[f >> 5] >> (f & 31)) & 1u) hit &= ~(1u << c);
+    }
+  }
+  return hit;
+}
+
+// The same work with sorted tiles.  A tile warp goes through a strip of
+// blocks, each in up to two phases (its listed pairs when the list is built
+// anew, then the new ones); a separate function, because the state that takes
+// costs the small plans 16% of a solve (261 us to 309 at p = 100).
+template <bool CLASSES>
+__device__ __forceinline__ void sorted_collision_warp(const Dev& P, int item, int nlist, int strip, TileMem* M, int mode) {
+  const int lane = threadIdx.x & 31;
+  const bool rebuild = mode == LISTED ? false : P.ctl[0] != 0u;
+  const bool lister = item < nlist;
+  const bool sorted = !rebuild;
+  float res = 0.f;
+  int idle = 0;  // inactive entries put on the list or left on it, less entries turned active
+  // list warp
+  unsigned n = 0, chunk = (unsigned)item;
+  // tile warp: its blocks t0, t0 + step, ... (cnt of them) of segment s, the
+  // current one q, those with near pairs; the current phase's pairs by row
+  // (todo; was: those active before)
+  int s = 0, t0 = 0, step = 0, cnt = 0, q = -1, I = 0, J = 0, rid = 0;
+  uint32_t live = 0u, todo = 0u, was = 0u;
+  unsigned tincl = 0, total = 0, base = 0;
+  bool scan = false, next = true, open = false;
+  if (lister) {
+    if (rebuild || mode == LISTING) return;
+    n = mode == LISTED ? *P.work_count : *P.work_count_prev;
+  } else {
+    const int nseg = P.vo ? 1 : P.eta, w = item - nlist;
+    if (w < P.ntp) {
+      s = nseg - 1; t0 = w; cnt = 1;
+    } else {
+      step = (P.ntp + strip - 1) / strip;
+      const int v = w - P.ntp;
+      s = nseg - 2 - v / step;
+      t0 = v - (nseg - 2 - s) * step;
+      cnt = (P.ntp - t0 + step - 1) / step;
+    }
+    bool meet = lane < cnt;
+    if (sorted && meet) {
+      int a, b;
+      tile_of(P.nt, t0 + lane * step, a, b);
+      const int4 A = P.box[(size_t)s * P.nt + a], B = P.box[(size_t)s * P.nt + b];
+      meet = A.x <= B.z && B.x <= A.z && A.y <= B.w && B.y <= A.w;
+    }
+    live = __ballot_sync(FULL, meet);
+    if (live == 0u) return;
+  }
+  for (;;) {
+    // the next 32 pairs
+    int pi = 0, pj = 0, ps = s, r = 0, c = 0;
+    uint32_t fid = 0u;
+    bool on = false, prev = false;
+    const unsigned long long t = 32ull * chunk + lane;
+    if (lister) {
+      if (32ull * chunk >= n) break;  // warp-uniform
+      on = t < n;
+      if (on) {
+        const uint32_t entry = P.work[t];
+        prev = (entry & ACTIVE) != 0u;
+        entry_pair(P, entry, fid, ps, pi, pj);
+      }
+    } else {
+      uint32_t row = ((uint32_t)s * P.ntp + t0 + q * step) * TILE + lane;
+      if (base >= total) {
+        if (open) {  // end of a phase: activity, membership and entries of its pairs
+          open = false;
+          __syncwarp();
+          const uint32_t acts = mode == LISTING ? (was & todo) : M->act[lane];
+          const uint32_t keep = mode == LISTING ? todo : acts | (was & todo);
+          if (scan) {  // (a rebuild: no list warp writes these words)
+            if (acts != was) P.bits[row] = acts;
+            P.listed[row] = keep;
+          } else if (!sorted) {
+            if (acts) atomicOr(P.bits + row, acts);
+            if (keep) P.listed[row] |= keep;
+          } else {
+            for (uint32_t w = keep; w; w &= w - 1u) {
+              const int k = __ffs(w) - 1;
+              const uint32_t f = pair_slot(P, s, rid, M->id[k]);
+              if ((acts >> k) & 1u) atomicOr(P.bits + (f >> 5), 1u << (f & 31));
+              atomicOr(P.listed + (f >> 5), 1u << (f & 31));
+            }
+          }
+          idle += __popc(keep & ~acts);
+          if (__any_sync(FULL, keep != 0u)) {
+            unsigned at = claim_entries(P, __popc(keep));
+            for (uint32_t w = keep; w; w &= w - 1u, ++at) {
+              const int k = __ffs(w) - 1;
+              const uint32_t f = !scan && sorted ? pair_slot(P, s, rid, M->id[k]) : row * TILE + k;
+              if (at < P.cap) P.work[at] = f | (((acts >> k) & 1u) ? ACTIVE : 0u);
+            }
+          }
+        }
+        // the next phase: a block's listed pairs (rebuild), then its tile's new ones
+        base = total = 0;
+        scan = next;
+        if (next) {
+          if (++q >= cnt) break;
+          next = false;
+          if (!rebuild) continue;
+          row = ((uint32_t)s * P.ntp + t0 + q * step) * TILE + lane;
+          todo = P.listed[row];
+          was = P.bits[row];
+          tile_of(P.nt, t0 + q * step, I, J);
+        } else {
+          next = true;
+          was = 0u;
+          if (!((live >> q) & 1u)) continue;
+          tile_of(P.nt, t0 + q * step, I, J);
+          todo = tile_candidates(P, s, t0 + q * step, I, J, sorted, M, rid);
+        }
+        if (!__any_sync(FULL, todo != 0u)) continue;
+        open = true;
+        if (mode == LISTING) continue;
+        M->act[lane] = 0u;
+        __syncwarp();
+        tincl = warp_inclusive(__popc(todo));
+        total = __shfl_sync(FULL, tincl, 31);
+      }
+      const unsigned g = base + lane;
+      base += 32;
+      on = g < total;
+      nth_pair(todo, tincl, total, g, r, c);
+      const uint32_t pw = __shfl_sync(FULL, was, r);
+      prev = on && ((pw >> c) & 1u);
+      pi = I * TILE + r;
+      pj = J * TILE + c;
+      fid = (row - lane + r) * TILE + c;
+      const int ra = __shfl_sync(FULL, rid, r);
+      if (sorted && on) {
+        const int ca = M->id[c];
+        pi = min(ra, ca);
+        pj = max(ra, ca);
+        fid = pair_slot(P, s, pi, pj);
+      }
+    }
+    bool act = false;
+    if (on) act = pair_factor<CLASSES>(P, ps, pi, pj, fid, prev, res);
+    if (lister) {
+      if (on) idle += entry_done(P, t, fid, prev, act);
+      chunk += (unsigned)nlist;
+    } else if (act) {
+      atomicOr(&M->act[r], 1u << c);
+    }
+  }
+  if (__any_sync(FULL, idle != 0)) {
+    idle = __reduce_add_sync(FULL, idle);
+    if (lane == 0 && idle != 0) atomicAdd(P.ctl + 1, (unsigned)idle);
   }
   if (__any_sync(FULL, res > 0.f)) {  // only pairs active before have a residual
     res = warp_max(res);

@@ -47,6 +47,30 @@ def test_any_worklist_gives_the_same_iterates():
             assert np.array_equal(a.trajectory().cpu().numpy(), b.trajectory().cpu().numpy()), n
 
 
+@pytest.mark.parametrize("p,eta,iters", [(2047, 21, 40), (2880, 11, 20)])
+def test_sorted_tiles_give_the_dense_iterates(p, eta, iters):
+    """Plans large enough for sorted tiles, over several sorts, with new fixed
+    ends in between (boxes widened, not sorted anew) and an imported state."""
+    import paper_1311_4527_gb300 as pk
+    inst = workloads.small_square(p, eta, seed=90 + p)
+    moved = (0.98 * inst.start + 0.02 * inst.start.mean(0), inst.goal)
+    shrunk = 0.9 * inst.radius  # so that the moved starts stay clear of one another
+    out = []
+    for flags in (0, pk.PLAN_DENSE_STATE):
+        with pk.Planner.from_instance(inst, flags=flags) as pl:
+            pl.set_params(radius=shrunk)
+            zs = []
+            for n in (3, iters - 3):
+                pl.iterate(n)
+                zs.append((pl.trajectory().cpu().numpy(), pl.info()["active_coll"]))
+            pl.set_endpoints(*moved)
+            pl.iterate(9)
+            zs.append((pl.trajectory().cpu().numpy(), pl.info()["active_coll"]))
+        out.append(zs)
+    for (zg, ag), (zd, ad) in zip(*out):
+        assert np.array_equal(zg, zd) and ag == ad
+
+
 @pytest.mark.parametrize("eta", [30, 31, 32, 33, 63, 64])
 def test_break_point_counts_around_a_node_warp(eta):
     """One iteration from an oracle iterate, with as many break-points as fill
