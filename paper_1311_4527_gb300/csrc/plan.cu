@@ -427,47 +427,103 @@ __device__ __forceinline__ float least_so_far(const unsigned long long* out) {
   return sqrtf((float)__longlong_as_double((long long)__ldcg(out))) * 1.000001f;
 }
 
+// plan_check's words: pair and wall minima (bits), endpoint error (bits),
+// finished blocks, the cost blocks' shares, an upper bound of the pairs' minimum.
+constexpr int CHECK_COST_BLOCKS = 64, CHECK_SHARES = 4, CHECK_KNOWN = CHECK_SHARES + CHECK_COST_BLOCKS;
+
 // A candidate's squared ratio into the global minimum.
 __device__ __forceinline__ void offer_ratio(double q, unsigned long long* out) {
   const unsigned long long v = (unsigned long long)__double_as_longlong(q);
   if (q >= 0.0 && v < __ldcg(out)) atomicMin(out, v);
 }
 
-// Pairs of one (segment s, agent tile pair): min over i < j of
-// dist^2 / (r_i + r_j)^2, dist the smallest distance between the agents over
-// the segment (the origin against their relative motion).  256 threads, four
-// rows each, lane = column.
-__device__ __forceinline__ void check_pairs(const Dev& P, int block, unsigned long long* out) {
-  constexpr int PER = TILE * TILE / 256;
-  const int s = block / P.ntp, tp = block - s * P.ntp;
-  const int2 IJ = P.tiles[tp];
-  const int E1 = P.eta + 1;
-  const int j = IJ.y * TILE + (threadIdx.x & 31);
-  float2 zjl = mk(0.f, 0.f), zjh = zjl;
-  float rj = 1.f;
-  if (j < P.p) { zjl = P.z[(size_t)j * E1 + s]; zjh = P.z[(size_t)j * E1 + s + 1]; rj = P.radius[j]; }
-  float lo[PER], least = INFINITY;
+// Agent i's ends of segment s.
+__device__ __forceinline__ float4 ends_of(const Dev& P, int i, int s) {
+  const float2* z = P.z + (size_t)i * (P.eta + 1) + s;
+  return pack(z[0], z[1]);
+}
+
+// Bounds of the pair with segments zi, zj and radius sum R: the smallest
+// distance between the agents over the segment (the origin against their
+// relative motion) over R.
+__device__ __forceinline__ Bounds pair_bounds(float4 zi, float4 zj, float R) {
+  const float2 cl = lo2(zj) - lo2(zi), ch = hi2(zj) - hi2(zi);
+  return ratio_bounds(sqrtf(dist2_origin_segment(cl, ch)), fmaxf(maxabs2(cl), maxabs2(ch)), R);
+}
+
+// A first upper bound of the smallest pair ratio, for a block of tiles that
+// starts with tile t: three quarters of the pairs of that tile's row group
+// with itself, two a thread (with any order of the agents some near neighbours
+// are among them, mostly), and what other blocks found (`known`).
+__device__ __forceinline__ float first_bound(const Dev& P, int t, const unsigned* known) {
+  const int s = t / P.ntp, I = P.tiles[t - s * P.ntp].x;
+  const int c = threadIdx.x & 31, j = I * TILE + c;
+  float least = __uint_as_float(__ldcg(known));
+  if (j < P.p) {
+    const float4 zj = ends_of(P, j, s);
+    // column c with rows 0-15 before it, and those after 15 for the first 16 columns
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int i = IJ.x * TILE + (threadIdx.x >> 5) + q * (256 / TILE);
-    lo[q] = INFINITY;
-    if (i < j && j < P.p) {
-      const float2 cl = zjl - P.z[(size_t)i * E1 + s], ch = zjh - P.z[(size_t)i * E1 + s + 1];
-      const float mag = fmaxf(maxabs2(cl), maxabs2(ch));
-      const Bounds b = ratio_bounds(sqrtf(dist2_origin_segment(cl, ch)), mag, P.radius[i] + rj);
-      lo[q] = b.lo;
-      least = fminf(least, b.hi);
+    for (int q = 0; q < 2; ++q) {
+      const int r = (threadIdx.x >> 5) + 8 * q, a = r < c ? r : TILE - 1 - r, i = I * TILE + a;
+      if (a != c && i < P.p) least = fminf(least, pair_bounds(ends_of(P, i, s), zj, P.radius[i] + P.radius[j]).hi);
     }
   }
-  least = fminf(block_min(least), least_so_far(out));
+  return block_min(least);
+}
+
+// Pairs of one (segment s, agent tile pair), one warp: min over i < j of
+// dist^2 / (r_i + r_j)^2.  A pair can only be the closest when its ratio is
+// at most the bound `least` of some other pair's, so its agents' segments are
+// within least (r_i + r_j): the bounding-circle filter with the radii times
+// `least` drops nearly every pair (and where FP32 squares are not safe, none).
+// Those left take the FP32 bounds, and FP64 where these leave them the
+// closest.
+__device__ __forceinline__ void check_tile(const Dev& P, int tile, float first, TileMem* M, unsigned* known,
+                                           unsigned long long* out) {
+  const int lane = threadIdx.x & 31;
+  const int s = tile / P.ntp;
+  const int2 IJ = P.tiles[tile - s * P.ntp];
+  const int i = IJ.x * TILE + lane, j = IJ.y * TILE + lane;
+  const bool vi = i < P.p, vj = j < P.p;
+  float4 zi = make_float4(0.f, 0.f, 0.f, 0.f), zj = zi;
+  float ri = 0.f, rj = 0.f;
+  if (vi) { zi = ends_of(P, i, s); ri = P.radius[i]; }
+  if (vj) { zj = ends_of(P, j, s); rj = P.radius[j]; }
+  bool safe = true;
+  auto circle = [&](float4 z, float r) {
+    const float2 m = 0.5f * (lo2(z) + hi2(z)), d = hi2(z) - lo2(z);
+    const float b = fmaf(0.5f, sqrtf(dot(d, d)), first * r);
+    safe = safe && dot(m, m) + b * b < 1e30f;
+    return make_float4(m.x, m.y, b, -bounding_offset(m, b));
+  };
+  const float4 ci = circle(zi, ri), cj = circle(zj, rj);
+  M->mx[lane] = cj.x; M->my[lane] = cj.y; M->b[lane] = cj.z; M->na[lane] = cj.w;
+  M->z[lane] = zj;
+  M->r[lane] = rj;
+  uint32_t near = __ballot_sync(FULL, vj);
+  __syncwarp();
+  if (!vi) near = 0u;
+  if (IJ.x == IJ.y) near &= (lane == 31) ? 0u : (~0u << (lane + 1));
+  if (__all_sync(FULL, safe)) near &= near_columns(ci, M);
+  if (!__any_sync(FULL, near != 0u)) return;
+  float least = first;
+  uint32_t hit = 0u;
+  for (uint32_t w = near; w; w &= w - 1u) {
+    const int c = __ffs(w) - 1;
+    const Bounds b = pair_bounds(zi, M->z[c], ri + M->r[c]);
+    if (!(b.lo > least)) hit |= 1u << c;
+    least = fminf(least, b.hi);
+  }
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int i = IJ.x * TILE + (threadIdx.x >> 5) + q * (256 / TILE);
-    if (!(i < j && j < P.p) || lo[q] > least) continue;
-    const float2 zil = P.z[(size_t)i * E1 + s], zih = P.z[(size_t)i * E1 + s + 1];
-    const double R = (double)P.radius[i] + (double)rj;
-    offer_ratio(origin_seg_dist2((double)zjl.x - (double)zil.x, (double)zjl.y - (double)zil.y,
-                                 (double)zjh.x - (double)zih.x, (double)zjh.y - (double)zih.y) / (R * R), out);
+  for (int o = 16; o > 0; o >>= 1) least = fminf(least, __shfl_xor_sync(FULL, least, o));
+  if (lane == 0 && least < __uint_as_float(__ldcg(known))) atomicMin(known, __float_as_uint(least));
+  for (uint32_t w = hit; w; w &= w - 1u) {
+    const int c = __ffs(w) - 1;
+    const float4 zc = M->z[c];
+    if (pair_bounds(zi, zc, ri + M->r[c]).lo > least) continue;
+    const double R = (double)ri + (double)M->r[c];
+    offer_ratio(origin_seg_dist2((double)zc.x - (double)zi.x, (double)zc.y - (double)zi.y, (double)zc.z - (double)zi.z,
+                                 (double)zc.w - (double)zi.w) / (R * R), out);
   }
 }
 
@@ -529,21 +585,27 @@ __device__ __forceinline__ void check_walls(const Dev& P, int nseg, int block, i
 // The whole check in one launch.  Blocks: `costs` for the total kinetic cost
 // sum c_{i,s} |z_i(s+1) - z_i(s)|^2 over the kinetic segments (each block's
 // share by a fixed tree, the blocks' shares in order, so the sum is
-// deterministic) and the largest endpoint error |z - start|, |z - goal|; one
-// per tile of pairs; the rest walls.  The last block to finish hands the four
-// numbers over and leaves the words as it found them.
-// words: pair and wall minima (bits), endpoint error (bits), finished blocks.
-constexpr int CHECK_COST_BLOCKS = 64;
+// deterministic) and the largest endpoint error |z - start|, |z - goal|;
+// `walls` for the walls; the rest a tile of pairs a warp.  The last block to finish hands the four numbers over
+// and leaves the words as it found them.
+// Every pair's FP32 distance took 90 us at p = 1,024, eta = 16 (a call 100); the
+// circle filter with a bound per block leaves a chain of loads per tile, a call
+// 37 (and 22 at p = 16, as before).  A first bound of all groups from a kernel
+// before is tighter, but its launch costs what it saves (34 at p = 1,024, 25
+// against 22-23 up to p = 64); two tiles a warp took 39.
 __device__ __forceinline__ void init_check_words(unsigned long long* words) {
   words[0] = words[1] = 0x7ff0000000000000ull;  // +inf
   words[2] = words[3] = 0ull;
+  words[CHECK_KNOWN] = 0x7f800000ull;            // +inf (32 bits)
 }
 __global__ void __launch_bounds__(256) check_kernel(Dev P, const double* ccost, const float2* start,
-                                                    const float2* goal, int s_lo, int nseg, int costs, int pairs,
-                                                    double* part, unsigned long long* words, double* out) {
+                                                    const float2* goal, int s_lo, int nseg, int costs, int walls,
+                                                    unsigned long long* words, double* out) {
   __shared__ double sc[256], se[256];
+  __shared__ TileMem mem[8];
   __shared__ bool last;
   const int block = (int)blockIdx.x, tid = threadIdx.x;
+  double* part = reinterpret_cast<double*>(words + CHECK_SHARES);
   if (block < costs) {
     const int E1 = P.eta + 1, stride = costs * 256;
     double c = 0.0, e = 0.0;
@@ -575,10 +637,13 @@ __global__ void __launch_bounds__(256) check_kernel(Dev P, const double* ccost, 
       part[block] = sc[0];
       if (se[0] > 0.0) atomicMax(words + 2, (unsigned long long)__double_as_longlong(se[0]));
     }
-  } else if (block < costs + pairs) {
-    check_pairs(P, block - costs, words);
+  } else if (block < costs + walls) {
+    check_walls(P, nseg, block - costs, walls, words + 1);
   } else {
-    check_walls(P, nseg, block - costs - pairs, (int)gridDim.x - costs - pairs, words + 1);
+    const int tile = (block - costs - walls) * 8;
+    unsigned* known = reinterpret_cast<unsigned*>(words + CHECK_KNOWN);
+    const float first = first_bound(P, tile, known);
+    if (tile + (tid >> 5) < nseg * P.ntp) check_tile(P, tile + (tid >> 5), first, mem + (tid >> 5), known, words);
   }
   __syncthreads();
   if (tid == 0) {
@@ -1315,7 +1380,7 @@ Layout layout_for(const plan_config* c) {
   L.status = take(4);
   L.count = take(16);
   L.ccost = take(p * eta * 8);  // FP64 kinetic coefficients for plan_check
-  L.chk = take((4 + CHECK_COST_BLOCKS) * 8);  // plan_check: its words and the cost blocks' shares
+  L.chk = take((CHECK_KNOWN + 1) * 8);  // plan_check's words
   L.ekey = take(24);            // plan_set_endpoints: first violation, extent, finished blocks
   // a device copy of the endpoints of a device-checked update, made while
   // they are checked
@@ -2352,7 +2417,7 @@ plan_status plan_check(plan_t h, double* total_cost, double* min_pair_clearance,
   const int s_lo = h->vo ? 1 : 0;
   const int nseg = h->vo ? 1 : h->eta;
   const int costs = (int)std::min<long long>(((long long)h->p * h->eta + 255) / 256, CHECK_COST_BLOCKS);
-  const int pairs = h->p > 1 ? nseg * h->ntp : 0;
+  const int pairs = h->p > 1 ? (nseg * h->ntp + 7) / 8 : 0;  // blocks of eight tiles
   const long long nwall = (long long)h->nw * nseg * h->p;
   const int walls = (int)std::min<long long>((nwall + 255) / 256, 4096);
   // the last block writes the results into pinned host memory: a copy behind
@@ -2361,9 +2426,9 @@ plan_status plan_check(plan_t h, double* total_cost, double* min_pair_clearance,
   double* v = reinterpret_cast<double*>(h->h_res + 4);
   double* dv = nullptr;
   CK(cudaHostGetDevicePointer(reinterpret_cast<void**>(&dv), v, 0));
-  check_kernel<<<(unsigned)(costs + pairs + walls), 256, 0, h->stream>>>(
-      P, h->at<double>(h->L.ccost), h->at<float2>(h->L.start), h->at<float2>(h->L.goal), s_lo, nseg, costs, pairs,
-      reinterpret_cast<double*>(words + 4), words, dv);
+  check_kernel<<<(unsigned)(costs + walls + pairs), 256, 0, h->stream>>>(
+      P, h->at<double>(h->L.ccost), h->at<float2>(h->L.start), h->at<float2>(h->L.goal), s_lo, nseg, costs, walls,
+      words, dv);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(h->stream));
   if (total_cost) *total_cost = v[0];

@@ -59,3 +59,25 @@ def test_clearances_match_plain_fp64(p, eta, shift, march):
     for g in got:  # the same FP64 arithmetic on the same FP32 values, in another order
         assert g["min_pair_clearance"] == pytest.approx(pair, rel=1e-13) if math.isfinite(pair) else math.isinf(g["min_pair_clearance"])
         assert g["min_wall_clearance"] == pytest.approx(wall, rel=1e-12, abs=1e-12 * (1 + shift))
+
+
+@pytest.mark.parametrize("p,eta,far", [(300, 2, 0.0), (513, 1, 0.0), (70, 2, 1e12), (70, 2, 1e17)])
+def test_bounding_circles_drop_no_closest_pair(p, eta, far):
+    """Sparse plans, where the first bound drops nearly every block of pairs
+    (the closest pair is planted in two groups, the bound comes from others),
+    and an agent beyond the range of FP32 squares, where nothing may be dropped."""
+    import paper_1311_4527_gb300 as pk
+    inst = workloads.small_square(p, eta, seed=180 + p)
+    rng = np.random.default_rng(p)
+    f32 = lambda a: np.asarray(a, np.float32).astype(np.float64)
+    with pk.Planner(f32(inst.start), f32(inst.goal), inst.radius, eta, walls=inst.walls) as pl:
+        z = f32(inst.start[:, None] + rng.normal(0, 0.02, size=(p, eta + 1, 2)))
+        z[p - 1, eta] = f32(z[1, eta] + 0.11 * inst.radius[1])
+        if far:
+            z[p // 2, :, 0] = np.float32(far)
+        P = p * (p - 1) // 2
+        pl.import_state(z, np.zeros((eta, P, 4, 2)), np.zeros((eta, p, 2, 2)), np.zeros((4, eta, p, 2, 2)), 0)
+        got = [pl.check() for _ in range(2)]
+    pair, _ = _clearances(z, f32(inst.radius), np.zeros((0, 4)))
+    for g in got:  # the same FP64 arithmetic on the same FP32 values, in another order
+        assert g["min_pair_clearance"] == pytest.approx(pair, rel=1e-13)
