@@ -10,8 +10,7 @@
 //                    fixed-point consensus sums
 //   node_kernel      z = sum m / count per free break-point
 //
-// Dense state, three: test_kernel (tests, with the kinetic, wall and velocity
-// factors whole), prox_kernel (the minimizer of every active pair) and
+// Dense state: test_kernel (every factor, the pairs' records streamed) and
 // node_kernel.
 //
 // Iterations after the first are replayed from captured CUDA graphs.
@@ -45,9 +44,6 @@ __device__ __forceinline__ void pdl_begin() {
 }
 
 // The single-planner kernels: thin wrappers over the per-warp work.
-constexpr int TEST_WARPS = 4;
-constexpr int TEST_ROWS = TILE / TEST_WARPS;
-
 // Gated state, every factor in one launch.  The first CTAs take the worklist
 // (long chains: a minimizer each), then the tiles of the last segment (early
 // in a solve it spans each agent's whole way, and nearly all its pairs take
@@ -86,17 +82,21 @@ __global__ void __launch_bounds__(32 * FACTOR_WARPS, 6) factor_kernel(Dev P, Fac
   else collision_warp<CLASSES>(P, item, nlist, mem + warp, G.mode);
 }
 
-// Dense state, pass 1: the first CTAs take the kinetic, wall and velocity
-// warps, the rest a collision tile each.
-__global__ void __launch_bounds__(32 * TEST_WARPS, 8) test_kernel(Dev P, int seg_ctas, int seg_warps) {
+// Dense state, every factor in one launch: the first CTAs take the kinetic,
+// wall and velocity warps, the rest a block of 32 x 32 pairs each.  Bound by
+// the u records where these are many (67 MB read and written per iteration at
+// p = 512, eta = 16), else by the chain from a row's records to its minimizers.
+template <int WARPS, int AHEAD>
+__global__ void __launch_bounds__(32 * WARPS, WARPS == 16 ? 1 : 4) test_kernel(Dev P, int seg_ctas, int seg_warps) {
+  __shared__ TestMem mem;
   pdl_begin();
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.res_cur = 0u;
   if ((int)blockIdx.x < seg_ctas) {
-    const int w = (int)blockIdx.x * TEST_WARPS + (threadIdx.x >> 5);
+    const int w = (int)blockIdx.x * WARPS + (threadIdx.x >> 5);
     if (w < seg_warps) segment_warp(P, w);
     return;
   }
-  test_block<TEST_ROWS>(P, blockIdx.x - seg_ctas);
+  test_block<TILE / WARPS, AHEAD, true>(P, blockIdx.x - seg_ctas, &mem);
 }
 
 // Worklist items are dealt to warps round-robin (item t to warp t mod W,
@@ -107,16 +107,6 @@ __device__ __forceinline__ unsigned long long dealt_first(unsigned long long& st
   const unsigned long long W = (gridDim.x * blockDim.x) >> 5;
   stride = 32ull * W;
   return (unsigned long long)(threadIdx.x & 31) * W + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-}
-
-// Dense state, pass 2: groups of 32 consecutive worklist entries (pairs of
-// one tile, so of one segment: the lanes take the same branches), consecutive
-// groups on different CTAs, so that they spread over the SMs.
-__global__ void __launch_bounds__(256) prox_kernel(Dev P) {
-  pdl_begin();
-  const unsigned long long nc = *P.work_count, G = gridDim.x, wpb = blockDim.x >> 5;
-  const unsigned long long v = (threadIdx.x >> 5) * G + blockIdx.x;
-  for (unsigned long long t = 32ull * v + (threadIdx.x & 31); t < nc; t += 32ull * G * wpb) prox_item(P, P.work[t]);
 }
 
 // Where an iteration is recorded for the backward pass: z^k, the kinetic u^k,
@@ -1540,7 +1530,6 @@ struct plan_s {
   int sorted_at = 0;    // iteration of the last sort
   bool fresh = true;  // no worklist yet: the next iteration runs in two launches (FactorMode)
   int sms = 0;        // SMs of the device
-  int prox_grid = 0;  // CTAs of the dense state's minimizer pass (resident CTAs per SM x SMs)
   cudaStream_t cap = nullptr;    // private stream for capturing the iteration graphs
   bool profiling = false;        // plan_profile: per-kernel event timing
   cudaEvent_t pev[6] = {};
@@ -1686,14 +1675,11 @@ plan_status drop_worklist(plan_t h) {
   return PLAN_OK;
 }
 
-plan_status ensure_prox_grid(plan_t h) {
-  if (h->prox_grid == 0) {
-    int dev = 0, sms = 0, nb = 0;
+plan_status ensure_sms(plan_t h) {
+  if (h->sms == 0) {
+    int dev = 0;
     CK(cudaGetDevice(&dev));
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, prox_kernel, 256, 0));
-    h->prox_grid = std::max(1, sms * std::max(nb, 1));
-    h->sms = sms;
+    CK(cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev));
   }
   return PLAN_OK;
 }
@@ -1793,10 +1779,18 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = null
   const bool prof = h->profiling;
   if (prof) CK(cudaEventRecord(h->pev[0], ms));
   if (P.dense) {
-    const int segc = (segw + TEST_WARPS - 1) / TEST_WARPS;
-    CK(launch_pdl(test_kernel, (unsigned)(segc + (size_t)h->eta * h->ntp), 32u * TEST_WARPS, ms, P, segc, segw));
+    // warps per block of pairs: as many as spread its rows and minimizers
+    // while the GPU holds all blocks at once, four (with four rows of records
+    // under way each) where it is the records that take the time.  Measured
+    // (us per iteration of standard ADMM, eta = 16, with 4 / 8 / 16 warps):
+    // 48 blocks 13.6 / 11.1 / 10.0, 240 blocks 14.2 / 12.2 / 13.4, 2,176
+    // blocks 28.7 / 29.4 / 47.6.
+    const size_t blocks = (size_t)h->eta * h->ntp;
+    const int warps = blocks <= (size_t)h->sms ? 16 : blocks <= (size_t)8 * h->sms ? 8 : 4;
+    auto kern = warps == 16 ? test_kernel<16, 2> : warps == 8 ? test_kernel<8, 2> : test_kernel<4, 4>;
+    const int segc = (segw + warps - 1) / warps;
+    CK(launch_pdl(kern, (unsigned)(segc + blocks), 32u * warps, ms, P, segc, segw));
     if (prof) CK(cudaEventRecord(h->pev[1], ms));
-    CK(launch_pdl(prox_kernel, (unsigned)h->prox_grid, 256u, ms, P));
   } else {
     FactorGrid G;
     const int nseg = h->vo ? 1 : h->eta;
@@ -1844,7 +1838,7 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = null
 // One iteration: replay a captured CUDA graph of the three kernels when one
 // fits (past the rho warm-up, not profiling), else launch them directly.
 plan_status run_iteration(plan_t h) {
-  plan_status st = ensure_prox_grid(h);
+  plan_status st = ensure_sms(h);
   if (st == PLAN_OK && h->sorted && h->k - h->sorted_at >= SORT_EVERY) st = sort_agents(h);
   if (st != PLAN_OK) return st;
   const bool graphable = h->cap && !h->profiling && h->k >= h->graph_from() && !h->fresh;
@@ -1918,7 +1912,7 @@ plan_status run_graph_runs(plan_t h, int& n, int len, cudaGraphExec_t* execs) {
 }
 
 plan_status run_iterations(plan_t h, int n) {
-  plan_status st = ensure_prox_grid(h);
+  plan_status st = ensure_sms(h);
   if (st != PLAN_OK) return st;
   if (n > 0 && h->fresh) {
     if ((st = run_iteration(h)) != PLAN_OK) return st;
@@ -2763,7 +2757,7 @@ plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, char* zb_in, ch
   const unsigned node_grid = (unsigned)((h->p * (h->eta + 1) + 255) / 256);
   // a thread per edge group that may be active (more CTAs than that only cost their launch)
   const long long items = (long long)(1 + h->nw + h->nv) * h->eta * h->p + (long long)h->eta * h->p * (h->p - 1) / 2;
-  const unsigned grid = (unsigned)std::min<long long>((items + 127) / 128, 2ll * h->prox_grid);
+  const unsigned grid = (unsigned)std::min<long long>((items + 127) / 128, 6ll * h->sms);
   for (int q = n - 1; q >= 0 && st == PLAN_OK && e == cudaSuccess; --q) {
     const AdjDev D = adj_dev(h, A, q, zb_in, zb_out);
     e = launch_pdl(bw_scatter_kernel, grid, 128u, ms, D);
@@ -2783,7 +2777,7 @@ plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, char* zb_in, ch
 // iteration 0 has no residual slot before it; the rest is the same for all of
 // them, the iteration number coming from AdjDev::k0.
 plan_status segment_steps(plan_t h, const AdjLayout& A, int n, char* zb_in, char* zb_out) {
-  plan_status st = ensure_prox_grid(h);
+  plan_status st = ensure_sms(h);
   if (st != PLAN_OK) return st;
   if (solo(h)) {
     Tape T = adj_tape(h, A);
@@ -3084,7 +3078,7 @@ plan_status plan_backward(plan_t h, int K, const float* dL_dz, float* d_start, f
   if (st != PLAN_OK) return st;
   if (!h->adj_valid || K != h->adj_K)
     return fail(PLAN_EINVAL, "plan_backward(K = %d) needs the state left by plan_unroll(K)", K);
-  if ((st = ensure_prox_grid(h)) != PLAN_OK) return st;
+  if ((st = ensure_sms(h)) != PLAN_OK) return st;
   const int C = h->adj_C;
   const AdjLayout A = adj_layout(h, K, C);
   const size_t p = h->p, nodes = p * (h->eta + 1);
@@ -3305,6 +3299,7 @@ template <int TROWS>
 __global__ void __launch_bounds__(32 * (TILE / TROWS)) batch_test_kernel(const Dev* tab, const int* pre,
                                                                           int n, const uint8_t* frozen) {
   __shared__ Dev sP;
+  __shared__ TestMem mem;
   __shared__ int sb, sblk;
   if (threadIdx.x == 0) {
     const int b = find_member(pre, n, blockIdx.x);
@@ -3315,7 +3310,7 @@ __global__ void __launch_bounds__(32 * (TILE / TROWS)) batch_test_kernel(const D
   __syncthreads();
   if (frozen[sb]) return;
   if (sblk == 0 && threadIdx.x == 0) *sP.res_cur = 0u;
-  test_block<TROWS>(sP, sblk);
+  test_block<TROWS, 4, false>(sP, sblk, &mem);
 }
 
 // Table entry of a factor-pass warp: the member, and an item of its own
@@ -3667,8 +3662,8 @@ plan_status plan_batch_create(int n, const plan_config* cfgs, const float* const
   if (e == cudaSuccess) e = cudaMemcpyAsync(B->shapes, shapes.data(), n * sizeof(BatchShape), cudaMemcpyHostToDevice, B->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(B->frozen, B->h_frozen.data(), n, cudaMemcpyHostToDevice, B->stream);
   if (e != cudaSuccess) { plan_batch_destroy(B); return fail(PLAN_ECUDA, "batch setup failed: %s", cudaGetErrorString(e)); }
-  st = ensure_prox_grid(B->m[0]);
-  if (st == PLAN_OK) { B->prox_grid = std::max(1, B->m[0]->prox_grid / 4); st = batch_tables(B); }
+  st = ensure_sms(B->m[0]);
+  if (st == PLAN_OK) { B->prox_grid = std::max(1, 3 * B->m[0]->sms / 4); st = batch_tables(B); }
   if (st != PLAN_OK) { plan_batch_destroy(B); return st; }
   *out = B;
   return PLAN_OK;

@@ -13,8 +13,9 @@
 //   Node pass, consensus_warp: z = sum m / count per free break-point (step
 //     5), and the per-segment records the next factor pass starts from.
 // Dense state: test_block (every pair's u record streamed, lane = column
-//   agent) and segment_warp in one launch, then prox_item over the worklist of
-//   active pairs, then the node pass.
+//   agent, then prox_item for the active ones) and segment_warp in one launch,
+//   then the node pass.  (A batch runs prox_item over its worklists in a launch
+//   of its own.)
 //
 // Step 7 needs z^{k+1}, which exists only after every factor ran, so x^{k+1}
 // of the active factors is stored and u^{k+1} = u^k + alpha (x^{k+1} -
@@ -442,17 +443,65 @@ __device__ __forceinline__ void tile_of(int nt, int t, int& I, int& J) {
   J = i + (t - tile_pair(nt, i, i));
 }
 
+// Dense state: the collision minimizer (Eq. coll_minimizer_problem through
+// App. C/D/I) of an active pair, one thread.
+__device__ __forceinline__ void prox_item(const Dev& P, uint32_t fid) {
+  const int E1 = P.eta + 1;
+  const uint32_t row = fid >> 5, c = fid & 31;
+  const uint32_t blk = row >> 5, r = row & 31;
+  const int s = (int)(blk / P.ntp);
+  int I, J;
+  tile_of(P.nt, (int)(blk - (uint32_t)s * P.ntp), I, J);
+  const int i = I * TILE + r, j = J * TILE + c;
+  const float scale = P.fix[0], bound = P.fix[1];  // loaded beside the minimizer
+  const float4 a = P.ulo[fid], b = P.uhi[fid];
+  const float2 nil = P.z[(size_t)i * E1 + s] - lo2(a), nih = P.z[(size_t)i * E1 + s + 1] - lo2(b);
+  const float2 njl = P.z[(size_t)j * E1 + s] - hi2(a), njh = P.z[(size_t)j * E1 + s + 1] - hi2(b);
+  float2 xil, xih, xjl, xjh;
+  const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
+  if (P.noenergy) {
+    int cil, cih, cjl, cjh;
+    end_classes(P, i, s, pin_lo, pin_hi, cil, cih);
+    end_classes(P, j, s, pin_lo, pin_hi, cjl, cjh);
+    coll_minimizer_classes(nil, nih, njl, njh, cil, cih, cjl, cjh, P.radius[i] + P.radius[j],
+                           P.rho, xil, xih, xjl, xjh);
+  } else {
+    coll_minimizer(nil, nih, njl, njh, pin_lo, pin_hi, P.radius[i] + P.radius[j], P.rho,
+                   xil, xih, xjl, xjh);
+  }
+  P.xlo[fid] = pack(xil, xjl);
+  P.xhi[fid] = pack(xih, xjh);
+  if (!pin_lo) {
+    contribute(P, scale, bound, i, s, xil + lo2(a));
+    contribute(P, scale, bound, j, s, xjl + hi2(a));
+  }
+  if (!pin_hi) {
+    contribute(P, scale, bound, i, s + 1, xih + lo2(b));
+    contribute(P, scale, bound, j, s + 1, xjh + hi2(b));
+  }
+}
+
 // Dense state, pass 1: one CTA of TILE / TROWS warps per (segment s, agent
 // tiles I <= J) block of 32 x 32 collision factors; each warp takes TROWS
 // rows (the launch shape the batched autotuner varies), lane = column agent j,
-// and the row agents' data is held one per lane and broadcast by shuffles.
-// Per row, the warp streams the u records of its 32 pairs, finishes the
-// pending dual update (step 7 of the previous iteration), forms n = z - u
-// (step 1), runs the collision test (steps 2-3: weight rho0 or 0), stores the
-// records and the row's activity bits, and appends its active pairs to the
-// global worklist.
-template <int TROWS>
-__device__ __forceinline__ void test_block(const Dev& P, int blk) {
+// and the row agents' data is broadcast from shared memory.  Per row, the warp
+// streams the u records of its 32 pairs, finishes the pending dual update
+// (step 7 of the previous iteration), forms n = z - u (step 1), runs the
+// collision test (steps 2-3: weight rho0 or 0), stores the records and the
+// row's activity bits and lists its active pairs.  A single plan's block then
+// runs their minimizers itself (LOCAL, its own list in shared memory: a kernel
+// of its own behind a global worklist cost 5 us of each iteration: 34.7 to 28.7
+// us at p = 512, eta = 16, 19.2 to 10.0 at p = 40); a batch
+// appends them to the members' worklists, which one launch shares out.
+struct TestMem {
+  float4 z[TILE], was[TILE];  // break-points of the row agents: z^k and (standard ADMM) z^{k-1}
+  float r[TILE];
+  uint32_t word[TILE];
+  unsigned listed;
+  uint16_t list[TILE * TILE];
+};
+template <int TROWS, int AHEAD, bool LOCAL>
+__device__ __forceinline__ void test_block(const Dev& P, int blk, TestMem* M) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int E1 = P.eta + 1;
   float res = 0.f;
@@ -464,76 +513,98 @@ __device__ __forceinline__ void test_block(const Dev& P, int blk) {
   const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
   const int r0 = warp * TROWS;
   const int nrows = min(TROWS, P.p - I * TILE - r0);
+  if (LOCAL) {
+    if (threadIdx.x == 0) M->listed = 0u;
+    __syncthreads();
+  }
   if (nrows > 0) {  // warp-uniform
     // column agent of this lane
     const int j = J * TILE + lane;
-    const bool vj = j < P.p;
-    float2 zjl = mk(0.f, 0.f), zjh = zjl;
+    const bool vj = j < P.p, every = P.admm || P.keep;
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 zj = none, pj = none;
     float rj = 0.f;
-    if (vj) { zjl = P.z[(size_t)j * E1 + s]; zjh = P.z[(size_t)j * E1 + s + 1]; rj = P.radius[j]; }
-    // row agents, held by the first nrows lanes
-    float2 ill = mk(0.f, 0.f), ilh = ill;
-    float rl = 0.f;
-    uint32_t wordl = 0u;
-    if (lane < nrows) {
-      const int il = I * TILE + r0 + lane;
-      ill = P.z[(size_t)il * E1 + s]; ilh = P.z[(size_t)il * E1 + s + 1]; rl = P.radius[il];
-      wordl = P.bits[(size_t)blk * TILE + r0 + lane];
+    if (vj) {
+      const size_t n = (size_t)j * E1 + s;
+      zj = pack(P.z[n], P.z[n + 1]);
+      if (P.admm) pj = pack(P.z_next[n], P.z_next[n + 1]);
+      rj = P.radius[j];
     }
-#pragma unroll 2
-    for (int q = 0; q < nrows; ++q) {
-      const int r = r0 + q;
-      const uint32_t word = __shfl_sync(FULL, wordl, q);
-      const bool valid = vj && (!diag || r < lane);
-      const float ri = __shfl_sync(FULL, rl, q);
-      float2 uil = mk(0.f, 0.f), ujl = uil, uih = uil, ujh = uil;
-      const size_t row = (size_t)blk * TILE + r;
-      const size_t fid = row * TILE + lane;
-      const float2 zil = mk(__shfl_sync(FULL, ill.x, q), __shfl_sync(FULL, ill.y, q));
-      const float2 zih = mk(__shfl_sync(FULL, ilh.x, q), __shfl_sync(FULL, ilh.y, q));
-      const bool bprev = (word >> lane) & 1u;  // set only for valid pairs
-      if (valid) {
-        const float4 a = P.ulo[fid], b = P.uhi[fid];
-        uil = lo2(a); ujl = hi2(a); uih = lo2(b); ujh = hi2(b);
+    if (lane < nrows) {
+      const int i = I * TILE + r0 + lane;
+      const size_t n = (size_t)i * E1 + s;
+      M->z[r0 + lane] = pack(P.z[n], P.z[n + 1]);
+      if (P.admm) M->was[r0 + lane] = pack(P.z_next[n], P.z_next[n + 1]);
+      M->r[r0 + lane] = P.radius[i];
+      M->word[r0 + lane] = P.bits[(size_t)blk * TILE + r0 + lane];
+    }
+    __syncwarp();
+    for (int q0 = 0; q0 < nrows; q0 += AHEAD) {
+      float4 ua[AHEAD], ub[AHEAD];
+      // the group's records, all loads under way before the first is used
+#pragma unroll
+      for (int g = 0; g < AHEAD; ++g) {
+        const int r = r0 + q0 + g;
+        ua[g] = ub[g] = none;
+        if (q0 + g < nrows && vj && (!diag || r < lane) && (every || ((M->word[r] >> lane) & 1u))) {
+          const size_t fid = ((size_t)blk * TILE + r) * TILE + lane;
+          ua[g] = P.ulo[fid];
+          ub[g] = P.uhi[fid];
+        }
       }
-      if (bprev) {
-        // finish step 7 of the previous iteration for this pair
-        const float4 xa = P.xlo[fid], xb = P.xhi[fid];
-        uil = finish_u(true, pin_lo, false, uil, lo2(xa), zil, P.alpha, res);
-        ujl = finish_u(true, pin_lo, false, ujl, hi2(xa), zjl, P.alpha, res);
-        uih = finish_u(true, pin_hi, false, uih, lo2(xb), zih, P.alpha, res);
-        ujh = finish_u(true, pin_hi, false, ujh, hi2(xb), zjh, P.alpha, res);
-      } else if (P.admm && valid) {
-        // standard ADMM: the pair was feasible, so x^k = z^{k-1} - u^{k-1}
-        const float2 pil = P.z_next[(size_t)(I * TILE + r) * E1 + s];
-        const float2 pih = P.z_next[(size_t)(I * TILE + r) * E1 + s + 1];
-        const float2 pjl = P.z_next[(size_t)j * E1 + s], pjh = P.z_next[(size_t)j * E1 + s + 1];
-        uil = finish_u_feasible(pin_lo, uil, pil, zil, P.alpha, res);
-        ujl = finish_u_feasible(pin_lo, ujl, pjl, zjl, P.alpha, res);
-        uih = finish_u_feasible(pin_hi, uih, pih, zih, P.alpha, res);
-        ujh = finish_u_feasible(pin_hi, ujh, pjh, zjh, P.alpha, res);
-      } else if (!P.keep) {
-        uil = ujl = uih = ujh = mk(0.f, 0.f);  // reset rule: inactive edges carry u = 0
-      }
-      if (pin_lo) { uil = mk(0.f, 0.f); ujl = uil; }
-      if (pin_hi) { uih = mk(0.f, 0.f); ujh = uih; }
-      const bool act = valid && collides((zjl - ujl) - (zil - uil), (zjh - ujh) - (zih - uih), ri + rj);
-      if (valid) {
-        P.ulo[fid] = pack(uil, ujl);
-        P.uhi[fid] = pack(uih, ujh);
-      }
-      const uint32_t nword = __ballot_sync(FULL, act);
-      if (nword != word && lane == 0) P.bits[row] = nword;
-      if (nword) {
-        unsigned base = 0;
-        if (lane == 0) base = atomicAdd(P.work_count, (unsigned)__popc(nword));
-        base = __shfl_sync(FULL, base, 0);
-        if (act) P.work[base + __popc(nword & ((1u << lane) - 1u))] = (uint32_t)fid;
+#pragma unroll
+      for (int g = 0; g < AHEAD; ++g) {
+        if (q0 + g >= nrows) break;  // warp-uniform
+        const int r = r0 + q0 + g;
+        const bool valid = vj && (!diag || r < lane);
+        const size_t row = (size_t)blk * TILE + r, fid = row * TILE + lane;
+        const float4 zi = M->z[r];
+        const uint32_t word = M->word[r];
+        const bool bprev = (word >> lane) & 1u;  // set only for valid pairs
+        float2 uil = lo2(ua[g]), ujl = hi2(ua[g]), uih = lo2(ub[g]), ujh = hi2(ub[g]);
+        if (bprev) {
+          // finish step 7 of the previous iteration for this pair
+          const float4 xa = P.xlo[fid], xb = P.xhi[fid];
+          uil = finish_u(true, pin_lo, false, uil, lo2(xa), lo2(zi), P.alpha, res);
+          ujl = finish_u(true, pin_lo, false, ujl, hi2(xa), lo2(zj), P.alpha, res);
+          uih = finish_u(true, pin_hi, false, uih, lo2(xb), hi2(zi), P.alpha, res);
+          ujh = finish_u(true, pin_hi, false, ujh, hi2(xb), hi2(zj), P.alpha, res);
+        } else if (P.admm && valid) {
+          // standard ADMM: the pair was feasible, so x^k = z^{k-1} - u^{k-1}
+          const float4 pi = M->was[r];
+          uil = finish_u_feasible(pin_lo, uil, lo2(pi), lo2(zi), P.alpha, res);
+          ujl = finish_u_feasible(pin_lo, ujl, lo2(pj), lo2(zj), P.alpha, res);
+          uih = finish_u_feasible(pin_hi, uih, hi2(pi), hi2(zi), P.alpha, res);
+          ujh = finish_u_feasible(pin_hi, ujh, hi2(pj), hi2(zj), P.alpha, res);
+        }
+        // (reset rule: inactive edges carry u = 0, and were not loaded)
+        if (pin_lo) { uil = mk(0.f, 0.f); ujl = uil; }
+        if (pin_hi) { uih = mk(0.f, 0.f); ujh = uih; }
+        const bool act = valid && collides((lo2(zj) - ujl) - (lo2(zi) - uil), (hi2(zj) - ujh) - (hi2(zi) - uih),
+                                           M->r[r] + rj);
+        if (valid) {
+          P.ulo[fid] = pack(uil, ujl);
+          P.uhi[fid] = pack(uih, ujh);
+        }
+        const uint32_t nword = __ballot_sync(FULL, act);
+        if (nword != word && lane == 0) P.bits[row] = nword;
+        if (nword) {
+          unsigned base = 0;
+          if (lane == 0) base = atomicAdd(LOCAL ? &M->listed : P.work_count, (unsigned)__popc(nword));
+          base = __shfl_sync(FULL, base, 0) + __popc(nword & ((1u << lane) - 1u));
+          if (act && LOCAL) M->list[base] = (uint16_t)(r * TILE + lane);
+          if (act && !LOCAL) P.work[base] = (uint32_t)fid;
+        }
       }
     }
   }
   res = warp_max(res);
   if (lane == 0 && res > 0.f && P.res_prev) atomic_max_nonneg(P.res_prev, res);
+  if (LOCAL) {
+    __syncthreads();
+    const unsigned n = M->listed;
+    for (unsigned t = threadIdx.x; t < n; t += blockDim.x) prox_item(P, (uint32_t)blk * TILE * TILE + M->list[t]);
+  }
 }
 
 // Bounding-circle filter of the gated state.  Agent i's segment lies in the
@@ -1161,45 +1232,6 @@ __device__ __forceinline__ void sorted_collision_warp(const Dev& P, int item, in
   if (__any_sync(FULL, res > 0.f)) {  // only pairs active before have a residual
     res = warp_max(res);
     if (lane == 0 && P.res_prev) atomic_max_nonneg(P.res_prev, res);
-  }
-}
-
-// Dense state, pass 2: the collision minimizer (Eq. coll_minimizer_problem
-// through App. C/D/I) of every active pair in the worklist, one thread per
-// pair.
-__device__ __forceinline__ void prox_item(const Dev& P, uint32_t fid) {
-  const int E1 = P.eta + 1;
-  const uint32_t row = fid >> 5, c = fid & 31;
-  const uint32_t blk = row >> 5, r = row & 31;
-  const int s = (int)(blk / P.ntp);
-  int I, J;
-  tile_of(P.nt, (int)(blk - (uint32_t)s * P.ntp), I, J);
-  const int i = I * TILE + r, j = J * TILE + c;
-  const float scale = P.fix[0], bound = P.fix[1];  // loaded beside the minimizer
-  const float4 a = P.ulo[fid], b = P.uhi[fid];
-  const float2 nil = P.z[(size_t)i * E1 + s] - lo2(a), nih = P.z[(size_t)i * E1 + s + 1] - lo2(b);
-  const float2 njl = P.z[(size_t)j * E1 + s] - hi2(a), njh = P.z[(size_t)j * E1 + s + 1] - hi2(b);
-  float2 xil, xih, xjl, xjh;
-  const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
-  if (P.noenergy) {
-    int cil, cih, cjl, cjh;
-    end_classes(P, i, s, pin_lo, pin_hi, cil, cih);
-    end_classes(P, j, s, pin_lo, pin_hi, cjl, cjh);
-    coll_minimizer_classes(nil, nih, njl, njh, cil, cih, cjl, cjh, P.radius[i] + P.radius[j],
-                           P.rho, xil, xih, xjl, xjh);
-  } else {
-    coll_minimizer(nil, nih, njl, njh, pin_lo, pin_hi, P.radius[i] + P.radius[j], P.rho,
-                   xil, xih, xjl, xjh);
-  }
-  P.xlo[fid] = pack(xil, xjl);
-  P.xhi[fid] = pack(xih, xjh);
-  if (!pin_lo) {
-    contribute(P, scale, bound, i, s, xil + lo2(a));
-    contribute(P, scale, bound, j, s, xjl + hi2(a));
-  }
-  if (!pin_hi) {
-    contribute(P, scale, bound, i, s + 1, xih + lo2(b));
-    contribute(P, scale, bound, j, s + 1, xjh + hi2(b));
   }
 }
 

@@ -124,3 +124,18 @@ def test_backward_by_graph_and_by_one_cta_match_single_launches(p, eta, K, C):
             assert torch.equal(pl.trajectory(), ref.trajectory())
             for a, b in zip(pl.backward(g), ref.backward(g)):
                 assert torch.allclose(a, b, rtol=1e-5, atol=1e-6 * float(b.abs().max()))
+
+
+@pytest.mark.parametrize("p,eta", [(33, 3), (200, 8), (384, 17)])
+def test_dense_blocks_of_each_size_equal_the_batch(p, eta):
+    """A single plan's blocks of pairs (16, 8 and 4 warps, minimizers run by
+    the block) against the batch's (minimizers from the members' worklists)."""
+    import paper_1311_4527_gb300 as pk
+    inst = workloads.small_square(p, eta, seed=140 + p)
+    for flags in (pk.PLAN_DENSE_STATE, pk.PLAN_U_KEEP, pk.PLAN_ADMM):
+        with pk.Planner.from_instance(inst, flags=flags) as a, pk.PlannerBatch([inst], flags=flags) as b:
+            for n in (1, 2, 9):
+                a.iterate(n)
+                b.iterate(n)
+                assert np.array_equal(a.trajectory().cpu().numpy(), b.trajectory(0).cpu().numpy()), (flags, n)
+            assert a.info()["active_coll"] > 0
