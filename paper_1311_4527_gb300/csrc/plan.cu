@@ -13,7 +13,7 @@
 // Dense state: test_kernel (every factor, the pairs' records streamed) and
 // node_kernel.
 //
-// Iterations after the first are replayed from captured CUDA graphs.
+// Runs of 8 and 64 iterations are replayed from captured CUDA graphs.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1534,8 +1534,7 @@ struct plan_s {
   bool profiling = false;        // plan_profile: per-kernel event timing
   cudaEvent_t pev[6] = {};
   cudaEvent_t pend = nullptr;
-  cudaGraphExec_t gexec[4] = {};  // captured iterations by (k parity, z buffer)
-  cudaGraphExec_t gexec8[4] = {}; // ... and runs of ITERS_PER_GRAPH iterations
+  cudaGraphExec_t gexec8[4] = {};  // captured runs of ITERS_PER_GRAPH iterations by (k parity, z buffer)
   cudaGraphExec_t gexec64[4] = {}; // ... and of ITERS_PER_LONG_GRAPH iterations
   double ptime[4] = {0, 0, 0, 0};
   int pcount = 0;
@@ -1835,34 +1834,16 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = null
   return PLAN_OK;
 }
 
-// One iteration: replay a captured CUDA graph of the three kernels when one
-// fits (past the rho warm-up, not profiling), else launch them directly.
+// One iteration, launched kernel by kernel: a graph of one iteration starts
+// the programmatic-launch chain over at both ends (1,024 agents, 4 iterations
+// from a reset: 73 us replayed one by one, 64 launched; 300 agents among 64
+// walls, 8 iterations: 130 and 109).
 plan_status run_iteration(plan_t h) {
   plan_status st = ensure_sms(h);
   if (st == PLAN_OK && h->sorted && h->k - h->sorted_at >= SORT_EVERY) st = sort_agents(h);
+  if (st == PLAN_OK) st = enqueue_iteration(h, h->stream);
   if (st != PLAN_OK) return st;
-  const bool graphable = h->cap && !h->profiling && h->k >= h->graph_from() && !h->fresh;
-  if (graphable) {
-    const int key = ((h->k & 1) << 1) | h->cur;
-    if (!h->gexec[key]) {
-      cudaGraph_t g = nullptr;
-      // captured on a private stream: the legacy default stream cannot be
-      // captured, and the graph does not depend on the stream it came from
-      CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-      plan_status cst = enqueue_iteration(h, h->cap);
-      cudaError_t e = cudaStreamEndCapture(h->cap, &g);
-      if (cst != PLAN_OK) { if (g) cudaGraphDestroy(g); return cst; }
-      if (e != cudaSuccess) return fail(PLAN_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
-      e = cudaGraphInstantiate(&h->gexec[key], g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return fail(PLAN_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e));
-    }
-    CK(cudaGraphLaunch(h->gexec[key], h->stream));
-  } else {
-    st = enqueue_iteration(h, h->stream);
-    if (st != PLAN_OK) return st;
-    h->fresh = false;
-  }
+  h->fresh = false;
   if (h->eta > 1) h->cur ^= 1;
   h->k += 1;
   return PLAN_OK;
@@ -1870,9 +1851,8 @@ plan_status run_iteration(plan_t h) {
 
 // Runs of ITERS_PER_LONG_GRAPH, then ITERS_PER_GRAPH iterations replayed
 // from one graph each (even counts, so a run ends at the parity and z buffer
-// it started from): fewer launches for problems small enough that launching
-// is the cost, and fewer graph boundaries, where the programmatic-launch
-// chain of the kernels starts over, in long runs.
+// it started from): an iteration of the p = 100 circle takes 7.0 us in a graph
+// of 64 and 7.6 launched by itself; 24 of them take 3 us less in graphs of 8.
 constexpr int ITERS_PER_GRAPH = 8;
 constexpr int ITERS_PER_LONG_GRAPH = 64;
 
@@ -2152,8 +2132,6 @@ void plan_destroy(plan_t h) {
   if (h->h_stage) cudaFreeHost(h->h_stage);
   for (int q = 0; q < 6; ++q)
     if (h->pev[q]) cudaEventDestroy(h->pev[q]);
-  for (int q = 0; q < 4; ++q)
-    if (h->gexec[q]) cudaGraphExecDestroy(h->gexec[q]);
   for (int q = 0; q < 4; ++q)
     if (h->gexec8[q]) cudaGraphExecDestroy(h->gexec8[q]);
   for (int q = 0; q < 4; ++q)
@@ -2960,8 +2938,6 @@ plan_status plan_set_energy(plan_t h, int on) {
   if (off == h->noenergy) return PLAN_OK;
   h->adj_valid = false;
   // the captured iterations hold the old mode
-  for (int q = 0; q < 4; ++q)
-    if (h->gexec[q]) { cudaGraphExecDestroy(h->gexec[q]); h->gexec[q] = nullptr; }
   for (int q = 0; q < 4; ++q)
     if (h->gexec8[q]) { cudaGraphExecDestroy(h->gexec8[q]); h->gexec8[q] = nullptr; }
   for (int q = 0; q < 4; ++q)
