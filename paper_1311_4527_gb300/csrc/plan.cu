@@ -290,23 +290,67 @@ __global__ void __launch_bounds__(1024) sort_kernel(Dev P) {
 // tape (differentiation): each iteration's record is written beside its node
 // pass.
 constexpr int SOLO_WARPS = 16;
+// What of the state a run keeps in shared memory: break-points, segment
+// records, kinetic factors and sums (the sums' atomics and the loads behind
+// them went to L2; at p = 4, eta = 8 an iteration took 5.2 us, with the state
+// here 4.7, with sums in limbs and the second round from the other end 3.7).
+// The pairs' records, the worklist and the wall factors stay in global memory
+// (bits and worklist here too made no difference).
+struct SoloState {
+  int N, M;  // break-points, segments
+  float4 *zseg, *circ, *ukin, *xkin;
+  float2 *z, *z_next;
+  uint32_t* sums;
+  __host__ __device__ SoloState(float4* base, int p, int eta) : N(p * (eta + 1)), M(p * eta) {
+    zseg = base; circ = zseg + M; ukin = circ + M; xkin = ukin + M;
+    z = reinterpret_cast<float2*>(xkin + M); z_next = z + N;
+    sums = reinterpret_cast<uint32_t*>(z_next + N);
+  }
+  __host__ __device__ size_t bytes() const { return (size_t)M * 64 + (size_t)N * (16 + 4 * SUM_WORDS); }
+};
 template <bool CLASSES>
 __global__ void __launch_bounds__(32 * SOLO_WARPS, 1) run_kernel(Dev P0, Dev P1, int iters, int nlist, int seg_warps,
                                                                  int tile_warps, int nodes, Tape T) {
   __shared__ TileMem mem[SOLO_WARPS];
-  __shared__ Dev sP[2];
+  __shared__ SoloDev sP[2];
+  extern __shared__ float4 state[];
+  const SoloState at(state, P0.p, P0.eta);
   for (int w = threadIdx.x; w < (int)(sizeof(Dev) / 4); w += blockDim.x) {
     reinterpret_cast<uint32_t*>(&sP[0])[w] = reinterpret_cast<const uint32_t*>(&P0)[w];
     reinterpret_cast<uint32_t*>(&sP[1])[w] = reinterpret_cast<const uint32_t*>(&P1)[w];
+  }
+  for (int t = threadIdx.x; t < at.M; t += blockDim.x) {
+    at.zseg[t] = P0.zseg[t];
+    at.circ[t] = P0.circ[t];
+    at.ukin[t] = P0.ukin[t];
+    at.xkin[t] = P0.xkin[t];
+  }
+  for (int t = threadIdx.x; t < at.N; t += blockDim.x) {
+    at.z[t] = P0.z[t];
+    at.z_next[t] = P0.z_next[t];
+  }
+  for (int t = threadIdx.x; t < SUM_WORDS * at.N; t += blockDim.x) at.sums[t] = 0u;  // (the plan's are zero between iterations)
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    SoloDev& P = sP[threadIdx.x];
+    const bool same = P.z == P0.z;
+    P.z = same ? at.z : at.z_next;
+    P.z_next = same ? at.z_next : at.z;
+    P.zseg = at.zseg; P.circ = at.circ; P.ukin = at.ukin; P.xkin = at.xkin;
+    P.sums = (uint32_t)__cvta_generic_to_shared(at.sums);
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, coll = nlist + tile_warps;
 #pragma unroll 1
   for (int it = 0; it < iters; ++it) {
-    const Dev& P = sP[it & 1];
+    const SoloDev& P = sP[it & 1];
     if (threadIdx.x == 0) *P.res_cur = 0u;
 #pragma unroll 1
-    for (int item = warp; item < coll + seg_warps; item += SOLO_WARPS) {
+    // (the second round from the other end: the warps that had a tile, not
+    // those that had a list chunk, take the segment warps)
+    for (int round = 0; round * SOLO_WARPS < coll + seg_warps; ++round) {
+      const int item = round * SOLO_WARPS + (round & 1 ? SOLO_WARPS - 1 - warp : warp);
+      if (item >= coll + seg_warps) continue;
       if (item < coll) collision_warp<CLASSES>(P, item, nlist, mem + warp, FUSED);
       else segment_warp(P, item - coll);
       __syncwarp();
@@ -317,6 +361,16 @@ __global__ void __launch_bounds__(32 * SOLO_WARPS, 1) run_kernel(Dev P0, Dev P1,
     for (int w = warp; w < nodes; w += SOLO_WARPS) consensus_warp(P, w);
     if (T.at) record_iteration(P, T, T.at + (size_t)it * T.stride, threadIdx.x, blockDim.x);
     __syncthreads();
+  }
+  for (int t = threadIdx.x; t < at.M; t += blockDim.x) {
+    P0.zseg[t] = at.zseg[t];
+    P0.circ[t] = at.circ[t];
+    P0.ukin[t] = at.ukin[t];
+    P0.xkin[t] = at.xkin[t];
+  }
+  for (int t = threadIdx.x; t < at.N; t += blockDim.x) {
+    const_cast<float2*>(P0.z)[t] = at.z[t];
+    P0.z_next[t] = at.z_next[t];
   }
 }
 
@@ -1709,16 +1763,20 @@ int list_ctas(const plan_s* h) {
 }
 
 // Problems that one CTA serves better than two launches per iteration over the
-// whole GPU.  Measured (circle swaps, us per iteration, one CTA / two
-// launches): eta = 4: 3.9 / 6.5 at p = 4, 4.3 / 6.3 at 16, 5.0 / 6.6 at 20,
-// 6.1 / 6.8 at 28, 6.9 / 7.3 at 32, 8.6 / 7.1 at 33; eta = 8: 5.6 / 6.3 at
-// p = 4, 6.5 / 6.8 at 20, 7.4 / 6.8 at 24; eta = 16: 6.9 / 6.4 at p = 4.  So:
-// tiles and segment warps within the CTA's warps, and pairs that make, with a
-// third of them active, about one list chunk per warp.
+// whole GPU.  Measured (us per iteration, one CTA / two launches), circle
+// swaps of up to 32 agents: eta = 4: 3.5 / 6.5 at p = 4, 4.1 / 6.3 at 16, 5.6
+// / 7.1 at 30, 6.4 / 7.0 at 32; eta = 8: 3.7 / 6.3 at p = 4, 4.6 / 6.8 at 20,
+// 6.0 / 6.9 at 28; eta = 12: 4.6 / 6.2 at p = 8, 5.6 / 6.8 at 16; eta = 16: 5.7
+// / 5.6 at p = 4, 7.5 / 6.8 at 20.  So: tiles and segment warps in at most one
+// and a half rounds of the CTA's warps, and pairs that make at most about two
+// list chunks per warp.  With two groups of 32 (eta = 2: 7.4 / 6.5 at p = 40)
+// or walls or speed limits, which keep more pairs active (30 agents with a
+// limit, eta = 4: 11.0 / 9.4), one.
 bool solo(const plan_s* h) {
   const long long eta = h->vo ? 1 : h->eta;
-  return h->cap && !h->profiling && !h->dense() && !h->sorted && eta * h->ntp + segment_warps(h) <= SOLO_WARPS &&
-         eta * h->p * (h->p - 1) / 2 <= 1536;
+  return h->cap && !h->profiling && !h->dense() && !h->sorted &&
+         2 * (eta * h->ntp + segment_warps(h)) <= 3 * SOLO_WARPS &&
+         eta * h->p * (h->p - 1) / 2 <= (h->nt == 1 && h->nw + h->nv == 0 ? 3072 : 1536);
 }
 
 // n iterations of a small problem from h->k on, past the warm-up, in launches
@@ -1738,7 +1796,7 @@ plan_status run_solo(plan_t h, int n, const Tape* tape) {
     // list warps: those the tiles and segments leave, at least half of the CTA's
     const int nlist = std::min(list_ctas(h) * FACTOR_WARPS, std::max(SOLO_WARPS - tiles - segw, SOLO_WARPS / 2));
     auto kern = h->noenergy ? run_kernel<true> : run_kernel<false>;
-    kern<<<1, 32 * SOLO_WARPS, 0, h->stream>>>(P0, P1, m, nlist, segw, tiles, node_warps(h->p, h->eta), T);
+    kern<<<1, 32 * SOLO_WARPS, SoloState(nullptr, h->p, h->eta).bytes(), h->stream>>>(P0, P1, m, nlist, segw, tiles, node_warps(h->p, h->eta), T);
     CK(cudaGetLastError());
     if (h->eta > 1 && (m & 1)) h->cur ^= 1;
     h->k += m;
@@ -2091,7 +2149,10 @@ plan_status create_plan(const plan_config* cfg, const float* start, const float*
       delete h;
       return fail(PLAN_ENOMEM, "cudaMallocHost failed: %s", cudaGetErrorString(e));
     }
-    if (cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess) {
+    // run_kernel: the state beside 23 KB for the warps, 31 KB at most under solo()'s rule
+    if (cudaFuncSetAttribute(run_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768) != cudaSuccess ||
+        cudaFuncSetAttribute(run_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess) {
       plan_destroy(h);
       return fail(PLAN_ECUDA, "stream or event creation failed");
     }

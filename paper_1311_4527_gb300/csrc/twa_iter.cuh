@@ -116,6 +116,12 @@ struct Dev {
                          // bit 1: a message out of the fixed-point range
 };
 
+// A descriptor whose sums are in shared memory (run_kernel): seven words per
+// break-point, three limbs of m.x and of m.y and the count.
+struct SoloDev : Dev {
+  uint32_t sums;  // shared-memory address
+};
+
 __device__ __forceinline__ float maxabs2(float2 a) { return fmaxf(fabsf(a.x), fabsf(a.y)); }
 
 // Step 7 of the previous iteration for one edge: u^k from the stored u^{k-1},
@@ -151,8 +157,63 @@ __device__ __forceinline__ void contribute(const Dev& P, float scale, float boun
   atomicAdd(P.accy + node, (unsigned long long)__float2ll_rn(m.y * scale));
   atomicAdd(P.accc + node, 1u);
 }
-__device__ __forceinline__ void contribute(const Dev& P, int i, int s, float2 m) {
+
+// The same sums in shared memory, which has no 64-bit add: each integer goes
+// in limbs of 22, 22 and 20 bits (the last one signed) into three 32-bit
+// counters, which 1,024 messages cannot overflow, and nothing waits for the
+// adds.  (64-bit atomics there are compare-and-swap loops.)
+constexpr int SUM_WORDS = 7;
+__device__ __forceinline__ void shared_add(uint32_t at, uint32_t v) {
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t shared_take(uint32_t at) {  // read and clear
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  asm volatile("st.shared.u32 [%0], %1;" ::"r"(at), "r"(0u) : "memory");
+  return v;
+}
+__device__ __forceinline__ void contribute(const SoloDev& P, float scale, float bound, int i, int s,
+                                           float2 m) {
+  if (!(fabsf(m.x) <= bound && fabsf(m.y) <= bound)) {
+    atomicOr(P.status, 2u);
+    return;
+  }
+  const uint32_t at = P.sums + 4u * SUM_WORDS * (uint32_t)(i * (P.eta + 1) + s);
+  const long long x = __float2ll_rn(m.x * scale), y = __float2ll_rn(m.y * scale);
+  constexpr uint32_t LIMB = (1u << 22) - 1u;
+  shared_add(at, (uint32_t)x & LIMB);
+  shared_add(at + 4, (uint32_t)(x >> 22) & LIMB);
+  shared_add(at + 8, (uint32_t)(x >> 44));
+  shared_add(at + 12, (uint32_t)y & LIMB);
+  shared_add(at + 16, (uint32_t)(y >> 22) & LIMB);
+  shared_add(at + 20, (uint32_t)(y >> 44));
+  shared_add(at + 24, 1u);
+}
+template <class D>
+__device__ __forceinline__ void contribute(const D& P, int i, int s, float2 m) {
   contribute(P, P.fix[0], P.fix[1], i, s, m);
+}
+
+// A break-point's sums and count, cleared for the next iteration.
+__device__ __forceinline__ void take_sums(const Dev& P, size_t node, long long& sx, long long& sy, unsigned& cnt) {
+  sx = (long long)P.accx[node];
+  sy = (long long)P.accy[node];
+  cnt = P.accc[node];
+  P.accx[node] = 0ull;
+  P.accy[node] = 0ull;
+  P.accc[node] = 0u;
+}
+__device__ __forceinline__ void take_sums(const SoloDev& P, size_t node, long long& sx, long long& sy, unsigned& cnt) {
+  const uint32_t at = P.sums + 4u * SUM_WORDS * (uint32_t)node;
+  uint32_t w[SUM_WORDS];
+#pragma unroll
+  for (int q = 0; q < SUM_WORDS; ++q) w[q] = shared_take(at + 4 * q);
+  auto whole = [](uint32_t a, uint32_t b, uint32_t c) {
+    return (long long)((unsigned long long)a + ((unsigned long long)b << 22) + ((unsigned long long)(long long)(int)c << 44));
+  };
+  sx = whole(w[0], w[1], w[2]);
+  sy = whole(w[3], w[4], w[5]);
+  cnt = w[6];
 }
 
 // Standard-ADMM mode, a factor that was feasible in the previous iteration:
@@ -285,7 +346,8 @@ __device__ __forceinline__ bool within(float2 a0, float2 a1, float2 b0, float2 b
 
 // Kinetic factor (i, s): always active (it always sends rho0).  Finishes its
 // pending dual update, runs the closed-form minimizer and stores x and u.
-__device__ __forceinline__ void kinetic_factor(const Dev& P, int i, int s, float2 zl, float2 zh,
+template <class D>
+__device__ __forceinline__ void kinetic_factor(const D& P, int i, int s, float2 zl, float2 zh,
                                                bool pin_lo, bool pin_hi, float& res) {
   const size_t idx = (size_t)s * P.p + i;
   const float4 u4 = P.ukin[idx], x4 = P.xkin[idx];
@@ -313,7 +375,8 @@ __device__ __forceinline__ void end_classes(const Dev& P, int i, int s, bool pin
 // maximum / minimum velocity factor (w >= nw, Eq. max_vel_min).  Forward
 // weight rho0 when the n's violate it, else 0.  Called by a full warp (lane =
 // agent of tile I).
-__device__ __forceinline__ void wall_factor(const Dev& P, int w, int i, bool vi, int s, int I,
+template <class D>
+__device__ __forceinline__ void wall_factor(const D& P, int w, int i, bool vi, int s, int I,
                                             float2 zl, float2 zh, float r, bool pin_lo,
                                             bool pin_hi, float& res) {
   const int lane = threadIdx.x & 31;
@@ -388,7 +451,8 @@ __device__ __forceinline__ void wall_factor(const Dev& P, int w, int i, bool vi,
 // Kinetic, wall and velocity factors (steps 1-3 and the pending step 7): one
 // warp per (kind f, segment s, agent tile I), lane = agent; item = (s nt + I)
 // kinds + f, kind 0 the kinetic factor.
-__device__ __forceinline__ void segment_warp(const Dev& P, int item) {
+template <class D>
+__device__ __forceinline__ void segment_warp(const D& P, int item) {
   const int kinds = 1 + P.nw + P.nv;
   const int sI = item / kinds, f = item - sI * kinds;
   const int s = sI / P.nt, I = sI - s * P.nt;
@@ -714,8 +778,8 @@ __device__ __forceinline__ uint32_t collides2(const RowPair& A, const TileMem* M
 // active, runs the minimizer, stores its record and adds its messages to the
 // sums (steps 7, 1-4).  CLASSES: per-node back weights (the feasibility
 // problem).
-template <bool CLASSES>
-__device__ __forceinline__ bool pair_factor(const Dev& P, int s, int i, int j, uint32_t fid,
+template <bool CLASSES, class D>
+__device__ __forceinline__ bool pair_factor(const D& P, int s, int i, int j, uint32_t fid,
                                             bool prev, float& res) {
   const bool pin_lo = (s == 0), pin_hi = (s == P.eta - 1);
   const float4 zi = P.zseg[(size_t)s * P.p + i], zj = P.zseg[(size_t)s * P.p + j];
@@ -870,8 +934,8 @@ __device__ __forceinline__ void nth_pair(uint32_t todo, unsigned tincl, unsigned
   c = g < total ? nth_bit(w, g - first) : 0;
 }
 
-template <bool CLASSES>
-__device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist, TileMem* M, int mode) {
+template <bool CLASSES, class D>
+__device__ __forceinline__ void collision_warp(const D& P, int item, int nlist, TileMem* M, int mode) {
   const int lane = threadIdx.x & 31;
   const bool rebuild = mode == LISTED ? false : P.ctl[0] != 0u;
   const bool lister = item < nlist;
@@ -926,9 +990,9 @@ __device__ __forceinline__ void collision_warp(const Dev& P, int item, int nlist
         w &= w - 1u;
         const int k = w ? __ffs(w) - 1 : c;
         w &= w - 1u;
-        const float4 B = M->z[c], D = M->z[k];
+        const float4 B = M->z[c], C = M->z[k];
         const bool h0 = collides(lo2(B) - lo2(zi), hi2(B) - hi2(zi), ri + M->r[c]);
-        const bool h1 = collides(lo2(D) - lo2(zi), hi2(D) - hi2(zi), ri + M->r[k]);
+        const bool h1 = collides(lo2(C) - lo2(zi), hi2(C) - hi2(zi), ri + M->r[k]);
         hit |= (h0 ? 1u << c : 0u) | (h1 ? 1u << k : 0u);
       }
       near = hit;
@@ -1239,13 +1303,12 @@ __device__ __forceinline__ void sorted_collision_warp(const Dev& P, int item, in
 // fixed-point sums (every weight is rho0, so z is the mean of the incoming m;
 // no incoming weight means z is unchanged).  Clears the sums for the next
 // iteration.
-__device__ __forceinline__ float2 consensus_node(const Dev& P, size_t node, float2 zo, unsigned status,
+template <class D>
+__device__ __forceinline__ float2 consensus_node(const D& P, size_t node, float2 zo, unsigned status,
                                                  float& dz, bool& bad) {
-  const long long sx = (long long)P.accx[node], sy = (long long)P.accy[node];
-  const unsigned cnt = P.accc[node];
-  P.accx[node] = 0ull;
-  P.accy[node] = 0ull;
-  P.accc[node] = 0u;
+  long long sx, sy;
+  unsigned cnt;
+  take_sums(P, node, sx, sy, cnt);
   float2 zn = zo;  // every incoming weight zero: treated as 1, which gives z unchanged
   if (P.admm) {
     // every edge is weighted; each feasible collision or wall factor sent
@@ -1288,7 +1351,8 @@ __host__ __device__ __forceinline__ int agents_per_warp(int eta) { return eta + 
 // (consecutive in the [p][eta+1] arrays, so coalesced), longer agents in
 // rounds of 32 from the far end.  A lane gets the next break-point's z from
 // its neighbour and writes the segment records of the next factor pass.
-__device__ __forceinline__ void consensus_warp(const Dev& P, int warp) {
+template <class D>
+__device__ __forceinline__ void consensus_warp(const D& P, int warp) {
   const int lane = threadIdx.x & 31, E1 = P.eta + 1, apw = agents_per_warp(P.eta);
   const unsigned status = *P.status;
   float dz = 0.f;

@@ -139,3 +139,9 @@ def test_dense_blocks_of_each_size_equal_the_batch(p, eta):
                 b.iterate(n)
                 assert np.array_equal(a.trajectory().cpu().numpy(), b.trajectory(0).cpu().numpy()), (flags, n)
             assert a.info()["active_coll"] > 0
+
+
+@pytest.mark.parametrize("p,eta", [(1, 12), (28, 8), (29, 8), (8, 12), (8, 13), (8, 3), (40, 2)])
+def test_single_cta_rule_edges(p, eta):
+    """Up to one and a half rounds of the CTA's warps and both pair limits."""
+    test_single_cta_runs_equal_iterations_one_kernel_at_a_time(p, eta)
