@@ -114,13 +114,17 @@ __device__ __forceinline__ unsigned long long dealt_first(unsigned long long& st
 // (both counts zeroed before).
 struct Tape {
   char* at;  // the iteration's slot (null: nothing is recorded)
-  size_t stride, z, ukin, count, fid, ucl, uch, scount, sidx, su;
+  size_t stride, z, inv, ukin, count, fid, ucl, uch, scount, sidx, su;
+  int *last, *slast;  // by pair slot and by segment factor: the iteration it was recorded in last
+  const int* k0;      // the slot's iteration is *k0 + q
+  int q;
   int from_list;  // the worklist holds every active pair (it cannot run out): else from the bits
 };
 
 // Records the iteration of descriptor P after its factor pass; threads t0, t0
 // + nt, ... (whole warps).
-__device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, char* slot, unsigned t0, unsigned nt) {
+__device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, char* slot, int q, unsigned t0, unsigned nt) {
+  const int k = *T.k0 + q;
   float2* tz = reinterpret_cast<float2*>(slot + T.z);
   float4* tukin = reinterpret_cast<float4*>(slot + T.ukin);
   uint32_t* tfid = reinterpret_cast<uint32_t*>(slot + T.fid);
@@ -159,7 +163,8 @@ __device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, ch
       at = __shfl_sync(FULL, at, 31) + (incl - cnt);
       for (uint32_t w = word; w; w &= w - 1u, ++at) {
         const uint32_t f = first + (uint32_t)(__ffs(w) - 1);
-        tfid[at] = f;
+        tfid[at] = f | (T.last[f] == k - 1 ? WAS_ACTIVE : 0u);
+        T.last[f] = k;
         tucl[at] = P.ulo[f];
         tuch[at] = P.uhi[f];
       }
@@ -168,7 +173,8 @@ __device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, ch
       const unsigned i = t % P.p, ws = t / P.p;
       if ((P.wbits[(size_t)ws * P.nt + i / TILE] >> (i % TILE)) & 1u) {
         const unsigned at = atomicAdd(tscount, 1u);
-        tsidx[at] = t;
+        tsidx[at] = t | (T.slast[t] == k - 1 ? WAS_ACTIVE : 0u);
+        T.slast[t] = k;
         tsu[at] = P.uwall[t];
       }
     }
@@ -177,7 +183,8 @@ __device__ __forceinline__ void record_iteration(const Dev& P, const Tape& T, ch
 
 // Node pass.
 constexpr int NODE_WARPS = 2;
-__device__ __forceinline__ void node_pass(const Dev& P) {
+template <class D>
+__device__ __forceinline__ void node_pass(const D& P) {
   const int warp = (int)blockIdx.x * NODE_WARPS + (threadIdx.x >> 5);
   if (blockIdx.x == 0 && threadIdx.x == 0) advance_worklist(P, false);
   consensus_warp(P, warp);
@@ -189,10 +196,10 @@ __global__ void __launch_bounds__(32 * NODE_WARPS) node_kernel(Dev P) {
 // The node pass beside the record of the iteration (the CTAs past node_ctas),
 // which like it needs the factor pass only.  A kernel of its own: the tape's
 // parameters cost the plain pass 0.1 us of each iteration.
-__global__ void __launch_bounds__(32 * NODE_WARPS) node_record_kernel(Dev P, Tape T, int node_ctas) {
+__global__ void __launch_bounds__(32 * NODE_WARPS) node_record_kernel(Taped<Dev> P, Tape T, int node_ctas) {
   pdl_begin();
   if ((int)blockIdx.x < node_ctas) node_pass(P);
-  else record_iteration(P, T, T.at, (blockIdx.x - node_ctas) * blockDim.x + threadIdx.x, (gridDim.x - node_ctas) * blockDim.x);
+  else record_iteration(P, T, T.at, T.q, (blockIdx.x - node_ctas) * blockDim.x + threadIdx.x, (gridDim.x - node_ctas) * blockDim.x);
 }
 
 // The segment records of the factor pass after z, a fixed end or a radius was
@@ -308,11 +315,12 @@ struct SoloState {
   }
   __host__ __device__ size_t bytes() const { return (size_t)M * 64 + (size_t)N * (16 + 4 * SUM_WORDS); }
 };
-template <bool CLASSES>
+template <bool CLASSES, bool TAPE>
 __global__ void __launch_bounds__(32 * SOLO_WARPS, 1) run_kernel(Dev P0, Dev P1, int iters, int nlist, int seg_warps,
                                                                  int tile_warps, int nodes, Tape T) {
   __shared__ TileMem mem[SOLO_WARPS];
-  __shared__ SoloDev sP[2];
+  using Local = std::conditional_t<TAPE, Taped<SoloDev>, SoloDev>;
+  __shared__ Local sP[2];
   extern __shared__ float4 state[];
   const SoloState at(state, P0.p, P0.eta);
   for (int w = threadIdx.x; w < (int)(sizeof(Dev) / 4); w += blockDim.x) {
@@ -332,7 +340,7 @@ __global__ void __launch_bounds__(32 * SOLO_WARPS, 1) run_kernel(Dev P0, Dev P1,
   for (int t = threadIdx.x; t < SUM_WORDS * at.N; t += blockDim.x) at.sums[t] = 0u;  // (the plan's are zero between iterations)
   __syncthreads();
   if (threadIdx.x < 2) {
-    SoloDev& P = sP[threadIdx.x];
+    Local& P = sP[threadIdx.x];
     const bool same = P.z == P0.z;
     P.z = same ? at.z : at.z_next;
     P.z_next = same ? at.z_next : at.z;
@@ -343,8 +351,11 @@ __global__ void __launch_bounds__(32 * SOLO_WARPS, 1) run_kernel(Dev P0, Dev P1,
   const int warp = threadIdx.x >> 5, coll = nlist + tile_warps;
 #pragma unroll 1
   for (int it = 0; it < iters; ++it) {
-    const SoloDev& P = sP[it & 1];
-    if (threadIdx.x == 0) *P.res_cur = 0u;
+    const Local& P = sP[it & 1];
+    if (threadIdx.x == 0) {
+      *P.res_cur = 0u;
+      if constexpr (TAPE) sP[it & 1].inv = reinterpret_cast<double*>(T.at + (size_t)it * T.stride + T.inv);
+    }
 #pragma unroll 1
     // (the second round from the other end: the warps that had a tile, not
     // those that had a list chunk, take the segment warps)
@@ -359,7 +370,7 @@ __global__ void __launch_bounds__(32 * SOLO_WARPS, 1) run_kernel(Dev P0, Dev P1,
     if (threadIdx.x == 32 * (SOLO_WARPS - 1)) advance_worklist(P, false);
 #pragma unroll 1
     for (int w = warp; w < nodes; w += SOLO_WARPS) consensus_warp(P, w);
-    if (T.at) record_iteration(P, T, T.at + (size_t)it * T.stride, threadIdx.x, blockDim.x);
+    if (TAPE) record_iteration(P, T, T.at + (size_t)it * T.stride, T.q + it, threadIdx.x, blockDim.x);
     __syncthreads();
   }
   for (int t = threadIdx.x; t < at.M; t += blockDim.x) {
@@ -1570,7 +1581,8 @@ plan_status check_endpoints(int p, const float* start, const float* goal, const 
 // A captured segment of the backward pass and what it was captured for.
 struct SegmentGraph {
   int n, parity, cur;
-  bool first, zb;
+  bool first;
+  int phase;
   cudaGraphExec_t exec;
 };
 
@@ -1820,7 +1832,7 @@ plan_status run_solo(plan_t h, int n, const Tape* tape) {
     const int segw = segment_warps(h), tiles = (h->vo ? 1 : h->eta) * h->ntp;
     // list warps: those the tiles and segments leave, at least half of the CTA's
     const int nlist = std::min(list_ctas(h) * FACTOR_WARPS, std::max(SOLO_WARPS - tiles - segw, SOLO_WARPS / 2));
-    auto kern = h->noenergy ? run_kernel<true> : run_kernel<false>;
+    auto kern = tape ? run_kernel<false, true> : h->noenergy ? run_kernel<true, false> : run_kernel<false, false>;
     kern<<<1, 32 * SOLO_WARPS, SoloState(nullptr, h->p, h->eta).bytes(), h->stream>>>(P0, P1, m, nlist, segw, tiles, node_warps(h->p, h->eta), T);
     CK(cudaGetLastError());
     if (h->eta > 1 && (m & 1)) h->cur ^= 1;
@@ -1898,9 +1910,12 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = null
   // the node pass also sets up the next iteration's worklist, so it runs even
   // when there is no free break-point (eta = 1)
   const int node_ctas = (node_warps(h->p, h->eta) + NODE_WARPS - 1) / NODE_WARPS;
-  if (tape)
-    CK(launch_pdl(node_record_kernel, (unsigned)(node_ctas + record_ctas(h)), 32u * NODE_WARPS, ms, P, *tape, node_ctas));
-  else
+  if (tape) {
+    Taped<Dev> N;
+    static_cast<Dev&>(N) = P;
+    N.inv = reinterpret_cast<double*>(tape->at + tape->inv);
+    CK(launch_pdl(node_record_kernel, (unsigned)(node_ctas + record_ctas(h)), 32u * NODE_WARPS, ms, N, *tape, node_ctas));
+  } else
     CK(launch_pdl(node_kernel, (unsigned)node_ctas, 32u * NODE_WARPS, ms, P));
   if (prof) {
     CK(cudaEventRecord(h->pend, ms));
@@ -2175,8 +2190,9 @@ plan_status create_plan(const plan_config* cfg, const float* start, const float*
       return fail(PLAN_ENOMEM, "cudaMallocHost failed: %s", cudaGetErrorString(e));
     }
     // run_kernel: the state beside 23 KB for the warps, 31 KB at most under solo()'s rule
-    if (cudaFuncSetAttribute(run_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768) != cudaSuccess ||
-        cudaFuncSetAttribute(run_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768) != cudaSuccess ||
+    auto allow = [](auto kern) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768); };
+    if (allow(run_kernel<false, false>) != cudaSuccess || allow(run_kernel<true, false>) != cudaSuccess ||
+        allow(run_kernel<false, true>) != cudaSuccess ||
         cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess) {
       plan_destroy(h);
       return fail(PLAN_ECUDA, "stream or event creation failed");
@@ -2575,23 +2591,23 @@ __global__ void begin_segment_kernel(char* a, char* b, size_t stride, int n, int
 __global__ void __launch_bounds__(128) bw_scatter_kernel(AdjDev A) {
   pdl_begin();
   A.k += *A.k0;
-  const unsigned n = (unsigned)(A.eta * A.p) + *A.count + *A.scount;
+  const unsigned n = *A.count + *A.scount;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
     bw_scatter_item(A, t);
 }
 
-__global__ void bw_node_kernel(AdjDev A) {
-  pdl_begin();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < A.p * (A.eta + 1)) bw_node(A, t);
-}
-
-__global__ void __launch_bounds__(128) bw_factor_kernel(AdjDev A) {
+// One adjoint step.  Bound by its chain (entry, records, minimizer adjoint,
+// FP64 atomics).  With the u adjoints' sums and the nodes in launches of their
+// own an iteration of the backward pass took 3.3 us more (p = 64, eta = 8,
+// 128 iterations: 4.05 ms the whole gradient, now 3.63).
+__global__ void __launch_bounds__(128) bw_step_kernel(AdjDev A) {
   pdl_begin();
   A.k += *A.k0;
-  const unsigned n = (unsigned)(A.eta * A.p) + *A.count + *A.scount;
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
-    bw_factor_item(A, t);
+  const unsigned nodes = (unsigned)(A.p * (A.eta + 1)), n = nodes + bw_factors(A);
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    if (t < nodes) bw_node(A, (int)t);
+    else bw_factor_item<false>(A, t - nodes);
+  }
 }
 
 // A small problem's adjoint steps of a whole segment, last iteration first, by
@@ -2602,21 +2618,27 @@ __global__ void __launch_bounds__(32 * SOLO_WARPS, 1) bw_run_kernel(AdjDev A, in
   auto back = [&](auto*& p) {
     p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(reinterpret_cast<const char*>(p) - stride);
   };
+  const unsigned gated = *A.count + *A.scount;
+  for (unsigned t = threadIdx.x; t < gated; t += blockDim.x) bw_scatter_item(A, t);
+  __syncthreads();
 #pragma unroll 1
   for (int it = 0; it < iters; ++it) {
-    const unsigned n = (unsigned)(A.eta * A.p) + *A.count + *A.scount, nodes = (unsigned)(A.p * (A.eta + 1));
-    for (unsigned t = threadIdx.x; t < n; t += blockDim.x) bw_scatter_item(A, t);
+    // (mbar from a pass over the nodes: one SM has too few FP64 units to form
+    // it at every edge, 5 % of the whole gradient at p = 20, eta = 8)
+    const unsigned n = bw_factors(A), nodes = (unsigned)(A.p * (A.eta + 1));
+    for (unsigned t = threadIdx.x; t < nodes; t += blockDim.x) {
+      A.mbar[t] = node_mbar(A, t);  // (not used at the fixed ends)
+      bw_node(A, (int)t);
+    }
     __syncthreads();
-    for (unsigned t = threadIdx.x; t < nodes; t += blockDim.x) bw_node(A, (int)t);
-    __syncthreads();
-    for (unsigned t = threadIdx.x; t < n; t += blockDim.x) bw_factor_item(A, t);
+    for (unsigned t = threadIdx.x; t < n; t += blockDim.x) bw_factor_item<true>(A, t);
     __syncthreads();
     A.k -= 1;
-    double2* in = const_cast<double2*>(A.zb_in);
-    A.zb_in = A.zb_out;
-    A.zb_out = in;
+    double2 *zb = const_cast<double2*>(A.zb_in), *S = const_cast<double2*>(A.S_in);
+    A.zb_in = A.zb_out; A.zb_out = A.zb_clear; A.zb_clear = zb;
+    A.S_in = A.S_out; A.S_out = A.S_clear; A.S_clear = S;
     if (it + 1 < iters) {  // the tape slot of the iteration before
-      back(A.z); back(A.ukin); back(A.fid); back(A.ucl); back(A.uch); back(A.count); back(A.sidx); back(A.su);
+      back(A.z); back(A.inv); back(A.ukin); back(A.fid); back(A.ucl); back(A.uch); back(A.count); back(A.sidx); back(A.su);
       back(A.scount);
     }
   }
@@ -2675,9 +2697,9 @@ struct AdjLayout {
   size_t ck_bytes, ck0;
   int nck;
   size_t cap, slot_bytes, tape0;
-  size_t t_z, t_ukin, t_count, t_fid, t_ucl, t_uch;  // within one tape slot
+  size_t t_z, t_inv, t_ukin, t_count, t_fid, t_ucl, t_uch;  // within one tape slot
   size_t t_scount, t_sidx, t_su, scap;
-  size_t ubk, ubl, ubh, stamp, ubs, sstamp, zbA, zbB, S, cnt, mbar, gs, gg, gr, gc, k0;
+  size_t ubk, ubl, ubh, stamp, last, ubs, sstamp, slast, zb, S, node3, mbar, gs, gg, gr, gc, k0;
   size_t total;
 };
 
@@ -2691,6 +2713,7 @@ AdjLayout adj_layout(plan_t h, int K, int C) {
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o = a256(o + std::max<size_t>(bytes, 1)); return at; };
   A.t_z = take(p * E1 * 8);
+  A.t_inv = take(p * E1 * 8);
   A.t_ukin = take(eta * p * 16);
   A.t_count = take(4);
   A.t_fid = take(A.cap * 4);
@@ -2708,12 +2731,13 @@ AdjLayout adj_layout(plan_t h, int K, int C) {
   A.ubl = take(h->slots * 16);
   A.ubh = take(h->slots * 16);
   A.stamp = take(h->slots * 4);
+  A.last = take(h->slots * 4);
   A.ubs = take(A.scap * 16);
   A.sstamp = take(A.scap * 4);
-  A.zbA = take(p * E1 * 16);
-  A.zbB = take(p * E1 * 16);
-  A.S = take(p * E1 * 16);
-  A.cnt = take(p * E1 * 4);
+  A.slast = take(A.scap * 4);
+  A.node3 = a256(p * E1 * 16);  // three buffers each
+  A.zb = take(3 * A.node3);
+  A.S = take(3 * A.node3);
   A.mbar = take(p * E1 * 8);
   A.gs = take(p * 16);
   A.gg = take(p * 16);
@@ -2765,13 +2789,14 @@ plan_status snapshot(plan_t h, const AdjLayout& A, int idx, bool save) {
 }
 
 Tape adj_tape(plan_t h, const AdjLayout& A) {
-  return {h->adj + A.tape0, A.slot_bytes, A.t_z, A.t_ukin, A.t_count, A.t_fid, A.t_ucl, A.t_uch, A.t_scount, A.t_sidx,
-          A.t_su, !h->dense() && lists_every_pair(h) ? 1 : 0};
+  return {h->adj + A.tape0, A.slot_bytes, A.t_z, A.t_inv, A.t_ukin, A.t_count, A.t_fid, A.t_ucl, A.t_uch, A.t_scount,
+          A.t_sidx, A.t_su, reinterpret_cast<int*>(h->adj + A.last), reinterpret_cast<int*>(h->adj + A.slast),
+          reinterpret_cast<const int*>(h->adj + A.k0), 0, !h->dense() && lists_every_pair(h) ? 1 : 0};
 }
 
 // Adjoint of the iteration `slot` of a segment (iterations count from the
 // segment's first, AdjDev::k0).
-AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, char* zb_in, char* zb_out) {
+AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, int phase) {
   AdjDev D{};
   D.p = h->p; D.eta = h->eta; D.ntp = h->ntp; D.k = slot;
   D.rho = h->cfg.rho0;
@@ -2785,6 +2810,7 @@ AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, char* zb_in, char* zb_out
   D.vlim = h->at<float>(h->L.vlim);
   char* t = h->adj + A.tape0 + (size_t)slot * A.slot_bytes;
   D.z = reinterpret_cast<const float2*>(t + A.t_z);
+  D.inv = reinterpret_cast<const double*>(t + A.t_inv);
   D.ukin = reinterpret_cast<const float4*>(t + A.t_ukin);
   D.count = reinterpret_cast<const unsigned*>(t + A.t_count);
   D.fid = reinterpret_cast<const uint32_t*>(t + A.t_fid);
@@ -2800,11 +2826,12 @@ AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, char* zb_in, char* zb_out
   D.ubh = reinterpret_cast<float4*>(h->adj + A.ubh);
   D.stamp = reinterpret_cast<int*>(h->adj + A.stamp);
   D.k0 = reinterpret_cast<const int*>(h->adj + A.k0);
-  D.zb_in = reinterpret_cast<const double2*>(zb_in);
-  D.zb_out = reinterpret_cast<double2*>(zb_out);
-  D.S = reinterpret_cast<double2*>(h->adj + A.S);
-  D.cnt = reinterpret_cast<unsigned*>(h->adj + A.cnt);
+  auto buffer = [&](size_t at, int turn) {
+    return reinterpret_cast<double2*>(h->adj + at + (size_t)((phase + turn) % 3) * A.node3);
+  };
+  D.zb_in = buffer(A.zb, 0); D.zb_out = buffer(A.zb, 1); D.zb_clear = buffer(A.zb, 2);
   D.mbar = reinterpret_cast<float2*>(h->adj + A.mbar);
+  D.S_in = buffer(A.S, 0); D.S_out = buffer(A.S, 1); D.S_clear = buffer(A.S, 2);
   D.g_start = reinterpret_cast<double2*>(h->adj + A.gs);
   D.g_goal = reinterpret_cast<double2*>(h->adj + A.gg);
   D.g_r = reinterpret_cast<double*>(h->adj + A.gr);
@@ -2815,7 +2842,7 @@ AdjDev adj_dev(plan_t h, const AdjLayout& A, int slot, char* zb_in, char* zb_out
 // One segment of the backward pass on the given stream: n iterations from h->k
 // recorded, then their adjoint steps, last iteration first (no state change
 // on the host).
-plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, char* zb_in, char* zb_out, cudaStream_t ms) {
+plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, int phase, cudaStream_t ms) {
   const int k0 = h->k, c0 = h->cur;
   const bool fresh = h->fresh;
   Tape T = adj_tape(h, A);
@@ -2824,6 +2851,7 @@ plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, char* zb_in, ch
   for (int q = 0; q < n && st == PLAN_OK && e == cudaSuccess; ++q) {
     st = enqueue_iteration(h, ms, &T);
     T.at += T.stride;
+    T.q += 1;
     h->fresh = false;
     if (h->eta > 1) h->cur ^= 1;
     h->k += 1;
@@ -2831,29 +2859,24 @@ plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, char* zb_in, ch
   h->k = k0;
   h->cur = c0;
   h->fresh = fresh;
-  const unsigned node_grid = (unsigned)((h->p * (h->eta + 1) + 255) / 256);
-  // a thread per edge group that may be active (more CTAs than that only cost their launch)
-  const long long items = (long long)(1 + h->nw + h->nv) * h->eta * h->p + (long long)h->eta * h->p * (h->p - 1) / 2;
+  // a thread per break-point and edge group that may be active (more CTAs than that only cost their launch)
+  const long long items = (long long)(2 + h->nw + h->nv) * h->eta * h->p + h->p + (long long)h->eta * h->p * (h->p - 1) / 2;
   const unsigned grid = (unsigned)std::min<long long>((items + 127) / 128, 6ll * h->sms);
-  for (int q = n - 1; q >= 0 && st == PLAN_OK && e == cudaSuccess; --q) {
-    const AdjDev D = adj_dev(h, A, q, zb_in, zb_out);
-    e = launch_pdl(bw_scatter_kernel, grid, 128u, ms, D);
-    if (e == cudaSuccess) e = launch_pdl(bw_node_kernel, node_grid, 256u, ms, D);
-    if (e == cudaSuccess) e = launch_pdl(bw_factor_kernel, grid, 128u, ms, D);
-    std::swap(zb_in, zb_out);
-  }
+  if (st == PLAN_OK && e == cudaSuccess) e = launch_pdl(bw_scatter_kernel, grid, 128u, ms, adj_dev(h, A, n - 1, phase));
+  for (int q = n - 1; q >= 0 && st == PLAN_OK && e == cudaSuccess; --q)
+    e = launch_pdl(bw_step_kernel, grid, 128u, ms, adj_dev(h, A, q, phase + n - 1 - q));
   if (st == PLAN_OK && e != cudaSuccess) st = fail(PLAN_ECUDA, "adjoint launch failed: %s", cudaGetErrorString(e));
   return st;
 }
 
 // The same, run: by one CTA for a small problem; else replayed from a graph,
-// kept with the plan (six launches an iteration, each about 6 us of host time
+// kept with the plan (six launches an iteration then, each about 6 us of host time
 // when made one by one, bound the backward pass at any size: 34 us an
 // iteration at p = 64).  Segments differ in their length, in the parity and z
 // buffer of their first iteration, in where the adjoint of z stands, and
 // iteration 0 has no residual slot before it; the rest is the same for all of
 // them, the iteration number coming from AdjDev::k0.
-plan_status segment_steps(plan_t h, const AdjLayout& A, int n, char* zb_in, char* zb_out) {
+plan_status segment_steps(plan_t h, const AdjLayout& A, int n, int phase) {
   plan_status st = ensure_sms(h);
   if (st != PLAN_OK) return st;
   if (solo(h)) {
@@ -2862,27 +2885,28 @@ plan_status segment_steps(plan_t h, const AdjLayout& A, int n, char* zb_in, char
     while (h->k < end && (h->fresh || h->k < h->graph_from())) {  // the first one has no worklist yet
       if ((st = enqueue_iteration(h, h->stream, &T)) != PLAN_OK) return st;
       T.at += T.stride;
+      T.q += 1;
       h->fresh = false;
       if (h->eta > 1) h->cur ^= 1;
       h->k += 1;
     }
     if (h->k < end && (st = run_solo(h, end - h->k, &T)) != PLAN_OK) return st;
-    bw_run_kernel<<<1, 32 * SOLO_WARPS, 0, h->stream>>>(adj_dev(h, A, n - 1, zb_in, zb_out), n, A.slot_bytes);
+    bw_run_kernel<<<1, 32 * SOLO_WARPS, 0, h->stream>>>(adj_dev(h, A, n - 1, phase), n, A.slot_bytes);
     CK(cudaGetLastError());
     return PLAN_OK;
   }
   if (h->profiling) {  // each kernel is timed on its own: launched one by one
-    if ((st = enqueue_segment(h, A, n, zb_in, zb_out, h->stream)) != PLAN_OK) return st;
+    if ((st = enqueue_segment(h, A, n, phase, h->stream)) != PLAN_OK) return st;
   } else {
-    const SegmentGraph key = {n, h->k & 1, h->cur, h->k == 0, zb_in == h->adj + A.zbA, nullptr};
+    const SegmentGraph key = {n, h->k & 1, h->cur, h->k == 0, phase, nullptr};
     const SegmentGraph* found = nullptr;
     for (const SegmentGraph& g : h->adj_graphs)
-      if (g.n == key.n && g.parity == key.parity && g.cur == key.cur && g.first == key.first && g.zb == key.zb) found = &g;
+      if (g.n == key.n && g.parity == key.parity && g.cur == key.cur && g.first == key.first && g.phase == key.phase) found = &g;
     if (!found) {
-      if (h->adj_graphs.size() >= 8) drop_segment_graphs(h);
+      if (h->adj_graphs.size() >= 12) drop_segment_graphs(h);
       cudaGraph_t g = nullptr;
       CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-      st = enqueue_segment(h, A, n, zb_in, zb_out, h->cap);
+      st = enqueue_segment(h, A, n, phase, h->cap);
       cudaError_t e = cudaStreamEndCapture(h->cap, &g);
       SegmentGraph made = key;
       if (st == PLAN_OK && e == cudaSuccess) e = cudaGraphInstantiate(&made.exec, g, 0);
@@ -3161,14 +3185,14 @@ plan_status plan_backward(plan_t h, int K, const float* dL_dz, float* d_start, f
   CK(cudaMemsetAsync(h->adj + A.ubk, 0, (size_t)h->eta * p * 16, h->stream));
   CK(cudaMemsetAsync(h->adj + A.stamp, 0xff, h->slots * 4, h->stream));
   CK(cudaMemsetAsync(h->adj + A.sstamp, 0xff, A.scap * 4, h->stream));
-  CK(cudaMemsetAsync(h->adj + A.S, 0, nodes * 16, h->stream));
-  CK(cudaMemsetAsync(h->adj + A.cnt, 0, nodes * 4, h->stream));
+  CK(cudaMemsetAsync(h->adj + A.last, 0x80, h->slots * 4, h->stream));  // (no iteration's number)
+  CK(cudaMemsetAsync(h->adj + A.slast, 0x80, A.scap * 4, h->stream));
+  CK(cudaMemsetAsync(h->adj + A.zb, 0, A.S + 3 * A.node3 - A.zb, h->stream));
   CK(cudaMemsetAsync(h->adj + A.gs, 0, A.gc + p * h->eta * 8 - A.gs, h->stream));
   bw_init_kernel<<<(unsigned)((nodes + 255) / 256), 256, 0, h->stream>>>(
-      (int)nodes, reinterpret_cast<const float2*>(dL_dz), reinterpret_cast<double2*>(h->adj + A.zbA));
+      (int)nodes, reinterpret_cast<const float2*>(dL_dz), reinterpret_cast<double2*>(h->adj + A.zb));
   CK(cudaGetLastError());
-  char* zb_in = h->adj + A.zbA;
-  char* zb_out = h->adj + A.zbB;
+  int phase = 0;  // which of the three buffers is read
   const int nseg = A.nck - 1;
   for (int seg = nseg - 1; seg >= 0; --seg) {
     const int c0 = seg * C, n = std::min(K, c0 + C) - c0;
@@ -3180,13 +3204,13 @@ plan_status plan_backward(plan_t h, int K, const float* dL_dz, float* d_start, f
     begin_segment_kernel<<<1, 64, 0, h->stream>>>(h->adj + A.tape0 + A.t_count, h->adj + A.tape0 + A.t_scount,
                                                   A.slot_bytes, n, reinterpret_cast<int*>(h->adj + A.k0), c0);
     CK(cudaGetLastError());
-    if ((st = segment_steps(h, A, n, zb_in, zb_out)) != PLAN_OK) return st;
-    if (n & 1) std::swap(zb_in, zb_out);
+    if ((st = segment_steps(h, A, n, phase)) != PLAN_OK) return st;
+    phase = (phase + n) % 3;
   }
-  const AdjDev D = adj_dev(h, A, 0, zb_in, zb_out);
+  const AdjDev D = adj_dev(h, A, 0, phase);
   const double norm = (h->cfg.flags & (PLAN_COST_UNNORM | PLAN_VO)) ? 1.0 : 1.0 / ((double)p * h->eta);
   bw_final_kernel<<<(unsigned)((p + 127) / 128), 128, 0, h->stream>>>(
-      D, reinterpret_cast<const double2*>(zb_in), norm, (h->cfg.flags & PLAN_COST_PER_SEGMENT) ? 1 : 0,
+      D, D.zb_in, norm, (h->cfg.flags & PLAN_COST_PER_SEGMENT) ? 1 : 0,
       reinterpret_cast<float2*>(d_start), reinterpret_cast<float2*>(d_goal), d_radius, d_cost_w);
   CK(cudaGetLastError());
   // leave the plan at iteration K, as plan_unroll did

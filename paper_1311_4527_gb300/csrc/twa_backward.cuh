@@ -8,9 +8,14 @@
 //   z^{k+1}_v = (1 / c_v) sum over the c_v active edges e at v of (x_e + u^k_e)
 //   u^{k+1}_e = u^k_e + alpha (x_e - z^{k+1}_v) on active edges at free nodes.
 // Given zbar = dL/dz^{k+1} and ubar = dL/du^{k+1}, the adjoint step is
-//   zhat_v = zbar_v - alpha sum_e ubar_e,   mbar_v = zhat_v / c_v   (pass 1, 2)
-//   xbar_e = mbar_v + alpha ubar_e,          nbar = (dg/dn)^T xbar   (pass 3)
+//   zhat_v = zbar_v - alpha sum_e ubar_e,   mbar_v = zhat_v / c_v
+//   xbar_e = mbar_v + alpha ubar_e,          nbar = (dg/dn)^T xbar
 //   dL/dz^k_v = sum_e nbar_e,   dL/du^k_e = ubar_e + mbar_v - nbar_e.
+// One pass over the factors per iteration: whoever computes dL/du^k of an edge
+// adds alpha times it to the sum that iteration k - 1 will read, if the edge
+// was active in that one too (a flag of the tape; the kinetic edges always
+// are), and mbar is formed where it is read, from the counts on the tape.  The
+// sums and the adjoint of z go through three buffers: read, added to, cleared.
 // At fixed nodes z is the start or goal, x is unused and u stays 0.  A
 // collision edge's u^{k+1} matters only if the factor is active in both k and
 // k+1 (else it is reset or unused), so its adjoint is kept with the iteration
@@ -23,6 +28,9 @@
 #include "twa_iter.cuh"
 
 namespace {
+
+// Flag of a tape entry: the factor was active in the iteration before too.
+constexpr uint32_t WAS_ACTIVE = 0x80000000u;
 
 struct AdjDev {
   int p, eta, ntp, k;       // k: iteration (kernels add *k0, the first one of their segment)
@@ -37,12 +45,13 @@ struct AdjDev {
   const float* vlim;        // [nv][p][eta]
   // the tape of iteration k
   const float2* z;          // z^k, [p][eta+1]
+  const double* inv;        // 1 / active edges of a break-point (0 without one), [p][eta+1]
   const float4* ukin;       // u^k of the kinetic edges, [eta][p]
-  const uint32_t* fid;      // collision slots active in iteration k
+  const uint32_t* fid;      // collision slots active in iteration k (with WAS_ACTIVE)
   const float4* ucl;        // their u^k at the lower break-point: (u_i, u_j)
   const float4* uch;        // ... at the upper break-point
   const unsigned* count;    // how many
-  const uint32_t* sidx;     // gated segment factors active in iteration k: (g eta + s) p + i
+  const uint32_t* sidx;     // gated segment factors active in iteration k: (g eta + s) p + i (with WAS_ACTIVE)
   const float4* su;         // their u^k (lower, upper)
   const unsigned* scount;   // how many
   // adjoint state
@@ -55,9 +64,11 @@ struct AdjDev {
   int* sstamp;              // ... and the iteration that wrote them
   const double2* zb_in;     // dL/dz^{k+1}
   double2* zb_out;          // dL/dz^k, accumulated
-  double2* S;               // alpha * sum of u adjoints per node
-  unsigned* cnt;            // active edges per node
-  float2* mbar;             // per node
+  double2* zb_clear;        // the next step's zb_out
+  const double2* S_in;      // alpha * sum of u adjoints per node, for this iteration
+  double2* S_out;           // ... for the one before it, accumulated
+  double2* S_clear;
+  float2* mbar;             // per node, where a pass before the factors' forms it (bw_run_kernel)
   double2* g_start;         // [p]
   double2* g_goal;          // [p]
   double* g_r;              // [p]
@@ -86,76 +97,79 @@ __device__ __forceinline__ float4 live_ub(const AdjDev& A, const float4* ub, uin
   return A.stamp[f] == A.k + 1 ? v : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__device__ __forceinline__ void scatter_edge(const AdjDev& A, int i, int s, float2 ub) {
-  const size_t node = (size_t)i * (A.eta + 1) + s;
-  atomic_add2(A.S + node, mk(A.alpha * ub.x, A.alpha * ub.y));
-  atomicAdd(A.cnt + node, 1u);
+__device__ __forceinline__ void scatter_edge(const AdjDev& A, double2* S, int i, int s, float2 ub) {
+  atomic_add2(S + (size_t)i * (A.eta + 1) + s, mk(A.alpha * ub.x, A.alpha * ub.y));
+}
+// The two ends of one agent's segment s (nothing at fixed ends).
+__device__ __forceinline__ void scatter_ends(const AdjDev& A, double2* S, int i, int s, float2 lo, float2 hi) {
+  if (s > 0) scatter_edge(A, S, i, s, lo);
+  if (s + 1 < A.eta) scatter_edge(A, S, i, s + 1, hi);
 }
 
-// Pass 1: alpha * u adjoints and edge counts into the nodes.
+// The gated edges' part of S_in for the last iteration of a segment, whose
+// activity was not known when the iteration behind it (the next segment's
+// first) took its step.
 __device__ __forceinline__ void bw_scatter_item(const AdjDev& A, unsigned t) {
-  const unsigned nkin = (unsigned)(A.eta * A.p);
   const unsigned ncoll = *A.count;
-  if (t >= nkin + ncoll) {  // a gated segment factor
-    const uint32_t g = A.sidx[t - nkin - ncoll];
+  double2* S = const_cast<double2*>(A.S_in);
+  if (t >= ncoll) {  // a gated segment factor
+    const uint32_t g = A.sidx[t - ncoll] & ~WAS_ACTIVE;
     const int i = (int)(g % A.p), s = (int)((g / A.p) % A.eta);
-    const float4 ub = (A.sstamp[g] == A.k + 1) ? A.ubs[g] : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (s > 0) scatter_edge(A, i, s, lo2(ub));
-    if (s + 1 < A.eta) scatter_edge(A, i, s + 1, hi2(ub));
+    if (A.sstamp[g] != A.k + 1) return;
+    const float4 ub = A.ubs[g];
+    scatter_ends(A, S, i, s, lo2(ub), hi2(ub));
     return;
   }
-  if (t < nkin) {
-    const int s = (int)(t / A.p), i = (int)(t - (unsigned)s * A.p);
-    if (A.vo && s == 0) return;
-    const float4 ub = A.ubk[t];
-    if (s > 0) scatter_edge(A, i, s, lo2(ub));
-    if (s + 1 < A.eta) scatter_edge(A, i, s + 1, hi2(ub));
-    return;
-  }
-  const uint32_t f = A.fid[t - nkin];
+  const uint32_t f = A.fid[t] & ~WAS_ACTIVE;
+  if (A.stamp[f] != A.k + 1) return;
   int s, i, j;
   decode_slot(A, f, s, i, j);
-  const float4 bl = live_ub(A, A.ubl, f), bh = live_ub(A, A.ubh, f);
-  if (s > 0) { scatter_edge(A, i, s, lo2(bl)); scatter_edge(A, j, s, hi2(bl)); }
-  if (s + 1 < A.eta) { scatter_edge(A, i, s + 1, lo2(bh)); scatter_edge(A, j, s + 1, hi2(bh)); }
+  const float4 bl = A.ubl[f], bh = A.ubh[f];
+  scatter_ends(A, S, i, s, lo2(bl), lo2(bh));
+  scatter_ends(A, S, j, s, hi2(bl), hi2(bh));
 }
 
-// Pass 2 per node: mbar at free nodes, start / goal gradients at fixed ones;
-// clears the sums and the next adjoint of z.
+// Per break-point: the start / goal gradients at the fixed ends, and the
+// buffers of the next step cleared.
 __device__ __forceinline__ void bw_node(const AdjDev& A, int t) {
   const int E1 = A.eta + 1;
   const int i = t / E1, s = t - i * E1;
-  const double2 zb = A.zb_in[t];
-  if (s == 0) {
-    A.g_start[i].x += zb.x; A.g_start[i].y += zb.y;
-  } else if (s == A.eta) {
-    A.g_goal[i].x += zb.x; A.g_goal[i].y += zb.y;
-  } else {
-    const unsigned c = A.cnt[t];
-    const double2 S = A.S[t];
-    const double inv = c ? 1.0 / (double)c : 0.0;
-    A.mbar[t] = mk((float)((zb.x - S.x) * inv), (float)((zb.y - S.y) * inv));
+  if (s == 0 || s == A.eta) {
+    const double2 zb = A.zb_in[t];
+    double2* g = s == 0 ? A.g_start : A.g_goal;
+    g[i].x += zb.x;
+    g[i].y += zb.y;
   }
-  A.S[t] = make_double2(0.0, 0.0);
-  A.cnt[t] = 0u;
-  A.zb_out[t] = make_double2(0.0, 0.0);
+  A.S_clear[t] = make_double2(0.0, 0.0);
+  A.zb_clear[t] = make_double2(0.0, 0.0);
 }
 
-// Per edge of pass 3: xbar, and the u adjoint once nbar is known.
+// mbar of a free node.
+__device__ __forceinline__ float2 node_mbar(const AdjDev& A, size_t node) {
+  const double2 zb = A.zb_in[node], S = A.S_in[node];
+  const double inv = A.inv[node];
+  return mk((float)((zb.x - S.x) * inv), (float)((zb.y - S.y) * inv));
+}
+
+// Per edge: xbar, and the u adjoint once nbar is known.  MBAR: mbar was formed
+// by a pass over the nodes.
+template <bool MBAR>
 __device__ __forceinline__ float2 edge_xbar(const AdjDev& A, bool fixed, int i, int s, float2 ub,
                                            float2& mb) {
   if (fixed) { mb = mk(0.f, 0.f); return mb; }
-  mb = A.mbar[(size_t)i * (A.eta + 1) + s];
+  const size_t node = (size_t)i * (A.eta + 1) + s;
+  mb = MBAR ? A.mbar[node] : node_mbar(A, node);
   return mk(mb.x + A.alpha * ub.x, mb.y + A.alpha * ub.y);
 }
 __device__ __forceinline__ float2 edge_ubar(bool fixed, float2 ub, float2 mb, float2 nb) {
   return fixed ? mk(0.f, 0.f) : mk(ub.x + mb.x - nb.x, ub.y + mb.y - nb.y);
 }
 
-// Pass 3 for a wall or velocity-limit factor (gated like a collision factor).
+// A wall or velocity-limit factor (gated like a collision factor).
+template <bool MBAR>
 __device__ __forceinline__ void bw_seg_item(const AdjDev& A, unsigned w) {
   const int E1 = A.eta + 1;
-  const uint32_t g = A.sidx[w];
+  const uint32_t entry = A.sidx[w], g = entry & ~WAS_ACTIVE;
   const int i = (int)(g % A.p), s = (int)((g / A.p) % A.eta);
   const int kind = (int)(g / ((uint32_t)A.p * A.eta));
   const bool pin_lo = (s == 0), pin_hi = (s == A.eta - 1);
@@ -163,8 +177,8 @@ __device__ __forceinline__ void bw_seg_item(const AdjDev& A, unsigned w) {
   const float2 nl = A.z[(size_t)i * E1 + s] - lo2(u), nh = A.z[(size_t)i * E1 + s + 1] - hi2(u);
   const float4 ub = (A.sstamp[g] == A.k + 1) ? A.ubs[g] : make_float4(0.f, 0.f, 0.f, 0.f);
   float2 ml, mh;
-  const float2 xl = edge_xbar(A, pin_lo, i, s, lo2(ub), ml);
-  const float2 xh = edge_xbar(A, pin_hi, i, s + 1, hi2(ub), mh);
+  const float2 xl = edge_xbar<MBAR>(A, pin_lo, i, s, lo2(ub), ml);
+  const float2 xh = edge_xbar<MBAR>(A, pin_hi, i, s + 1, hi2(ub), mh);
   float2 bl, bh;
   if (kind < A.nw) {
     const float4 W = A.walls[kind];
@@ -177,16 +191,19 @@ __device__ __forceinline__ void bw_seg_item(const AdjDev& A, unsigned w) {
   }
   atomic_add2(A.zb_out + (size_t)i * E1 + s, bl);
   atomic_add2(A.zb_out + (size_t)i * E1 + s + 1, bh);
-  A.ubs[g] = pack(edge_ubar(pin_lo, lo2(ub), ml, bl), edge_ubar(pin_hi, hi2(ub), mh, bh));
+  const float4 un = pack(edge_ubar(pin_lo, lo2(ub), ml, bl), edge_ubar(pin_hi, hi2(ub), mh, bh));
+  A.ubs[g] = un;
   A.sstamp[g] = A.k;
+  if (entry & WAS_ACTIVE) scatter_ends(A, A.S_out, i, s, lo2(un), hi2(un));
 }
 
-// Pass 3: the adjoint of one factor's minimizer.
+// The adjoint of one factor's minimizer (t past the break-points).
+template <bool MBAR>
 __device__ __forceinline__ void bw_factor_item(const AdjDev& A, unsigned t) {
   const int E1 = A.eta + 1;
   const unsigned nkin = (unsigned)(A.eta * A.p);
   const unsigned ncoll = *A.count;
-  if (t >= nkin + ncoll) { bw_seg_item(A, t - nkin - ncoll); return; }
+  if (t >= nkin + ncoll) { bw_seg_item<MBAR>(A, t - nkin - ncoll); return; }
   if (t < nkin) {
     const int s = (int)(t / A.p), i = (int)(t - (unsigned)s * A.p);
     if (A.vo && s == 0) return;
@@ -195,19 +212,21 @@ __device__ __forceinline__ void bw_factor_item(const AdjDev& A, unsigned t) {
     const float2 nl = A.z[(size_t)i * E1 + s] - lo2(u), nh = A.z[(size_t)i * E1 + s + 1] - hi2(u);
     const float4 ub = A.ubk[t];
     float2 ml, mh;
-    const float2 xl = edge_xbar(A, pin_lo, i, s, lo2(ub), ml);
-    const float2 xh = edge_xbar(A, pin_hi, i, s + 1, hi2(ub), mh);
+    const float2 xl = edge_xbar<MBAR>(A, pin_lo, i, s, lo2(ub), ml);
+    const float2 xh = edge_xbar<MBAR>(A, pin_hi, i, s + 1, hi2(ub), mh);
     float2 bl, bh;
     float cb;
     energy_vjp(nl, nh, A.rho, pin_lo, pin_hi, A.cost[(size_t)i * A.eta + s], xl, xh, bl, bh, cb);
     atomic_add2(A.zb_out + (size_t)i * E1 + s, bl);
     atomic_add2(A.zb_out + (size_t)i * E1 + s + 1, bh);
-    A.ubk[t] = pack(edge_ubar(pin_lo, lo2(ub), ml, bl), edge_ubar(pin_hi, hi2(ub), mh, bh));
+    const float4 un = pack(edge_ubar(pin_lo, lo2(ub), ml, bl), edge_ubar(pin_hi, hi2(ub), mh, bh));
+    A.ubk[t] = un;
+    scatter_ends(A, A.S_out, i, s, lo2(un), hi2(un));
     A.g_c[(size_t)i * A.eta + s] += (double)cb;
     return;
   }
   const unsigned w = t - nkin;
-  const uint32_t f = A.fid[w];
+  const uint32_t entry = A.fid[w], f = entry & ~WAS_ACTIVE;
   int s, i, j;
   decode_slot(A, f, s, i, j);
   const bool pin_lo = (s == 0), pin_hi = (s == A.eta - 1);
@@ -217,10 +236,10 @@ __device__ __forceinline__ void bw_factor_item(const AdjDev& A, unsigned t) {
   const float2 njl = A.z[(size_t)j * E1 + s] - hi2(a), njh = A.z[(size_t)j * E1 + s + 1] - hi2(b);
   const float4 bl = live_ub(A, A.ubl, f), bh = live_ub(A, A.ubh, f);
   float2 mil, mjl, mih, mjh;
-  const float2 xil = edge_xbar(A, pin_lo, i, s, lo2(bl), mil);
-  const float2 xjl = edge_xbar(A, pin_lo, j, s, hi2(bl), mjl);
-  const float2 xih = edge_xbar(A, pin_hi, i, s + 1, lo2(bh), mih);
-  const float2 xjh = edge_xbar(A, pin_hi, j, s + 1, hi2(bh), mjh);
+  const float2 xil = edge_xbar<MBAR>(A, pin_lo, i, s, lo2(bl), mil);
+  const float2 xjl = edge_xbar<MBAR>(A, pin_lo, j, s, hi2(bl), mjl);
+  const float2 xih = edge_xbar<MBAR>(A, pin_hi, i, s + 1, lo2(bh), mih);
+  const float2 xjh = edge_xbar<MBAR>(A, pin_hi, j, s + 1, hi2(bh), mjh);
   float2 nbil, nbih, nbjl, nbjh;
   float Rb;
   coll_vjp(nil, nih, njl, njh, pin_lo, pin_hi, A.radius[i] + A.radius[j], A.rho, xil, xih, xjl,
@@ -231,9 +250,20 @@ __device__ __forceinline__ void bw_factor_item(const AdjDev& A, unsigned t) {
   atomic_add2(A.zb_out + (size_t)j * E1 + s + 1, nbjh);
   atomicAdd(A.g_r + i, (double)Rb);
   atomicAdd(A.g_r + j, (double)Rb);
-  A.ubl[f] = pack(edge_ubar(pin_lo, lo2(bl), mil, nbil), edge_ubar(pin_lo, hi2(bl), mjl, nbjl));
-  A.ubh[f] = pack(edge_ubar(pin_hi, lo2(bh), mih, nbih), edge_ubar(pin_hi, hi2(bh), mjh, nbjh));
+  const float4 ul = pack(edge_ubar(pin_lo, lo2(bl), mil, nbil), edge_ubar(pin_lo, hi2(bl), mjl, nbjl));
+  const float4 uh = pack(edge_ubar(pin_hi, lo2(bh), mih, nbih), edge_ubar(pin_hi, hi2(bh), mjh, nbjh));
+  A.ubl[f] = ul;
+  A.ubh[f] = uh;
   A.stamp[f] = A.k;
+  if (entry & WAS_ACTIVE) {
+    scatter_ends(A, A.S_out, i, s, lo2(ul), lo2(uh));
+    scatter_ends(A, A.S_out, j, s, hi2(ul), hi2(uh));
+  }
+}
+
+// Factors of an adjoint step.
+__device__ __forceinline__ unsigned bw_factors(const AdjDev& A) {
+  return (unsigned)(A.eta * A.p) + *A.count + *A.scount;
 }
 
 }  // namespace

@@ -122,6 +122,17 @@ struct SoloDev : Dev {
   uint32_t sums;  // shared-memory address
 };
 
+// A descriptor whose node pass also notes 1 / counts for the backward pass.
+template <class Base>
+struct Taped : Base {
+  double* inv;  // [p][eta+1]
+};
+__device__ __forceinline__ void note_count(const Dev&, size_t, unsigned) {}
+template <class Base>
+__device__ __forceinline__ void note_count(const Taped<Base>& P, size_t node, unsigned cnt) {
+  P.inv[node] = cnt ? 1.0 / (double)cnt : 0.0;
+}
+
 __device__ __forceinline__ float maxabs2(float2 a) { return fmaxf(fabsf(a.x), fabsf(a.y)); }
 
 // Step 7 of the previous iteration for one edge: u^k from the stored u^{k-1},
@@ -1309,6 +1320,7 @@ __device__ __forceinline__ float2 consensus_node(const D& P, size_t node, float2
   long long sx, sy;
   unsigned cnt;
   take_sums(P, node, sx, sy, cnt);
+  note_count(P, node, cnt);
   float2 zn = zo;  // every incoming weight zero: treated as 1, which gives z unchanged
   if (P.admm) {
     // every edge is weighted; each feasible collision or wall factor sent
