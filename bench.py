@@ -35,15 +35,14 @@ METRIC = "factor-updates/s and time-to-converge (1 GB300) vs FP64 CPU oracle; % 
 UNIT = "factor-updates/s"
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of
-# the current pass-1 kernels on square1024_eta16 (gated: two launches of one
-# capture, profiles/test_rows_kernel_square1024.md; dense: one single-pass
-# capture of two launches, profiles/test_kernel_traffic_square1024.md).
-TRAFFIC_SQUARE1024 = {"gated": 10.49e6, "dense": 486.32e6}
-# Warp instructions executed per launch of the gated pass-1 kernel on
-# square1024_eta16 (smsp__inst_executed.sum of a two-launch capture,
-# profiles/test_rows_kernel_square1024.md): the work the issue-rate
-# roofline divides by the kernel time.
-WARP_INST_SQUARE1024 = {"gated": 7.017e6}
+# the factor kernels on square1024_eta16 (gated: the mean of three launches,
+# profiles/factor_kernel_square1024.md; dense: of two,
+# profiles/test_kernel_traffic_square1024.md).
+TRAFFIC_SQUARE1024 = {"gated": 10.94e6, "dense": 223.3e6}
+# Warp instructions executed per launch of factor_kernel on square1024_eta16
+# (smsp__inst_executed.sum, the mean of the same launches): the work the
+# issue-rate roofline divides by the kernel time.
+WARP_INST_SQUARE1024 = {"gated": 5.932e6}
 
 
 def factor_counts(inst):
@@ -52,11 +51,12 @@ def factor_counts(inst):
 
 
 def dense_coll_bytes(inst):
-    """Algorithmic HBM bytes of the collision test pass under the dense state
-    model: per collision factor its 8-float u record read and written (64 B)
-    plus 2 bits of activity (read and written)."""
+    """Algorithmic HBM bytes of the collision factors under the dense state
+    model with the reset rule: per collision factor its 8-float u record
+    written (32 B; those of the few active ones are also read) plus 2 bits of
+    activity (read and written)."""
     c = factor_counts(inst)
-    return c["coll"] * 64 + c["coll"] * 2 / 8
+    return c["coll"] * 32 + c["coll"] * 2 / 8
 
 
 def dense_bytes_per_iter(inst):
@@ -629,11 +629,11 @@ def main():
             t = ktimes["test"] / 1e3
             ach = b / t / 1e9
             traffic = TRAFFIC_SQUARE1024["dense"] if inst.name == "square1024_eta16" else None
-            return {"bound": "hbm", "kernel": "test_kernel<dense> (with the kinetic and wall blocks)",
+            return {"bound": "hbm", "kernel": "test_kernel (dense; every factor)",
                     "achieved": ach,
                     "peak": hbm_peak, "unit": "GB/s", "frac": ach / hbm_peak, "traffic": traffic,
                     "peak_kind": f"{peak_kind} (copy bandwidth)",
-                    "note": f"algorithmic bytes {b:.4g} per launch (64 B u record read+written "
+                    "note": f"algorithmic bytes {b:.4g} per launch (32 B u record written "
                             f"and 2 bits per collision factor) / live kernel time "
                             f"{ktimes['test'] * 1e3:.1f} us"}
         # gated state: the bounding-circle filter leaves no per-factor bytes or
@@ -643,7 +643,7 @@ def main():
         pk_i = issue_peak_g(sm_max)
         ach = winst / t / 1e9 if winst else None
         own = TRAFFIC_SQUARE1024["gated"] if inst.name == "square1024_eta16" else None
-        return {"bound": "issue", "kernel": "test_rows_kernel (gated; with the kinetic and wall blocks)",
+        return {"bound": "issue", "kernel": "factor_kernel (gated; every factor)",
                 "achieved": ach, "peak": pk_i, "unit": "G warp-instructions/s",
                 "frac": ach / pk_i if ach else None, "traffic": own,
                 "peak_kind": f"derived: {sm_count()} SMs x 4 schedulers x 1 warp instruction/cycle "
@@ -668,7 +668,7 @@ def main():
         "kernel_ms": kt,
         "wall_s": wall,
         "clocks": clk,
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": 2 * args.steps,
         "roofline": roofline_for(args.mode, kt),
     }
     if not args.quick:

@@ -225,11 +225,11 @@ plan_status plan_check(plan_t plan, double* total_cost, double* min_pair_clearan
 /* Per-kernel timing of the next iterations (CUDA events on the plan's
  * stream).  enable = 1 starts collecting (and synchronises once per
  * iteration, so timings are taken without overlap between iterations);
- * enable = 0 stops and writes the average milliseconds per iteration of the
- * three kernels to ms[0..3] = {pass 1: collision tests, with the kinetic
- * factors and wall tests in the same launch; pass 2: wall and collision
- * minimizers; 0 (no separate kinetic / wall launch); consensus} and their
- * count to *iterations (either may be NULL).  Errors: PLAN_EINVAL (a batch
+ * enable = 0 stops and writes the average milliseconds per iteration of its
+ * kernels to ms[0..3] = {factor pass: every factor's test and minimizer;
+ * about 0 (no separate minimizer launch, what is left is the distance of two
+ * events); 0; node pass} and their count to *iterations (either may be
+ * NULL).  Errors: PLAN_EINVAL (a batch
  * member), PLAN_ECUDA. */
 plan_status plan_profile(plan_t plan, int enable, float* ms, int* iterations);
 
@@ -274,10 +274,10 @@ plan_status plan_batch_import_state(plan_batch_t batch, int member, const float*
 plan_status plan_batch_export_state(plan_batch_t batch, int member, float* z, float* u_coll,
                                     float* u_kin, float* u_wall, uint8_t* act_coll,
                                     uint8_t* act_wall);
-/* Time the launch-shape candidates (rows per warp of the collision test
- * {4, 8, 16}, or 32: one warp per tile with lane = row agent, gated state
- * only; minimizer CTAs per SM {1, 2, 4} x the base grid; iterations per
- * graph {2, 8}) on this batch, iters_per_candidate iterations each (they are
+/* Time the launch-shape candidates (rows per warp of the dense state's
+ * collision test {4, 8, 16}, 32 with the gated state; minimizer CTAs per SM
+ * {1, 2, 4} x the base grid, dense state; iterations per graph {2, 8}; with
+ * the gated state only the last one changes a launch) on this batch, iters_per_candidate iterations each (they are
  * real iterations: results do not depend on the shape), and keep the fastest.
  * choice: 3 host ints receiving the chosen values (may be NULL). */
 plan_status plan_batch_autotune(plan_batch_t batch, int iters_per_candidate, int* choice);

@@ -479,9 +479,9 @@ class Planner:
         _check(_lib.plan_profile(self._h, 1, None, None))
 
     def profile_stop(self):
-        """Average ms per iteration of the three passes: test (collision
-        tests with the kinetic factors and wall tests in the same launch),
-        minimizer (walls and pairs) and consensus."""
+        """Average ms per iteration of its kernels: test (the factor pass,
+        tests and minimizers of every factor), minimizer (about 0: no launch
+        of its own) and consensus (the node pass)."""
         ms = (c_float * 4)()
         n = c_int(0)
         _check(_lib.plan_profile(self._h, 0, ms, byref(n)))

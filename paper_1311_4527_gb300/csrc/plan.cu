@@ -1651,7 +1651,7 @@ struct plan_s {
     P.vlim = at<float>(L.vlim);
     P.wnode = at<uint8_t>(L.wnode);
     P.rho = rho_at(kk);
-    // pass 1 of iteration kk finishes the dual step of iteration kk - 1, so
+    // the factor pass of iteration kk finishes the dual step of iteration kk - 1, so
     // the printed step alpha / rho takes the rho of that iteration
     P.alpha = (cfg.flags & PLAN_U_LITERAL) ? cfg.alpha / rho_at(kk > 0 ? kk - 1 : 0) : cfg.alpha;
     // keeping u on inactive edges (or standard ADMM, which updates every u)
@@ -2009,7 +2009,7 @@ plan_status run_iterations(plan_t h, int n) {
 }
 
 // Residual of the last completed iteration (k - 1): its consensus part was
-// written by consensus_kernel, the primal part comes from residual_kernel.
+// written by the node pass, the primal part comes from residual_kernel.
 plan_status read_residual(plan_t h, float* out) {
   if (h->k == 0) { *out = INFINITY; return PLAN_OK; }
   Dev P = h->dev(h->k);

@@ -99,7 +99,7 @@ struct Dev {
   int* inv;              // [eta][p] place of an agent
   int4* box;             // [eta][nt] box of the circles at 32 places (x, y least, x, y largest;
                          // floats as ordered integers)
-  uint32_t* work;        // collision worklist (dense state: the active slots of this iteration)
+  uint32_t* work;        // collision worklist (dense batches: the active slots of this iteration)
   unsigned cap;          // its capacity
   uint32_t* listed;      // [eta * ntp * 32] pairs on the worklist (gated state)
   unsigned* work_count;  // its length, by iteration parity: entries are appended here
@@ -556,7 +556,7 @@ __device__ __forceinline__ void prox_item(const Dev& P, uint32_t fid) {
   }
 }
 
-// Dense state, pass 1: one CTA of TILE / TROWS warps per (segment s, agent
+// Dense state: one CTA of TILE / TROWS warps per (segment s, agent
 // tiles I <= J) block of 32 x 32 collision factors; each warp takes TROWS
 // rows (the launch shape the batched autotuner varies), lane = column agent j,
 // and the row agents' data is broadcast from shared memory.  Per row, the warp
