@@ -718,6 +718,7 @@ __global__ void __launch_bounds__(256) check_kernel(Dev P, const double* ccost, 
 // Primal residual max |x^k - z^k| over weighted edges, without changing state
 // (the same finishing arithmetic the next factor_kernel will apply).
 __global__ void residual_kernel(Dev P) {
+  pdl_begin();
   float res = 0.f;
   const int lane = threadIdx.x & 31;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -784,6 +785,14 @@ __global__ void residual_kernel(Dev P) {
   }
   res = warp_max(res);
   if (lane == 0 && res > 0.f) atomic_max_nonneg(P.res_prev, res);
+}
+
+// One word into pinned host memory, in the launch chain (with the residual's own
+// launch in it too, 8 us less a reading than by a copy engine behind it: p = 4,
+// 100 iterations with four readings 450 us, now 418).
+__global__ void report_kernel(const unsigned* value, unsigned* host) {
+  pdl_begin();
+  *host = *value;
 }
 
 // bytes (a multiple of 8) from src to dst, both on 16-byte boundaries.
@@ -2013,9 +2022,10 @@ plan_status run_iterations(plan_t h, int n) {
 plan_status read_residual(plan_t h, float* out) {
   if (h->k == 0) { *out = INFINITY; return PLAN_OK; }
   Dev P = h->dev(h->k);
-  residual_kernel<<<h->eta > 0 ? 304 : 1, 256, 0, h->stream>>>(P);
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(h->h_res, P.res_prev, 4, cudaMemcpyDeviceToHost, h->stream));
+  unsigned* host = nullptr;
+  CK(cudaHostGetDevicePointer(reinterpret_cast<void**>(&host), h->h_res, 0));
+  CK(launch_pdl(residual_kernel, 304u, 256u, h->stream, P));
+  CK(launch_pdl(report_kernel, 1u, 1u, h->stream, (const unsigned*)P.res_prev, host));
   CK(cudaStreamSynchronize(h->stream));
   uint32_t bitsv = *h->h_res;
   float v;
