@@ -13,8 +13,7 @@
 //        E'' = sum w_v (<v, tau>^2 + g_v <v, n>),
 //        dE'/dv = w_v (<v, tau> n - g_v tau),  dE'/dR = -sum w_v <v, tau>;
 //  * the single-hinge direction n = v / |v|: dphi = <tau, dv> / |v|;
-//  * an end of the arc of a fixed-end minimizer, <q, n> = R:
-//    dphi = (dR - <dq, n>) / <q, tau>.
+//  * an end of an arc, <q, n> = R: dphi = (dR - <dq, n>) / <q, tau>.
 // Kinetic minimizer (Appendix E): linear in n, rational in c.
 #pragma once
 #include "twa_math.cuh"
@@ -78,11 +77,14 @@ TWA_DEV void disk_free_vjp(float2 a, float2 b, float wl, float wh, float R, floa
   end_vjp(a, vlbar, n, R, abar, Rbar, phib);
   end_vjp(b, vhbar, n, R, bbar, Rbar, phib);
   switch (tag) {
+    case DISK_GLOBAL: stationary_vjp(a, b, wl, wh, R, n, phib, abar, bbar, Rbar); break;
     case DISK_A_INNER: inner_vjp(a, n, phib, abar); break;
     case DISK_B_INNER: inner_vjp(b, n, phib, bbar); break;
+    case DISK_A_TANGENT: tangent_vjp(b, n, phib, bbar, Rbar); break;
+    case DISK_B_TANGENT: tangent_vjp(a, n, phib, abar, Rbar); break;
     default: {
-      // a stationary point of the hinges that are positive there (both, but
-      // for a winner within rounding of a single-hinge direction)
+      // the (1, 0) fallback wins only where it is itself a minimiser: a
+      // stationary point of the hinges that are positive there
       const float ml = (R - dot(a, n) > 0.f) ? wl : 0.f, mh = (R - dot(b, n) > 0.f) ? wh : 0.f;
       stationary_vjp(a, b, ml, mh, R, n, phib, abar, bbar, Rbar);
     }

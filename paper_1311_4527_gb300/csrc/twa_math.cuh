@@ -27,10 +27,11 @@
 // mu <= lambda1, i.e. t = lambda1 - mu >= 0 is the unique root of the
 // decreasing secular function (R s1 / t)^2 + (R s2 / (d + t))^2 = 1,
 // d = lambda2 - lambda1 (hard case: s1 = 0 and R |s2| < d gives t = 0).
-// m_a is the energy at a / |a| when that direction lies in its arc; when it
-// does not, the arc's best point is an end <b,n> = R, where the energy still
-// falls on the arc's outside (the b hinge starts with slope zero), so it is
-// not the minimum of E and needs no candidate.  m_b likewise.
+// m_a / m_b are closed form: the arc point closest in angle to a (or b).
+// Where that point is an end of the arc, <b, n> = R, the energy still falls on
+// the arc's outside, so in exact arithmetic it is never below E(n_f); to
+// rounding it ties with it, and is a candidate for that reason: which of two
+// tying candidates wins is part of the FP32 results (see trs_global).
 //
 // Capsule (wall) regions use the same hinge energy with
 // h(n) = max(<xL,n>, <xR,n>) + r, which is the disk energy of one end circle
@@ -73,11 +74,11 @@ TWA_DEV float dot(float2 a, float2 b) { return fmaf(a.x, b.x, a.y * b.y); }
 TWA_DEV float cross(float2 a, float2 b) { return fmaf(a.x, b.y, -(a.y * b.x)); }
 TWA_DEV float2 axpy(float s, float2 a, float2 b) { return mk(fmaf(s, a.x, b.x), fmaf(s, a.y, b.y)); }  // s a + b
 TWA_DEV float2 perp(float2 a) { return mk(-a.y, a.x); }
-TWA_DEV float2 normalized(float2 a) {
+// a / |a|; dd: |a|^2, where the caller sums it in an order of its own.
+TWA_DEV float2 normalized(float2 a, float dd) {
 #ifdef __CUDA_ARCH__
   // one reciprocal square root (2 ulp) where |a|^2 is a normal float; the
   // directions are unit to a few ulp either way
-  const float dd = dot(a, a);
   if (dd > 1e-30f && dd < 1e30f) {
     const float s = rsqrtf(dd);
     return mk(a.x * s, a.y * s);
@@ -86,6 +87,7 @@ TWA_DEV float2 normalized(float2 a) {
   float n = hypotf(a.x, a.y);
   return n > 0.f ? mk(a.x / n, a.y / n) : mk(1.f, 0.f);
 }
+TWA_DEV float2 normalized(float2 a) { return normalized(a, dot(a, a)); }
 
 // Fast division (2 ulp for divisors of normal magnitude; every divisor here
 // is a length, a curvature or a secular variable far from the float limits)
@@ -207,59 +209,76 @@ TWA_DEV float hinge_E(float2 a, float2 b, float wl, float wh, float R, float2 n)
   return fmaf(0.5f * wl * ga, ga, 0.5f * wh * gb * gb);
 }
 
+// n1 e1 + n2 e2, e1 = perp(e2).
+TWA_DEV float2 in_frame(float n1, float n2, float2 e2) {
+  return mk(fmaf(n2, e2.x, -(n1 * e2.y)), fmaf(n1, e2.x, n2 * e2.y));
+}
+
 // Global minimiser(s) of f(n) = wl (R - <a,n>)^2 + wh (R - <b,n>)^2 on the
 // unit circle.  Writes 1 or 2 directions (2 only for exact ties).
-// The longest chain of the iteration, so its arithmetic is kept short: a, b
-// and R are scaled by a power of two to R in [1, 2) (exact), after which the
-// squares below stay in range for |a|, |b| up to 1e9 R and plain square roots
-// serve; the Newton loop needs no bracket (below).
+// The order of the operations, fused or not, is part of the results: where a
+// candidate of another kind ties with the root to rounding, the last bit
+// decides which one wins, and with it the branch that the adjoint
+// differentiates (and, head on, the side on which the pair passes).  A form
+// with a shorter chain (plain square roots, a climb without a bracket, no arc
+// ends) took 4.1 us an iteration for 4.8 of the p = 4 circle's, but parted from
+// these results by up to 2e-4 in 2 % of gradients of circle swaps, and by whole
+// detours in one pass of 300.
 TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
                                        float2* out) {
-  const float sc = pow2_inverse(R);
-  a = sc * a; b = sc * b; R *= sc;
   const float2 wa = wl * a, wb = wh * b;
   const float m11 = fmaf(wa.x, a.x, wb.x * b.x);
   const float m22 = fmaf(wa.y, a.y, wb.y * b.y);
   const float m12 = fmaf(wa.x, a.y, wb.x * b.y);
   const float2 S = wa + wb;
   const float hd = 0.5f * (m11 - m22);
-  const float disc = sqrtf(fmaf(hd, hd, m12 * m12));
+  const float disc = hypotf(hd, m12);
   const float d = 2.f * disc;  // lambda2 - lambda1 >= 0
   const float q = fabsf(hd) + disc;
-  float2 e2 = (hd >= 0.f) ? mk(q, m12) : mk(m12, q);
-  e2 = (disc > 0.f) ? normalized(e2) : mk(1.f, 0.f);
+  const float2 e2 = (disc > 0.f) ? normalized((hd >= 0.f) ? mk(q, m12) : mk(m12, q), fmaf(m12, m12, q * q)) : mk(1.f, 0.f);
   const float2 e1 = perp(e2);
-  const float s1 = dot(S, e1), s2 = dot(S, e2);
-  const float Sn = sqrtf(fmaf(s1, s1, s2 * s2));
+  const float s1 = cross(e2, S), s2 = dot(S, e2);
+  const float Sn = hypotf(s1, s2);
   if (!(Sn > 0.f)) { out[0] = e1; out[1] = -e1; return 2; }
-  const float A1 = R * fabsf(s1), A2 = R * fabsf(s2), RS = R * Sn;
-  if (A1 <= 1e-7f * RS && A2 < d) {  // hard case: t = 0
+  const float A1 = R * fabsf(s1), A2 = R * fabsf(s2);
+  if (A1 <= 1e-7f * R * Sn && A2 < d) {  // hard case: t = 0
     const float n2 = R * s2 / d;
     const float n1 = sqrtf(fmaxf(0.f, fmaf(-n2, n2, 1.f)));
-    out[0] = axpy(n1, e1, n2 * e2);
-    out[1] = axpy(-n1, e1, n2 * e2);
+    out[0] = in_frame(n1, n2, e2);
+    out[1] = mk(fmaf(n1, e2.y, n2 * e2.x), fmaf(n2, e2.y, -(n1 * e2.x)));
     return 2;
   }
-  // Root of 1/|n(t)| = 1, |n(t)|^2 = phi = (A1/t)^2 + (A2/(d+t))^2.  1/|n(t)|
-  // is concave and increasing (Moré-Sorensen), so Newton from a point left of
-  // the root (phi >= 1 there) climbs to it without passing it, and every
-  // step is t += (sqrt(phi) - 1) phi / (q1^2/t + q2^2/(d+t)).
-  float t = fmaxf(fmaxf(A1, RS - d), 1e-12f * RS);
+  // Root of h(t) = phi(t)^{-1/2} - 1 with phi = (A1/t)^2 + (A2/(d+t))^2.
+  // 1/|n(t)| is concave and increasing (Moré-Sorensen), so Newton from the
+  // left bracket end, where h <= 0, climbs monotonically to the root.
+  float lo = fmaxf(fmaxf(A1, R * Sn - d), 0.f), hi = R * Sn;
+  if (lo > hi) lo = hi;
+  float t = lo > 0.f ? lo : 0.5f * hi;
 #pragma unroll 1
   for (int it = 0; it < 40; ++it) {
     TWA_ITER_HOOK(0);
     const float it_ = fdiv(1.f, t), id = fdiv(1.f, d + t);
     const float q1 = A1 * it_, q2 = A2 * id;
-    const float w1 = q1 * q1, w2 = q2 * q2;
-    const float phi = w1 + w2;
-    const float step = (phi * frsqrt(phi) - 1.f) * fdiv(phi, fmaf(w1, it_, w2 * id));
-    t += step;
-    // FP32 noise in phi limits t to ~1e-7 relative; stop at 1e-6
-    if (!(step > 1e-6f * t)) break;
+    const float phi = q1 * q1 + q2 * q2;
+    const float ip = frsqrt(phi);
+    const float h = ip - 1.f;
+    if (h > 0.f) hi = t; else lo = t;
+    if (h == 0.f) break;
+    const float dh = ip * ip * ip * fmaf(q1 * q1, it_, q2 * q2 * id);
+    float tn = fmaf(-h, fdiv(1.f, dh), t);
+    if (!(tn > lo && tn < hi)) tn = 0.5f * (lo + hi);
+    // FP32 noise in h limits t to ~1e-7 relative; stop at 1e-6
+    const bool done = fabsf(tn - t) <= 1e-6f * t || hi - lo <= 1e-6f * hi;
+    t = tn;
+    if (done) break;
   }
-  // (n1, n2) = (R s1 / t, R s2 / (d + t)) up to its length, which is 1 to the
-  // error of t; only their ratio is used
-  out[0] = normalized(axpy(s1 * (d + t), e1, (s2 * t) * e2));
+  // the smaller component from the root, the other from the unit length
+  const float p1 = (t > 0.f) ? fdiv(R * s1, t) : copysignf(INFINITY, s1);
+  const float p2 = fdiv(R * s2, d + t);
+  const bool first = fabsf(p1) <= fabsf(p2);
+  const float c = first ? p1 : p2;
+  const float rest = copysignf(sqrtf(fmaxf(0.f, fmaf(-c, c, 1.f))), first ? s2 : s1);
+  out[0] = normalized(first ? in_frame(p1, rest, e2) : in_frame(rest, p2, e2));
   return 1;
 }
 
@@ -317,9 +336,9 @@ TWA_DEV void tangent_normals(float2 q, float R, float2& t0, float2& t1) {
   float L2 = dot(q, q);
   float s = sqrtf(fmaxf(fmaf(-R, R, L2), 0.f));
   float inv = fdiv(1.f, L2);
-  float2 pq = perp(q), Rq = R * q;
-  t0 = inv * axpy(s, pq, Rq);
-  t1 = inv * axpy(-s, pq, Rq);
+  const float2 sp = s * perp(q);  // (fused in this order: see trs_global)
+  t0 = inv * axpy(R, q, sp);
+  t1 = inv * axpy(R, q, -sp);
 }
 
 // Direction in the arc {n : <q,n> >= R} (|q| >= R) maximising <w, n>.
@@ -345,36 +364,35 @@ TWA_DEV float2 arc_argmax(float2 q, float R, float2 w) {
 
 // Kinds of winning direction of the free disk minimizer (Best::tag).
 enum DiskTag {
+  DISK_DEFAULT = 0,  // the (1, 0) fallback
   DISK_GLOBAL = 1,   // global minimiser n_f of the both-stretched piece f
-  DISK_A_INNER = 2,  // a / |a|, where b's hinge is zero
-  DISK_B_INNER = 4   // b / |b|, where a's hinge is zero
+  DISK_A_INNER = 2,  // a / |a| on the arc where b's hinge is zero
+  DISK_A_TANGENT = 3,  // an end of that arc, <b, n> = R
+  DISK_B_INNER = 4,  // b / |b| on the arc where a's hinge is zero
+  DISK_B_TANGENT = 5   // an end of that arc, <a, n> = R
 };
 
 // Separating direction of the free disk minimizer and the kind of candidate
 // it came from.
 TWA_DEV float2 disk_dir_free(float2 a, float2 b, float wl, float wh, float R, int& tag) {
-  float2 c[2];
-  const int nc = trs_global(a, b, wl, wh, R, c);
   Best best;
-  best.n = c[0];
-  best.E = hinge_E(a, b, wl, wh, R, c[0]);
-  best.tag = DISK_GLOBAL;
-  if (nc > 1) best.offer(c[1], hinge_E(a, b, wl, wh, R, c[1]), DISK_GLOBAL);
-  // a / |a| where b's hinge is zero there, and the same with a and b
-  // exchanged (an end within 1e-15 of the centre has no direction)
-  const float aa = dot(a, a), bb = dot(b, b), tiny = 1e-30f * R * R, ab = dot(a, b);
-  if (aa > tiny) {
-    const float ia = frsqrt(aa);
-    if (ab * ia >= R) {
-      const float2 n = ia * a;
-      best.offer(n, hinge_E(a, b, wl, wh, R, n), DISK_A_INNER);
-    }
-  }
-  if (bb > tiny) {
-    const float ib = frsqrt(bb);
-    if (ab * ib >= R) {
-      const float2 n = ib * b;
-      best.offer(n, hinge_E(a, b, wl, wh, R, n), DISK_B_INNER);
+  best.init();
+  best.offer(mk(1.f, 0.f), hinge_E(a, b, wl, wh, R, mk(1.f, 0.f)), DISK_DEFAULT);
+  float2 c[2];
+  int nc = trs_global(a, b, wl, wh, R, c);
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    if (k < nc) best.offer(c[k], hinge_E(a, b, wl, wh, R, c[k]), DISK_GLOBAL);
+  // side 0: b's hinge can be zero, best a-term on that arc; side 1: the same
+  // with a and b exchanged (one copy of the code, run twice)
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    const float2 q = side ? a : b, w = side ? b : a;
+    if (dot(q, q) >= R * R) {
+      bool tg;
+      float2 n = arc_argmax(q, R, w, tg);
+      best.offer(n, hinge_E(a, b, wl, wh, R, n),
+                 side ? (tg ? DISK_B_TANGENT : DISK_B_INNER) : (tg ? DISK_A_TANGENT : DISK_A_INNER));
     }
   }
   tag = best.tag;
