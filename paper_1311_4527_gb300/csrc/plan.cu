@@ -1282,7 +1282,7 @@ __global__ void vo_target_kernel(int p, const float2* start, const float2* dest,
   const float2 d = dest[i] - start[i];
   const float L = hypotf(d.x, d.y);
   const float sc = (L > step) ? step / L : 1.f;
-  goal[i] = start[i] + sc * d;
+  goal[i] = axpy(sc, d, start[i]);
 }
 
 __global__ void vo_advance_kernel(int p, int eta, const float2* z, const float2* dest, float frac,
@@ -1291,7 +1291,7 @@ __global__ void vo_advance_kernel(int p, int eta, const float2* z, const float2*
   float dist = 0.f;
   if (i < p) {
     const float2 x0 = start[i], x1 = z[(size_t)i * (eta + 1) + 1];
-    const float2 xn = x0 + frac * (x1 - x0);
+    const float2 xn = axpy(frac, x1 - x0, x0);
     start[i] = xn;
     const float2 d = dest[i] - xn;
     dist = hypotf(d.x, d.y);
