@@ -1830,14 +1830,14 @@ bool solo(const plan_s* h) {
 // GPU to others now and then).  tape: where to record them, or null.
 constexpr int SOLO_ITERS = 512;
 plan_status run_solo(plan_t h, int n, const Tape* tape) {
+  Tape T{};
+  if (tape) T = *tape;
   while (n > 0) {
     const int m = std::min(n, SOLO_ITERS), c0 = h->cur;
     const Dev P0 = h->dev(h->k);
     if (h->eta > 1) h->cur ^= 1;
     const Dev P1 = h->dev(h->k + 1);
     h->cur = c0;
-    Tape T{};
-    if (tape) T = *tape;
     const int segw = segment_warps(h), tiles = (h->vo ? 1 : h->eta) * h->ntp;
     // list warps: those the tiles and segments leave, at least half of the CTA's
     const int nlist = std::min(list_ctas(h) * FACTOR_WARPS, std::max(SOLO_WARPS - tiles - segw, SOLO_WARPS / 2));
@@ -1847,6 +1847,8 @@ plan_status run_solo(plan_t h, int n, const Tape* tape) {
     if (h->eta > 1 && (m & 1)) h->cur ^= 1;
     h->k += m;
     n -= m;
+    T.at += (size_t)m * T.stride;  // the next launch records behind this one
+    T.q += m;
   }
   return PLAN_OK;
 }
