@@ -608,9 +608,18 @@ __device__ double wall_ratio2(const Dev& P, float4 W, float2 a, float2 b, float 
   return d2 / ((double)ri * (double)ri);
 }
 
-// One thread per (wall, segment, agent), grid-stride over whole blocks.  A
-// wall that the FP32 test finds crossed is 0 within its bound only if the
-// crossing is not one of rounding, so it asks for FP64 like a distance of 0.
+// Do the segments cross, by the signs of FP32 cross products?
+__device__ __forceinline__ bool seem_to_cross(float2 a, float2 b, float2 c0, float2 c1) {
+  const float o1 = cross(b - a, c0 - a), o2 = cross(b - a, c1 - a);
+  const float o3 = cross(c1 - c0, a - c0), o4 = cross(c1 - c0, b - c0);
+  return ((o1 < 0.f && o2 > 0.f) || (o1 > 0.f && o2 < 0.f)) && ((o3 < 0.f && o4 > 0.f) || (o3 > 0.f && o4 < 0.f));
+}
+
+// One thread per (wall, segment, agent), grid-stride over whole blocks.  The
+// distance of the nearest end from the other segment bounds the distance from
+// above whether the two cross or not (an agent that moves along a wall's line
+// beyond its end seems to cross it by rounding, and is far away); a crossing
+// asks for FP64 like a distance of 0.
 __device__ __forceinline__ void check_walls(const Dev& P, int nseg, int block, int blocks, unsigned long long* out) {
   const int E1 = P.eta + 1;
   const long long n = (long long)P.nw * nseg * P.p;
@@ -628,8 +637,10 @@ __device__ __forceinline__ void check_walls(const Dev& P, int nseg, int block, i
       const float2 c0 = mk(W.x, W.y), c1 = mk(W.z, W.w);
       // the differences the distances are made of
       const float mag = fmaxf(fmaxf(maxabs2(a - c0), maxabs2(a - c1)), fmaxf(maxabs2(b - c0), maxabs2(b - c1)));
-      const Bounds q = ratio_bounds(sqrtf(dist2_segment_segment(a, b, c0, c1)), mag, ri);
-      lo = q.lo;
+      const float ends = fminf(fminf(dist2_point_segment(a, c0, c1), dist2_point_segment(b, c0, c1)),
+                               fminf(dist2_point_segment(c0, a, b), dist2_point_segment(c1, a, b)));
+      const Bounds q = ratio_bounds(sqrtf(ends), mag, ri);
+      lo = seem_to_cross(a, b, c0, c1) ? -1.f : q.lo;
       hi = q.hi;
     }
     const float least = fminf(block_min(hi), least_so_far(out));

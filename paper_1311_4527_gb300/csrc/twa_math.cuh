@@ -151,17 +151,6 @@ TWA_DEV float dist2_point_segment(float2 q, float2 p0, float2 p1) {
   return dist2_origin_segment(p0 - q, p1 - q);
 }
 
-// Squared distance between segments [a0, a1] and [b0, b1].
-TWA_DEV float dist2_segment_segment(float2 a0, float2 a1, float2 b0, float2 b1) {
-  float d1 = cross(a1 - a0, b0 - a0), d2 = cross(a1 - a0, b1 - a0);
-  float d3 = cross(b1 - b0, a0 - b0), d4 = cross(b1 - b0, a1 - b0);
-  if (((d1 < 0.f && d2 > 0.f) || (d1 > 0.f && d2 < 0.f)) &&
-      ((d3 < 0.f && d4 > 0.f) || (d3 > 0.f && d4 < 0.f)))
-    return 0.f;
-  float m = fminf(dist2_point_segment(a0, b0, b1), dist2_point_segment(a1, b0, b1));
-  return fminf(m, fminf(dist2_point_segment(b0, a0, a1), dist2_point_segment(b1, a0, a1)));
-}
-
 // Keep the best (lowest E, then smallest angle) candidate direction.  tag
 // records which kind of candidate won (read by the adjoint; dead otherwise).
 struct Best {
