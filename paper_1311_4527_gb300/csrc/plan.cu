@@ -447,17 +447,28 @@ __device__ __forceinline__ double origin_seg_dist2(double ax, double ay, double 
   return fma(cx, cx, cy * cy);
 }
 
+// Distance of the origin from the segment p0 -> p1 in FP32, without squaring a
+// cross product (which underflows already at coordinates of 1e-11).
+__device__ __forceinline__ float origin_seg_dist(float2 p0, float2 p1) {
+  const float2 d = p1 - p0;
+  const float dd = dot(d, d), t = -dot(p0, d);
+  if (dd <= 1e-28f || t <= 0.f) return sqrtf(dot(p0, p0));
+  if (t >= dd) return sqrtf(dot(p1, p1));
+  return fabsf(cross(p0, d)) * frsqrt(dd);
+}
+
 // Distance bounds of one ratio in FP32: the distance of the origin from the
 // segment cl -> ch (or any other distance d found from coordinates of size
 // mag), with an error of at most 4e-6 mag (sixty times the rounding of one
-// operation on such coordinates, of which the distance takes about ten), over
-// the radius sum R.  Beyond the range where FP32 squares are safe the bounds
-// are those that always ask for FP64.
+// operation on such coordinates, of which the distance takes about ten) + 1e-14
+// (segments shorter than that are taken for points), over the radius sum R.
+// Beyond the range where FP32 squares are safe the bounds are those that
+// always ask for FP64.
 struct Bounds { float lo, hi; };
 __device__ __forceinline__ Bounds ratio_bounds(float d, float mag, float R) {
   Bounds b = {-1.f, INFINITY};
   if (mag < 1e15f && d < INFINITY) {
-    const float err = fmaf(4e-6f, mag, 1e-18f);
+    const float err = fmaf(4e-6f, mag, 1e-14f);
     b.lo = (d - err) / R * 0.999999f;
     b.hi = (d + err) / R * 1.000001f;
   }
@@ -503,7 +514,7 @@ __device__ __forceinline__ float4 ends_of(const Dev& P, int i, int s) {
 // relative motion) over R.
 __device__ __forceinline__ Bounds pair_bounds(float4 zi, float4 zj, float R) {
   const float2 cl = lo2(zj) - lo2(zi), ch = hi2(zj) - hi2(zi);
-  return ratio_bounds(sqrtf(dist2_origin_segment(cl, ch)), fmaxf(maxabs2(cl), maxabs2(ch)), R);
+  return ratio_bounds(origin_seg_dist(cl, ch), fmaxf(maxabs2(cl), maxabs2(ch)), R);
 }
 
 // A first upper bound of the smallest pair ratio, for a block of tiles that
@@ -541,14 +552,15 @@ __device__ __forceinline__ void check_tile(const Dev& P, int tile, float first, 
   const int i = IJ.x * TILE + lane, j = IJ.y * TILE + lane;
   const bool vi = i < P.p, vj = j < P.p;
   float4 zi = make_float4(0.f, 0.f, 0.f, 0.f), zj = zi;
-  float ri = 0.f, rj = 0.f;
+  float ri = 1.f, rj = 1.f;
   if (vi) { zi = ends_of(P, i, s); ri = P.radius[i]; }
   if (vj) { zj = ends_of(P, j, s); rj = P.radius[j]; }
   bool safe = true;
   auto circle = [&](float4 z, float r) {
     const float2 m = 0.5f * (lo2(z) + hi2(z)), d = hi2(z) - lo2(z);
     const float b = fmaf(0.5f, sqrtf(dot(d, d)), first * r);
-    safe = safe && dot(m, m) + b * b < 1e30f;
+    const float q = dot(m, m) + b * b;
+    safe = safe && q < 1e30f && q > 1e-30f;
     return make_float4(m.x, m.y, b, -bounding_offset(m, b));
   };
   const float4 ci = circle(zi, ri), cj = circle(zj, rj);
@@ -637,9 +649,9 @@ __device__ __forceinline__ void check_walls(const Dev& P, int nseg, int block, i
       const float2 c0 = mk(W.x, W.y), c1 = mk(W.z, W.w);
       // the differences the distances are made of
       const float mag = fmaxf(fmaxf(maxabs2(a - c0), maxabs2(a - c1)), fmaxf(maxabs2(b - c0), maxabs2(b - c1)));
-      const float ends = fminf(fminf(dist2_point_segment(a, c0, c1), dist2_point_segment(b, c0, c1)),
-                               fminf(dist2_point_segment(c0, a, b), dist2_point_segment(c1, a, b)));
-      const Bounds q = ratio_bounds(sqrtf(ends), mag, ri);
+      const float ends = fminf(fminf(origin_seg_dist(c0 - a, c1 - a), origin_seg_dist(c0 - b, c1 - b)),
+                               fminf(origin_seg_dist(a - c0, b - c0), origin_seg_dist(a - c1, b - c1)));
+      const Bounds q = ratio_bounds(ends, mag, ri);
       lo = seem_to_cross(a, b, c0, c1) ? -1.f : q.lo;
       hi = q.hi;
     }
