@@ -282,15 +282,18 @@ TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
 // minimum.  Writes 0 or 1 direction; used by the wall minimizer, whose capsule
 // restricts each end circle to a half-plane of directions.
 TWA_NOINLINE int trs_local(float2 a, float2 b, float wl, float wh, float R, float2* out) {
-  const float sc = pow2_inverse(R);
+  // lengths to R in [1, 2) and weights to [1, 2), by powers of two: the direction
+  // is the same and the products below stay in range
+  const float sc = pow2_inverse(R), sw = pow2_inverse(fmaxf(wl, wh));
   a = sc * a; b = sc * b; R *= sc;
+  wl *= sw; wh *= sw;
   const float2 wa = wl * a, wb = wh * b;
   const float m11 = fmaf(wa.x, a.x, wb.x * b.x);
   const float m22 = fmaf(wa.y, a.y, wb.y * b.y);
   const float m12 = fmaf(wa.x, a.y, wb.x * b.y);
   const float2 S = wa + wb;
   const float hd = 0.5f * (m11 - m22);
-  const float disc = sqrtf(fmaf(hd, hd, m12 * m12));
+  const float disc = hypotf(hd, m12);
   const float d = 2.f * disc;
   if (!(d > 0.f)) return 0;
   const float q = fabsf(hd) + disc;
