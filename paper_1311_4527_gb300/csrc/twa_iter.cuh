@@ -410,7 +410,8 @@ __device__ __forceinline__ void wall_factor(const D& P, int w, int i, bool vi, i
       const float b = fmaf(0.5f, sqrtf(dot(d, d)), r);
       const float L = fmaxf(fmaxf(maxabs2(c0), maxabs2(c1)), maxabs2(m));
       const float reach = fmaf(1e-5f, L, 1.0001f * b);
-      if (!__any_sync(FULL, vi && !(dist2_point_segment(m, c0, c1) > reach * reach))) return;
+      // (coordinates whose squares' products overflow: no wall is left out)
+      if (!__any_sync(FULL, vi && !(L < 1e9f && dist2_point_segment(m, c0, c1) > reach * reach))) return;
     }
   }
   const size_t idx = ((size_t)w * P.eta + s) * P.p + i;
