@@ -1806,19 +1806,24 @@ cudaError_t launch_pdl(void (*kern)(Args...), unsigned grid, unsigned block, cud
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-// Where a kernel may write a caller's buffer in place: device memory of the
-// current device on a 16-byte boundary, or (host destinations) pinned host
-// memory.  Anything else gives null, and goes by cudaMemcpyAsync, which also
-// finds a bad pointer.
-cudaError_t kernel_pointer(float* z, int on_device, float** dst) {
+// Where a kernel may write a caller's buffer of `bytes` in place: device memory
+// of the current device on a 16-byte boundary, or (host destinations) pinned
+// host memory, at its first and at its last byte.  Anything else gives null,
+// and goes by cudaMemcpyAsync, which also finds a bad pointer and a buffer
+// that ends too early.
+cudaError_t kernel_pointer(float* z, size_t bytes, int on_device, float** dst) {
   *dst = nullptr;
   if (reinterpret_cast<uintptr_t>(z) & 15) return cudaSuccess;
-  cudaPointerAttributes a;
   int dev = 0;
-  cudaError_t e = cudaPointerGetAttributes(&a, z);
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  cudaPointerAttributes a, last;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaPointerGetAttributes(&a, z);
+  if (e == cudaSuccess) e = cudaPointerGetAttributes(&last, reinterpret_cast<char*>(z) + bytes - 1);
   if (e != cudaSuccess) return e;
-  if (on_device ? (a.type == cudaMemoryTypeDevice && a.device == dev) : a.type == cudaMemoryTypeHost)
+  const auto fits = [&](const cudaPointerAttributes& q) {
+    return on_device ? q.type == cudaMemoryTypeDevice && q.device == dev : q.type == cudaMemoryTypeHost;
+  };
+  if (fits(a) && fits(last) && a.devicePointer && static_cast<char*>(last.devicePointer) == static_cast<char*>(a.devicePointer) + bytes - 1)
     *dst = static_cast<float*>(a.devicePointer);
   return cudaSuccess;
 }
@@ -2463,7 +2468,7 @@ plan_status plan_get_trajectory(plan_t h, float* z, int on_device) {
   // 139 KB to pinned memory at the end of a re-planning step of 1,024 agents:
   // 47.2 us the step, now 45.4)
   float* dst = nullptr;
-  CK(kernel_pointer(z, on_device, &dst));
+  CK(kernel_pointer(z, bytes, on_device, &dst));
   if (dst) {
     const unsigned n = (unsigned)(bytes / 16 + 1);
     CK(launch_pdl(copy_kernel, std::min((n + 255) / 256, 4u * 152u), 256u, h->stream, (const float4*)src,
