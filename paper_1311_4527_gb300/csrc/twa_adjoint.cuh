@@ -28,9 +28,9 @@ TWA_DEV void end_vjp(float2 w, float2 vbar, float2 n, float R, float2& wbar, flo
   if (g > 0.f) {
     const float2 t = perp(n);
     const float vn = dot(vbar, n);
-    wbar = vbar - vn * n;
+    wbar = axpy(-vn, n, vbar);
     Rbar += vn;
-    phibar += g * dot(vbar, t) - dot(w, t) * vn;
+    phibar += fmaf(g, dot(vbar, t), -(dot(w, t) * vn));
   } else {
     wbar = vbar;
   }
@@ -42,19 +42,19 @@ TWA_DEV void stationary_vjp(float2 a, float2 b, float wl, float wh, float R, flo
   const float2 t = perp(n);
   const float an = dot(a, n), bn = dot(b, n), at = dot(a, t), bt = dot(b, t);
   const float ga = R - an, gb = R - bn;
-  const float E2 = wl * (at * at + ga * an) + wh * (bt * bt + gb * bn);
-  const float scale = wl * (dot(a, a) + R * R) + wh * (dot(b, b) + R * R);
+  const float E2 = fmaf(wl, fmaf(at, at, ga * an), wh * fmaf(bt, bt, gb * bn));
+  const float scale = fmaf(wl, fmaf(R, R, dot(a, a)), wh * fmaf(R, R, dot(b, b)));
   if (!(E2 > 1e-6f * scale)) return;  // degenerate stationary point: no rotation
   const float k = phibar / E2;
-  abar = abar - (k * wl) * (at * n - ga * t);
-  bbar = bbar - (k * wh) * (bt * n - gb * t);
-  Rbar += k * (wl * at + wh * bt);
+  abar = axpy(-(k * wl), axpy(at, n, -ga * t), abar);
+  bbar = axpy(-(k * wh), axpy(bt, n, -gb * t), bbar);
+  Rbar = fmaf(k, fmaf(wl, at, wh * bt), Rbar);
 }
 
 // n = w / |w|
 TWA_DEV void inner_vjp(float2 w, float2 n, float phibar, float2& wbar) {
   const float nw = hypotf(w.x, w.y);
-  if (nw > 0.f) wbar = wbar + (phibar / nw) * perp(n);
+  if (nw > 0.f) wbar = axpy(phibar / nw, perp(n), wbar);
 }
 
 // <q, n> = R
@@ -63,7 +63,7 @@ TWA_DEV void tangent_vjp(float2 q, float2 n, float phibar, float2& qbar, float& 
   if (fabsf(qt) > 1e-6f * hypotf(q.x, q.y)) {
     const float k = phibar / qt;
     Rbar += k;
-    qbar = qbar - k * n;
+    qbar = axpy(-k, n, qbar);
   }
 }
 
@@ -146,23 +146,23 @@ TWA_DEV void energy_vjp(float2 n_lo, float2 n_hi, float rho, bool pin_lo, bool p
   if (pin_lo) {
     // x_hi = (rho n_hi + 2 c n_lo) / (2 c + rho)
     const float inv = 1.f / (2.f * c + rho);
-    nbl = xbl + (2.f * c * inv) * xbh;
+    nbl = axpy(2.f * c * inv, xbh, xbl);
     nbh = (rho * inv) * xbh;
     cbar = 2.f * rho * inv * inv * dot(xbh, n_lo - n_hi);
     return;
   }
   if (pin_hi) {
     const float inv = 1.f / (2.f * c + rho);
-    nbh = xbh + (2.f * c * inv) * xbl;
+    nbh = axpy(2.f * c * inv, xbl, xbh);
     nbl = (rho * inv) * xbl;
     cbar = 2.f * rho * inv * inv * dot(xbl, n_hi - n_lo);
     return;
   }
   // x_lo = (rho n_lo + 2 c s) / (4 c + rho), x_hi likewise, s = n_lo + n_hi
-  const float inv = 1.f / (4.f * c + rho);
+  const float inv = 1.f / fmaf(4.f, c, rho);
   const float2 sb = (2.f * c * inv) * (xbl + xbh);
-  nbl = (rho * inv) * xbl + sb;
-  nbh = (rho * inv) * xbh + sb;
+  nbl = axpy(rho * inv, xbl, sb);
+  nbh = axpy(rho * inv, xbh, sb);
   cbar = 2.f * rho * inv * inv * dot(xbl - xbh, n_hi - n_lo);
 }
 
@@ -249,7 +249,7 @@ TWA_DEV void velocity_vjp(float2 nl, float2 nh, bool pin_lo, bool pin_hi, float 
   auto proj = [&](float2 g) {  // (I - u u^T) g / L
     if (!(L > 0.f)) return mk(0.f, 0.f);
     const float gu = dot(g, u);
-    return (1.f / L) * (g - gu * u);
+    return (1.f / L) * axpy(-gu, u, g);
   };
   if (pin_lo) {  // x_lo = n_lo, x_hi = n_lo - C u
     const float2 pd = (-C) * proj(xbh);

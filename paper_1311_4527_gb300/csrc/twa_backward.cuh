@@ -159,7 +159,7 @@ __device__ __forceinline__ float2 edge_xbar(const AdjDev& A, bool fixed, int i, 
   if (fixed) { mb = mk(0.f, 0.f); return mb; }
   const size_t node = (size_t)i * (A.eta + 1) + s;
   mb = MBAR ? A.mbar[node] : node_mbar(A, node);
-  return mk(mb.x + A.alpha * ub.x, mb.y + A.alpha * ub.y);
+  return axpy(A.alpha, ub, mb);
 }
 __device__ __forceinline__ float2 edge_ubar(bool fixed, float2 ub, float2 mb, float2 nb) {
   return fixed ? mk(0.f, 0.f) : mk(ub.x + mb.x - nb.x, ub.y + mb.y - nb.y);
