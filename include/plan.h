@@ -276,10 +276,12 @@ plan_status plan_batch_export_state(plan_batch_t batch, int member, float* z, fl
                                     uint8_t* act_wall);
 /* Time the launch-shape candidates (rows per warp of the dense state's
  * collision test {4, 8, 16}, 32 with the gated state; minimizer CTAs per SM
- * {1, 2, 4} x the base grid, dense state; iterations per graph {2, 8}; with
- * the gated state only the last one changes a launch) on this batch, iters_per_candidate iterations each (they are
- * real iterations: results do not depend on the shape), and keep the fastest.
- * choice: 3 host ints receiving the chosen values (may be NULL). */
+ * {1, 2, 4} x the base grid, dense state; iterations per graph {2, 8}) on this
+ * batch, iters_per_candidate iterations each (they are real iterations:
+ * results do not depend on the shape), and keep the fastest.  With the gated
+ * state only the iterations per graph change a launch, and only they are
+ * chosen; the other two stay as they were.
+ * choice: 3 host ints receiving the values kept (may be NULL). */
 plan_status plan_batch_autotune(plan_batch_t batch, int iters_per_candidate, int* choice);
 /* Set the launch shape directly (for example one found by the autotuner on
  * another batch of the same instances): rows_per_warp in {4, 8, 16, 32},

@@ -3914,7 +3914,11 @@ plan_status plan_batch_autotune(plan_batch_t B, int iters_per_candidate, int* ch
         CK(cudaEventSynchronize(e1));
         float ms = 0.f;
         CK(cudaEventElapsedTime(&ms, e0, e1));
-        if (ms / iters < best) { best = ms / iters; bt = tr[a]; bm = mu[c]; bg = gl[g]; }
+        if (ms / iters < best) {
+          best = ms / iters;
+          bg = gl[g];
+          if (B->dense) { bt = tr[a]; bm = mu[c]; }  // (no launch of the gated state depends on them)
+        }
       }
   B->trows = bt; B->prox_mult = bm; B->glen = bg;
   cudaEventDestroy(e0);
