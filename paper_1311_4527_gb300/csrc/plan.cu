@@ -1393,9 +1393,7 @@ size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
 // against 34.2 / 39.8; 4,095, 4 (25,000) 49.2 / 54.8 against 47.5 / 57.5;
 // 6,000, 4 (53,000) 98 / 112 against 81 / 107; 4,095, 16 (124,000) 119 / 124
 // against 66 / 94.
-#ifndef SORT_MIN
-#define SORT_MIN 40000
-#endif
+constexpr size_t SORT_MIN = 40000;
 constexpr int SORT_EVERY = 16;
 
 // plan_set_endpoints checks new endpoints on the device up to this many
@@ -2051,10 +2049,12 @@ plan_status run_iterations(plan_t h, int n) {
 // written by the node pass, the primal part comes from residual_kernel.
 plan_status read_residual(plan_t h, float* out) {
   if (h->k == 0) { *out = INFINITY; return PLAN_OK; }
+  const plan_status st = ensure_sms(h);
+  if (st != PLAN_OK) return st;
   Dev P = h->dev(h->k);
   unsigned* host = nullptr;
   CK(cudaHostGetDevicePointer(reinterpret_cast<void**>(&host), h->h_res, 0));
-  CK(launch_pdl(residual_kernel, 304u, 256u, h->stream, P));
+  CK(launch_pdl(residual_kernel, 2u * (unsigned)h->sms, 256u, h->stream, P));
   CK(launch_pdl(report_kernel, 1u, 1u, h->stream, (const unsigned*)P.res_prev, host));
   CK(cudaStreamSynchronize(h->stream));
   uint32_t bitsv = *h->h_res;
@@ -2470,8 +2470,10 @@ plan_status plan_get_trajectory(plan_t h, float* z, int on_device) {
   float* dst = nullptr;
   CK(kernel_pointer(z, bytes, on_device, &dst));
   if (dst) {
+    const plan_status sst = ensure_sms(h);
+    if (sst != PLAN_OK) return sst;
     const unsigned n = (unsigned)(bytes / 16 + 1);
-    CK(launch_pdl(copy_kernel, std::min((n + 255) / 256, 4u * 152u), 256u, h->stream, (const float4*)src,
+    CK(launch_pdl(copy_kernel, std::min((n + 255) / 256, 4u * (unsigned)h->sms), 256u, h->stream, (const float4*)src,
                   reinterpret_cast<float4*>(dst), bytes));
   } else {
     CK(cudaMemcpyAsync(z, src, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
@@ -2910,9 +2912,9 @@ plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, int phase, cuda
 }
 
 // The same, run: by one CTA for a small problem; else replayed from a graph,
-// kept with the plan (six launches an iteration then, each about 6 us of host time
-// when made one by one, bound the backward pass at any size: 34 us an
-// iteration at p = 64).  Segments differ in their length, in the parity and z
+// kept with the plan (launched one by one, an iteration's three take about 6 us
+// of host time each; with six launches an iteration, in an earlier form, that
+// bound the backward pass at any size: 34 us an iteration at p = 64).  Segments differ in their length, in the parity and z
 // buffer of their first iteration, in where the adjoint of z stands, and
 // iteration 0 has no residual slot before it; the rest is the same for all of
 // them, the iteration number coming from AdjDev::k0.
