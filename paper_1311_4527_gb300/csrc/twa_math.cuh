@@ -726,8 +726,9 @@ TWA_DEV void velocity_prox(float2 n_lo, float2 n_hi, int cl, int ch, float C, fl
   if (cl == 2 || (ch == 0 && cl != 0)) { x_hi = axpy(-C, u, n_lo); return; }
   if (ch == 2 || (cl == 0 && ch != 0)) { x_lo = axpy(C, u, n_hi); return; }
   const float2 m = 0.5f * (n_lo + n_hi);
-  x_lo = axpy(0.5f * C, u, m);
-  x_hi = axpy(-0.5f * C, u, m);
+  const float2 h = (0.5f * C) * u;  // rounded before it is added (the order of operations: see trs_global)
+  x_lo = m + h;
+  x_hi = m - h;
 }
 
 }  // namespace twa
