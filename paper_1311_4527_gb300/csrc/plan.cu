@@ -300,7 +300,8 @@ constexpr int SOLO_WARPS = 16;
 // What of the state a run keeps in shared memory: break-points, segment
 // records, kinetic factors and sums (the sums' atomics and the loads behind
 // them went to L2; at p = 4, eta = 8 an iteration took 5.2 us, with the state
-// here 4.7, with sums in limbs and the second round from the other end 3.7).
+// here 4.7, with sums in limbs and the second round from the other end 3.7; 4.3
+// with the minimizers' present form).
 // The pairs' records, the worklist and the wall factors stay in global memory
 // (bits and worklist here too made no difference).
 struct SoloState {
@@ -812,7 +813,7 @@ __global__ void residual_kernel(Dev P) {
 
 // One word into pinned host memory, in the launch chain (with the residual's own
 // launch in it too, 8 us less a reading than by a copy engine behind it: p = 4,
-// 100 iterations with four readings 450 us, now 418).
+// 100 iterations with four readings 450 us, then 418).
 __global__ void report_kernel(const unsigned* value, unsigned* host) {
   pdl_begin();
   *host = *value;
@@ -1389,10 +1390,10 @@ size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
 // Sorted tiles pay where the segments before the last have at least this many
 // blocks of pairs.  Measured (us per iteration, squares, first 4 / after 200
 // iterations, agents' order against sorted): p = 1,536, eta = 16 (18,000
-// blocks) 26.5 / 25.2 against 27.5 / 29.2; 2,048, 16 (31,000) 39.2 / 37.8
-// against 34.2 / 39.8; 4,095, 4 (25,000) 49.2 / 54.8 against 47.5 / 57.5;
-// 6,000, 4 (53,000) 98 / 112 against 81 / 107; 4,095, 16 (124,000) 119 / 124
-// against 66 / 94.
+// blocks) 20.8 / 22.1 against 27.9 / 30.6; 2,048, 16 (31,000) 30.6 / 32.8
+// against 33.5 / 40.9; 4,095, 4 (25,000) 42.2 / 51.7 against 47.4 / 61.0;
+// 6,000, 4 (53,000) 83 / 103 against 81 / 111; 4,095, 16 (124,000) 93 / 102
+// against 69 / 99.
 constexpr size_t SORT_MIN = 40000;
 constexpr int SORT_EVERY = 16;
 
@@ -1836,14 +1837,14 @@ int list_ctas(const plan_s* h) {
 
 // Problems that one CTA serves better than two launches per iteration over the
 // whole GPU.  Measured (us per iteration, one CTA / two launches), circle
-// swaps of up to 32 agents: eta = 4: 3.5 / 6.5 at p = 4, 4.1 / 6.3 at 16, 5.6
-// / 7.1 at 30, 6.4 / 7.0 at 32; eta = 8: 3.7 / 6.3 at p = 4, 4.6 / 6.8 at 20,
-// 6.0 / 6.9 at 28; eta = 12: 4.6 / 6.2 at p = 8, 5.6 / 6.8 at 16; eta = 16: 5.7
-// / 5.6 at p = 4, 7.5 / 6.8 at 20.  So: tiles and segment warps in at most one
+// swaps of up to 32 agents: eta = 4: 4.1 / 7.1 at p = 4, 4.1 / 7.2 at 16, 6.0
+// / 8.1 at 30, 6.4 / 7.9 at 32; eta = 8: 4.3 / 6.8 at p = 4, 4.4 / 6.8 at 20,
+// 6.5 / 7.8 at 28; eta = 12: 4.8 / 6.6 at p = 8, 5.2 / 6.8 at 16; eta = 16: 6.1
+// / 6.6 at p = 4, 7.1 / 6.5 at 20.  So: tiles and segment warps in at most one
 // and a half rounds of the CTA's warps, and pairs that make at most about two
-// list chunks per warp.  With two groups of 32 (eta = 2: 7.4 / 6.5 at p = 40)
+// list chunks per warp.  With two groups of 32 (eta = 2: 7.3 / 6.4 at p = 40)
 // or walls or speed limits, which keep more pairs active (30 agents with a
-// limit, eta = 4: 11.0 / 9.4), one.
+// limit, eta = 4: 13.4 / 8.5), one.
 bool solo(const plan_s* h) {
   const long long eta = h->vo ? 1 : h->eta;
   return h->cap && !h->profiling && !h->dense() && !h->sorted &&
@@ -1914,8 +1915,8 @@ plan_status enqueue_iteration(plan_t h, cudaStream_t ms, const Tape* tape = null
     // while the GPU holds all blocks at once, four (with four rows of records
     // under way each) where it is the records that take the time.  Measured
     // (us per iteration of standard ADMM, eta = 16, with 4 / 8 / 16 warps):
-    // 48 blocks 13.6 / 11.1 / 10.0, 240 blocks 14.2 / 12.2 / 13.4, 2,176
-    // blocks 28.7 / 29.4 / 47.6.
+    // 48 blocks 10.6 / 10.3 / 9.1, 240 blocks 12.3 / 11.0 / 11.7, 2,176
+    // blocks 25.8 / 26.8 / 45.4.
     const size_t blocks = (size_t)h->eta * h->ntp;
     const int warps = blocks <= (size_t)h->sms ? 16 : blocks <= (size_t)8 * h->sms ? 8 : 4;
     auto kern = warps == 16 ? test_kernel<16, 2> : warps == 8 ? test_kernel<8, 2> : test_kernel<4, 4>;
@@ -1986,8 +1987,8 @@ plan_status run_iteration(plan_t h) {
 
 // Runs of ITERS_PER_LONG_GRAPH, then ITERS_PER_GRAPH iterations replayed
 // from one graph each (even counts, so a run ends at the parity and z buffer
-// it started from): an iteration of the p = 100 circle takes 7.0 us in a graph
-// of 64 and 7.6 launched by itself; 24 of them take 3 us less in graphs of 8.
+// it started from): an iteration of the p = 100 circle takes 8.4 us in a graph
+// of 64 and 8.8 launched by itself; 24 of them take 2 us less in graphs of 8.
 constexpr int ITERS_PER_GRAPH = 8;
 constexpr int ITERS_PER_LONG_GRAPH = 64;
 
@@ -2641,7 +2642,8 @@ __global__ void __launch_bounds__(128) bw_scatter_kernel(AdjDev A) {
 // One adjoint step.  Bound by its chain (entry, records, minimizer adjoint,
 // FP64 atomics).  With the u adjoints' sums and the nodes in launches of their
 // own an iteration of the backward pass took 3.3 us more (p = 64, eta = 8,
-// 128 iterations: 4.05 ms the whole gradient, now 3.63).
+// 128 iterations: 4.05 ms the whole gradient, then 3.63; 3.85 with the
+// minimizers' present form).
 __global__ void __launch_bounds__(128) bw_step_kernel(AdjDev A) {
   pdl_begin();
   A.k += *A.k0;
@@ -2914,10 +2916,11 @@ plan_status enqueue_segment(plan_t h, const AdjLayout& A, int n, int phase, cuda
 // The same, run: by one CTA for a small problem; else replayed from a graph,
 // kept with the plan (launched one by one, an iteration's three take about 6 us
 // of host time each; with six launches an iteration, in an earlier form, that
-// bound the backward pass at any size: 34 us an iteration at p = 64).  Segments differ in their length, in the parity and z
-// buffer of their first iteration, in where the adjoint of z stands, and
-// iteration 0 has no residual slot before it; the rest is the same for all of
-// them, the iteration number coming from AdjDev::k0.
+// bound the backward pass at any size: 34 us an iteration at p = 64).  Segments
+// differ in their length, in the parity and z buffer of their first iteration,
+// in where the adjoint of z stands, and iteration 0 has no residual slot before
+// it; the rest is the same for all of them, the iteration number coming from
+// AdjDev::k0.
 plan_status segment_steps(plan_t h, const AdjLayout& A, int n, int phase) {
   plan_status st = ensure_sms(h);
   if (st != PLAN_OK) return st;

@@ -210,8 +210,8 @@ TWA_DEV float2 in_frame(float n1, float n2, float2 e2) {
 // decides which one wins, and with it the branch that the adjoint
 // differentiates (and, head on, the side on which the pair passes).  A form
 // with a shorter chain (plain square roots, a climb without a bracket, no arc
-// ends) took 4.1 us an iteration for 4.8 of the p = 4 circle's, but parted from
-// these results by up to 2e-4 in 2 % of gradients of circle swaps, and by whole
+// ends) took 4.2 us an iteration for 4.8 of the p = 4 circle's, but parted from
+// these results by up to 2e-4 in 3 % of gradients of circle swaps, and by whole
 // detours in one pass of 300.
 TWA_NOINLINE int trs_global(float2 a, float2 b, float wl, float wh, float R,
                                        float2* out) {
